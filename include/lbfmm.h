@@ -90,7 +90,8 @@ typedef struct lbf_options {
                              per-kernel tracing skips graph-replayed kernels */
     int fmm64;            /* arithmetic of the accurate (double) FMM operator: 0 double,
                              1 double-float (pairs of floats, ~48-bit significands; this
-                             GPU issues float 64 times faster than double) */
+                             GPU issues float 64 times faster than double).  Stored leaf
+                             rows are double in both */
     int schur;            /* how the preconditioner applies S^-1 (S = D - F E, Sec. 5, Eq.
                              matrix_eqns_c): LBF_SCHUR_AUTO, LBF_SCHUR_GJ or LBF_SCHUR_LU */
     int p2p_warps;        /* near-field tile: warps (leaves) per block of the leaf pass,
@@ -139,7 +140,10 @@ const char *lbf_status_string(int status);
 /* Bytes of device workspace a plan over these islands needs (synchronous, host
  * only).  The quadtree part is an estimate from N and leaf_size unless
  * opt->box_capacity is set; lbf_plan_create reports the exact need if the
- * estimate was short. */
+ * estimate was short.  The last part holds the accurate forward operator's leaf
+ * rows (near field and local evaluation, 8 bytes an entry, up to 64 GB): a plan
+ * given a workspace without it, or whose tree needs more, forms them on the fly
+ * in every application. */
 int lbf_workspace_size(int M, const int64_t *island_ptr /* host, M+1 */, const lbf_options *opt,
                        size_t *bytes /* host out */);
 

@@ -502,6 +502,9 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
     // the float passes form coordinates across large level gaps in double-float
     const cx<df64> *udf = sizeof(R) == sizeof(float) ? (const cx<df64> *)pl->udf : nullptr;
     const bool dbl = sizeof(R) == sizeof(double);
+    // the accurate forward rows: near field, small W and X boxes and L2P stored (lbf_rows.cu)
+    const bool stored = sizeof(R) == sizeof(double) && MODE == fmm::kLeafForward && pl->rows;
+    const int xskip = stored ? pl->rows_thr : -1;
     const int kid_up = dbl ? LBF_KERNEL_UP : LBF_KERNEL_UP32;
     const int kid_down = dbl ? LBF_KERNEL_DOWN : LBF_KERNEL_DOWN32;
     const int kid_leaf = dbl ? LBF_KERNEL_LEAF : LBF_KERNEL_LEAF32;
@@ -527,14 +530,14 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
             LBF_LAUNCH_P(kid_down, fmm::k_down<R>, lbf_grid(pl, lbf_cdiv(T.nbox, wpb)), 32 * wpb,
                          smem, s, (int64_t)0, T.nbox, T.level, T.ix, T.iy, T.parent, T.vlist, T.nv,
                          T.xlist, T.nx, T.begin, T.end, g, P, binom, tpow, dsh, pl->xi, uloc, q, mp,
-                         loc, gate, 0, (unsigned *)nullptr, pl->dev_status, udf, pl->slab);
+                         loc, gate, 0, (unsigned *)nullptr, pl->dev_status, udf, xskip, pl->slab);
             LBF_CHECK_LAUNCH();
         } else if (pl->pull) {
             const int64_t grid = std::min<int64_t>(lbf_cdiv(T.nbox, wpb), 4 * (int64_t)std::max(pl->nsm, 1));
             LBF_LAUNCH_P(kid_down, fmm::k_down<R>, lbf_grid(pl, grid), 32 * wpb, smem, s, (int64_t)0,
                          T.nbox, T.level, T.ix, T.iy, T.parent, T.vlist, T.nv, T.xlist, T.nx, T.begin,
                          T.end, g, P, binom, tpow, dsh, pl->xi, uloc, q, mp, loc, gate, 2, pl->pull,
-                         pl->dev_status, udf, pl->slab);
+                         pl->dev_status, udf, xskip, pl->slab);
             LBF_CHECK_LAUNCH();
         } else {
             for (int l = 0; l < T.nlev; l++) {
@@ -543,11 +546,12 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
                 LBF_LAUNCH_P(kid_down, fmm::k_down<R>, lbf_grid(pl, lbf_cdiv(le - ls, wpb)), 32 * wpb,
                              smem, s, ls, le, T.level, T.ix, T.iy, T.parent, T.vlist, T.nv, T.xlist,
                              T.nx, T.begin, T.end, g, P, binom, tpow, dsh, pl->xi, uloc, q, mp, loc,
-                             gate, 1, (unsigned *)nullptr, pl->dev_status, udf, pl->slab);
+                             gate, 1, (unsigned *)nullptr, pl->dev_status, udf, xskip, pl->slab);
                 LBF_CHECK_LAUNCH();
             }
         }
     }
+    if (stored) return lbf_rows_apply(pl, sigma, v, gate, s);
     // Several right-hand sides in lockstep: the double forward rows' near field in one pass
     // that forms each pair's geometry once (k_near_multi), the leaf kernel adding it.  (The
     // float operator keeps a leaf pass per right-hand side: its pairs are cheap on the

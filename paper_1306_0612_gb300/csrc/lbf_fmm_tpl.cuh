@@ -421,7 +421,7 @@ k_down(int64_t ls, int64_t le, const int32_t *__restrict__ level,
                        const cx<R> *__restrict__ uloc, const cx<R> *__restrict__ q,
                        const cx<R> *__restrict__ mp, cx<R> *__restrict__ loc, const int *gate,
                        int with_l2l, unsigned *pull, int *status, const cx<df64> *__restrict__ udf,
-                       int64_t slab)
+                       int xskip, int64_t slab)
 {
     lbf_rhs(slab, q, mp, loc, gate, pull);
     if (gate_closed(gate)) return;
@@ -644,8 +644,9 @@ k_down(int64_t ls, int64_t le, const int32_t *__restrict__ level,
         have_c = true;
     };
     if constexpr (!kLocal<R>) need_centre();
-    // the X list's box records (at most 16), a lane per box, then broadcast
-    const int nxb = nx[b];
+    // the X list's box records (at most 16), a lane per box, then broadcast (left out for
+    // boxes of at most xskip nodes, whose X lists are near columns of the stored rows)
+    const int nxb = en[b] - bg[b] <= xskip ? 0 : nx[b];
     int xr_s = 0, xr_l = 0, xr_x = 0, xr_y = 0, xr_b = 0, xr_e = 0;
     if (lane < nxb) {
         xr_s = xlist[b * 16 + lane];
@@ -1297,7 +1298,7 @@ __global__ void k_leaf(int64_t nleaf, const int32_t *__restrict__ leaves,
 // term of the forward rows, 2 (1/2pi) (-Im Phi), to v (the leaf kernel wrote the rest).
 // A parallel alternative to shifting the expansions down the tree (L2L): no serial
 // chain, and the nodes of a leaf share their ancestors' coefficients in L1.
-__global__ void k_l2p_walk(int64_t N, int P, const int32_t *__restrict__ leaf_of,
+static __global__ void k_l2p_walk(int64_t N, int P, const int32_t *__restrict__ leaf_of,
                            const int32_t *__restrict__ level, const int32_t *__restrict__ ix,
                            const int32_t *__restrict__ iy, const int32_t *__restrict__ anc,
                            const float2 *__restrict__ u32, const cx<float> *__restrict__ loc,

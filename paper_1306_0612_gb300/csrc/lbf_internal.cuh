@@ -114,6 +114,12 @@ struct Border {
     double *sums = nullptr;          // Y, Lam
 };
 
+// A block of stored leaf rows (lbf_rows.cu): nrow rows of leaf `box` from node row0 on,
+// nchunk chunks of eight near columns from chunk `chunk` on, tiles from `tile` on
+struct __align__(16) RowItem {
+    int32_t box, row0, nrow, tile, chunk, nchunk, pad[2];
+};
+
 struct GmresState;  // device-side scalars (lbf_krylov.cu)
 
 struct lbf_plan {
@@ -168,6 +174,14 @@ struct lbf_plan {
     // expansion were written (nbox each)
     uint32_t *pull = nullptr;
     int nsm = 0;                // streaming multiprocessors of the plan's device
+    // stored leaf rows of the accurate forward operator (lbf_rows.cu; rows null: not stored)
+    double *rows = nullptr;
+    int32_t *rows_cols = nullptr;
+    RowItem *rows_items = nullptr;
+    int64_t rows_tiles = 0, rows_chunks = 0, rows_items_cap = 0;  // capacities
+    int64_t rows_nitem = 0;
+    int rows_split = 0;         // a small system: four warps share a block's columns
+    int rows_thr = 0;           // boxes of at most this many nodes enter W and X lists as pairs
     double *v = nullptr;        // (I + K - I) sigma = K sigma, doubled scaling
     double *bsig = nullptr;     // scalar beta . sigma
     double *red = nullptr;      // reduction partials
@@ -318,6 +332,10 @@ int lbf_cauchy_deriv(lbf_plan *pl, const double *x, bool weighted, double2 *out,
 // box (P2M + M2M); also writes q = (x, 0) and *bsig = sum_j x_j
 int lbf_multipoles(lbf_plan *pl, const double *x, int P, double2 *mp, const int *gate,
                    cudaStream_t s);
+// ---- stored leaf rows (lbf_rows.cu) ----------------------------------------------
+void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap);
+int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len);
+int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate, cudaStream_t s);
 int lbf_evaluate_impl(lbf_plan *pl, const double *sigma_sorted, const double *a, int64_t T,
                       const double *t, double *u, cudaStream_t s);
 int lbf_green_sum_impl(int64_t T, const double *t, int64_t S, const double *p,

@@ -218,6 +218,16 @@ class Plan:
             self.handle = None
 
 
+def _plan_workspace(nbytes, dev):
+    """(workspace, error): nbytes on dev, or what is free there with the allocator's error (a
+    plan without room for its stored rows forms them on the fly)."""
+    try:
+        return torch.empty(nbytes, dtype=torch.uint8, device=dev), None
+    except torch.cuda.OutOfMemoryError as e:
+        free = torch.cuda.mem_get_info(dev)[0]
+        return torch.empty(min(nbytes, int(0.95 * free)), dtype=torch.uint8, device=dev), e
+
+
 def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream, device):
     lib = load()
     opt = opt or lbf_default_options()
@@ -230,7 +240,8 @@ def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream,
     name = "lbf_plan_create_planar" if planar else "lbf_plan_create"
     for _ in range(6):
         nbytes = lbf_workspace_size(ptr, opt)
-        ws = torch.empty(nbytes, dtype=torch.uint8, device=dev)
+        ws, short = _plan_workspace(nbytes, dev)
+        nbytes = ws.numel()
         h = C.c_void_p()
         need = C.c_int64(0)
         geo = (_dptr(a, k * N, "nodes"), _dptr(da, k * N, "first derivatives"),
@@ -242,6 +253,8 @@ def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream,
         else:
             rc = lib.lbf_plan_create(C.byref(h), M, ptr.ctypes.data_as(_P), *geo,
                                      None if rot is None else rot.ctypes.data_as(_P), *tail)
+        if rc == LBF_EWORKSPACE and short is not None:
+            raise short
         if rc == LBF_EWORKSPACE and need.value > opt.box_capacity:
             opt = lbf_options.from_buffer_copy(opt)
             opt.box_capacity = int(need.value)

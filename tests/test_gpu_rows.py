@@ -1,0 +1,70 @@
+"""Stored leaf rows of the accurate forward operator (csrc/lbf_rows.cu): plans with and
+without room for them, against the oracle, where the tiles' edges fall differently."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as wl
+from gpu_util import L, dev, host, plan_for, rel_l2, zeros
+
+pytestmark = pytest.mark.gpu
+# the operator's own bound at these orders (p >= 24: truncation below 2e-12; rounding far less)
+TOL = 1e-10
+
+
+def short_plan(monkeypatch, g, **opt):
+    """The same plan in a workspace without room for the rows (they come last in it)."""
+    full = L.lbf_workspace_size
+    with monkeypatch.context() as m:
+        m.setattr(L, "lbf_workspace_size", lambda ptr, o: full(ptr, o) - 1024)
+        return plan_for(g, **opt)
+
+
+@pytest.mark.parametrize("fmm64", [0, 1])
+@pytest.mark.parametrize("leaf,p,depth", [
+    (1, 24, 30),     # one row a leaf, many chunks
+    (5, 26, 30),     # two row groups, the second with one row
+    (33, 35, 30),    # a leaf of more than 32 rows: two blocks where whole leaves go to a warp
+    (48, 63, 30),    # the most local columns
+    (1024, 26, 30),  # one or few leaves: every node a column of every row
+    (4, 26, 4),      # depth-capped leaves
+])
+def test_rows_against_the_oracle_and_the_unstored_rows(monkeypatch, leaf, p, depth, fmm64):
+    g = wl.star_caps(11, 5, np.array([64, 37, 201, 90, 333]))
+    v = np.random.default_rng(leaf).standard_normal(g.N + g.M)
+    ref = oracle.apply(g, v, 0)
+    opt = dict(leaf_size=leaf, p=p, max_depth=depth, fmm64=fmm64)
+    out = []
+    for plan in (plan_for(g, **opt), short_plan(monkeypatch, g, **opt)):
+        o = zeros(g.N + g.M)
+        L.lbf_apply(plan, L.LBF_OP_FULL, dev(v), o)
+        assert L.lbf_sync_status(plan) == L.LBF_OK
+        assert rel_l2(host(o), ref) < TOL
+        out.append(o)
+    assert rel_l2(host(out[0]), host(out[1])) < TOL
+
+
+def test_rows_of_whole_leaves_and_large_w_boxes():
+    """Leaves enough for a warp each (not shared by a thread block), with W boxes of more
+    than 4 (p + 1) nodes, whose M2P rows are columns: sampled rows against the oracle."""
+    g = wl.star_caps(3, 64, np.where(np.arange(64) % 8 == 0, 4096, 300))
+    plan = plan_for(g, leaf_size=8, p=26)
+    assert L.lbf_plan_info(plan)["nleaf"] > 4864
+    v = np.random.default_rng(1).standard_normal(g.N + g.M)
+    o = zeros(g.N + g.M)
+    L.lbf_apply(plan, L.LBF_OP_FULL, dev(v), o)
+    rows = np.random.default_rng(2).choice(g.N, 400, replace=False)
+    assert rel_l2(host(o)[rows], oracle.apply_rows(g, v, rows, 0)) < TOL
+
+
+def test_rows_repeat_and_zero_weights():
+    """Two applications agree bit for bit; a zero density gives zero rows."""
+    g = wl.star_caps(5, 7, 129)
+    plan = plan_for(g)
+    v = dev(np.random.default_rng(3).standard_normal(g.N))
+    a, b, z = zeros(g.N), zeros(g.N), torch.full((g.N,), 1.0, dtype=torch.float64, device=v.device)
+    L.lbf_apply(plan, L.LBF_OP_K_ONLY, v, a)
+    L.lbf_apply(plan, L.LBF_OP_K_ONLY, v, b)
+    L.lbf_apply(plan, L.LBF_OP_K_ONLY, zeros(g.N), z)
+    assert torch.equal(a, b) and torch.count_nonzero(z) == 0
