@@ -629,7 +629,7 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
     rc = lbf_geometry_gather(pl, s, tt.xi_o, tt.w_o, tt.d_o, tt.b_o);
     if (rc) return fail(rc);
     if ((rc = lbf_fmm_prepare(pl, s))) return fail(rc);
-    if ((rc = lbf_rows_build(pl, s, tt.iscr, tt.iscr_len))) return fail(rc);
+    if ((rc = lbf_rows_build(pl, s, tt.iscr, tt.iscr_len, tt.perm_alt))) return fail(rc);
     lbf_prof_mark(LBF_STAGE_GEOMETRY, 0, s);
     if (opt->border) {
         SortBufs sb{tt.keys, tt.keys_alt, tt.perm_alt};

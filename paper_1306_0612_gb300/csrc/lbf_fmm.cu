@@ -503,7 +503,9 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
     const cx<df64> *udf = sizeof(R) == sizeof(float) ? (const cx<df64> *)pl->udf : nullptr;
     const bool dbl = sizeof(R) == sizeof(double);
     // the accurate forward rows: near field, small W and X boxes and L2P stored (lbf_rows.cu)
-    const bool stored = sizeof(R) == sizeof(double) && MODE == fmm::kLeafForward && pl->rows;
+    const bool stored = sizeof(R) == sizeof(double) && pl->rows &&
+                        (MODE == fmm::kLeafForward ||
+                         (MODE == fmm::kLeafTranspose && pl->rows_rptr && pl->nrhs == 1));
     const int xskip = stored ? pl->rows_thr : -1;
     const int kid_up = dbl ? LBF_KERNEL_UP : LBF_KERNEL_UP32;
     const int kid_down = dbl ? LBF_KERNEL_DOWN : LBF_KERNEL_DOWN32;
@@ -551,7 +553,9 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
             }
         }
     }
-    if (stored) return lbf_rows_apply(pl, sigma, v, gate, s);
+    if (stored)
+        return MODE == fmm::kLeafForward ? lbf_rows_apply(pl, sigma, v, gate, s)
+                                         : lbf_rows_apply_t(pl, sigma, v, gate, s);
     // Several right-hand sides in lockstep: the double forward rows' near field in one pass
     // that forms each pair's geometry once (k_near_multi), the leaf kernel adding it.  (The
     // float operator keeps a leaf pass per right-hand side: its pairs are cheap on the

@@ -115,9 +115,10 @@ struct Border {
 };
 
 // A block of stored leaf rows (lbf_rows.cu): nrow rows of leaf `box` from node row0 on,
-// nchunk chunks of eight near columns from chunk `chunk` on, tiles from `tile` on
+// nchunk chunks of eight near columns from chunk `chunk` on (the first ncol columns are
+// nodes), tiles from `tile` on; leaf: the box's index among the leaves
 struct __align__(16) RowItem {
-    int32_t box, row0, nrow, tile, chunk, nchunk, pad[2];
+    int32_t box, row0, nrow, tile, chunk, nchunk, ncol, leaf;
 };
 
 struct GmresState;  // device-side scalars (lbf_krylov.cu)
@@ -179,7 +180,11 @@ struct lbf_plan {
     int32_t *rows_cols = nullptr;
     RowItem *rows_items = nullptr;
     int64_t rows_tiles = 0, rows_chunks = 0, rows_items_cap = 0;  // capacities
-    int64_t rows_nitem = 0;
+    int64_t rows_nitem = 0, rows_rev_cap = 0;
+    // transposed rows: row blocks of each leaf, where its nodes stand in other leaves'
+    // columns (rptr null: not stored), a value per column
+    int32_t *rows_block0 = nullptr, *rows_rptr = nullptr, *rows_rbase = nullptr;
+    double *rows_z = nullptr;
     int rows_split = 0;         // a small system: four warps share a block's columns
     int rows_thr = 0;           // boxes of at most this many nodes enter W and X lists as pairs
     double *v = nullptr;        // (I + K - I) sigma = K sigma, doubled scaling
@@ -334,7 +339,9 @@ int lbf_multipoles(lbf_plan *pl, const double *x, int P, double2 *mp, const int 
                    cudaStream_t s);
 // ---- stored leaf rows (lbf_rows.cu) ----------------------------------------------
 void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap);
-int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len);
+int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len,
+                   int32_t *leaf);
+int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate, cudaStream_t s);
 int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate, cudaStream_t s);
 int lbf_evaluate_impl(lbf_plan *pl, const double *sigma_sorted, const double *a, int64_t T,
                       const double *t, double *u, cudaStream_t s);

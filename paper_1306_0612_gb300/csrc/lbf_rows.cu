@@ -33,6 +33,12 @@
 // that halves the groups at each step adds them in 7 additions for 8 groups (lanes on
 // rows alone would leave 19 % of the lanes idle at 26 nodes a leaf, lanes on columns
 // alone would add 31 shuffled sums to 4 x 26 multiply-adds).
+//
+// The transposed rows (K^T tau)_i read the same tiles: near pairs are symmetric (b's columns
+// hold leaf t's nodes exactly when t's hold b's), so each leaf forms z = G_b^T tau_b over its
+// columns (k_rows_t) and a node adds its entry of every z it is a column of, in a fixed
+// order (k_rows_t_out), from a list per leaf of where its nodes begin in the others' columns.
+// The far field is Im(w_i Phi(xi_i)): the same local and M2P columns with two sums a row.
 #include <algorithm>
 
 #include "lbf_fmm_tpl.cuh"
@@ -55,6 +61,7 @@ constexpr int64_t kSmallLeaves = 4864;
 struct TreeLists {
     const int32_t *level, *ix, *iy, *parent, *begin, *end, *uptr, *uidx, *wptr, *widx, *xlist, *nx;
 };
+// (f(first node, end) in a fixed order)
 template <class F> __device__ __forceinline__ void for_ranges(const TreeLists &T, int b, int thr, F f)
 {
     for (int q = T.uptr[b]; q < T.uptr[b + 1]; q++) f(T.begin[T.uidx[q]], T.end[T.uidx[q]]);
@@ -114,15 +121,16 @@ __global__ void k_rows_count(int64_t nleaf, const int32_t *__restrict__ leaves, 
 
 // the row blocks of each leaf, a thread per leaf (groups spread evenly over its blocks)
 __global__ void k_rows_items(int64_t nleaf, const int32_t *__restrict__ leaves, TreeLists T,
-                             int lchunks, int groups, const int32_t *__restrict__ chunk0,
+                             int thr, int lchunks, int groups, const int32_t *__restrict__ chunk0,
                              const int32_t *__restrict__ block0, const int32_t *__restrict__ tile0,
-                             RowItem *__restrict__ items)
+                             RowItem *__restrict__ items, int32_t *__restrict__ leaf)
 {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= nleaf) return;
     const int b = leaves[t];
     const int n = T.end[b] - T.begin[b], g = (n + 3) / 4, nb = (g + groups - 1) / groups;
     const int ch = chunk0[t + 1] - chunk0[t];
+    for (int i = T.begin[b]; i < T.end[b]; i++) leaf[i] = (int32_t)t;
     for (int k = 0; k < nb; k++) {
         const int g0 = (int)((long long)g * k / nb), g1 = (int)((long long)g * (k + 1) / nb);
         RowItem it;
@@ -132,7 +140,8 @@ __global__ void k_rows_items(int64_t nleaf, const int32_t *__restrict__ leaves, 
         it.tile = tile0[t] + g0 * (ch + lchunks);
         it.chunk = chunk0[t];
         it.nchunk = ch;
-        it.pad[0] = it.pad[1] = 0;
+        it.ncol = (int)near_nodes(T, b, thr);
+        it.leaf = (int32_t)t;
         items[block0[t] + k] = it;
     }
 }
@@ -162,6 +171,35 @@ __global__ void k_rows_cols(int64_t nleaf, const int32_t *__restrict__ leaves, T
     if (m + lane < (m + 7) / 8 * 8) c[m + lane] = T.begin[b];
 }
 
+// For leaf t, the leaves whose columns hold its nodes, in the order of its own columns: their
+// number (base null) or where t's first node stands among all the columns.
+__global__ void k_rows_rev(int64_t nleaf, const int32_t *__restrict__ leaves, TreeLists T, int thr,
+                           const int32_t *__restrict__ chunk0, const int32_t *__restrict__ leaf,
+                           int32_t *__restrict__ count, const int32_t *__restrict__ ptr,
+                           int32_t *__restrict__ base)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= nleaf) return;
+    const int first = T.begin[leaves[t]];
+    int n = 0;
+    for_ranges(T, leaves[t], thr, [&](int s, int e) {
+        for (int j = s; j < e;) {
+            const int tb = leaf[j], b = leaves[tb];
+            if (base) {
+                int off = 0, at = 0;
+                for_ranges(T, b, thr, [&](int s2, int e2) {
+                    if (first >= s2 && first < e2) at = off + first - s2;
+                    off += e2 - s2;
+                });
+                base[ptr[t] + n] = chunk0[tb] * 8 + at;
+            }
+            n++;
+            j = T.end[b];
+        }
+    });
+    if (!base) count[t] = n;
+}
+
 // the entries, a warp per row block
 __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, TreeLists T, int thr,
                             BoxGeo g, int P, int lchunks, const int32_t *__restrict__ cols,
@@ -173,7 +211,7 @@ __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, Tr
     if (k >= nitem) return;
     const RowItem it = items[k];
     const int ng = (it.nrow + 3) / 4;
-    const int ncol = (int)near_nodes(T, it.box, thr);
+    const int ncol = it.ncol;
     const int nend = ncol + 2 * P * big_boxes(T, it.box, thr);
     double *t = rows + (int64_t)it.tile * 32 + lane;
     for (int c = 0; c < it.nchunk; c++) {
@@ -339,7 +377,7 @@ k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__r
     const int64_t k = split ? (int64_t)blockIdx.x : blockIdx.x * (int64_t)(blockDim.x >> 5) + wid;
     if (k >= nitem) return;
     const int4 i0 = ((const int4 *)items)[2 * k], i1 = ((const int4 *)items)[2 * k + 1];
-    const RowItem it{i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, {0, 0}};
+    const RowItem it{i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
     const int nk = it.nchunk + lchunks;
     const int k0 = split ? nk * wid / 4 : 0, k1 = split ? nk * (wid + 1) / 4 : nk;
     int row;
@@ -364,6 +402,123 @@ k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__r
         s = part[0][lane] + part[1][lane] + part[2][lane] + part[3][lane];
     }
     if (row < it.nrow) v[it.row0 + row] = s + 2.0 * *bsig;
+}
+
+// z = G^T tau over each leaf's columns, a warp per leaf, or (split) the four warps of a
+// thread block, a quarter of the columns each.  Four chunks at a time: a lane sums its rows'
+// parts of a column of each, and the four lanes of a column are added in 3 additions.
+__global__ void __launch_bounds__(128)
+k_rows_t(int64_t nleaf, const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
+         const double *__restrict__ rows, const double *__restrict__ tau, double *__restrict__ z,
+         const int *gate, int split)
+{
+    if (fmm::gate_closed(gate)) return;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t t = split ? (int64_t)blockIdx.x : blockIdx.x * (int64_t)(blockDim.x >> 5) + wid;
+    if (t >= nleaf) return;
+    for (int k = block0[t]; k < block0[t + 1]; k++) {
+        const RowItem it = items[k];
+        const int ng = (it.nrow + 3) / 4, nk = (it.ncol + 7) / 8;
+        const int k0 = split ? nk * wid / 4 : 0, k1 = split ? nk * (wid + 1) / 4 : nk;
+        double tv[kGroups];
+#pragma unroll
+        for (int q = 0; q < kGroups; q++) {
+            const int r = 4 * q + (lane >> 3);
+            tv[q] = r < it.nrow ? tau[it.row0 + r] : 0.0;
+        }
+        const double *tl = rows + ((int64_t)it.tile + (int64_t)k0 * ng) * 32 + lane;
+        for (int c = k0; c < k1; c += 4, tl += 128 * ng) {
+            double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+            for (int q = 0; q < kGroups; q++)
+                if (q < ng) {
+#pragma unroll
+                    for (int h = 0; h < 4; h++)
+                        if (c + h < k1) a[h] = fma(tl[32 * (h * ng + q)], tv[q], a[h]);
+                }
+            const bool u = (lane & 16) != 0, w = (lane & 8) != 0;
+            const double b0 = (u ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, u ? a[0] : a[2], 16);
+            const double b1 = (u ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, u ? a[1] : a[3], 16);
+            const double s = (w ? b1 : b0) + __shfl_xor_sync(0xffffffffu, w ? b0 : b1, 8);
+            const int h = (u ? 2 : 0) + (w ? 1 : 0);  // the chunk this lane's sum belongs to
+            if (c + h < k1) {
+                double *o = z + ((int64_t)it.chunk + c + h) * 8 + (lane & 7);
+                *o = k == block0[t] ? s : *o + s;
+            }
+        }
+    }
+}
+
+// v_i = Im(w_i Phi_far)/pi + 2 beta_i sum tau + the node's entries of the z vectors, a warp
+// per row block
+template <typename R>
+__global__ void __launch_bounds__(128)
+k_rows_t_out(int64_t nitem, const RowItem *__restrict__ items, const double *__restrict__ rows,
+             const int32_t *__restrict__ cols, const double *__restrict__ z,
+             const int32_t *__restrict__ rptr, const int32_t *__restrict__ rbase,
+             const int32_t *__restrict__ begin, const cx<R> *__restrict__ loc,
+             const cx<R> *__restrict__ mp, int P, int lchunks, const double2 *__restrict__ w,
+             const double *__restrict__ beta, const double *__restrict__ bsig,
+             double *__restrict__ v, const int *gate)
+{
+    if (fmm::gate_closed(gate)) return;
+    const int64_t k = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (k >= nitem) return;
+    const RowItem it = items[k];
+    const int ng = (it.nrow + 3) / 4;
+    double ai[kGroups], ar[kGroups];
+#pragma unroll
+    for (int q = 0; q < kGroups; q++) ai[q] = ar[q] = 0.0;
+    const int c0 = it.ncol >> 3, near = 8 * it.nchunk, par = lane & 1;
+    const double *t = rows + ((int64_t)it.tile + (int64_t)c0 * ng) * 32 + lane;
+    const int64_t lb = (int64_t)it.box * 2 * P;
+    for (int c = c0; c < it.nchunk + lchunks; c++, t += 32 * ng) {
+        // the real of this lane's column, and the other real of its coefficient: columns
+        // 2 l and 2 l + 1 hold -(1/pi) (Im, Re) of a power, to be met by (x, y) for the
+        // imaginary part of the sum and by (-y, x) for the real part
+        const int m = 8 * c + (lane & 7);
+        double si = 0.0, sr = 0.0;
+        if (m < near) {
+            const int j = cols[(int64_t)it.chunk * 8 + m];
+            if (m >= it.ncol && j < 0) {
+                const int e = -1 - j, odd = e & 1;
+                si = local_real(mp, e);
+                sr = odd ? local_real(mp, e - 1) : -local_real(mp, e + 1);
+            }
+        } else if (m < near + 2 * P) {
+            const int64_t e = lb + m - near;
+            si = local_real(loc, e);
+            sr = par ? local_real(loc, e - 1) : -local_real(loc, e + 1);
+        }
+#pragma unroll
+        for (int q = 0; q < kGroups; q++)
+            if (q < ng) {
+                const double e = t[32 * q];
+                ai[q] = fma(e, si, ai[q]);
+                ar[q] = fma(e, sr, ar[q]);
+            }
+    }
+    int grp = 0;
+#pragma unroll
+    for (int bit = 4; bit > 0; bit >>= 1) {
+        const bool up = (lane & bit) != 0;
+#pragma unroll
+        for (int q = 0; q < bit; q++) {
+            const double ki = up ? ai[q + bit] : ai[q], sdi = up ? ai[q] : ai[q + bit];
+            const double kr = up ? ar[q + bit] : ar[q], sdr = up ? ar[q] : ar[q + bit];
+            ai[q] = ki + __shfl_xor_sync(0xffffffffu, sdi, bit);
+            ar[q] = kr + __shfl_xor_sync(0xffffffffu, sdr, bit);
+        }
+        grp += up ? bit : 0;
+    }
+    const int row = 4 * grp + (lane >> 3);
+    if (row >= it.nrow) return;
+    const int i = it.row0 + row, at = i - begin[it.box];
+    double s = 0.0;
+    for (int e = rptr[it.leaf]; e < rptr[it.leaf + 1]; e++) s += z[(int64_t)rbase[e] + at];
+    const double2 ww = w[i];
+    v[i] = s - fma(ww.x, ai[0], ww.y * ar[0]) + 2.0 * (beta[i] * *bsig);
 }
 
 TreeLists lists_of(const Tree &T)
@@ -392,7 +547,7 @@ void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap)
     const int64_t cols = (N <= 1 << 18 ? 10 : 4) * (int64_t)o.leaf_size + 2 * (o.p + 1) + 48;
     // a chunk of columns serves every row group of its leaf (leaves hold about half of leaf_size)
     const int64_t tiles = (N * cols) / 32 + 4096;
-    const int64_t chunks = tiles / std::max(1, o.leaf_size / 16) + 4096;
+    const int64_t chunks = tiles / std::max(1, o.leaf_size / 10) + 4096;
     if (tiles > (int64_t)250000000) return;
     Arena &A = pl->arena;
     const size_t off = A.off;
@@ -400,8 +555,13 @@ void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap)
     pl->rows_tiles = tiles;
     pl->rows_chunks = chunks;
     pl->rows_items_cap = N / 4 + cap;
+    pl->rows_rev_cap = 12 * cap;
     pl->rows_items = A.get<RowItem>(pl->rows_items_cap);
     pl->rows_cols = A.get<int32_t>(8 * chunks);
+    pl->rows_block0 = A.get<int32_t>(cap + 1);
+    pl->rows_rptr = A.get<int32_t>(cap + 1);
+    pl->rows_rbase = A.get<int32_t>(pl->rows_rev_cap);
+    pl->rows_z = A.get<double>(8 * chunks);
     pl->rows = A.get<double>(32 * tiles);
     if (A.overflow && !full) {  // a workspace of the size without rows
         A.off = off;
@@ -410,7 +570,9 @@ void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap)
     }
 }
 
-int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len)
+// leaf: room for the leaf of each node (plan time)
+int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len,
+                   int32_t *leaf)
 {
     if (!pl->rows) return LBF_OK;
     Tree &T = pl->tree;
@@ -423,15 +585,17 @@ int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scrat
     pl->rows_split = small ? 1 : 0;
     const int groups = small ? kGroupsSmall : kGroups;
     const TreeLists tl = lists_of(T);
-    int32_t *chunks = scratch + 8, *blocks = chunks + nl + 1, *tiles = blocks + nl + 1;
+    int32_t *chunks = scratch + 8, *tiles = chunks + nl + 1, *blocks = pl->rows_block0;
     int32_t *sc = tiles + nl + 1;
-    const int64_t sc_len = scratch_len - 8 - 3 * (nl + 1);
+    const int64_t sc_len = scratch_len - 8 - 2 * (nl + 1);
     unsigned long long *total = (unsigned long long *)scratch;
     if (sc_len < nl / 1024 + 64 || T.nbox * 2 * P >= INT32_MAX) {
         pl->rows = nullptr;
         return LBF_OK;
     }
-    LBF_CUDA(cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (8 + 3 * (nl + 1)), s));
+    LBF_CUDA(cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (8 + 2 * (nl + 1)), s));
+    LBF_CUDA(cudaMemsetAsync(blocks, 0, sizeof(int32_t) * (nl + 1), s));
+    LBF_CUDA(cudaMemsetAsync(pl->rows_rptr, 0, sizeof(int32_t) * (nl + 1), s));
     LBF_LAUNCH(k_rows_count, lbf_cdiv(nl, 128), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, P,
                lch, groups, chunks, blocks, tiles, total);
     LBF_CHECK_LAUNCH();
@@ -450,12 +614,26 @@ int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scrat
     if ((rc = lbf_scan_i32(chunks, chunks, nl + 1, sc, sc_len, s))) return rc;
     if ((rc = lbf_scan_i32(tiles, tiles, nl + 1, sc, sc_len, s))) return rc;
     pl->rows_nitem = nitem;
-    LBF_LAUNCH(k_rows_items, lbf_cdiv(nl, 128), 128, 0, s, nl, T.leaves, tl, lch, groups, chunks,
-               blocks, tiles, pl->rows_items);
+    LBF_LAUNCH(k_rows_items, lbf_cdiv(nl, 128), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, lch,
+               groups, chunks, blocks, tiles, pl->rows_items, leaf);
     LBF_LAUNCH(k_rows_cols, lbf_cdiv(nl, 4), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, P, chunks,
                pl->rows_cols);
     LBF_LAUNCH(k_rows_fill, lbf_cdiv((int64_t)nitem, 4), 128, 0, s, (int64_t)nitem, pl->rows_items, tl,
                pl->rows_thr, geo_of(T), P, lch, pl->rows_cols, pl->xi, pl->w, pl->dself, pl->rows);
+    // the transposed rows' lists
+    LBF_LAUNCH(k_rows_rev, lbf_cdiv(nl, 128), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, chunks, leaf,
+               pl->rows_rptr, (const int32_t *)nullptr, (int32_t *)nullptr);
+    LBF_CHECK_LAUNCH();
+    if ((rc = lbf_scan_i32(pl->rows_rptr, pl->rows_rptr, nl + 1, sc, sc_len, s))) return rc;
+    int32_t nrev = 0;
+    LBF_CUDA(cudaMemcpyAsync(&nrev, pl->rows_rptr + nl, sizeof(nrev), cudaMemcpyDeviceToHost, s));
+    LBF_CUDA(cudaStreamSynchronize(s));
+    if (nrev > pl->rows_rev_cap) {
+        pl->rows_rptr = nullptr;  // transposed applications form their rows on the fly
+        return LBF_OK;
+    }
+    LBF_LAUNCH(k_rows_rev, lbf_cdiv(nl, 128), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, chunks, leaf,
+               (int32_t *)nullptr, (const int32_t *)pl->rows_rptr, pl->rows_rbase);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }
@@ -472,6 +650,28 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
         LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_apply<double>, grid, 128, 0, s, n, pl->rows_items,
                      pl->rows, pl->rows_cols, sigma, (const cx<double> *)pl->local,
                      (const cx<double> *)pl->mpole, pl->P, local_chunks(pl->P), pl->bsig, v, gate, pl->rows_split, pl->slab);
+    LBF_CHECK_LAUNCH();
+    return LBF_OK;
+}
+
+int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate, cudaStream_t s)
+{
+    const Tree &T = pl->tree;
+    const int64_t n = pl->rows_nitem;
+    LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t, pl->rows_split ? T.nleaf : lbf_cdiv(T.nleaf, 4), 128, 0, s,
+                 T.nleaf, pl->rows_block0, pl->rows_items, pl->rows, tau, pl->rows_z, gate,
+                 pl->rows_split);
+    const int lch = local_chunks(pl->P);
+    if (pl->qdf)
+        LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t_out<df64>, lbf_cdiv(n, 4), 128, 0, s, n, pl->rows_items,
+                     pl->rows, pl->rows_cols, pl->rows_z, pl->rows_rptr, pl->rows_rbase, T.begin,
+                     (const cx<df64> *)pl->local, (const cx<df64> *)pl->mpole, pl->P, lch, pl->w,
+                     pl->beta, pl->bsig, v, gate);
+    else
+        LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t_out<double>, lbf_cdiv(n, 4), 128, 0, s, n,
+                     pl->rows_items, pl->rows, pl->rows_cols, pl->rows_z, pl->rows_rptr,
+                     pl->rows_rbase, T.begin, (const cx<double> *)pl->local,
+                     (const cx<double> *)pl->mpole, pl->P, lch, pl->w, pl->beta, pl->bsig, v, gate);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }

@@ -68,3 +68,32 @@ def test_rows_repeat_and_zero_weights():
     L.lbf_apply(plan, L.LBF_OP_K_ONLY, v, b)
     L.lbf_apply(plan, L.LBF_OP_K_ONLY, zeros(g.N), z)
     assert torch.equal(a, b) and torch.count_nonzero(z) == 0
+
+
+@pytest.mark.parametrize("fmm64", [0, 1])
+@pytest.mark.parametrize("leaf,p,depth", [(1, 24, 30), (5, 26, 30), (33, 35, 30), (48, 63, 30),
+                                          (1024, 26, 30), (4, 26, 4)])
+def test_transposed_rows_against_the_oracle_and_the_unstored_rows(monkeypatch, leaf, p, depth, fmm64):
+    g = wl.star_caps(11, 5, np.array([64, 37, 201, 90, 333]))
+    v = np.random.default_rng(leaf).standard_normal(g.N + g.M)
+    ref = oracle.matrix(g).T @ v
+    opt = dict(leaf_size=leaf, p=p, max_depth=depth, fmm64=fmm64)
+    for plan in (plan_for(g, **opt), short_plan(monkeypatch, g, **opt)):
+        o = zeros(g.N + g.M)
+        L.lbf_apply(plan, L.LBF_OP_FULL | L.LBF_OP_TRANSPOSE, dev(v), o)
+        assert L.lbf_sync_status(plan) == L.LBF_OK
+        assert rel_l2(host(o), ref) < TOL
+
+
+def test_transposed_rows_of_whole_leaves_and_large_w_boxes():
+    """<K x, y> = <x, K^T y> where whole leaves go to a warp, some boxes' M2P rows are columns
+    and leaves of more than 32 rows have two blocks."""
+    g = wl.star_caps(3, 64, np.where(np.arange(64) % 8 == 0, 4096, 300))
+    for leaf in (8, 40):
+        plan = plan_for(g, leaf_size=leaf, p=26, border=0)
+        rng = np.random.default_rng(leaf)
+        x, y = dev(rng.standard_normal(g.N)), dev(rng.standard_normal(g.N))
+        kx, ky = zeros(g.N), zeros(g.N)
+        L.lbf_apply(plan, L.LBF_OP_K_ONLY, x, kx)
+        L.lbf_apply(plan, L.LBF_OP_K_ONLY | L.LBF_OP_TRANSPOSE, y, ky)
+        assert abs(float(kx @ y - x @ ky)) < TOL * float(kx.norm() * y.norm())
