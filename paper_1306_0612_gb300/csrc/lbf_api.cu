@@ -262,6 +262,7 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
     pl->region = (char *)A.take(big);
     pl->region_bytes = big;
     pl->V = o.border ? (double *)pl->region : nullptr;
+    lbf_emat_layout(pl, N, M, o);
     lbf_rows_layout(pl, N, o, cap);
 }
 

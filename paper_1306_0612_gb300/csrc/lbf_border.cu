@@ -35,6 +35,7 @@ namespace {
 
 constexpr double kEta = 3.0;
 constexpr int kMaxLevelsWalk = LBF_MAX_LEVELS + 1;
+constexpr int kEmatFloat = 128;
 
 template <typename R> struct __align__(2 * sizeof(R)) cz {
     R x, y;
@@ -1007,14 +1008,21 @@ static int pairs_to_boxes(lbf_plan *pl, cudaStream_t s, const int32_t *off, cons
     return lbf_radix_sort(sb.key, sb.key_alt, src, sb.val_alt, npairs, bits, work, work_len, s);
 }
 
-// Plan time, without the tree: the centres' planar images, the island moments and
-// S = D - F E into G (M x M).  work holds a counter and the entries summed directly.
+int lbf_centres_plane(lbf_plan *pl, cudaStream_t s)
+{
+    const int M = pl->M;
+    LBF_LAUNCH(k_mp_centres_plane, lbf_cdiv(M, 128), 128, 0, s, M, pl->centres, pl->bd.xc, pl->bd.lam,
+               pl->bd.live);
+    LBF_CHECK_LAUNCH();
+    return LBF_OK;
+}
+
+// Plan time, without the tree: the island moments and S = D - F E into G (M x M).  work holds a counter and the entries summed directly.
 int lbf_schur_build(lbf_plan *pl, cudaStream_t s, const double2 *xi_o, double *G, int32_t *work,
                     int64_t work_len)
 {
     const int M = pl->M;
     Border &B = pl->bd;
-    LBF_LAUNCH(k_mp_centres_plane, lbf_cdiv(M, 128), 128, 0, s, M, pl->centres, B.xc, B.lam, B.live);
     LBF_LAUNCH(k_mp_islands, M, 256, 0, s, M, B.P, pl->island_ptr, xi_o, B.zc, B.Rk, B.rk, B.slog,
                B.sell, B.mu, B.nu);
     int32_t *dcount = work, *dlist = work + 1;
@@ -1106,7 +1114,7 @@ int lbf_mp_build(lbf_plan *pl, cudaStream_t s, int32_t *work, int64_t work_len, 
         B.npartial = np;
         if (B.npartial > B.partial_cap) return LBF_EWORKSPACE;
     }
-    return LBF_OK;
+    return lbf_emat_build(pl, s);
 }
 
 // out = x + v + s E y (Morton order; v nullable) in precision prec.
@@ -1119,6 +1127,9 @@ int lbf_mp_apply(lbf_plan *pl, const double *y, const double *x, const double *v
     int M = pl->M;
     const int wpb = 4;
     bool f32 = prec == LBF_PREC_FP32 && B.loc32;
+    // E stored: double for the float operator too, up to kEmatFloat islands (there the tree in
+    // float, three launches, is as fast)
+    if (B.E && (!f32 || M <= kEmatFloat)) return lbf_emat_apply(pl, y, x, v, sc, out, gate, s);
     if (f32) {
         int P = B.P32;
         size_t smem = sizeof(cz<float>) * (size_t)wpb * P * 32;
@@ -1377,6 +1388,7 @@ int lbf_mp_apply_transpose(lbf_plan *pl, const double *tau, double sc, const dou
     Border &B = pl->bd;
     Tree &T = pl->tree;
     Geo g{T.xmin, T.ymin, T.L};
+    if (B.E) return lbf_emat_apply_transpose(pl, tau, sc, add, out, gate, s);
     int rc = lbf_multipoles(pl, tau, B.P, B.loc, gate, s);
     if (rc) return rc;
     LBF_LAUNCH(k_mp_tsum, 1, 1024, 0, s, pl->N, tau, B.ell, B.sums, gate);

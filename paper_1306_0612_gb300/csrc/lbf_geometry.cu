@@ -713,13 +713,15 @@ int lbf_border_start(lbf_plan *pl, cudaStream_t s0, const double2 *xi_o, double 
     LBF_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
     LBF_CUDA(cudaStreamCreateWithPriority(&pl->side, cudaStreamNonBlocking, hi));
     for (auto &e : pl->fork) LBF_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    int rc = lbf_centres_plane(pl, s0);  // read on both streams
+    if (rc) return rc;
     LBF_CUDA(cudaEventRecord(pl->fork[0], s0));
     const cudaStream_t s = pl->side;
     LBF_CUDA(cudaStreamWaitEvent(s, pl->fork[0], 0));
     lbf_prof_mark(LBF_STAGE_INVERSE, 1, s);
     // until the inverse starts, the first M^2 doubles of its scratch hold the list of
     // Schur entries summed directly (at most M^2 - M of them)
-    int rc = lbf_schur_build(pl, s, xi_o, S, (int32_t *)scratch, 2 * (int64_t)M * M);
+    rc = lbf_schur_build(pl, s, xi_o, S, (int32_t *)scratch, 2 * (int64_t)M * M);
     if (rc) return rc;
     if (pl->lu) {  // many islands: LU factors in double-float instead of the inverse
         if ((rc = lbf_schur_lu_factor(pl, s, scratch))) return rc;

@@ -106,6 +106,8 @@ struct Border {
     int32_t *p2l_ptr = nullptr, *p2l_src = nullptr;  // P2L centres per box (CSR)
     int32_t *near_ptr = nullptr, *near_src = nullptr;  // direct centres per leaf (CSR)
     int32_t *cp2l = nullptr, *cnear = nullptr;  // per centre: offsets into pairs_a / pairs_b (M + 1)
+    double *E = nullptr;             // E itself for a few hundred islands (lbf_emat.cu), or null
+    int nch = 0;                     // its chunks of eight centres
     double2 *loc = nullptr;          // local expansions of the log potential, box x P
     float2 *loc32 = nullptr;         // box x P32
     double2 *zc = nullptr;           // island node means
@@ -296,6 +298,7 @@ int lbf_schur_lu_apply(lbf_plan *pl, const double *f, double alpha, double *y, i
 // list of entries summed directly
 int lbf_schur_build(lbf_plan *pl, cudaStream_t s, const double2 *xi_o, double *G, int32_t *work,
                     int64_t work_len);
+int lbf_centres_plane(lbf_plan *pl, cudaStream_t s);  // the centres' planar images
 int lbf_mp_build(lbf_plan *pl, cudaStream_t s, int32_t *work, int64_t work_len, const SortBufs &sb);
 int lbf_mp_apply(lbf_plan *pl, const double *y, const double *x, const double *v, double sc,
                  double *out, const int *gate, cudaStream_t s, int prec);
@@ -337,6 +340,13 @@ int lbf_cauchy_deriv(lbf_plan *pl, const double *x, bool weighted, double2 *out,
 // box (P2M + M2M); also writes q = (x, 0) and *bsig = sum_j x_j
 int lbf_multipoles(lbf_plan *pl, const double *x, int P, double2 *mp, const int *gate,
                    cudaStream_t s);
+// ---- stored multiplier block (lbf_emat.cu) ---------------------------------------
+void lbf_emat_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o);
+int lbf_emat_build(lbf_plan *pl, cudaStream_t s);
+int lbf_emat_apply(lbf_plan *pl, const double *y, const double *x, const double *v, double sc,
+                   double *out, const int *gate, cudaStream_t s);
+int lbf_emat_apply_transpose(lbf_plan *pl, const double *tau, double sc, const double *add,
+                             double *out, const int *gate, cudaStream_t s);
 // ---- stored leaf rows (lbf_rows.cu) ----------------------------------------------
 void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap);
 int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len,

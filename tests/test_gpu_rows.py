@@ -97,3 +97,20 @@ def test_transposed_rows_of_whole_leaves_and_large_w_boxes():
         L.lbf_apply(plan, L.LBF_OP_K_ONLY, x, kx)
         L.lbf_apply(plan, L.LBF_OP_K_ONLY | L.LBF_OP_TRANSPOSE, y, ky)
         assert abs(float(kx @ y - x @ ky)) < TOL * float(kx.norm() * y.norm())
+
+
+@pytest.mark.parametrize("M,nodes", [(1, 40), (7, 33), (8, 32), (33, 48), (129, 40)])
+def test_stored_multiplier_block_both_ways(M, nodes):
+    """E y and E^T tau where the chunks of eight centres and blocks of 32 nodes end differently:
+    entries to the rounding of a logarithm, sums of at most 5,160 of them."""
+    g = wl.star_caps(17, M, nodes)
+    plan = plan_for(g, p=30)
+    rng = np.random.default_rng(M)
+    E = oracle.matrix(g)[:g.N, g.N:]
+    v = np.concatenate([np.zeros(g.N), rng.standard_normal(g.M)])
+    o = zeros(g.N + g.M)
+    L.lbf_apply(plan, L.LBF_OP_FULL, dev(v), o)
+    assert rel_l2(host(o)[:g.N], E @ v[g.N:]) < 1e-13
+    tau = rng.standard_normal(g.N)
+    L.lbf_apply(plan, L.LBF_OP_FULL | L.LBF_OP_TRANSPOSE, dev(np.concatenate([tau, np.zeros(g.M)])), o)
+    assert rel_l2(host(o)[g.N:], E.T @ tau) < 1e-13 * np.sqrt(g.N)
