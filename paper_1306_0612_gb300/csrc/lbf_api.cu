@@ -262,6 +262,7 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
     pl->region = (char *)A.take(big);
     pl->region_bytes = big;
     pl->V = o.border ? (double *)pl->region : nullptr;
+    lbf_m2l_layout(pl, o, cap);
     lbf_emat_layout(pl, N, M, o);
     lbf_rows_layout(pl, N, o, cap);
 }
@@ -310,6 +311,7 @@ static void layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A)
     v->gpart = A.get<double>((int64_t)pl->mdot_blocks * (m + 2));
     v->gs = (GmresState *)A.take(sizeof(GmresStateBytes));
     v->nearbuf = A.get<double>(N);
+    lbf_m2l_layout_rhs(pl, v, A);
     v->V = A.get<double>(pl->ldv * (m + 1));
     v->region = (char *)v->V;
     v->region_bytes = sizeof(double) * (size_t)pl->ldv * (m + 1);
@@ -356,6 +358,7 @@ lbf_plan lbf_view_at(const lbf_plan &v, int r)
     mv(o.red); mv(o.red_count); mv(o.fvec); mv(o.yvec); mv(o.tin); mv(o.tout); mv(o.vstep);
     mv(o.bd.partial); mv(o.bd.loc); mv(o.bd.loc32); mv(o.bd.sums); mv(o.H); mv(o.gw);
     mv(o.gx); mv(o.gb); mv(o.gpart); mv(o.gs); mv(o.V); mv(o.region); mv(o.nearbuf);
+    mv(o.m2l_X); mv(o.m2l_e); mv(o.m2l_out);
     o.nrhs = 1;
     o.slab = 0;
     return o;
@@ -514,7 +517,9 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
     int rc = check_islands(M, island_ptr, &N);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    if ((rc = lbf_fmm_init_attrs()) || (rc = lbf_border_init_attrs())) return rc;
+    if ((rc = lbf_fmm_init_attrs()) || (rc = lbf_border_init_attrs()) ||
+        (rc = lbf_m2l_init_attrs()))
+        return rc;
     lbf_plan *pl = new (std::nothrow) lbf_plan();
     if (!pl) return LBF_EINVAL;
     pl->N = N;
@@ -630,6 +635,7 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
     rc = lbf_geometry_gather(pl, s, tt.xi_o, tt.w_o, tt.d_o, tt.b_o);
     if (rc) return fail(rc);
     if ((rc = lbf_fmm_prepare(pl, s))) return fail(rc);
+    if ((rc = lbf_m2l_build(pl, s, tt.iscr, tt.iscr_len))) return fail(rc);
     if ((rc = lbf_rows_build(pl, s, tt.iscr, tt.iscr_len, tt.perm_alt))) return fail(rc);
     lbf_prof_mark(LBF_STAGE_GEOMETRY, 0, s);
     if (opt->border) {

@@ -530,16 +530,27 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
         const size_t smem = down_smem<R>(P, wpb);
         if (walk) {  // every box's own M2L + P2L, a warp per box, no chain
             LBF_LAUNCH_P(kid_down, fmm::k_down<R>, lbf_grid(pl, lbf_cdiv(T.nbox, wpb)), 32 * wpb,
+    // the double passes' M2L on the tensor cores (lbf_m2l.cu)
+    const int32_t *vptr = nullptr;
+    const cx<R> *trans = nullptr;
+    if (std::is_same<R, double>::value && pl->m2l_cap && MODE != fmm::kLeafDeriv) {
+        const int rc = lbf_m2l_apply(pl, gate, s);
+        if (rc) return rc;
+        vptr = pl->m2l_vptr;
+        trans = (const cx<R> *)pl->m2l_out;
+    }
                          smem, s, (int64_t)0, T.nbox, T.level, T.ix, T.iy, T.parent, T.vlist, T.nv,
                          T.xlist, T.nx, T.begin, T.end, g, P, binom, tpow, dsh, pl->xi, uloc, q, mp,
-                         loc, gate, 0, (unsigned *)nullptr, pl->dev_status, udf, xskip, pl->slab);
+                         loc, gate, 0, (unsigned *)nullptr, pl->dev_status, udf, xskip,
+                         vptr, trans, pl->slab);
             LBF_CHECK_LAUNCH();
         } else if (pl->pull) {
             const int64_t grid = std::min<int64_t>(lbf_cdiv(T.nbox, wpb), 4 * (int64_t)std::max(pl->nsm, 1));
             LBF_LAUNCH_P(kid_down, fmm::k_down<R>, lbf_grid(pl, grid), 32 * wpb, smem, s, (int64_t)0,
                          T.nbox, T.level, T.ix, T.iy, T.parent, T.vlist, T.nv, T.xlist, T.nx, T.begin,
                          T.end, g, P, binom, tpow, dsh, pl->xi, uloc, q, mp, loc, gate, 2, pl->pull,
-                         pl->dev_status, udf, xskip, pl->slab);
+                         pl->dev_status, udf, xskip,
+                         vptr, trans, pl->slab);
             LBF_CHECK_LAUNCH();
         } else {
             for (int l = 0; l < T.nlev; l++) {
@@ -548,7 +559,8 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
                 LBF_LAUNCH_P(kid_down, fmm::k_down<R>, lbf_grid(pl, lbf_cdiv(le - ls, wpb)), 32 * wpb,
                              smem, s, ls, le, T.level, T.ix, T.iy, T.parent, T.vlist, T.nv, T.xlist,
                              T.nx, T.begin, T.end, g, P, binom, tpow, dsh, pl->xi, uloc, q, mp, loc,
-                             gate, 1, (unsigned *)nullptr, pl->dev_status, udf, xskip, pl->slab);
+                             gate, 1, (unsigned *)nullptr, pl->dev_status, udf, xskip,
+                         vptr, trans, pl->slab);
                 LBF_CHECK_LAUNCH();
             }
         }

@@ -421,9 +421,10 @@ k_down(int64_t ls, int64_t le, const int32_t *__restrict__ level,
                        const cx<R> *__restrict__ uloc, const cx<R> *__restrict__ q,
                        const cx<R> *__restrict__ mp, cx<R> *__restrict__ loc, const int *gate,
                        int with_l2l, unsigned *pull, int *status, const cx<df64> *__restrict__ udf,
-                       int xskip, int64_t slab)
+                       int xskip, const int32_t *__restrict__ vptr,
+                       const cx<R> *__restrict__ trans, int64_t slab)
 {
-    lbf_rhs(slab, q, mp, loc, gate, pull);
+    lbf_rhs(slab, q, mp, loc, gate, pull, trans);
     if (gate_closed(gate)) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int nw = blockDim.x >> 5;
@@ -490,7 +491,20 @@ k_down(int64_t ls, int64_t le, const int32_t *__restrict__ level,
     if (with_l2l == 1 && level[b] >= 3) l2l();
     // M2L: (-1)^l t^(l+1) sum_k C(k+l, l) t^k a_k,  t = 1/(2 (dx + i dy))  (times 1/r below)
     cx<R> accF0 = mk<R>(0, 0), accF1 = mk<R>(0, 0);
-    if (P <= 16) {
+    if (trans) {
+        // the translations were formed on the tensor cores (lbf_m2l.cu, P <= 32): add this
+        // box's, a coefficient per lane, in list order
+        const cx<R> *tr = trans + (int64_t)vptr[b] * P;
+        const int nvb = nv[b];
+        if (lane < P) {
+#pragma unroll 4
+            for (int v = 0; v < nvb; v++) {
+                const cx<R> a = tr[(int64_t)v * P + lane];
+                accF0.x += a.x;
+                accF0.y += a.y;
+            }
+        }
+    } else if (P <= 16) {
         // two half-warps take two V-list boxes at a time; lane gl of a half-warp owns
         // coefficient gl, and the halves are summed at the end
         // the V list's boxes and offset indices are loaded once, a lane per entry (at most

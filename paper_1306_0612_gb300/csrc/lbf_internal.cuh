@@ -177,6 +177,16 @@ struct lbf_plan {
     // expansion were written (nbox each)
     uint32_t *pull = nullptr;
     int nsm = 0;                // streaming multiprocessors of the plan's device
+    // M2L on the tensor cores (lbf_m2l.cu; m2l_cap 0: in k_down): (source box, row) of every
+    // translation sorted by offset, each box's first row, first tile of each offset, the
+    // matrices' digits and exponents; per application the boxes' integers and exponents and
+    // a local expansion per translation
+    int64_t m2l_cap = 0, m2l_tiles = 0;
+    int2 *m2l_pairs = nullptr;
+    int32_t *m2l_vptr = nullptr, *m2l_tile0 = nullptr, *m2l_f = nullptr, *m2l_e = nullptr;
+    uint4 *m2l_img = nullptr;
+    long long *m2l_X = nullptr;
+    double *m2l_out = nullptr;
     // stored leaf rows of the accurate forward operator (lbf_rows.cu; rows null: not stored)
     double *rows = nullptr;
     int32_t *rows_cols = nullptr;
@@ -343,6 +353,12 @@ int lbf_multipoles(lbf_plan *pl, const double *x, int P, double2 *mp, const int 
 // ---- stored multiplier block (lbf_emat.cu) ---------------------------------------
 void lbf_emat_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o);
 int lbf_emat_build(lbf_plan *pl, cudaStream_t s);
+// ---- M2L on the tensor cores (lbf_m2l.cu) ----------------------------------------
+void lbf_m2l_layout(lbf_plan *pl, const lbf_options &o, int64_t cap);
+void lbf_m2l_layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A);
+int lbf_m2l_init_attrs();
+int lbf_m2l_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len);
+int lbf_m2l_apply(lbf_plan *pl, const int *gate, cudaStream_t s);
 int lbf_emat_apply(lbf_plan *pl, const double *y, const double *x, const double *v, double sc,
                    double *out, const int *gate, cudaStream_t s);
 int lbf_emat_apply_transpose(lbf_plan *pl, const double *tau, double sc, const double *add,
