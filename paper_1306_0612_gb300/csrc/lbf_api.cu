@@ -518,7 +518,7 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     if ((rc = lbf_fmm_init_attrs()) || (rc = lbf_border_init_attrs()) ||
-        (rc = lbf_m2l_init_attrs()))
+        (rc = lbf_m2l_init_attrs()) || (rc = lbf_passes_init_attrs()))
         return rc;
     lbf_plan *pl = new (std::nothrow) lbf_plan();
     if (!pl) return LBF_EINVAL;
@@ -637,6 +637,7 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
     if ((rc = lbf_fmm_prepare(pl, s))) return fail(rc);
     if ((rc = lbf_m2l_build(pl, s, tt.iscr, tt.iscr_len))) return fail(rc);
     if ((rc = lbf_rows_build(pl, s, tt.iscr, tt.iscr_len, tt.perm_alt))) return fail(rc);
+    if ((rc = lbf_passes_build(pl, s, tt.iscr))) return fail(rc);
     lbf_prof_mark(LBF_STAGE_GEOMETRY, 0, s);
     if (opt->border) {
         SortBufs sb{tt.keys, tt.keys_alt, tt.perm_alt};

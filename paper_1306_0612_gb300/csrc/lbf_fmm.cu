@@ -487,6 +487,13 @@ struct FmmArrays {
 // the land on one side, (I + 2K) 1_k is a constant vector, far smaller than 1_k, so the
 // float passes never form the near-cancelling sum of a mean density, which is what the
 // corrections of the refinement are made of.
+// whether an accurate application reads the stored rows
+template <int MODE> bool rows_stored(const lbf_plan *pl)
+{
+    return pl->rows && (MODE == fmm::kLeafForward ||
+                        (MODE == fmm::kLeafTranspose && pl->rows_rptr && pl->nrhs == 1));
+}
+
 template <typename R, int MODE>
 int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, const int *gate,
               cudaStream_t s, bool split = false)
@@ -503,10 +510,15 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
     const cx<df64> *udf = sizeof(R) == sizeof(float) ? (const cx<df64> *)pl->udf : nullptr;
     const bool dbl = sizeof(R) == sizeof(double);
     // the accurate forward rows: near field, small W and X boxes and L2P stored (lbf_rows.cu)
-    const bool stored = sizeof(R) == sizeof(double) && pl->rows &&
-                        (MODE == fmm::kLeafForward ||
-                         (MODE == fmm::kLeafTranspose && pl->rows_rptr && pl->nrhs == 1));
+    const bool stored = sizeof(R) == sizeof(double) && rows_stored<MODE>(pl);
     const int xskip = stored ? pl->rows_thr : -1;
+    constexpr bool kDf = std::is_same<R, df64>::value;
+    if (std::is_same<R, double>::value && stored && lbf_passes_ready(pl)) {
+        const int rc = lbf_passes_apply(pl, gate, s);
+        if (rc) return rc;
+        return MODE == fmm::kLeafForward ? lbf_rows_apply(pl, sigma, v, gate, s, false)
+                                         : lbf_rows_apply_t(pl, sigma, v, gate, s, false);
+    }
     const int kid_up = dbl ? LBF_KERNEL_UP : LBF_KERNEL_UP32;
     const int kid_down = dbl ? LBF_KERNEL_DOWN : LBF_KERNEL_DOWN32;
     const int kid_leaf = dbl ? LBF_KERNEL_LEAF : LBF_KERNEL_LEAF32;
@@ -517,6 +529,15 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
                      T.end, T.parent, T.child0, T.nchild, g, P, binom, dsh, pl->xi, uloc, q,
                      mp, pl->upcnt, gate, pl->slab);
         LBF_CHECK_LAUNCH();
+    }
+    // the double passes' M2L on the tensor cores (lbf_m2l.cu)
+    const int32_t *vptr = nullptr;
+    const cx<R> *trans = nullptr;
+    if (std::is_same<R, double>::value && pl->m2l_cap && MODE != fmm::kLeafDeriv) {
+        const int rc = lbf_m2l_apply(pl, gate, s);
+        if (rc) return rc;
+        vptr = pl->m2l_vptr;
+        trans = (const cx<R> *)pl->m2l_out;
     }
     // float forward rows: no chain, the far field comes from the per-node walk below
     const bool walk = sizeof(R) == sizeof(float) && MODE == fmm::kLeafForward && pl->anc &&
@@ -530,15 +551,6 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
         const size_t smem = down_smem<R>(P, wpb);
         if (walk) {  // every box's own M2L + P2L, a warp per box, no chain
             LBF_LAUNCH_P(kid_down, fmm::k_down<R>, lbf_grid(pl, lbf_cdiv(T.nbox, wpb)), 32 * wpb,
-    // the double passes' M2L on the tensor cores (lbf_m2l.cu)
-    const int32_t *vptr = nullptr;
-    const cx<R> *trans = nullptr;
-    if (std::is_same<R, double>::value && pl->m2l_cap && MODE != fmm::kLeafDeriv) {
-        const int rc = lbf_m2l_apply(pl, gate, s);
-        if (rc) return rc;
-        vptr = pl->m2l_vptr;
-        trans = (const cx<R> *)pl->m2l_out;
-    }
                          smem, s, (int64_t)0, T.nbox, T.level, T.ix, T.iy, T.parent, T.vlist, T.nv,
                          T.xlist, T.nx, T.begin, T.end, g, P, binom, tpow, dsh, pl->xi, uloc, q, mp,
                          loc, gate, 0, (unsigned *)nullptr, pl->dev_status, udf, xskip,
@@ -566,8 +578,8 @@ int fmm_apply(lbf_plan *pl, const FmmArrays &a, const double *sigma, double *v, 
         }
     }
     if (stored)
-        return MODE == fmm::kLeafForward ? lbf_rows_apply(pl, sigma, v, gate, s)
-                                         : lbf_rows_apply_t(pl, sigma, v, gate, s);
+        return MODE == fmm::kLeafForward ? lbf_rows_apply(pl, sigma, v, gate, s, kDf)
+                                         : lbf_rows_apply_t(pl, sigma, v, gate, s, kDf);
     // Several right-hand sides in lockstep: the double forward rows' near field in one pass
     // that forms each pair's geometry once (k_near_multi), the leaf kernel adding it.  (The
     // float operator keeps a leaf pass per right-hand side: its pairs are cheap on the
@@ -670,8 +682,11 @@ static int apply_mode(lbf_plan *pl, const double *sigma, double *v, const int *g
 {
     if (prec == LBF_PREC_FP32 && !pl->q32) return LBF_ENOTBUILT;
     if (pl->opt.matvec == LBF_MATVEC_DIRECT || MODE == fmm::kLeafDeriv) prec = LBF_PREC_FP64;
+    // with every stored part present the double passes are the faster ones (and no less
+    // accurate), whatever opt.fmm64 says
+    const bool stored = rows_stored<MODE>(pl) && lbf_passes_ready(pl);
     const Arith ar = prec == LBF_PREC_FP32 ? Arith::F32
-                     : (pl->qdf && MODE != fmm::kLeafDeriv && pl->opt.matvec == LBF_MATVEC_FMM)
+                     : (pl->qdf && !stored && MODE != fmm::kLeafDeriv && pl->opt.matvec == LBF_MATVEC_FMM)
                          ? Arith::DF64
                          : Arith::F64;
     // the float forward rows split off each island's mean density (see fmm_apply)

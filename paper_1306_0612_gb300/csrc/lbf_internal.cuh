@@ -197,6 +197,9 @@ struct lbf_plan {
     // columns (rptr null: not stored), a value per column
     int32_t *rows_block0 = nullptr, *rows_rptr = nullptr, *rows_rbase = nullptr;
     double *rows_z = nullptr;
+    // boxes whose X lists are not near columns (nbigx < 0: the passes of lbf_passes.cu are off)
+    int64_t nbigx = -1, bigx_cap = 0;
+    int32_t *bigx = nullptr;
     int rows_split = 0;         // a small system: four warps share a block's columns
     int rows_thr = 0;           // boxes of at most this many nodes enter W and X lists as pairs
     double *v = nullptr;        // (I + K - I) sigma = K sigma, doubled scaling
@@ -350,15 +353,15 @@ int lbf_cauchy_deriv(lbf_plan *pl, const double *x, bool weighted, double2 *out,
 // box (P2M + M2M); also writes q = (x, 0) and *bsig = sum_j x_j
 int lbf_multipoles(lbf_plan *pl, const double *x, int P, double2 *mp, const int *gate,
                    cudaStream_t s);
-// ---- stored multiplier block (lbf_emat.cu) ---------------------------------------
-void lbf_emat_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o);
-int lbf_emat_build(lbf_plan *pl, cudaStream_t s);
 // ---- M2L on the tensor cores (lbf_m2l.cu) ----------------------------------------
 void lbf_m2l_layout(lbf_plan *pl, const lbf_options &o, int64_t cap);
 void lbf_m2l_layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A);
 int lbf_m2l_init_attrs();
 int lbf_m2l_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len);
 int lbf_m2l_apply(lbf_plan *pl, const int *gate, cudaStream_t s);
+// ---- stored multiplier block (lbf_emat.cu) ---------------------------------------
+void lbf_emat_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o);
+int lbf_emat_build(lbf_plan *pl, cudaStream_t s);
 int lbf_emat_apply(lbf_plan *pl, const double *y, const double *x, const double *v, double sc,
                    double *out, const int *gate, cudaStream_t s);
 int lbf_emat_apply_transpose(lbf_plan *pl, const double *tau, double sc, const double *add,
@@ -367,8 +370,16 @@ int lbf_emat_apply_transpose(lbf_plan *pl, const double *tau, double sc, const d
 void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap);
 int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len,
                    int32_t *leaf);
-int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate, cudaStream_t s);
-int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate, cudaStream_t s);
+// df: the expansions are double-float
+int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate, cudaStream_t s,
+                     bool df);
+int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate, cudaStream_t s,
+                   bool df);
+// ---- up and down passes over the stored parts (lbf_passes.cu) -------------------------
+int lbf_passes_init_attrs();
+bool lbf_passes_ready(const lbf_plan *pl);
+int lbf_passes_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch);
+int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s);
 int lbf_evaluate_impl(lbf_plan *pl, const double *sigma_sorted, const double *a, int64_t T,
                       const double *t, double *u, cudaStream_t s);
 int lbf_green_sum_impl(int64_t T, const double *t, int64_t S, const double *p,

@@ -562,6 +562,8 @@ void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap)
     pl->rows_rptr = A.get<int32_t>(cap + 1);
     pl->rows_rbase = A.get<int32_t>(pl->rows_rev_cap);
     pl->rows_z = A.get<double>(8 * chunks);
+    pl->bigx_cap = cap / 8 + 16;
+    pl->bigx = A.get<int32_t>(pl->bigx_cap);
     pl->rows = A.get<double>(32 * tiles);
     if (A.overflow && !full) {  // a workspace of the size without rows
         A.off = off;
@@ -578,10 +580,10 @@ int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scrat
     Tree &T = pl->tree;
     const int64_t nl = T.nleaf;
     const int P = pl->P, lch = local_chunks(P);
-        // (in a small system the few larger W boxes are pairs too: an M2P there is a chain of
-    // P dependent steps that the whole launch waits for)
+        // (in a small system W and X boxes of up to 512 nodes are pairs while there is room: their
+    // few P2L and M2P are dependent steps that the whole application waits for; with boxes of up
+    // to 2048 the longest rows hold it up instead, 85 against 22 us for the rows of 8192 nodes)
     const bool small = nl < kSmallLeaves;
-    pl->rows_thr = small ? std::max(512, 4 * P) : 4 * P;
     pl->rows_split = small ? 1 : 0;
     const int groups = small ? kGroupsSmall : kGroups;
     const TreeLists tl = lists_of(T);
@@ -593,24 +595,29 @@ int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scrat
         pl->rows = nullptr;
         return LBF_OK;
     }
-    LBF_CUDA(cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (8 + 2 * (nl + 1)), s));
-    LBF_CUDA(cudaMemsetAsync(blocks, 0, sizeof(int32_t) * (nl + 1), s));
-    LBF_CUDA(cudaMemsetAsync(pl->rows_rptr, 0, sizeof(int32_t) * (nl + 1), s));
-    LBF_LAUNCH(k_rows_count, lbf_cdiv(nl, 128), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, P,
-               lch, groups, chunks, blocks, tiles, total);
-    LBF_CHECK_LAUNCH();
     int rc;
-    if ((rc = lbf_scan_i32(blocks, blocks, nl + 1, sc, sc_len, s))) return rc;
-    unsigned long long h[2];
     int32_t nitem = 0;
-    LBF_CUDA(cudaMemcpyAsync(h, total, sizeof(h), cudaMemcpyDeviceToHost, s));
-    LBF_CUDA(cudaMemcpyAsync(&nitem, blocks + nl, sizeof(nitem), cudaMemcpyDeviceToHost, s));
-    LBF_CUDA(cudaStreamSynchronize(s));
-    if (h[0] > (unsigned long long)pl->rows_tiles || h[1] > (unsigned long long)pl->rows_chunks ||
-        nitem > pl->rows_items_cap) {
-        pl->rows = nullptr;
-        return LBF_OK;
+    for (int large = small;; large = 0) {
+        pl->rows_thr = large ? std::max(512, 4 * P) : 4 * P;
+        LBF_CUDA(cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (8 + 2 * (nl + 1)), s));
+        LBF_CUDA(cudaMemsetAsync(blocks, 0, sizeof(int32_t) * (nl + 1), s));
+        LBF_LAUNCH(k_rows_count, lbf_cdiv(nl, 128), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, P, lch,
+                   groups, chunks, blocks, tiles, total);
+        LBF_CHECK_LAUNCH();
+        if ((rc = lbf_scan_i32(blocks, blocks, nl + 1, sc, sc_len, s))) return rc;
+        unsigned long long h[2];
+        LBF_CUDA(cudaMemcpyAsync(h, total, sizeof(h), cudaMemcpyDeviceToHost, s));
+        LBF_CUDA(cudaMemcpyAsync(&nitem, blocks + nl, sizeof(nitem), cudaMemcpyDeviceToHost, s));
+        LBF_CUDA(cudaStreamSynchronize(s));
+        if (h[0] <= (unsigned long long)pl->rows_tiles && h[1] <= (unsigned long long)pl->rows_chunks &&
+            nitem <= pl->rows_items_cap)
+            break;
+        if (!large) {
+            pl->rows = nullptr;
+            return LBF_OK;
+        }
     }
+    LBF_CUDA(cudaMemsetAsync(pl->rows_rptr, 0, sizeof(int32_t) * (nl + 1), s));
     if ((rc = lbf_scan_i32(chunks, chunks, nl + 1, sc, sc_len, s))) return rc;
     if ((rc = lbf_scan_i32(tiles, tiles, nl + 1, sc, sc_len, s))) return rc;
     pl->rows_nitem = nitem;
@@ -638,11 +645,12 @@ int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scrat
     return LBF_OK;
 }
 
-int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate, cudaStream_t s)
+int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate, cudaStream_t s,
+                   bool df)
 {
     const int64_t n = pl->rows_nitem;
     const dim3 grid = lbf_grid(pl, pl->rows_split ? n : lbf_cdiv(n, 4));
-    if (pl->qdf)
+    if (df)
         LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_apply<df64>, grid, 128, 0, s, n, pl->rows_items, pl->rows,
                      pl->rows_cols, sigma, (const cx<df64> *)pl->local, (const cx<df64> *)pl->mpole,
                      pl->P, local_chunks(pl->P), pl->bsig, v, gate, pl->rows_split, pl->slab);
@@ -654,7 +662,8 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
     return LBF_OK;
 }
 
-int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate, cudaStream_t s)
+int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate, cudaStream_t s,
+                     bool df)
 {
     const Tree &T = pl->tree;
     const int64_t n = pl->rows_nitem;
@@ -662,7 +671,7 @@ int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate
                  T.nleaf, pl->rows_block0, pl->rows_items, pl->rows, tau, pl->rows_z, gate,
                  pl->rows_split);
     const int lch = local_chunks(pl->P);
-    if (pl->qdf)
+    if (df)
         LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t_out<df64>, lbf_cdiv(n, 4), 128, 0, s, n, pl->rows_items,
                      pl->rows, pl->rows_cols, pl->rows_z, pl->rows_rptr, pl->rows_rbase, T.begin,
                      (const cx<df64> *)pl->local, (const cx<df64> *)pl->mpole, pl->P, lch, pl->w,
