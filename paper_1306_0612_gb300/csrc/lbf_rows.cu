@@ -171,8 +171,10 @@ __global__ void k_rows_cols(int64_t nleaf, const int32_t *__restrict__ leaves, T
     if (m + lane < (m + 7) / 8 * 8) c[m + lane] = T.begin[b];
 }
 
-// For leaf t, the leaves whose columns hold its nodes, in the order of its own columns: their
-// number (base null) or where t's first node stands among all the columns.
+// Per leaf, where its first node stands in the columns of the leaves that hold its nodes: a
+// thread per holding leaf goes through its own columns and appends to the lists of the leaves
+// it finds (base null: counts them), and k_rows_rev_sort puts each list in ascending order, so
+// that the sums over it do not depend on the atomics.
 __global__ void k_rows_rev(int64_t nleaf, const int32_t *__restrict__ leaves, TreeLists T, int thr,
                            const int32_t *__restrict__ chunk0, const int32_t *__restrict__ leaf,
                            int32_t *__restrict__ count, const int32_t *__restrict__ ptr,
@@ -180,24 +182,27 @@ __global__ void k_rows_rev(int64_t nleaf, const int32_t *__restrict__ leaves, Tr
 {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= nleaf) return;
-    const int first = T.begin[leaves[t]];
-    int n = 0;
+    int at = chunk0[t] * 8;
     for_ranges(T, leaves[t], thr, [&](int s, int e) {
         for (int j = s; j < e;) {
-            const int tb = leaf[j], b = leaves[tb];
-            if (base) {
-                int off = 0, at = 0;
-                for_ranges(T, b, thr, [&](int s2, int e2) {
-                    if (first >= s2 && first < e2) at = off + first - s2;
-                    off += e2 - s2;
-                });
-                base[ptr[t] + n] = chunk0[tb] * 8 + at;
-            }
-            n++;
-            j = T.end[b];
+            const int h = leaf[j], k = atomicAdd(&count[h], 1), next = T.end[leaves[h]];
+            if (base) base[ptr[h] + k] = at + (j - s);
+            j = next;
         }
+        at += e - s;
     });
-    if (!base) count[t] = n;
+}
+
+__global__ void k_rows_rev_sort(int64_t nleaf, const int32_t *__restrict__ ptr, int32_t *__restrict__ base)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= nleaf) return;
+    for (int i = ptr[t] + 1; i < ptr[t + 1]; i++) {
+        const int32_t v = base[i];
+        int k = i - 1;
+        for (; k >= ptr[t] && base[k] > v; k--) base[k + 1] = base[k];
+        base[k + 1] = v;
+    }
 }
 
 // the entries, a warp per row block
@@ -404,22 +409,25 @@ k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__r
     if (row < it.nrow) v[it.row0 + row] = s + 2.0 * *bsig;
 }
 
-// z = G^T tau over each leaf's columns, a warp per leaf, or (split) the four warps of a
-// thread block, a quarter of the columns each.  Four chunks at a time: a lane sums its rows'
-// parts of a column of each, and the four lanes of a column are added in 3 additions.
+// z = G^T tau over each leaf's columns, a thread block of four warps per leaf, a quarter of
+// the columns a warp (no sums between warps; a warp per leaf left the leaf with the most
+// columns, 1500 of a mean of 200, running alone: 582 us at 131,072 nodes).  Four chunks at a
+// time: a lane sums its rows' parts of a column of each, and the four lanes of a column are
+// added in 3 additions.
 __global__ void __launch_bounds__(128)
-k_rows_t(int64_t nleaf, const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
+k_rows_t(const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
          const double *__restrict__ rows, const double *__restrict__ tau, double *__restrict__ z,
-         const int *gate, int split)
+         const int *gate)
 {
     if (fmm::gate_closed(gate)) return;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t t = split ? (int64_t)blockIdx.x : blockIdx.x * (int64_t)(blockDim.x >> 5) + wid;
-    if (t >= nleaf) return;
-    for (int k = block0[t]; k < block0[t + 1]; k++) {
+    const int64_t t = blockIdx.x;
+    const int b0 = block0[t], b1 = block0[t + 1];
+    const bool u = (lane & 16) != 0, w = (lane & 8) != 0;
+    for (int k = b0; k < b1; k++) {
         const RowItem it = items[k];
         const int ng = (it.nrow + 3) / 4, nk = (it.ncol + 7) / 8;
-        const int k0 = split ? nk * wid / 4 : 0, k1 = split ? nk * (wid + 1) / 4 : nk;
+        const int k0 = nk * wid / 4, k1 = nk * (wid + 1) / 4;
         double tv[kGroups];
 #pragma unroll
         for (int q = 0; q < kGroups; q++) {
@@ -428,22 +436,26 @@ k_rows_t(int64_t nleaf, const int32_t *__restrict__ block0, const RowItem *__res
         }
         const double *tl = rows + ((int64_t)it.tile + (int64_t)k0 * ng) * 32 + lane;
         for (int c = k0; c < k1; c += 4, tl += 128 * ng) {
-            double a[4] = {0.0, 0.0, 0.0, 0.0};
+            double a[4];
 #pragma unroll
-            for (int q = 0; q < kGroups; q++)
-                if (q < ng) {
+            for (int h = 0; h < 4; h++) {
+                double e[kGroups];
+                const bool on = c + h < k1;
 #pragma unroll
-                    for (int h = 0; h < 4; h++)
-                        if (c + h < k1) a[h] = fma(tl[32 * (h * ng + q)], tv[q], a[h]);
-                }
-            const bool u = (lane & 16) != 0, w = (lane & 8) != 0;
-            const double b0 = (u ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, u ? a[0] : a[2], 16);
-            const double b1 = (u ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, u ? a[1] : a[3], 16);
-            const double s = (w ? b1 : b0) + __shfl_xor_sync(0xffffffffu, w ? b0 : b1, 8);
+                for (int q = 0; q < kGroups; q++) e[q] = on && q < ng ? tl[32 * (h * ng + q)] : 0.0;
+                double s = 0.0;
+#pragma unroll
+                for (int q = 0; q < kGroups; q++)
+                    if (q < ng) s = fma(e[q], tv[q], s);
+                a[h] = s;
+            }
+            const double s0 = (u ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, u ? a[0] : a[2], 16);
+            const double s1 = (u ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, u ? a[1] : a[3], 16);
+            const double s = (w ? s1 : s0) + __shfl_xor_sync(0xffffffffu, w ? s0 : s1, 8);
             const int h = (u ? 2 : 0) + (w ? 1 : 0);  // the chunk this lane's sum belongs to
             if (c + h < k1) {
                 double *o = z + ((int64_t)it.chunk + c + h) * 8 + (lane & 7);
-                *o = k == block0[t] ? s : *o + s;
+                *o = k == b0 ? s : *o + s;
             }
         }
     }
@@ -639,8 +651,10 @@ int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scrat
         pl->rows_rptr = nullptr;  // transposed applications form their rows on the fly
         return LBF_OK;
     }
+    LBF_CUDA(cudaMemsetAsync(tiles, 0, sizeof(int32_t) * nl, s));  // the lists' write positions
     LBF_LAUNCH(k_rows_rev, lbf_cdiv(nl, 128), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, chunks, leaf,
-               (int32_t *)nullptr, (const int32_t *)pl->rows_rptr, pl->rows_rbase);
+               tiles, (const int32_t *)pl->rows_rptr, pl->rows_rbase);
+    LBF_LAUNCH(k_rows_rev_sort, lbf_cdiv(nl, 128), 128, 0, s, nl, pl->rows_rptr, pl->rows_rbase);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }
@@ -667,9 +681,8 @@ int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate
 {
     const Tree &T = pl->tree;
     const int64_t n = pl->rows_nitem;
-    LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t, pl->rows_split ? T.nleaf : lbf_cdiv(T.nleaf, 4), 128, 0, s,
-                 T.nleaf, pl->rows_block0, pl->rows_items, pl->rows, tau, pl->rows_z, gate,
-                 pl->rows_split);
+    LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t, T.nleaf, 128, 0, s, pl->rows_block0, pl->rows_items,
+                 pl->rows, tau, pl->rows_z, gate);
     const int lch = local_chunks(pl->P);
     if (df)
         LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t_out<df64>, lbf_cdiv(n, 4), 128, 0, s, n, pl->rows_items,
