@@ -518,7 +518,7 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     if ((rc = lbf_fmm_init_attrs()) || (rc = lbf_border_init_attrs()) ||
-        (rc = lbf_m2l_init_attrs()) || (rc = lbf_passes_init_attrs()))
+        (rc = lbf_m2l_init_attrs()) || (rc = lbf_passes_init_attrs()) || (rc = lbf_evaluate_init_attrs()))
         return rc;
     lbf_plan *pl = new (std::nothrow) lbf_plan();
     if (!pl) return LBF_EINVAL;

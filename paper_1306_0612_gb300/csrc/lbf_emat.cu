@@ -16,39 +16,12 @@
 #include <algorithm>
 
 #include "lbf_fmm_tpl.cuh"
+#include "lbf_log.cuh"
 
 namespace {
 
 constexpr int kEmatIslands = 512;
 constexpr int64_t kEmatEntries = 100000000;
-
-// log a for positive normal a, table-driven (P. T. P. Tang, ACM TOMS 16, 1990): with
-// a = 2^e m, c the tabulated 1/m to 7 bits, r = c m - 1, |r| <= 2^-8,
-//   log a = e log 2 + log(1/c) + (r - r^2/2 + r^3/3 - ... + r^7/7),
-// the remainder below 2^-66: 12 double instructions.  The table: c_j = 128/(128 + j) rounded
-// to float (c m - 1 has one rounding, relative to r), formed by each thread block.
-struct LogTab {
-    double c[129], l[129];
-};
-
-__device__ __forceinline__ double log_tab(double a, const LogTab &t)
-{
-    const int hi = __double2hiint(a);
-    int e = (hi >> 20) - 1023;
-    const int j = ((hi & 0xfffff) + (1 << 12)) >> 13;  // m to the nearest 1/128, 0..128
-    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(a));
-    const double r = fma(m, t.c[j], -1.0);
-    // e as a double from the integer's bits (2^52 + 2^31 + e less 2^52 + 2^31)
-    const double ed = __hiloint2double(0x43300000, e ^ 0x80000000) - 4503601774854144.0;
-    double q = 1.0 / 7.0;
-    q = fma(q, r, -1.0 / 6.0);
-    q = fma(q, r, 1.0 / 5.0);
-    q = fma(q, r, -1.0 / 4.0);
-    q = fma(q, r, 1.0 / 3.0);
-    q = fma(q, r, -0.5);
-    const double r2 = r * r;
-    return fma(ed, LBF_LN2, t.l[j]) + fma(q, r2, r);
-}
 
 // E, a warp per (node block, chunk) in turn
 __global__ void k_emat_fill(int64_t N, int M, int nch, const double2 *__restrict__ xi,
@@ -57,11 +30,7 @@ __global__ void k_emat_fill(int64_t N, int M, int nch, const double2 *__restrict
                             double *__restrict__ E)
 {
     __shared__ LogTab tab;
-    for (int k = threadIdx.x; k < 129; k += blockDim.x) {
-        const double c = (double)(float)(128.0 / (128.0 + k));
-        tab.c[k] = c;
-        tab.l[k] = -log(c);
-    }
+    log_table(tab);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t nb = (N + 31) / 32, nw = gridDim.x * (int64_t)(blockDim.x >> 5);
@@ -82,7 +51,7 @@ __global__ void k_emat_fill(int64_t N, int M, int nch, const double2 *__restrict
                 const double2 z = xi[i];
                 const double dx = z.x - c.x, dy = z.y - c.y;
                 const double d2 = fma(dx, dx, dy * dy);
-                e -= d2 > 0x1p-1000 && d2 < 0x1p1000 ? log_tab(d2, tab) : log(d2);
+                e -= log_any(d2, tab);
             }
             e *= 1.0 / (2.0 * LBF_PI);
         }

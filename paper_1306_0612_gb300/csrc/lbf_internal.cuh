@@ -381,7 +381,12 @@ bool lbf_passes_ready(const lbf_plan *pl);
 int lbf_passes_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch);
 int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s);
 int lbf_evaluate_impl(lbf_plan *pl, const double *sigma_sorted, const double *a, int64_t T,
+int lbf_passes_up(lbf_plan *pl, const int *gate, cudaStream_t s);
                       const double *t, double *u, cudaStream_t s);
+// off-curve evaluation (lbf_evaluate.cu); its charges, and its charges and double multipoles
+int lbf_eval_charges(lbf_plan *pl, const double *sigma, cudaStream_t s);
+int lbf_eval_multipoles(lbf_plan *pl, const double *sigma, cudaStream_t s);
+int lbf_evaluate_init_attrs();
 int lbf_green_sum_impl(int64_t T, const double *t, int64_t S, const double *p,
                        const double *gamma, double *out, cudaStream_t s);
 

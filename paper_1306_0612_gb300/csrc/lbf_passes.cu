@@ -581,8 +581,8 @@ int lbf_passes_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch)
     return LBF_OK;
 }
 
-// multipoles and full local expansions of the charges pl->q
-int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s)
+// multipoles of the charges pl->q
+int lbf_passes_up(lbf_plan *pl, const int *gate, cudaStream_t s)
 {
     const Tree &T = pl->tree;
     const int P = pl->P, lch = (2 * P + 7) / 8;
@@ -598,7 +598,18 @@ int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s)
                      pl->rows_items, pl->rows, pl->tab_binom, (const cx<double> *)pl->tab_dshift, pl->q,
                      (cx<double> *)pl->mpole, pl->upcnt, gate, pl->slab);
     LBF_CHECK_LAUNCH();
-    const int rc = lbf_m2l_apply(pl, gate, s);
+    return LBF_OK;
+}
+
+// multipoles and full local expansions of the charges pl->q
+int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s)
+{
+    const Tree &T = pl->tree;
+    const int P = pl->P;
+    const bool small = T.nleaf < kSmallLeaves;
+    int rc = lbf_passes_up(pl, gate, s);
+    if (rc) return rc;
+    rc = lbf_m2l_apply(pl, gate, s);
     if (rc) return rc;
     if (pl->nbigx > 0)
         LBF_LAUNCH_P(LBF_KERNEL_DOWN, k_p2l_big, lbf_grid(pl, pl->nbigx), 128, kP2lSmem, s,
