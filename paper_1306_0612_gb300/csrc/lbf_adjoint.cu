@@ -7,7 +7,13 @@
 //   dL/dxi_j = d/dxi_j (ubar^T C z) - lam^T (dA/dxi_j) z.
 // Every term is a Cauchy-type sum (the derivative FMM), a node-target sum, or the
 // gradient of the multiplier potential; they are combined per node below.
-#include "lbf_internal.cuh"
+#include <algorithm>
+
+#include "lbf_fmm_tpl.cuh"
+
+using fmm::BoxGeo;
+using fmm::cx;
+using fmm::mk;
 
 namespace {
 
@@ -41,17 +47,50 @@ __device__ __forceinline__ void target_plane(const double *t, int64_t k, const R
     zy = finite ? p[1] / w : 0.0;
 }
 
-// per node (sorted): S1 = sum_t ubar_t/(xi - xi_t), S2 = sum_t ubar_t/(xi - xi_t)^2
-// (targets tiled through shared memory, projected by each block)
+// Per node (sorted order) the target sums, Power 1: S = sum_t ubar_t/(xi - xi_t), Power 2:
+// S = sum_t ubar_t/(xi - xi_t)^2.
+//
+// Few pairs (N T <= kDirectPairs): all of them (k_node_target, targets tiled through shared
+// memory and projected by each block).  More: the targets as sources of the FMM's downward
+// pass.  They are sorted by their Morton key on the nodes' quadtree, so that the targets of any
+// cell are one run of the sorted list, found by binary search; a box takes the targets of the
+// cells that are separated from it but whose parents touch its parent's (P2L, at most 27
+// cells), the expansions are shifted down, and a leaf adds the targets of the 3 x 3 cells around
+// it directly.  Nothing of it goes through the host, so the call stays asynchronous.  A
+// target is at least 3 half-widths from a box's centre, its nodes at most sqrt 2: kTerms = 48
+// terms leave (sqrt 2/3)^48 = 2e-16.  At 131,072 nodes and 4096 targets 21.3 ms of pairs (the
+// double pipe, 40 instructions a pair with the division) to 0.5 ms.
+constexpr int64_t kDirectPairs = 1 << 24;
+constexpr int kTerms = 48;
+
+template <int Power>
+__device__ __forceinline__ void target_term(double2 z, double2 t, double ub, double2 &s)
+{
+    const double dr = z.x - t.x, di = z.y - t.y;
+    const double d2 = fma(dr, dr, di * di);
+    const double id = d2 > 0x1p-120 && d2 < 0x1p120 ? fmm::rcp_near(d2) : 1.0 / d2;
+    // 1/d = conj(d)/|d|^2, 1/d^2 = conj(d)^2/|d|^4
+    const double er = dr * id, ei = -di * id;
+    if (Power == 1) {
+        s.x = fma(ub, er, s.x);
+        s.y = fma(ub, ei, s.y);
+    } else {
+        const double ur = ub * er;
+        s.x = fma(ur, er, fma(-ub * ei, ei, s.x));
+        s.y = fma(ur + ur, ei, s.y);
+    }
+}
+
+template <int Power>
 __global__ void k_node_target(int64_t N, const double2 *__restrict__ xi, int64_t T,
                               const double *__restrict__ t, Rot3 R, const double *__restrict__ ub,
-                              double2 *__restrict__ S1, double2 *__restrict__ S2)
+                              double2 *__restrict__ S)
 {
     __shared__ double2 tz[256];
     __shared__ double tu[256];
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const double2 z = i < N ? xi[i] : make_double2(0, 0);
-    double a1r = 0, a1i = 0, a2r = 0, a2i = 0;
+    double2 s = make_double2(0.0, 0.0);
     for (int64_t base = 0; base < T; base += 256) {
         __syncthreads();
         int64_t k = base + threadIdx.x;
@@ -64,20 +103,185 @@ __global__ void k_node_target(int64_t N, const double2 *__restrict__ xi, int64_t
         }
         __syncthreads();
         int n = (int)(T - base < 256 ? T - base : 256);
-        for (int m = 0; m < n; m++) {
-            const double dr = z.x - tz[m].x, di = z.y - tz[m].y;
-            const double id = 1.0 / fma(dr, dr, di * di);
-            // 1/d = conj(d)/|d|^2, 1/d^2 = conj(d)^2/|d|^4
-            const double er = dr * id, ei = -di * id;
-            a1r = fma(tu[m], er, a1r);
-            a1i = fma(tu[m], ei, a1i);
-            a2r = fma(tu[m], er * er - ei * ei, a2r);
-            a2i = fma(tu[m], 2.0 * er * ei, a2i);
-        }
+        for (int m = 0; m < n; m++) target_term<Power>(z, tz[m], tu[m], s);
     }
-    if (i < N) {
-        S1[i] = make_double2(a1r, a1i);
-        S2[i] = make_double2(a2r, a2i);
+    if (i < N) S[i] = s;
+}
+
+__device__ __forceinline__ uint64_t spread32(uint64_t v)
+{
+    v &= 0xffffffffull;
+    v = (v | (v << 16)) & 0x0000ffff0000ffffull;
+    v = (v | (v << 8)) & 0x00ff00ff00ff00ffull;
+    v = (v | (v << 4)) & 0x0f0f0f0f0f0f0f0full;
+    v = (v | (v << 2)) & 0x3333333333333333ull;
+    v = (v | (v << 1)) & 0x5555555555555555ull;
+    return v;
+}
+
+// key of each target's cell at depth D of the nodes' square, or past every cell's outside it
+__global__ void k_target_keys(int64_t T, const double *__restrict__ t, Rot3 R, BoxGeo g, int D,
+                              uint64_t *__restrict__ key, int32_t *__restrict__ idx)
+{
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= T) return;
+    double p[3], zx, zy;
+    bool fin;
+    target_plane(t, k, R, p, zx, zy, fin);
+    const double sc = g.invL * fmm::pow2<double>(D), top = fmm::pow2<double>(D);
+    const double fx = (zx - g.xmin) * sc, fy = (zy - g.ymin) * sc;
+    const bool in = fin && fx >= 0.0 && fy >= 0.0 && fx < top && fy < top;
+    key[k] = in ? spread32((uint64_t)fx) | (spread32((uint64_t)fy) << 1) : 1ull << (2 * D);
+    idx[k] = (int32_t)k;
+}
+
+// positions and weights in the sorted order
+__global__ void k_target_gather(int64_t T, const double *__restrict__ t, Rot3 R,
+                                const double *__restrict__ ub, const int32_t *__restrict__ idx,
+                                double2 *__restrict__ tz, double *__restrict__ tu)
+{
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= T) return;
+    const int64_t j = idx[k];
+    double p[3], zx, zy;
+    bool fin;
+    target_plane(t, j, R, p, zx, zy, fin);
+    tz[k] = make_double2(zx, zy);
+    tu[k] = fin ? ub[j] : 0.0;
+}
+
+// first sorted target with a key >= v
+__device__ __forceinline__ int lower_key(const uint64_t *__restrict__ key, int T, uint64_t v)
+{
+    int lo = 0, hi = T;
+    while (lo < hi) {
+        const int m = (lo + hi) >> 1;
+        if (key[m] < v) lo = m + 1;
+        else hi = m;
+    }
+    return lo;
+}
+// the targets of cell (x, y) of level l (none outside the square)
+__device__ __forceinline__ int2 cell_run(const uint64_t *__restrict__ key, int T, int D, int l, int x,
+                                         int y)
+{
+    if (x < 0 || y < 0 || x >= (1 << l) || y >= (1 << l)) return make_int2(0, 0);
+    const uint64_t k0 = (spread32((uint64_t)x) | (spread32((uint64_t)y) << 1)) << (2 * (D - l));
+    const int a = lower_key(key, T, k0);
+    return make_int2(a, lower_key(key, T, k0 + (1ull << (2 * (D - l)))));
+}
+
+// P2L of the separated cells' targets into each box, a warp per box:
+// b_l = (1/r) (-1)^l sum_t ubar_t tau_t^(l+1), tau_t = r/(c - xi_t)
+__global__ void __launch_bounds__(64)
+k_target_p2l(int64_t nbox, const int32_t *__restrict__ level, const int32_t *__restrict__ ix,
+             const int32_t *__restrict__ iy, BoxGeo g, int D, int T, const uint64_t *__restrict__ key,
+             const double2 *__restrict__ tz, const double *__restrict__ tu, cx<double> *__restrict__ loc)
+{
+    extern __shared__ __align__(16) unsigned char tp_sm[];
+    __shared__ int s_run[2][36], s_end[2][36];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    cx<double> *term_s = (cx<double> *)tp_sm + wid * kTerms * 33;
+    const int64_t b = blockIdx.x * 2ll + wid;
+    if (b >= nbox) return;
+    const int l = level[b], bx = ix[b], by = iy[b];
+    int total = 0;
+    for (int q0 = 0; q0 < 36; q0 += 32) {
+        const int q = q0 + lane;
+        int2 r = make_int2(0, 0);
+        if (l >= 2 && q < 36) {
+            const int x = 2 * ((bx >> 1) - 1) + q % 6, y = 2 * ((by >> 1) - 1) + q / 6;
+            if (abs(x - bx) > 1 || abs(y - by) > 1) r = cell_run(key, T, D, l, x, y);
+        }
+        int inc = r.y - r.x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        if (q < 36) {
+            s_end[wid][q] = total + inc;
+            s_run[wid][q] = r.x - (total + inc - (r.y - r.x));  // target = run + position
+        }
+        total += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    __syncwarp();
+    double cxd, cyd, ir;
+    box_centre_ir(g, l, bx, by, cxd, cyd, ir);
+    cx<double> s0 = mk<double>(0, 0), s1 = mk<double>(0, 0);
+    for (int base = 0; base < total; base += 32) {
+        const int at = base + lane;
+        cx<double> tau = mk<double>(0, 0), term = mk<double>(0, 0);
+        if (at < total) {
+            int q = 0;
+            while (at >= s_end[wid][q]) q++;
+            const int k = s_run[wid][q] + at;
+            const double2 z = tz[k];
+            tau = fmm::crcp(mk<double>((cxd - z.x) * ir, (cyd - z.y) * ir));
+            term = mk<double>(tu[k] * tau.x, tu[k] * tau.y);
+        }
+        for (int m = 0; m < kTerms; m++) {
+            term_s[m * 33 + lane] = (m & 1) ? mk<double>(-term.x, -term.y) : term;
+            term = fmm::cmul(term, tau);
+        }
+        __syncwarp();
+        const int n = min(32, total - base);
+        for (int m = 0; m < n; m++) {
+            s0.x += term_s[lane * 33 + m].x;
+            s0.y += term_s[lane * 33 + m].y;
+        }
+        if (lane + 32 < kTerms)
+            for (int m = 0; m < n; m++) {
+                s1.x += term_s[(lane + 32) * 33 + m].x;
+                s1.y += term_s[(lane + 32) * 33 + m].y;
+            }
+        __syncwarp();
+    }
+    loc[b * kTerms + lane] = mk<double>(s0.x * ir, s0.y * ir);
+    if (lane + 32 < kTerms) loc[b * kTerms + lane + 32] = mk<double>(s1.x * ir, s1.y * ir);
+}
+
+// S at the nodes of a leaf, a warp per leaf: the local expansion (phi = sum ubar/(z - xi_t), S2 =
+// -phi'), the targets of the cells around it, and those outside the square
+template <int Power>
+__global__ void __launch_bounds__(128)
+k_target_nodes(int64_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ level,
+               const int32_t *__restrict__ ix, const int32_t *__restrict__ iy,
+               const int32_t *__restrict__ bg, const int32_t *__restrict__ en, BoxGeo g, int D, int T,
+               const uint64_t *__restrict__ key, const double2 *__restrict__ tz,
+               const double *__restrict__ tu, const cx<double> *__restrict__ loc,
+               const double2 *__restrict__ xi, double2 *__restrict__ S)
+{
+    const int64_t w = blockIdx.x * 4ll + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (w >= nleaf) return;
+    const int b = leaves[w], l = level[b], bx = ix[b], by = iy[b];
+    // runs of the nine cells, and of the targets outside the square
+    int2 run = make_int2(0, 0);
+    if (lane < 9) run = cell_run(key, T, D, l, bx + lane % 3 - 1, by + lane / 3 - 1);
+    if (lane == 9) run = make_int2(lower_key(key, T, 1ull << (2 * D)), T);
+    double cxd, cyd, ir;
+    box_centre_ir(g, l, bx, by, cxd, cyd, ir);
+    const cx<double> *lb = loc + (int64_t)b * kTerms;
+    for (int i0 = bg[b]; i0 < en[b]; i0 += 32) {
+        const int i = i0 + lane;
+        const double2 z = xi[min(i, en[b] - 1)];
+        double2 s = make_double2(0.0, 0.0);
+        if (l >= 2) {
+            const cx<double> u = mk<double>((z.x - cxd) * ir, (z.y - cyd) * ir);
+            cx<double> h = lb[kTerms - 1];
+            if (Power == 2) h = mk<double>((kTerms - 1) * h.x, (kTerms - 1) * h.y);
+#pragma unroll 4
+            for (int m = kTerms - 2; m >= (Power == 2 ? 1 : 0); m--) {
+                const cx<double> c = lb[m];
+                h = fmm::cfma(h, u, Power == 2 ? mk<double>(m * c.x, m * c.y) : c);
+            }
+            s = Power == 2 ? make_double2(-h.x * ir, -h.y * ir) : make_double2(h.x, h.y);
+        }
+        for (int c = 0; c < 10; c++) {
+            const int a = __shfl_sync(0xffffffffu, run.x, c), e = __shfl_sync(0xffffffffu, run.y, c);
+            for (int k = a; k < e; k++) target_term<Power>(z, tz[k], tu[k], s);
+        }
+        if (i < en[b]) S[i] = s;
     }
 }
 
@@ -208,6 +412,52 @@ __global__ void k_grad_data(int64_t N, const double *__restrict__ lam, double *_
 
 }  // namespace
 
+// S of one power into S (N), scratch: the rest of the region from `free` on
+template <int Power>
+static int target_sums(lbf_plan *pl, int64_t T, const double *t, const double *ub, double2 *S,
+                       char *free, cudaStream_t s)
+{
+    const int64_t N = pl->N;
+    const Rot3 R = plan_rot(pl);
+    const Tree &Tr = pl->tree;
+    const int D = pl->opt.max_depth;
+    char *end = pl->region + pl->region_bytes;
+    auto take = [&](size_t bytes) {
+        char *p = (char *)(((uintptr_t)free + 255) & ~(uintptr_t)255);
+        free = p + bytes;
+        return p;
+    };
+    const int64_t scratch_len = 256 * lbf_cdiv(T, 1024) + T / 4 + 8192;
+    uint64_t *key = (uint64_t *)take(sizeof(uint64_t) * T), *key2 = (uint64_t *)take(sizeof(uint64_t) * T);
+    int32_t *idx = (int32_t *)take(sizeof(int32_t) * T), *idx2 = (int32_t *)take(sizeof(int32_t) * T);
+    double2 *tz = (double2 *)take(sizeof(double2) * T);
+    double *tu = (double *)take(sizeof(double) * T);
+    int32_t *scratch = (int32_t *)take(sizeof(int32_t) * scratch_len);
+    cx<double> *loc = (cx<double> *)take(sizeof(cx<double>) * Tr.nbox * kTerms);
+    if (pl->opt.matvec != LBF_MATVEC_FMM || T <= kDirectPairs / N || T > INT32_MAX / 2 || free > end ||
+        !pl->pull) {
+        LBF_LAUNCH(k_node_target<Power>, lbf_cdiv(N, 256), 256, 0, s, N, pl->xi, T, t, R, ub, S);
+        LBF_CHECK_LAUNCH();
+        return LBF_OK;
+    }
+    const BoxGeo g{Tr.xmin, Tr.ymin, Tr.L, (float)(1.0 / Tr.L), df64(1.0 / Tr.L), 1.0 / Tr.L};
+    LBF_LAUNCH(k_target_keys, lbf_cdiv(T, 256), 256, 0, s, T, t, R, g, D, key, idx);
+    LBF_CHECK_LAUNCH();
+    int rc = lbf_radix_sort(key, key2, idx, idx2, T, 2 * D + 1, scratch, scratch_len, s);
+    if (rc) return rc;
+    constexpr int smem = 2 * kTerms * 33 * (int)sizeof(cx<double>);
+    LBF_CUDA(cudaFuncSetAttribute(k_target_p2l, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    LBF_LAUNCH(k_target_gather, lbf_cdiv(T, 256), 256, 0, s, T, t, R, ub, idx, tz, tu);
+    LBF_LAUNCH(k_target_p2l, lbf_cdiv(Tr.nbox, 2), 64, smem, s, Tr.nbox, Tr.level, Tr.ix, Tr.iy, g, D,
+               (int)T, key, tz, tu, loc);
+    LBF_CHECK_LAUNCH();
+    if ((rc = lbf_mp_shift_down(pl, kTerms, (double2 *)loc, s))) return rc;
+    LBF_LAUNCH(k_target_nodes<Power>, lbf_cdiv(Tr.nleaf, 4), 128, 0, s, Tr.nleaf, Tr.leaves, Tr.level, Tr.ix,
+               Tr.iy, Tr.begin, Tr.end, g, D, (int)T, key, tz, tu, loc, pl->xi, S);
+    LBF_CHECK_LAUNCH();
+    return LBF_OK;
+}
+
 int lbf_gradient_data_impl(lbf_plan *pl, const double *lam, double *grad_g, cudaStream_t s)
 {
     if (pl->N > 0) LBF_LAUNCH(k_grad_data, lbf_cdiv(pl->N, 256), 256, 0, s, pl->N, lam, grad_g);
@@ -221,12 +471,13 @@ int lbf_evaluate_transpose_impl(lbf_plan *pl, int64_t T, const double *t, const 
     int64_t N = pl->N;
     int M = pl->M;
     // scratch: the GMRES basis region (unused outside a solve)
-    double2 *S1 = (double2 *)pl->region, *S2 = S1 + N;
-    double *sums = (double *)(S2 + N);
+    double2 *S1 = (double2 *)pl->region;
+    double *sums = (double *)(S1 + N);
     Rot3 R = plan_rot(pl);
     LBF_LAUNCH(k_sums3, 1, 1024, 0, s, T, ub, N, (const double *)nullptr, M,
                (const double *)nullptr, sums);
-    LBF_LAUNCH(k_node_target, lbf_cdiv(N, 256), 256, 0, s, N, pl->xi, T, t, R, ub, S1, S2);
+    const int rc = target_sums<1>(pl, T, t, ub, S1, (char *)(sums + 8), s);
+    if (rc) return rc;
     LBF_LAUNCH(k_sbar, lbf_cdiv(N, 256), 256, 0, s, N, pl->perm, pl->w, pl->beta, S1, sums, sbar);
     if (abar) LBF_LAUNCH(k_abar, lbf_cdiv((int64_t)M * 32, 256), 256, 0, s, M, pl->centres, T, t, R, ub, abar);
     LBF_CHECK_LAUNCH();
@@ -239,15 +490,14 @@ int lbf_gradient_nodes_impl(lbf_plan *pl, const double *sigma, const double *a, 
 {
     int64_t N = pl->N;
     int M = pl->M;
-    double2 *S1 = (double2 *)pl->region, *S2 = S1 + N, *Dl = S2 + N, *Dq = Dl + N, *Eg = Dq + N;
+    double2 *S2 = (double2 *)pl->region, *Dl = S2 + N, *Dq = Dl + N, *Eg = Dq + N;
     double *sg = (double *)(Eg + N), *lm = sg + N, *sums = lm + N;
-    Rot3 R = plan_rot(pl);
     int rc;
     if ((rc = lbf_permute_in(pl, sigma, sg, 0, s)) || (rc = lbf_permute_in(pl, lam, lm, 0, s)))
         return rc;
     LBF_LAUNCH(k_sums3, 1, 1024, 0, s, T, ub, N, lm, M, a, sums);
-    LBF_LAUNCH(k_node_target, lbf_cdiv(N, 256), 256, 0, s, N, pl->xi, T, t, R, ub, S1, S2);
     LBF_CHECK_LAUNCH();
+    if ((rc = target_sums<2>(pl, T, t, ub, S2, (char *)(sums + 8), s))) return rc;
     if ((rc = lbf_cauchy_deriv(pl, lm, false, Dl, s))) return rc;
     if ((rc = lbf_cauchy_deriv(pl, sg, true, Dq, s))) return rc;
     if ((rc = lbf_mp_gradient(pl, a, Eg, s))) return rc;

@@ -1399,6 +1399,19 @@ int lbf_mp_apply_transpose(lbf_plan *pl, const double *tau, double sc, const dou
     return LBF_OK;
 }
 
+int lbf_mp_shift_down(lbf_plan *pl, int P, double2 *loc, cudaStream_t s)
+{
+    const Tree &T = pl->tree;
+    const int cw = 8;
+    const int64_t grid = std::min<int64_t>(lbf_cdiv(T.nbox, cw), 4 * (int64_t)std::max(pl->nsm, 1));
+    LBF_CUDA(cudaFuncSetAttribute(k_mp_chain<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    LBF_LAUNCH(k_mp_chain<double>, grid, 32 * cw, l2l_smem<double>(P, cw), s, T.nbox, P, T.parent, T.level,
+               T.ix, T.iy, pl->tab_binom, (const cz<double> *)pl->tab_dshift, (cz<double> *)loc, pl->pull,
+               pl->dev_status, (const int *)nullptr, (int64_t)0);
+    LBF_CHECK_LAUNCH();
+    return LBF_OK;
+}
+
 // out_i = grad_i (E y)_i (sorted order, N double2), FP64
 int lbf_mp_gradient(lbf_plan *pl, const double *y, double2 *out, cudaStream_t s)
 {

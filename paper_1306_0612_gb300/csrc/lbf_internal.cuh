@@ -319,6 +319,8 @@ int lbf_mp_apply(lbf_plan *pl, const double *y, const double *x, const double *v
 int lbf_mp_apply_transpose(lbf_plan *pl, const double *tau, double sc, const double *add,
                            double *out, const int *gate, cudaStream_t s);
 // out_i = gradient of (E y)_i with respect to (Re xi_i, Im xi_i), sorted order, FP64
+// L2L of the expansions loc (nbox x P, P <= LBF_MAX_TERMS) from level 3 on, in place
+int lbf_mp_shift_down(lbf_plan *pl, int P, double2 *loc, cudaStream_t s);
 int lbf_mp_gradient(lbf_plan *pl, const double *y, double2 *out, cudaStream_t s);
 int lbf_geometry_out_impl(const lbf_plan *pl, double *xi, double *normal, double *weight,
                           double *arc, cudaStream_t s);
@@ -379,14 +381,14 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
 int lbf_passes_init_attrs();
 bool lbf_passes_ready(const lbf_plan *pl);
 int lbf_passes_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch);
-int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s);
-int lbf_evaluate_impl(lbf_plan *pl, const double *sigma_sorted, const double *a, int64_t T,
 int lbf_passes_up(lbf_plan *pl, const int *gate, cudaStream_t s);
-                      const double *t, double *u, cudaStream_t s);
+int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s);
 // off-curve evaluation (lbf_evaluate.cu); its charges, and its charges and double multipoles
 int lbf_eval_charges(lbf_plan *pl, const double *sigma, cudaStream_t s);
 int lbf_eval_multipoles(lbf_plan *pl, const double *sigma, cudaStream_t s);
 int lbf_evaluate_init_attrs();
+int lbf_evaluate_impl(lbf_plan *pl, const double *sigma_sorted, const double *a, int64_t T,
+                      const double *t, double *u, cudaStream_t s);
 int lbf_green_sum_impl(int64_t T, const double *t, int64_t S, const double *p,
                        const double *gamma, double *out, cudaStream_t s);
 
