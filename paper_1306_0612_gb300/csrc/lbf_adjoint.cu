@@ -58,8 +58,8 @@ __device__ __forceinline__ void target_plane(const double *t, int64_t k, const R
 // cells), the expansions are shifted down, and a leaf adds the targets of the 3 x 3 cells around
 // it directly.  Nothing of it goes through the host, so the call stays asynchronous.  A
 // target is at least 3 half-widths from a box's centre, its nodes at most sqrt 2: kTerms = 48
-// terms leave (sqrt 2/3)^48 = 2e-16.  At 131,072 nodes and 4096 targets 21.3 ms of pairs (the
-// double pipe, 40 instructions a pair with the division) to 0.5 ms.
+// terms leave (sqrt 2/3)^48 = 2e-16.  At 131,072 nodes and 4096 targets 21.3 ms of pairs (both
+// powers, with a division) a call to 1.9 ms, 0.7 of it P2L, 0.4 the shifts.
 constexpr int64_t kDirectPairs = 1 << 24;
 constexpr int kTerms = 48;
 
@@ -171,50 +171,54 @@ __device__ __forceinline__ int2 cell_run(const uint64_t *__restrict__ key, int T
     return make_int2(a, lower_key(key, T, k0 + (1ull << (2 * (D - l)))));
 }
 
-// P2L of the separated cells' targets into each box, a warp per box:
+// P2L of the separated cells' targets into each box, a thread block of four warps per box, the
+// targets' chunks of 32 dealt to the warps in turn:
 // b_l = (1/r) (-1)^l sum_t ubar_t tau_t^(l+1), tau_t = r/(c - xi_t)
-__global__ void __launch_bounds__(64)
-k_target_p2l(int64_t nbox, const int32_t *__restrict__ level, const int32_t *__restrict__ ix,
+__global__ void __launch_bounds__(128)
+k_target_p2l(const int32_t *__restrict__ level, const int32_t *__restrict__ ix,
              const int32_t *__restrict__ iy, BoxGeo g, int D, int T, const uint64_t *__restrict__ key,
              const double2 *__restrict__ tz, const double *__restrict__ tu, cx<double> *__restrict__ loc)
 {
     extern __shared__ __align__(16) unsigned char tp_sm[];
-    __shared__ int s_run[2][36], s_end[2][36];
+    __shared__ int s_run[36], s_end[36], s_total;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     cx<double> *term_s = (cx<double> *)tp_sm + wid * kTerms * 33;
-    const int64_t b = blockIdx.x * 2ll + wid;
-    if (b >= nbox) return;
+    const int64_t b = blockIdx.x;
     const int l = level[b], bx = ix[b], by = iy[b];
-    int total = 0;
-    for (int q0 = 0; q0 < 36; q0 += 32) {
-        const int q = q0 + lane;
-        int2 r = make_int2(0, 0);
-        if (l >= 2 && q < 36) {
-            const int x = 2 * ((bx >> 1) - 1) + q % 6, y = 2 * ((by >> 1) - 1) + q / 6;
-            if (abs(x - bx) > 1 || abs(y - by) > 1) r = cell_run(key, T, D, l, x, y);
+    if (wid == 0) {
+        int total = 0;
+        for (int q0 = 0; q0 < 36; q0 += 32) {
+            const int q = q0 + lane;
+            int2 r = make_int2(0, 0);
+            if (l >= 2 && q < 36) {
+                const int x = 2 * ((bx >> 1) - 1) + q % 6, y = 2 * ((by >> 1) - 1) + q / 6;
+                if (abs(x - bx) > 1 || abs(y - by) > 1) r = cell_run(key, T, D, l, x, y);
+            }
+            int inc = r.y - r.x;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += v;
+            }
+            if (q < 36) {
+                s_end[q] = total + inc;
+                s_run[q] = r.x - (total + inc - (r.y - r.x));  // target = run + position
+            }
+            total += __shfl_sync(0xffffffffu, inc, 31);
         }
-        int inc = r.y - r.x;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += v;
-        }
-        if (q < 36) {
-            s_end[wid][q] = total + inc;
-            s_run[wid][q] = r.x - (total + inc - (r.y - r.x));  // target = run + position
-        }
-        total += __shfl_sync(0xffffffffu, inc, 31);
+        if (lane == 0) s_total = total;
     }
-    __syncwarp();
+    __syncthreads();
+    const int total = s_total;
     double cxd, cyd, ir;
     box_centre_ir(g, l, bx, by, cxd, cyd, ir);
     cx<double> s0 = mk<double>(0, 0), s1 = mk<double>(0, 0);
-    for (int base = 0; base < total; base += 32) {
+    for (int base = 32 * wid; base < total; base += 128) {
         const int at = base + lane;
         cx<double> tau = mk<double>(0, 0), term = mk<double>(0, 0);
         if (at < total) {
             int q = 0;
-            while (at >= s_end[wid][q]) q++;
-            const int k = s_run[wid][q] + at;
+            while (at >= s_end[q]) q++;
+            const int k = s_run[q] + at;
             const double2 z = tz[k];
             tau = fmm::crcp(mk<double>((cxd - z.x) * ir, (cyd - z.y) * ir));
             term = mk<double>(tu[k] * tau.x, tu[k] * tau.y);
@@ -236,52 +240,75 @@ k_target_p2l(int64_t nbox, const int32_t *__restrict__ level, const int32_t *__r
             }
         __syncwarp();
     }
-    loc[b * kTerms + lane] = mk<double>(s0.x * ir, s0.y * ir);
-    if (lane + 32 < kTerms) loc[b * kTerms + lane + 32] = mk<double>(s1.x * ir, s1.y * ir);
+    // the warps' sums, through the terms' memory
+    term_s[lane] = s0;
+    if (lane + 32 < kTerms) term_s[lane + 32] = s1;
+    __syncthreads();
+    if (threadIdx.x < kTerms) {
+        const cx<double> *p = (const cx<double> *)tp_sm + threadIdx.x;
+        cx<double> s = p[0];
+        for (int w = 1; w < 4; w++) {
+            s.x += p[w * kTerms * 33].x;
+            s.y += p[w * kTerms * 33].y;
+        }
+        loc[b * kTerms + threadIdx.x] = mk<double>(s.x * ir, s.y * ir);
+    }
 }
 
-// S at the nodes of a leaf, a warp per leaf: the local expansion (phi = sum ubar/(z - xi_t), S2 =
-// -phi'), the targets of the cells around it, and those outside the square
+// S at the nodes of a leaf, a thread block of four warps per leaf: the targets of the cells
+// around it and those outside the square (a large leaf between large empty cells has
+// thousands), and the local expansion (phi = sum ubar/(z - xi_t), S2 = -phi').  A chunk of 32
+// nodes at a time: TP >= n lanes on the nodes, 128 / TP groups of lanes on every so many of the
+// targets, their sums added in order.
 template <int Power>
 __global__ void __launch_bounds__(128)
-k_target_nodes(int64_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ level,
+k_target_nodes(const int32_t *__restrict__ leaves, const int32_t *__restrict__ level,
                const int32_t *__restrict__ ix, const int32_t *__restrict__ iy,
                const int32_t *__restrict__ bg, const int32_t *__restrict__ en, BoxGeo g, int D, int T,
                const uint64_t *__restrict__ key, const double2 *__restrict__ tz,
                const double *__restrict__ tu, const cx<double> *__restrict__ loc,
                const double2 *__restrict__ xi, double2 *__restrict__ S)
 {
-    const int64_t w = blockIdx.x * 4ll + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (w >= nleaf) return;
-    const int b = leaves[w], l = level[b], bx = ix[b], by = iy[b];
+    __shared__ int2 run[10];
+    __shared__ double2 part[128];
+    const int b = leaves[blockIdx.x], l = level[b], bx = ix[b], by = iy[b], tid = threadIdx.x;
     // runs of the nine cells, and of the targets outside the square
-    int2 run = make_int2(0, 0);
-    if (lane < 9) run = cell_run(key, T, D, l, bx + lane % 3 - 1, by + lane / 3 - 1);
-    if (lane == 9) run = make_int2(lower_key(key, T, 1ull << (2 * D)), T);
+    if (tid < 9) run[tid] = cell_run(key, T, D, l, bx + tid % 3 - 1, by + tid / 3 - 1);
+    if (tid == 9) run[9] = make_int2(lower_key(key, T, 1ull << (2 * D)), T);
+    __syncthreads();
     double cxd, cyd, ir;
     box_centre_ir(g, l, bx, by, cxd, cyd, ir);
     const cx<double> *lb = loc + (int64_t)b * kTerms;
     for (int i0 = bg[b]; i0 < en[b]; i0 += 32) {
-        const int i = i0 + lane;
-        const double2 z = xi[min(i, en[b] - 1)];
+        const int n = min(32, en[b] - i0);
+        const int TP = n <= 1 ? 1 : 1 << (32 - __clz(n - 1)), G = 128 / TP;
+        const int r = tid & (TP - 1), grp = tid / TP;
+        const double2 z = xi[i0 + min(r, n - 1)];
         double2 s = make_double2(0.0, 0.0);
-        if (l >= 2) {
-            const cx<double> u = mk<double>((z.x - cxd) * ir, (z.y - cyd) * ir);
-            cx<double> h = lb[kTerms - 1];
-            if (Power == 2) h = mk<double>((kTerms - 1) * h.x, (kTerms - 1) * h.y);
-#pragma unroll 4
-            for (int m = kTerms - 2; m >= (Power == 2 ? 1 : 0); m--) {
-                const cx<double> c = lb[m];
-                h = fmm::cfma(h, u, Power == 2 ? mk<double>(m * c.x, m * c.y) : c);
+        for (int c = 0; c < 10; c++)
+            for (int k = run[c].x + grp; k < run[c].y; k += G) target_term<Power>(z, tz[k], tu[k], s);
+        part[tid] = s;
+        __syncthreads();
+        if (tid < n) {
+            for (int w = 1; w < G; w++) {
+                s.x += part[w * TP + tid].x;
+                s.y += part[w * TP + tid].y;
             }
-            s = Power == 2 ? make_double2(-h.x * ir, -h.y * ir) : make_double2(h.x, h.y);
+            if (l >= 2) {
+                const cx<double> u = mk<double>((z.x - cxd) * ir, (z.y - cyd) * ir);
+                cx<double> h = lb[kTerms - 1];
+                if (Power == 2) h = mk<double>((kTerms - 1) * h.x, (kTerms - 1) * h.y);
+#pragma unroll 4
+                for (int m = kTerms - 2; m >= (Power == 2 ? 1 : 0); m--) {
+                    const cx<double> c = lb[m];
+                    h = fmm::cfma(h, u, Power == 2 ? mk<double>(m * c.x, m * c.y) : c);
+                }
+                s = Power == 2 ? make_double2(s.x - h.x * ir, s.y - h.y * ir)
+                               : make_double2(s.x + h.x, s.y + h.y);
+            }
+            S[i0 + tid] = s;
         }
-        for (int c = 0; c < 10; c++) {
-            const int a = __shfl_sync(0xffffffffu, run.x, c), e = __shfl_sync(0xffffffffu, run.y, c);
-            for (int k = a; k < e; k++) target_term<Power>(z, tz[k], tu[k], s);
-        }
-        if (i < en[b]) S[i] = s;
+        __syncthreads();
     }
 }
 
@@ -445,15 +472,14 @@ static int target_sums(lbf_plan *pl, int64_t T, const double *t, const double *u
     LBF_CHECK_LAUNCH();
     int rc = lbf_radix_sort(key, key2, idx, idx2, T, 2 * D + 1, scratch, scratch_len, s);
     if (rc) return rc;
-    constexpr int smem = 2 * kTerms * 33 * (int)sizeof(cx<double>);
+    constexpr int smem = 4 * kTerms * 33 * (int)sizeof(cx<double>);
     LBF_CUDA(cudaFuncSetAttribute(k_target_p2l, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     LBF_LAUNCH(k_target_gather, lbf_cdiv(T, 256), 256, 0, s, T, t, R, ub, idx, tz, tu);
-    LBF_LAUNCH(k_target_p2l, lbf_cdiv(Tr.nbox, 2), 64, smem, s, Tr.nbox, Tr.level, Tr.ix, Tr.iy, g, D,
-               (int)T, key, tz, tu, loc);
+    LBF_LAUNCH(k_target_p2l, Tr.nbox, 128, smem, s, Tr.level, Tr.ix, Tr.iy, g, D, (int)T, key, tz, tu, loc);
     LBF_CHECK_LAUNCH();
     if ((rc = lbf_mp_shift_down(pl, kTerms, (double2 *)loc, s))) return rc;
-    LBF_LAUNCH(k_target_nodes<Power>, lbf_cdiv(Tr.nleaf, 4), 128, 0, s, Tr.nleaf, Tr.leaves, Tr.level, Tr.ix,
-               Tr.iy, Tr.begin, Tr.end, g, D, (int)T, key, tz, tu, loc, pl->xi, S);
+    LBF_LAUNCH(k_target_nodes<Power>, Tr.nleaf, 128, 0, s, Tr.leaves, Tr.level, Tr.ix, Tr.iy,
+                Tr.begin, Tr.end, g, D, (int)T, key, tz, tu, loc, pl->xi, S);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }

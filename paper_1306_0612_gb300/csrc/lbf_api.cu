@@ -264,6 +264,7 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
     pl->V = o.border ? (double *)pl->region : nullptr;
     lbf_m2l_layout(pl, o, cap);
     lbf_emat_layout(pl, N, M, o);
+    if (o.border) lbf_mp_layout_pairs(pl, M);
     lbf_rows_layout(pl, N, o, cap);
 }
 

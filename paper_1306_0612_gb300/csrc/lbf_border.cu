@@ -943,6 +943,36 @@ __global__ void k_zero_i32(int32_t *p, int64_t n)
     if (i < n) p[i] = 0;
 }
 
+// The P coefficients of every (box, centre) pair's P2L at unit strength, a thread per pair
+// (box from the lists' offsets by bisection): c_0 = log|c - xi_m|, c_l = (-1)^(l+1) tau^l / l.
+__global__ void k_mp_pair_exp(int64_t npair, int64_t nbox, int P, const int32_t *__restrict__ ptr,
+                              const int32_t *__restrict__ src, const int32_t *__restrict__ level,
+                              const int32_t *__restrict__ ix, const int32_t *__restrict__ iy, Geo g,
+                              const double2 *__restrict__ xc, cz<double> *__restrict__ out)
+{
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q >= npair) return;
+    int64_t lo = 0, hi = nbox - 1;  // the last box whose list starts at or before q
+    while (lo < hi) {
+        const int64_t m = (lo + hi + 1) >> 1;
+        if (ptr[m] <= q) lo = m;
+        else hi = m - 1;
+    }
+    double cx, cy, r;
+    centre_of(g, level[lo], ix[lo], iy[lo], cx, cy, r);
+    const double ir = 1.0 / r;
+    const double2 xm = xc[src[q]];
+    const double dx = cx - xm.x, dy = cy - xm.y;
+    const cz<double> tau = zinv(cz<double>{dx * ir, dy * ir});
+    cz<double> *o = out + q * P, pw = tau;
+    o[0] = cz<double>{0.5 * log(dx * dx + dy * dy), 0.0};
+    for (int l = 1; l < P; l++) {
+        const double f = ((l & 1) ? 1.0 : -1.0) / l;
+        o[l] = cz<double>{pw.x * f, pw.y * f};
+        pw = zmul(pw, tau);
+    }
+}
+
 template <typename R> size_t l2l_smem(int P, int wpb)
 {
     return (P * P * sizeof(R) + 15) / 16 * 16 + sizeof(cz<R>) * (size_t)wpb * 2 * P;
@@ -1114,7 +1144,34 @@ int lbf_mp_build(lbf_plan *pl, cudaStream_t s, int32_t *work, int64_t work_len, 
         B.npartial = np;
         if (B.npartial > B.partial_cap) return LBF_EWORKSPACE;
     }
+    if (n_p2l > B.p2l_exp_cap) B.p2l_exp = nullptr;
+    if (B.p2l_exp && n_p2l > 0) {
+        LBF_LAUNCH(k_mp_pair_exp, lbf_cdiv(n_p2l, 128), 128, 0, s, n_p2l, T.nbox, B.Pe, B.p2l_ptr, B.p2l_src,
+                   T.level, T.ix, T.iy, g, B.xc, (cz<double> *)B.p2l_exp);
+        LBF_CHECK_LAUNCH();
+    }
     return lbf_emat_build(pl, s);
+}
+
+// 400 pairs a centre (measured 320 at 16,384 islands, 190 at 407): 200 kB of 512-byte
+// expansions each
+void lbf_mp_layout_pairs(lbf_plan *pl, int M)
+{
+    Border &B = pl->bd;
+    B.p2l_exp = nullptr;
+    B.p2l_exp_cap = 0;
+    if (B.use_E) return;  // E y needs no expansions
+    Arena &A = pl->arena;
+    const size_t off = A.off;
+    const bool full = A.overflow;
+    B.p2l_exp_cap = std::min<int64_t>(400 * (int64_t)M, B.pair_cap);
+    B.p2l_exp = A.get<double2>(B.p2l_exp_cap * B.Pe);
+    if (A.overflow && !full) {
+        A.off = off;
+        A.overflow = false;
+        B.p2l_exp_cap = 0;
+        B.p2l_exp = nullptr;
+    }
 }
 
 // out = x + v + s E y (Morton order; v nullable) in precision prec.
@@ -1157,6 +1214,19 @@ int lbf_mp_apply(lbf_plan *pl, const double *y, const double *x, const double *v
                      B.ell, B.sums, x, v, sc, out, gate, pl->anc, pl->u32, chain ? 0 : 1,
                      chain ? (const cz<float> *)pl->u32 : (const cz<float> *)nullptr, B.nodebase,
                      B.partial, pl->slab);
+    } else if (B.p2l_exp && pl->pull) {
+        // stored expansions, double whatever opt.fmm64 says
+        const int rc = lbf_mp_chain_apply(pl, y, gate, s);
+        if (rc) return rc;
+        if (B.nchunks)
+            LBF_LAUNCH(k_mp_near<double>, lbf_grid(pl, lbf_cdiv(B.nchunks, 8)), 256, 0, s, B.nchunks,
+                       B.chunk_leaf, B.chunk_k, B.near_ptr, B.near_src, T.begin, T.end, pl->xi,
+                       B.xc, y, B.nodebase, B.partial, gate, pl->slab);
+        LBF_LAUNCH_P(LBF_KERNEL_ESUM, k_mp_eval<double>, lbf_grid(pl, lbf_cdiv(pl->N, 256)), 256, 0,
+                     s, pl->N, B.Pe, pl->xi, B.leaf_of, T.level, T.ix, T.iy, g,
+                     (const cz<double> *)B.loc, B.near_ptr, B.near_src, B.glob, B.nglob_h, B.xc, y,
+                     B.ell, B.sums, x, v, sc, out, gate, T.parent, (const float2 *)nullptr, 0,
+                     (const cz<double> *)nullptr, B.nodebase, B.partial, pl->slab);
     } else if (pl->udf) {
         // the accurate operator in double-float (P2L terms formed in double)
         int P = B.Pe;

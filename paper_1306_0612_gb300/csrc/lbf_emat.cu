@@ -160,6 +160,7 @@ void lbf_emat_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o)
 {
     Border &B = pl->bd;
     B.E = nullptr;
+    B.use_E = false;
     B.nch = (M + 7) / 8;
     if (!o.border || M > kEmatIslands || N * (int64_t)M > kEmatEntries) return;
     Arena &A = pl->arena;
@@ -170,6 +171,8 @@ void lbf_emat_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o)
         A.off = off;
         A.overflow = false;
         B.E = nullptr;
+    } else {
+        B.use_E = true;
     }
 }
 

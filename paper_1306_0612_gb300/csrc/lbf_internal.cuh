@@ -108,6 +108,9 @@ struct Border {
     int32_t *cp2l = nullptr, *cnear = nullptr;  // per centre: offsets into pairs_a / pairs_b (M + 1)
     double *E = nullptr;             // E itself for a few hundred islands (lbf_emat.cu), or null
     int nch = 0;                     // its chunks of eight centres
+    bool use_E = false;              // whether the layout holds E
+    double2 *p2l_exp = nullptr;      // Pe coefficients of each (box, centre) pair at y = 1, or null
+    int64_t p2l_exp_cap = 0;         // room, in pairs
     double2 *loc = nullptr;          // local expansions of the log potential, box x P
     float2 *loc32 = nullptr;         // box x P32
     double2 *zc = nullptr;           // island node means
@@ -319,6 +322,8 @@ int lbf_mp_apply(lbf_plan *pl, const double *y, const double *x, const double *v
 int lbf_mp_apply_transpose(lbf_plan *pl, const double *tau, double sc, const double *add,
                            double *out, const int *gate, cudaStream_t s);
 // out_i = gradient of (E y)_i with respect to (Re xi_i, Im xi_i), sorted order, FP64
+// room for the (box, centre) pairs' expansions, dropped when the workspace has none
+void lbf_mp_layout_pairs(lbf_plan *pl, int M);
 // L2L of the expansions loc (nbox x P, P <= LBF_MAX_TERMS) from level 3 on, in place
 int lbf_mp_shift_down(lbf_plan *pl, int P, double2 *loc, cudaStream_t s);
 int lbf_mp_gradient(lbf_plan *pl, const double *y, double2 *out, cudaStream_t s);
@@ -381,6 +386,7 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
 int lbf_passes_init_attrs();
 bool lbf_passes_ready(const lbf_plan *pl);
 int lbf_passes_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch);
+int lbf_mp_chain_apply(lbf_plan *pl, const double *y, const int *gate, cudaStream_t s);
 int lbf_passes_up(lbf_plan *pl, const int *gate, cudaStream_t s);
 int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s);
 // off-curve evaluation (lbf_evaluate.cu); its charges, and its charges and double multipoles

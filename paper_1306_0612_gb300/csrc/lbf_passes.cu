@@ -6,7 +6,8 @@
 //   k_p2l_big   P2L of the few boxes whose X lists are not near columns;
 //   k_l2l       each box's translations added up and its parent's expansion shifted to it,
 //               in one launch: warps take the boxes in index order and wait (bounded) for
-//               the parent, which a running warp took earlier.
+//               the parent, which a running warp took earlier; also the chain of the
+//               multiplier potential's expansions.
 //
 // P2M: with the stored powers a node and coefficient take two multiply-adds a real where
 // the recurrence took six double instructions and left the lanes past a leaf's last node
@@ -235,20 +236,83 @@ k_p2l_big(int n, const int32_t *__restrict__ list, const int32_t *__restrict__ l
 
 constexpr unsigned kL2lSpins = 1u << 24;
 
-// Every box's local expansion: its translations (list order), its P2L part where it has
-// one (in loc already), and from level 3 on its parent's expansion shifted down,
+// What a box's expansion takes beside its parent's: of the density block its translations and
+// its P2L part where it has one (in loc already); of the multiplier potential (lbf_border.cu)
+// the stored expansions of its centres times their strengths y.
+struct Own {
+    const int32_t *ptr;        // first translation, or first (box, centre) pair, of each box
+    const cx<double> *part;    // P coefficients each
+    const int32_t *src;        // the pairs' centres (null: translations, with weight 1 / r)
+    const double *y;
+    const int32_t *bg, *en, *nx;
+    int thr;
+    double *sums;              // pairs: [0] = sum y, [1] = sum of y lam over the finite centres
+    const int32_t *kind;
+    const double *lam;
+    int M;
+};
+
+__device__ __forceinline__ cx<double> own_part(const Own &w, int64_t b, int P, int lane, int v0, int dv,
+                                               double ir, const cx<double> *loc)
+{
+    cx<double> o = mk<double>(0, 0);
+    if (lane >= P) return o;
+    const int v1 = w.ptr[b + 1];
+    if (w.src) {
+#pragma unroll 4
+        for (int v = w.ptr[b] + v0; v < v1; v += dv) {
+            const cx<double> a = w.part[(int64_t)v * P + lane];
+            const double y = w.y[w.src[v]];
+            o.x = fma(y, a.x, o.x);
+            o.y = fma(y, a.y, o.y);
+        }
+        return o;
+    }
+#pragma unroll 4
+    for (int v = w.ptr[b] + v0; v < v1; v += dv) {
+        const cx<double> a = w.part[(int64_t)v * P + lane];
+        o.x += a.x;
+        o.y += a.y;
+    }
+    o.x *= ir;
+    o.y *= ir;
+    if (v0 == 0 && w.nx[b] && w.en[b] - w.bg[b] > w.thr) {
+        const cx<double> x = fmm::ldcg_cx(&loc[b * P + lane]);
+        o.x += x.x;
+        o.y += x.y;
+    }
+    return o;
+}
+
+// the sums of the strengths, by the warp that has box 0
+__device__ __forceinline__ void strength_sums(const Own &w, int lane)
+{
+    double Y = 0.0, Lam = 0.0;
+    for (int m = lane; m < w.M; m += 32) {
+        Y += w.y[m];
+        if (w.kind[m]) Lam = fma(w.y[m], w.lam[m], Lam);
+    }
+    Y = fmm::wsum(Y);
+    Lam = fmm::wsum(Lam);
+    if (lane == 0) {
+        w.sums[0] = Y;
+        w.sums[1] = Lam;
+    }
+}
+
+// Every box's local expansion: its own part, and from level 3 on its parent's expansion
+// shifted down,
 //   b'_l = (2d)^-l sum_{k >= l} C(k, l) d^k b_k.
 // pull: the words of k_down's chain ([1] finished warps, [2] epoch, [3] box counter, then
 // nbox words unused here and nbox epochs in which a box was finished).
 __global__ void __launch_bounds__(256)
 k_l2l(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_t *__restrict__ ix,
-      const int32_t *__restrict__ iy, const int32_t *__restrict__ parent,
-      const int32_t *__restrict__ bg, const int32_t *__restrict__ en, const int32_t *__restrict__ nx,
-      int thr, const int32_t *__restrict__ vptr, const cx<double> *__restrict__ trans, BoxGeo g,
+      const int32_t *__restrict__ iy, const int32_t *__restrict__ parent, Own w, BoxGeo g,
       const double *__restrict__ binom, const cx<double> *__restrict__ dtab, cx<double> *loc,
       unsigned *pull, int *status, const int *gate, int64_t slab)
 {
-    lbf_rhs(slab, trans, loc, pull, gate);
+    lbf_rhs(slab, loc, pull, gate, w.y, w.sums);
+    if (!w.src) lbf_rhs(slab, w.part);
     if (fmm::gate_closed(gate)) return;
     __shared__ double Cd[32 * 32];
     __shared__ cx<double> As[8][32];
@@ -273,24 +337,9 @@ k_l2l(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_t *__r
         if (lane == 0) bi = atomicAdd(&pull[3], 1u);
         const int64_t b = (int64_t)__shfl_sync(0xffffffffu, bi, 0);
         if (b >= nbox) break;
-        const int lv = level[b], p = parent[b], v0 = vptr[b], v1 = vptr[b + 1];
-        cx<double> own = mk<double>(0, 0);
-        if (lane < P) {
-#pragma unroll 4
-            for (int v = v0; v < v1; v++) {
-                const cx<double> a = trans[(int64_t)v * P + lane];
-                own.x += a.x;
-                own.y += a.y;
-            }
-            const double ir = g.invL * fmm::pow2<double>(lv + 1);
-            own.x *= ir;
-            own.y *= ir;
-            if (nx[b] && en[b] - bg[b] > thr) {
-                const cx<double> x = fmm::ldcg_cx(&loc[b * P + lane]);
-                own.x += x.x;
-                own.y += x.y;
-            }
-        }
+        const int lv = level[b], p = parent[b];
+        if (w.sums && b == 0) strength_sums(w, lane);
+        const cx<double> own = own_part(w, b, P, lane, 0, 1, g.invL * fmm::pow2<double>(lv + 1), loc);
         if (lv >= 3) {
             const int d = (ix[b] & 1) + 2 * (iy[b] & 1);
             const cx<double> *dp = fmm::dpow(dtab, d), *inv = fmm::d2inv(dtab, d);
@@ -439,14 +488,12 @@ k_up_small(const int32_t *__restrict__ leaves, const int32_t *__restrict__ ix,
 // parent together, and take a quarter of the shift's terms each (a half-warp an eighth).
 __global__ void __launch_bounds__(128)
 k_l2l_small(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_t *__restrict__ ix,
-            const int32_t *__restrict__ iy, const int32_t *__restrict__ parent,
-            const int32_t *__restrict__ bg, const int32_t *__restrict__ en,
-            const int32_t *__restrict__ nx, int thr, const int32_t *__restrict__ vptr,
-            const cx<double> *__restrict__ trans, BoxGeo g, const double *__restrict__ binom,
-            const cx<double> *__restrict__ dtab, cx<double> *loc, unsigned *pull, int *status,
-            const int *gate, int64_t slab)
+            const int32_t *__restrict__ iy, const int32_t *__restrict__ parent, Own w, BoxGeo g,
+            const double *__restrict__ binom, const cx<double> *__restrict__ dtab, cx<double> *loc,
+            unsigned *pull, int *status, const int *gate, int64_t slab)
 {
-    lbf_rhs(slab, trans, loc, pull, gate);
+    lbf_rhs(slab, loc, pull, gate, w.y, w.sums);
+    if (!w.src) lbf_rhs(slab, w.part);
     if (fmm::gate_closed(gate)) return;
     __shared__ double Cd[32 * 32];
     __shared__ cx<double> As[4][32], part[4][32], own[4][32];
@@ -468,26 +515,11 @@ k_l2l_small(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_
         const int64_t b = (int64_t)s_ticket;
         const unsigned epoch = s_epoch;
         if (b >= nbox) break;
-        const int lv = level[b], p = parent[b], v1 = vptr[b + 1];
-        const double ir = g.invL * fmm::pow2<double>(lv + 1);
+        const int lv = level[b], p = parent[b];
         const int d = (ix[b] & 1) + 2 * (iy[b] & 1);
         const cx<double> dk = fmm::dpow(dtab, d)[lane], iv = fmm::d2inv(dtab, d)[lane];
-        if (lane < P) {
-            cx<double> o = mk<double>(0, 0);
-            for (int v = vptr[b] + wid; v < v1; v += 4) {
-                const cx<double> a = trans[(int64_t)v * P + lane];
-                o.x += a.x;
-                o.y += a.y;
-            }
-            o.x *= ir;
-            o.y *= ir;
-            if (wid == 0 && nx[b] && en[b] - bg[b] > thr) {
-                const cx<double> x = fmm::ldcg_cx(&loc[b * P + lane]);
-                o.x += x.x;
-                o.y += x.y;
-            }
-            own[wid][lane] = o;
-        }
+        if (w.sums && b == 0 && wid == 3) strength_sums(w, lane);
+        own[wid][lane] = own_part(w, b, P, lane, wid, 4, g.invL * fmm::pow2<double>(lv + 1), loc);
         if (lv >= 3) {
             if (threadIdx.x == 0) {
                 unsigned spins = 0;
@@ -561,6 +593,23 @@ BoxGeo geo_of(const Tree &T)
 
 }  // namespace
 
+static int l2l(lbf_plan *pl, int P, const Own &w, cx<double> *loc, int kid, const int *gate,
+               cudaStream_t s)
+{
+    const Tree &T = pl->tree;
+    const int64_t nsm = std::max(pl->nsm, 1);
+    if (T.nleaf < kSmallLeaves)
+        LBF_LAUNCH_P(kid, k_l2l_small, lbf_grid(pl, std::min<int64_t>(T.nbox, 8 * nsm)), 128, 0, s, T.nbox,
+                     P, T.level, T.ix, T.iy, T.parent, w, geo_of(T), pl->tab_binom,
+                     (const cx<double> *)pl->tab_dshift, loc, pl->pull, pl->dev_status, gate, pl->slab);
+    else
+        LBF_LAUNCH_P(kid, k_l2l, lbf_grid(pl, std::min<int64_t>(lbf_cdiv(T.nbox, 8), 4 * nsm)), 256, 0, s,
+                     T.nbox, P, T.level, T.ix, T.iy, T.parent, w, geo_of(T), pl->tab_binom,
+                     (const cx<double> *)pl->tab_dshift, loc, pl->pull, pl->dev_status, gate, pl->slab);
+    LBF_CHECK_LAUNCH();
+    return LBF_OK;
+}
+
 // whether the plan's double applications take these passes
 bool lbf_passes_ready(const lbf_plan *pl) { return pl->rows && pl->m2l_cap && pl->nbigx >= 0; }
 
@@ -606,7 +655,6 @@ int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s)
 {
     const Tree &T = pl->tree;
     const int P = pl->P;
-    const bool small = T.nleaf < kSmallLeaves;
     int rc = lbf_passes_up(pl, gate, s);
     if (rc) return rc;
     rc = lbf_m2l_apply(pl, gate, s);
@@ -615,22 +663,34 @@ int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s)
         LBF_LAUNCH_P(LBF_KERNEL_DOWN, k_p2l_big, lbf_grid(pl, pl->nbigx), 128, kP2lSmem, s,
                      (int)pl->nbigx, pl->bigx, T.level, T.ix, T.iy, T.begin, T.end, T.xlist, T.nx,
                      geo_of(T), P, pl->xi, pl->q, (cx<double> *)pl->local, gate, pl->slab);
-    if (small)
-        LBF_LAUNCH_P(LBF_KERNEL_DOWN, k_l2l_small,
-                     lbf_grid(pl, std::min<int64_t>(T.nbox, 8 * (int64_t)std::max(pl->nsm, 1))), 128, 0, s,
-                     T.nbox, P, T.level, T.ix, T.iy, T.parent, T.begin, T.end, T.nx, pl->rows_thr,
-                     pl->m2l_vptr, (const cx<double> *)pl->m2l_out, geo_of(T), pl->tab_binom,
-                     (const cx<double> *)pl->tab_dshift, (cx<double> *)pl->local, pl->pull,
-                     pl->dev_status, gate, pl->slab);
-    else
-        LBF_LAUNCH_P(LBF_KERNEL_DOWN, k_l2l,
-                     lbf_grid(pl, std::min<int64_t>(lbf_cdiv(T.nbox, 8), 4 * (int64_t)std::max(pl->nsm, 1))),
-                     256, 0, s, T.nbox, P, T.level, T.ix, T.iy, T.parent, T.begin, T.end, T.nx,
-                     pl->rows_thr, pl->m2l_vptr, (const cx<double> *)pl->m2l_out, geo_of(T),
-                     pl->tab_binom, (const cx<double> *)pl->tab_dshift, (cx<double> *)pl->local,
-                     pl->pull, pl->dev_status, gate, pl->slab);
-    LBF_CHECK_LAUNCH();
-    return LBF_OK;
+    Own w{};
+    w.ptr = pl->m2l_vptr;
+    w.part = (const cx<double> *)pl->m2l_out;
+    w.bg = T.begin;
+    w.en = T.end;
+    w.nx = T.nx;
+    w.thr = pl->rows_thr;
+    return l2l(pl, P, w, (cx<double> *)pl->local, LBF_KERNEL_DOWN, gate, s);
+}
+
+// Full local expansions of the multiplier potential E y (P = 32 terms, lbf_border.cu) and its
+// sums of the strengths, from the stored expansions of the (box, centre) pairs: the P2L formed
+// every pair's powers and logarithm again in each application, 7.1 ms for 5.3 million pairs
+// where the stored coefficients are 0.4 ms of HBM, then wrote and read every expansion once
+// more for the chain.
+int lbf_mp_chain_apply(lbf_plan *pl, const double *y, const int *gate, cudaStream_t s)
+{
+    const Border &B = pl->bd;
+    Own w{};
+    w.ptr = B.p2l_ptr;
+    w.part = (const cx<double> *)B.p2l_exp;
+    w.src = B.p2l_src;
+    w.y = y;
+    w.sums = B.sums;
+    w.kind = B.kind;
+    w.lam = B.lam;
+    w.M = pl->M;
+    return l2l(pl, B.Pe, w, (cx<double> *)B.loc, LBF_KERNEL_ESUM, gate, s);
 }
 
 int lbf_passes_init_attrs()
