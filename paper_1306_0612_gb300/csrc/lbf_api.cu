@@ -135,6 +135,10 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
         pl->mpole = A.get<double2>(cap * P);
         pl->local = A.get<double2>(cap * P);
     }
+    if (o.matvec == LBF_MATVEC_DIRECT) {
+        pl->dpart = A.get<double2>(lbf_cdiv(N, 32) * 32 * lbf_direct_runs(N));
+        pl->dcount = A.get<unsigned>(lbf_cdiv(N, 32));
+    }
     if (o.matvec == LBF_MATVEC_FMM || o.border) {
         pl->upcnt = A.get<int32_t>(cap);
         pl->pull = A.get<uint32_t>(2 * cap + 4);
@@ -281,6 +285,8 @@ static void layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A)
     const Border &B = pl->bd;
     const bool fmm = o.matvec == LBF_MATVEC_FMM, f32 = o.precision == LBF_PRECISION_FP32_REFINE;
     v->q = A.get<double2>(N);
+    v->dpart = fmm ? nullptr : A.get<double2>(lbf_cdiv(N, 32) * 32 * lbf_direct_runs(N));
+    v->dcount = fmm ? nullptr : A.get<unsigned>(lbf_cdiv(N, 32));
     v->mpole = fmm ? A.get<double2>(cap * P) : nullptr;
     v->local = fmm ? A.get<double2>(cap * P) : nullptr;
     v->upcnt = fmm || o.border ? A.get<int32_t>(cap) : nullptr;
@@ -359,7 +365,7 @@ lbf_plan lbf_view_at(const lbf_plan &v, int r)
     mv(o.red); mv(o.red_count); mv(o.fvec); mv(o.yvec); mv(o.tin); mv(o.tout); mv(o.vstep);
     mv(o.bd.partial); mv(o.bd.loc); mv(o.bd.loc32); mv(o.bd.sums); mv(o.H); mv(o.gw);
     mv(o.gx); mv(o.gb); mv(o.gpart); mv(o.gs); mv(o.V); mv(o.region); mv(o.nearbuf);
-    mv(o.m2l_X); mv(o.m2l_e); mv(o.m2l_out);
+    mv(o.dpart); mv(o.dcount); mv(o.m2l_X); mv(o.m2l_e); mv(o.m2l_out);
     o.nrhs = 1;
     o.slab = 0;
     return o;
@@ -606,6 +612,7 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
         CK(cudaMemcpyAsync(pl->tabdf_dshift, d2.data(), sizeof(float) * d2.size(), cudaMemcpyHostToDevice, s));
         CK(cudaStreamSynchronize(s));  // the host vectors end with this scope
     }
+    if (pl->dcount) CK(cudaMemsetAsync(pl->dcount, 0, sizeof(unsigned) * lbf_cdiv(N, 32), s));
     if (pl->upcnt) CK(cudaMemsetAsync(pl->upcnt, 0, sizeof(int32_t) * cap, s));
     if (pl->pull) CK(cudaMemsetAsync(pl->pull, 0, sizeof(uint32_t) * (2 * cap + 4), s));
     CK(cudaMemcpyAsync(pl->tab_tpow, tpow.data(), sizeof(double2) * tpow.size(), cudaMemcpyHostToDevice, s));

@@ -183,50 +183,69 @@ __global__ void k_island_means(int M, const int64_t *__restrict__ ptr, const int
     if (lane == 0) mean[wg] = (e > b && mean[M] != 0.0) ? acc / (double)(e - b) : 0.0;
 }
 
-// Direct O(N^2) Cauchy sums with the same outputs as the leaf kernel's modes
-// (tiled through shared memory).
+// Direct O(N^2) Cauchy sums with the same outputs as the leaf kernel's modes: a warp per 32
+// nodes and run of sources, a node a lane, every lane reading the same source.  A run's sums
+// go to part; the warp that finishes a group of 32 nodes last adds its runs in order (one run:
+// no sums of sums) and writes the rows.  A thread block per 256 nodes over all sources left
+// one island of 256 nodes to a single SM: 220 us an application, now 8.
 template <int MODE>
-__global__ void k_direct(int64_t N, const double2 *__restrict__ xi, const double2 *__restrict__ q,
-                         const double *__restrict__ sigma, const double *__restrict__ dself,
-                         const double2 *__restrict__ w, const double *__restrict__ beta,
-                         const double *__restrict__ bsig, double *__restrict__ v, const int *gate,
-                         int64_t slab)
+__global__ void __launch_bounds__(128)
+k_direct(int64_t N, const double2 *__restrict__ xi, const double2 *__restrict__ q,
+         const double *__restrict__ sigma, const double *__restrict__ dself,
+         const double2 *__restrict__ w, const double *__restrict__ beta,
+         const double *__restrict__ bsig, double *__restrict__ v, const int *gate, int nrun,
+         double2 *part, unsigned *count, int64_t slab)
 {
-    lbf_rhs(slab, q, sigma, bsig, v, gate);
+    lbf_rhs(slab, q, sigma, bsig, v, gate, part, count);
     if (fmm::gate_closed(gate)) return;
-    __shared__ double2 sx[256], sq[256];
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    double2 z = i < N ? xi[i] : make_double2(0, 0);
-    double accI = 0.0, ar = 0.0, ai = 0.0;
-    for (int64_t base = 0; base < N; base += 256) {
-        int64_t j = base + threadIdx.x;
-        __syncthreads();
-        if (j < N) { sx[threadIdx.x] = xi[j]; sq[threadIdx.x] = q[j]; }
-        __syncthreads();
-        int n = (int)(N - base < 256 ? N - base : 256);
-        for (int m = 0; m < n; m++) {
-            if (base + m == i) continue;
-            double dr = sx[m].x - z.x, di = sx[m].y - z.y;
-            double2 qq = sq[m];
-            double ir2 = fmm::rcp(fma(dr, dr, di * di));
-            if (MODE == fmm::kLeafForward) {
-                accI = fma(fma(qq.y, dr, -qq.x * di), ir2, accI);
-            } else if (MODE == fmm::kLeafTranspose) {
-                ar = fma(fma(qq.x, dr, qq.y * di), ir2, ar);
-                ai = fma(fma(qq.y, dr, -qq.x * di), ir2, ai);
-            } else {
-                double er = (dr * dr - di * di) * ir2 * ir2, ei = -2 * dr * di * ir2 * ir2;
-                ar = fma(qq.x, er, fma(-qq.y, ei, ar));
-                ai = fma(qq.x, ei, fma(qq.y, er, ai));
-            }
+    const int64_t wg = blockIdx.x * 4ll + (threadIdx.x >> 5), ngrp = (N + 31) / 32;
+    const int lane = threadIdx.x & 31;
+    if (wg >= ngrp * nrun) return;
+    const int64_t grp = wg / nrun, run = wg % nrun, i = 32 * grp + lane;
+    const double2 z = i < N ? xi[i] : make_double2(0, 0);
+    double ar = 0.0, ai = 0.0;
+    const int64_t j1 = N * (run + 1) / nrun;
+#pragma unroll 2
+    for (int64_t j = N * run / nrun; j < j1; j++) {
+        const double2 zj = xi[j], qq = q[j];
+        if (j == i) continue;
+        const double dr = zj.x - z.x, di = zj.y - z.y;
+        const double ir2 = fmm::rcp(fma(dr, dr, di * di));
+        if (MODE == fmm::kLeafForward) {
+            ai = fma(fma(qq.y, dr, -qq.x * di), ir2, ai);
+        } else if (MODE == fmm::kLeafTranspose) {
+            ar = fma(fma(qq.x, dr, qq.y * di), ir2, ar);
+            ai = fma(fma(qq.y, dr, -qq.x * di), ir2, ai);
+        } else {
+            const double er = (dr * dr - di * di) * ir2 * ir2, ei = -2 * dr * di * ir2 * ir2;
+            ar = fma(qq.x, er, fma(-qq.y, ei, ar));
+            ai = fma(qq.x, ei, fma(qq.y, er, ai));
+        }
+    }
+    if (nrun > 1) {
+        part[wg * 32 + lane] = make_double2(ar, ai);
+        __threadfence();
+        __syncwarp();
+        unsigned c = 0;
+        if (lane == 0) c = atomicAdd(&count[grp], 1u);
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if (c != (unsigned)nrun - 1u) return;
+        if (lane == 0) count[grp] = 0u;  // ready for the next application
+        __threadfence();
+        ar = ai = 0.0;
+#pragma unroll 4
+        for (int r = 0; r < nrun; r++) {
+            const double2 p = __ldcg(&part[(grp * nrun + r) * 32 + lane]);
+            ar += p.x;
+            ai += p.y;
         }
     }
     if (i >= N) return;
     if (MODE == fmm::kLeafForward) {
-        v[i] = 2.0 * (accI * (1.0 / (2.0 * LBF_PI)) + dself[i] * sigma[i] + *bsig);
+        v[i] = 2.0 * (ai * (1.0 / (2.0 * LBF_PI)) + dself[i] * sigma[i] + *bsig);
     } else if (MODE == fmm::kLeafTranspose) {
-        double2 ww = w[i];
-        double im = -(ww.x * ai + ww.y * ar);
+        const double2 ww = w[i];
+        const double im = -(ww.x * ai + ww.y * ar);
         v[i] = 2.0 * (im * (1.0 / (2.0 * LBF_PI)) + dself[i] * sigma[i] + beta[i] * *bsig);
     } else {
         ((double2 *)v)[i] = make_double2(-ar, -ai);
@@ -528,8 +547,10 @@ static int apply_mode(lbf_plan *pl, const double *sigma, double *v, const int *g
     if (rc) return rc;
     int64_t N = pl->N;
     if (pl->opt.matvec == LBF_MATVEC_DIRECT) {
-        LBF_LAUNCH_P(LBF_KERNEL_DIRECT, k_direct<MODE>, lbf_grid(pl, lbf_cdiv(N, 256)), 256, 0, s, N,
-                     pl->xi, pl->q, sigma, pl->dself, pl->w, pl->beta, pl->bsig, v, gate, pl->slab);
+        const int nrun = lbf_direct_runs(N);
+        LBF_LAUNCH_P(LBF_KERNEL_DIRECT, k_direct<MODE>, lbf_grid(pl, lbf_cdiv(lbf_cdiv(N, 32) * nrun, 4)),
+                     128, 0, s, N, pl->xi, pl->q, sigma, pl->dself, pl->w, pl->beta, pl->bsig, v, gate,
+                     nrun, pl->dpart, pl->dcount, pl->slab);
         LBF_CHECK_LAUNCH();
         return LBF_OK;
     }

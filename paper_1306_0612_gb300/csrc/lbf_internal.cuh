@@ -191,6 +191,9 @@ struct lbf_plan {
     long long *m2l_X = nullptr;
     double *m2l_out = nullptr;
     // stored leaf rows of the accurate forward operator (lbf_rows.cu; rows null: not stored)
+    // direct sums: partial sums of the runs of sources, finished runs per 32 nodes
+    double2 *dpart = nullptr;
+    unsigned *dcount = nullptr;
     double *rows = nullptr;
     int32_t *rows_cols = nullptr;
     RowItem *rows_items = nullptr;
@@ -373,6 +376,12 @@ int lbf_emat_apply(lbf_plan *pl, const double *y, const double *x, const double 
                    double *out, const int *gate, cudaStream_t s);
 int lbf_emat_apply_transpose(lbf_plan *pl, const double *tau, double sc, const double *add,
                              double *out, const int *gate, cudaStream_t s);
+// runs of sources of the direct sums: about 2400 warps (four a scheduler), runs of at least 4
+static inline int lbf_direct_runs(int64_t N)
+{
+    const int64_t ngrp = lbf_cdiv(N, 32), r = 2432 / ngrp, m = N / 4;
+    return (int)(r < 1 ? 1 : r < m ? r : m < 1 ? 1 : m);
+}
 // ---- stored leaf rows (lbf_rows.cu) ----------------------------------------------
 void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap);
 int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len,
