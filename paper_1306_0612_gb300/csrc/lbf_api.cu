@@ -235,9 +235,11 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
     }
     int m = o.restart;
     pl->ldv = (n + 31) / 32 * 32;
-    // blocks of the Arnoldi reductions: about 2048 unknowns each, at most 2 per SM (a
-    // small system's steps would otherwise pay for hundreds of near-empty blocks)
-    pl->mdot_blocks = (int)std::min<int64_t>(lbf_gmres_blocks(), std::max<int64_t>(1, lbf_cdiv(n, 2048)));
+    // blocks of the Arnoldi reductions: about 1024 unknowns each, at most 2 per SM (a
+    // small system's steps would otherwise pay for hundreds of near-empty blocks; 16
+    // right-hand sides of 9,808 unknowns: 23.1 ms with 2048 a block, 22.4 with 1024, 22.6
+    // with 512)
+    pl->mdot_blocks = (int)std::min<int64_t>(lbf_gmres_blocks(), std::max<int64_t>(1, lbf_cdiv(n, 1024)));
     if (o.border) {
         pl->H = A.get<double>((int64_t)(m + 1) * m + 2 * (m + 1) + 2 * m + 2 * (m + 1) + m);
         pl->gw = A.get<double>(n);

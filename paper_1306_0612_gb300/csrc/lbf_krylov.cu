@@ -279,26 +279,34 @@ __global__ void k_arnoldi(int64_t n, const T *__restrict__ V, int64_t ldv, const
         }
     }
     __syncthreads();
+    // Hessenberg column j: h = h1 + h2, and the previous rotations, brought to shared memory by
+    // the block (a load of each by the one thread that rotates them was a chain of j trips to L2)
+    double *hs = sh, *cps = sh + (m + 2), *sps = cps + (m + 2);  // ws is free by now
+    if (mode == 2) {
+        for (int k = threadIdx.x; k <= j; k += blockDim.x) {
+            hs[k] = hbuf[k] + hbuf[(m + 1) + k];
+            cps[k] = k < j ? cs[k] : 0.0;
+            sps[k] = k < j ? sn[k] : 0.0;
+        }
+    }
+    __syncthreads();
+    double *Hj = H + (int64_t)j * (m + 1);
     if (threadIdx.x == 0) {
         *count = 0u;
         if (mode == 2) {
-            // Hessenberg column j: h = h1 + h2, H[j+1][j] = ||w||
-            double *Hj = H + (int64_t)j * (m + 1);
-            for (int k = 0; k <= j; k++) Hj[k] = hbuf[k] + hbuf[(m + 1) + k];
             double hn = sqrt(acc[0]);
-            Hj[j + 1] = hn;
-            // apply the previous Givens rotations, then a new one zeroing H[j+1][j]
+            // apply the previous Givens rotations, then a new one zeroing H[j+1][j] = ||w||
+            double a = hs[0], b = hn;
             for (int k = 0; k < j; k++) {
-                double a = Hj[k], b = Hj[k + 1];
-                Hj[k] = cs[k] * a + sn[k] * b;
-                Hj[k + 1] = -sn[k] * a + cs[k] * b;
+                const double c = cps[k], s = sps[k], h = hs[k + 1];
+                hs[k] = c * a + s * h;
+                a = -s * a + c * h;
             }
-            double a = Hj[j], b = Hj[j + 1];
             double rr = hypot(a, b);
             double c = rr > 0.0 ? a / rr : 1.0, s = rr > 0.0 ? b / rr : 0.0;
             cs[j] = c;
             sn[j] = s;
-            Hj[j] = rr;
+            hs[j] = rr;
             Hj[j + 1] = 0.0;
             gv[j + 1] = -s * gv[j];
             gv[j] = c * gv[j];
@@ -310,6 +318,10 @@ __global__ void k_arnoldi(int64_t n, const T *__restrict__ V, int64_t ldv, const
             if (conv) st->converged = 1;
             if (conv || st->it >= st->maxit || j + 1 >= m || !(hn > 0.0)) st->go = 0;
         }
+    }
+    if (mode == 2) {
+        __syncthreads();
+        for (int k = threadIdx.x; k <= j; k += blockDim.x) Hj[k] = hs[k];
     }
 }
 
