@@ -142,6 +142,7 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
     if (o.matvec == LBF_MATVEC_FMM || o.border) {
         pl->upcnt = A.get<int32_t>(cap);
         pl->pull = A.get<uint32_t>(2 * cap + 4);
+        pl->loc_e = A.get<int32_t>(cap);
     }
     if (o.matvec == LBF_MATVEC_FMM && o.fmm64) {
         pl->qdf = A.get<double2>(N);   // cx<df64>: 16 B per node
@@ -293,6 +294,7 @@ static void layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A)
     v->local = fmm ? A.get<double2>(cap * P) : nullptr;
     v->upcnt = fmm || o.border ? A.get<int32_t>(cap) : nullptr;
     v->pull = fmm || o.border ? A.get<uint32_t>(2 * cap + 4) : nullptr;
+    v->loc_e = fmm || o.border ? A.get<int32_t>(cap) : nullptr;
     v->qdf = fmm && o.fmm64 ? (void *)A.get<double2>(N) : nullptr;
     v->q32 = f32 ? A.get<float2>(N) : nullptr;
     v->mpole32 = f32 && fmm ? A.get<float2>(cap * (o.p32 + 1)) : nullptr;
@@ -367,7 +369,7 @@ lbf_plan lbf_view_at(const lbf_plan &v, int r)
     mv(o.red); mv(o.red_count); mv(o.fvec); mv(o.yvec); mv(o.tin); mv(o.tout); mv(o.vstep);
     mv(o.bd.partial); mv(o.bd.loc); mv(o.bd.loc32); mv(o.bd.sums); mv(o.H); mv(o.gw);
     mv(o.gx); mv(o.gb); mv(o.gpart); mv(o.gs); mv(o.V); mv(o.region); mv(o.nearbuf);
-    mv(o.dpart); mv(o.dcount); mv(o.m2l_X); mv(o.m2l_e); mv(o.m2l_out);
+    mv(o.dpart); mv(o.dcount); mv(o.m2l_X); mv(o.m2l_e); mv(o.m2l_out); mv(o.loc_e);
     o.nrhs = 1;
     o.slab = 0;
     return o;

@@ -189,6 +189,7 @@ struct lbf_plan {
     int32_t *m2l_vptr = nullptr, *m2l_tile0 = nullptr, *m2l_f = nullptr, *m2l_e = nullptr;
     uint4 *m2l_img = nullptr;
     long long *m2l_X = nullptr;
+    int32_t *loc_e = nullptr;   // exponents of the integer local expansions (lbf_passes.cu)
     double *m2l_out = nullptr;
     // stored leaf rows of the accurate forward operator (lbf_rows.cu; rows null: not stored)
     // direct sums: partial sums of the runs of sources, finished runs per 32 nodes
@@ -368,7 +369,7 @@ void lbf_m2l_layout(lbf_plan *pl, const lbf_options &o, int64_t cap);
 void lbf_m2l_layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A);
 int lbf_m2l_init_attrs();
 int lbf_m2l_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len);
-int lbf_m2l_apply(lbf_plan *pl, const int *gate, cudaStream_t s);
+int lbf_m2l_apply(lbf_plan *pl, const int *gate, cudaStream_t s, bool fixed = false);
 // ---- stored multiplier block (lbf_emat.cu) ---------------------------------------
 void lbf_emat_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o);
 int lbf_emat_build(lbf_plan *pl, cudaStream_t s);

@@ -36,6 +36,7 @@
 // expansions keep the double loop in k_down.
 #include <algorithm>
 
+#include "lbf_fixed.cuh"
 #include "lbf_fmm_tpl.cuh"
 #include "lbf_tc.cuh"
 
@@ -51,24 +52,8 @@ constexpr int kM2lSmem = kSl * (kABytes + kBBytes);
 constexpr int kM2lThreads = 512;
 constexpr int kNoffs = 49;              // offsets (dx + 3) 7 + dy + 3
 constexpr unsigned kM2lSpins = 1u << 24;
-constexpr int kBadExp = 1 << 20;        // exponent of a box with an infinity or NaN
 
-__host__ __device__ inline int real_pitch(int P) { return (2 * P + 7) / 8 * 8; }
 __host__ __device__ inline int tile_cols(int P) { return (2 * P + 15) / 16 * 16; }
-
-// v as an integer in units of 2^(e - 54), rounded, |v| < 2^e: its double bits with the
-// exponent lowered by `drop`; top: the largest lowered exponent field of the set (> 0)
-__device__ __forceinline__ long long fixed54(long long bits, int drop, int top)
-{
-    const int E = (int)((bits >> 52) & 0x7ff);
-    if (E == 0) return 0;  // zero (a subnormal is far below any unit here)
-    const int d = top - (E - drop);
-    if (d > 60) return 0;
-    unsigned long long m = ((unsigned long long)bits & 0xfffffffffffffull) | 0x10000000000000ull;
-    m <<= 1;
-    if (d > 0) m = (m + (1ull << (d - 1))) >> d;
-    return bits < 0 ? -(long long)m : (long long)m;
-}
 
 // the seven base-256 digits of x (|x| <= 2^54), most significant first, each plus 128
 __device__ __forceinline__ unsigned long long digits(long long x)
@@ -105,7 +90,7 @@ __global__ void k_m2l_fix(int64_t nbox, int P, const cx<double> *__restrict__ mp
         bad |= E == 0x7ff;
         if (E) top = max(top, E - (m >> 2));
     }
-    for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    top = __reduce_max_sync(0xffffffffu, top);
     bad = __any_sync(0xffffffffu, bad);
     const int pitch = real_pitch(P);
 #pragma unroll
@@ -231,22 +216,6 @@ __global__ void k_m2l_place(int64_t nbox, const int32_t *__restrict__ ix, const 
 }
 
 // ---- per application -----------------------------------------------------------------
-
-// w 2^E (|w| < 2^63) as a double, rounded half up, without the double pipe
-__device__ __forceinline__ double pack_double(long long w, int E)
-{
-    unsigned long long m = w < 0 ? (unsigned long long)-w : (unsigned long long)w;
-    if (m == 0) return 0.0;
-    const int lz = __clzll((long long)m);
-    m <<= lz;
-    const int ef = 1023 + 63 - lz + E;
-    const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // hidden bit at 52, may carry
-    unsigned long long bits;
-    if (ef <= 0) bits = 0;
-    else if (ef >= 2047) bits = 0x7ff0000000000000ull;
-    else bits = ((unsigned long long)(ef - 1) << 52) + r;
-    return __longlong_as_double((long long)(bits | (w < 0 ? 0x8000000000000000ull : 0ull)));
-}
 
 __global__ void __launch_bounds__(kM2lThreads, 1)
 k_m2l_tc(int P, const int32_t *__restrict__ tile0, const int2 *__restrict__ pairs,
@@ -509,13 +478,15 @@ int lbf_m2l_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratc
     return LBF_OK;
 }
 
-// m2l_out from the plan's (or view's) double multipoles
-int lbf_m2l_apply(lbf_plan *pl, const int *gate, cudaStream_t s)
+// m2l_out from the plan's (or view's) multipoles, of which m2l_X and m2l_e hold the integers
+// already where `fixed` is set (lbf_passes.cu)
+int lbf_m2l_apply(lbf_plan *pl, const int *gate, cudaStream_t s, bool fixed)
 {
     if (!pl->m2l_tiles) return LBF_OK;
     const Tree &T = pl->tree;
-    LBF_LAUNCH_P(LBF_KERNEL_DOWN, k_m2l_fix, lbf_grid(pl, lbf_cdiv(T.nbox, 8)), 256, 0, s, T.nbox, pl->P,
-                 (const cx<double> *)pl->mpole, pl->m2l_X, pl->m2l_e, gate, pl->slab);
+    if (!fixed)
+        LBF_LAUNCH_P(LBF_KERNEL_DOWN, k_m2l_fix, lbf_grid(pl, lbf_cdiv(T.nbox, 8)), 256, 0, s, T.nbox, pl->P,
+                     (const cx<double> *)pl->mpole, pl->m2l_X, pl->m2l_e, gate, pl->slab);
     const int64_t grid = std::min<int64_t>(pl->m2l_tiles, std::max(pl->nsm, 1));
     LBF_LAUNCH_P(LBF_KERNEL_DOWN, k_m2l_tc, lbf_grid(pl, grid), kM2lThreads, kM2lSmem, s, pl->P, pl->m2l_tile0,
                  pl->m2l_pairs, pl->m2l_X, pl->m2l_e, (const uint4 *)pl->m2l_img, pl->m2l_f, pl->m2l_out,

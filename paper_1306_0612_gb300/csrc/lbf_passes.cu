@@ -1,7 +1,7 @@
 // The upward and downward passes of a double application on a plan whose leaf rows
 // (lbf_rows.cu) and translations (lbf_m2l.cu) are stored, P <= 32:
 //
-//   k_up_rows   P2M from the rows' local columns (the powers u_i^l of the leaf's nodes are
+//   k_up        P2M from the rows' local columns (the powers u_i^l of the leaf's nodes are
 //               there already), then M2M by the warp that completes a box's last child;
 //   k_p2l_big   P2L of the few boxes whose X lists are not near columns;
 //   k_l2l       each box's translations added up and its parent's expansion shifted to it,
@@ -11,20 +11,21 @@
 //
 // P2M: with the stored powers a node and coefficient take two multiply-adds a real where
 // the recurrence took six double instructions and left the lanes past a leaf's last node
-// idle (26 of 32 at 16.8 million nodes).  L2L: a warp a box, the two halves of a warp
-// sharing each coefficient's sum, so a box's shift is (P + 1)/2 dependent steps where the
-// half-warp form of k_down takes P + 1; and no shared-memory staging but the shift matrix
-// and one expansion a warp, so an SM holds 64 warps.
+// idle (26 of 32 at 16.8 million nodes).
 //
-// A small system is a chain of some ten to seventeen levels that nothing hides, and a warp
-// issues a double instruction every 64 cycles: there a thread block of four warps, on the
-// SM's four schedulers, takes a leaf or a box (k_up_small, k_l2l_small).  Four warps a box
-// lower a level's shift from P + 1 dependent steps to 4.  Up and down at 8192 nodes 122 to
-// 63 us and 75 to 46 us; at 7130 leaves an application 907 to 863 us, at 16,150 the two forms
-// are equal, at 647,307 the block form takes 10.4 + 10.9 ms where the warp form takes
-// 8.0 + 8.6 (of 10.5 + 28.7 with the passes of lbf_fmm_tpl.cuh).
+// Shifts on the integer pipes.  A shift is a triangle of binomials between powers of
+// 2d = +-1 +- i,
+//   M2M  a_l  = d^l     sum_{k <= l} C(l, k) (2d)^-k a'_k,
+//   L2L  b'_l = (2d)^-l sum_{k >= l} C(k, l) d^k b_k,
+// and this GPU issues a double multiply-add every 64 cycles per scheduler, a 32 x 32 -> 64 bit
+// integer one every few.  The expansions are integers of 54 bits below the box's largest
+// (lbf_fixed.cuh, the form the translations take too), the powers of 1 + i are additions,
+// swaps and shifts, C(l, k) and 2^(31-k) C(k, l) are below 2^31, and a sum of at most 32
+// products of a 56-bit integer is exact in two 64-bit accumulators (28 low bits, the rest):
+// one rounding a coefficient and level, 2^-54 of the box's largest.  FIXMEFIG
 #include <algorithm>
 
+#include "lbf_fixed.cuh"
 #include "lbf_fmm_tpl.cuh"
 
 using fmm::BoxGeo;
@@ -33,7 +34,6 @@ using fmm::mk;
 
 namespace {
 
-constexpr int64_t kSmallLeaves = 12000;
 constexpr int kP2lSmem = 4 * 32 * 33 * 16;
 constexpr int kGroups = 8;  // row groups of a block at most (lbf_rows.cu)
 
@@ -41,12 +41,12 @@ constexpr int kGroups = 8;  // row groups of a block at most (lbf_rows.cu)
 // leaf's row blocks, four chunks at a time.  Column 2 l of a row holds -(1/pi) Im u^l, column 2 l + 1 -(1/pi) Re u^l:
 // an even lane adds their parts of both reals of coefficient l, an odd lane likewise, and
 // one exchange leaves the real part on the even lane, the imaginary part on the odd one.
-__device__ __forceinline__ void leaf_p2m(int64_t t, int b, int P,
+__device__ __forceinline__ void leaf_p2m(int64_t t, int P,
                                          const int32_t *__restrict__ block0,
                                          const RowItem *__restrict__ items,
                                          const double *__restrict__ rows,
-                                         const double2 *__restrict__ q, double *__restrict__ a,
-                                         int lane, int cbeg, int cend)
+                                         const double2 *__restrict__ q, double *a, int lane,
+                                         int cbeg, int cend)
 {
     const int k0 = block0[t], k1 = block0[t + 1];
     const bool odd = (lane & 1) != 0, u = (lane & 16) != 0, w = (lane & 8) != 0;
@@ -79,91 +79,7 @@ __device__ __forceinline__ void leaf_p2m(int64_t t, int b, int P,
         const double b1 = (u ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, u ? s[1] : s[3], 16);
         const double v = (w ? b1 : b0) + __shfl_xor_sync(0xffffffffu, w ? b0 : b1, 8);
         const int h = (u ? 2 : 0) + (w ? 1 : 0), m = 8 * (c + h) + (lane & 7);
-        if (c + h < cend && m < 2 * P) a[(int64_t)b * 2 * P + m] = v * LBF_PI;
-    }
-}
-
-// P2M per leaf, then M2M by the warp that completes a box's last child
-// (a_l = d^l sum_{k <= l} C(l, k) (2d)^-k a'_k, two children at a time, one a half-warp:
-// lane j of a half sums the rows l = j and P - 1 - j of the triangle in one loop)
-__global__ void __launch_bounds__(128)
-k_up_rows(int64_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ ix,
-          const int32_t *__restrict__ iy, const int32_t *__restrict__ parent,
-          const int32_t *__restrict__ child0, const int32_t *__restrict__ nchild, int P, int lchunks,
-          const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
-          const double *__restrict__ rows, const double *__restrict__ binom,
-          const cx<double> *__restrict__ dtab, const double2 *__restrict__ q, cx<double> *mp,
-          int *cnt, const int *gate, int64_t slab)
-{
-    lbf_rhs(slab, q, mp, cnt, gate);
-    if (fmm::gate_closed(gate)) return;
-    __shared__ double Cl[32 * 32];
-    __shared__ cx<double> As[4][2][32];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int e = threadIdx.x; e < P * P; e += blockDim.x) {
-        const int k = e / P, l = e % P;
-        Cl[e] = k <= l ? binom[l * LBF_MAX_TERMS + k] : 0.0;  // C(l, k)
-    }
-    __syncthreads();
-    const int64_t t = blockIdx.x * 4ll + wid;
-    if (t >= nleaf) return;
-    const int b = leaves[t];
-    leaf_p2m(t, b, P, block0, items, rows, q, (double *)mp, lane, 0, lchunks);
-    const int hf = lane >> 4, j = lane & 15;
-    const unsigned hmask = hf ? 0xffff0000u : 0x0000ffffu;
-    const int nr = (P + 1) / 2, r1 = j < nr ? j : 0, r2 = P - 1 - r1, n1 = r1 + 1;
-    cx<double> *Ah = As[wid][hf];
-    for (int cur = b;;) {
-        const int p = parent[cur];
-        if (p < 0) break;
-        __threadfence();
-        __syncwarp();
-        int last = 0;
-        if (lane == 0) {
-            last = atomicAdd(&cnt[p], 1) == nchild[p] - 1;
-            if (last) cnt[p] = 0;  // ready for the next application
-        }
-        last = __shfl_sync(0xffffffffu, last, 0);
-        if (!last) break;
-        __threadfence();
-        cx<double> a1 = mk<double>(0, 0), a2 = mk<double>(0, 0);
-        const int cend = child0[p] + nchild[p];
-        for (int c0 = child0[p]; c0 < cend; c0 += 2) {
-            const int c = c0 + hf;
-            if (c < cend) {
-                const int d = (ix[c] & 1) + 2 * (iy[c] & 1);
-                const cx<double> *inv = fmm::d2inv(dtab, d);
-                for (int k = j; k < P; k += 16)
-                    Ah[k] = fmm::cmul(fmm::ldcg_cx(&mp[(int64_t)c * P + k]), inv[k]);
-                __syncwarp(hmask);
-                cx<double> acc = mk<double>(0, 0), s1 = mk<double>(0, 0);
-                for (int it = 0; it <= P; it++) {
-                    const bool first = it < n1;
-                    if (it == n1) {
-                        s1 = acc;
-                        acc = mk<double>(0, 0);
-                    }
-                    const int k = first ? it : it - n1, l = first ? r1 : r2;
-                    const cx<double> a = Ah[k];
-                    const double cc = Cl[k * P + l];
-                    acc.x = fma(cc, a.x, acc.x);
-                    acc.y = fma(cc, a.y, acc.y);
-                }
-                const cx<double> *dp = fmm::dpow(dtab, d);
-                a1 = fmm::cfma(dp[r1], s1, a1);
-                a2 = fmm::cfma(dp[r2], acc, a2);
-                __syncwarp(hmask);
-            }
-        }
-        a1.x += __shfl_xor_sync(0xffffffffu, a1.x, 16);
-        a1.y += __shfl_xor_sync(0xffffffffu, a1.y, 16);
-        a2.x += __shfl_xor_sync(0xffffffffu, a2.x, 16);
-        a2.y += __shfl_xor_sync(0xffffffffu, a2.y, 16);
-        if (j < nr) {
-            if (hf == 0) mp[(int64_t)p * P + r1] = a1;
-            else if (r2 != r1) mp[(int64_t)p * P + r2] = a2;
-        }
-        cur = p;
+        if (c + h < cend && m < 2 * P) a[m] = v * LBF_PI;
     }
 }
 
@@ -234,8 +150,6 @@ k_p2l_big(int n, const int32_t *__restrict__ list, const int32_t *__restrict__ l
     loc[(int64_t)b * P + lane] = mk<double>(s.x * ir, s.y * ir);
 }
 
-constexpr unsigned kL2lSpins = 1u << 24;
-
 // What a box's expansion takes beside its parent's: of the density block its translations and
 // its P2L part where it has one (in loc already); of the multiplier potential (lbf_border.cu)
 // the stored expansions of its centres times their strengths y.
@@ -300,50 +214,266 @@ __device__ __forceinline__ void strength_sums(const Own &w, int lane)
     }
 }
 
+// ---- shifts of integer expansions ------------------------------------------------------
+
+// (x + iy) times (2d)^k up to the power of two 2^(k/2) (k even) or 2^((k-1)/2) (k odd), for
+// n = k (2h + 1) mod 8, 2d = sqrt 2 e^(i (2h + 1) pi/4): i^(n/2), times 1 + i when n is odd
+__device__ __forceinline__ void mul_pow(long long &x, long long &y, int n)
+{
+    if (n & 1) {
+        const long long t = x - y;
+        y = x + y;
+        x = t;
+    }
+    if (n & 2) {
+        const long long t = x;
+        x = -y;
+        y = t;
+    }
+    if (n & 4) {
+        x = -x;
+        y = -y;
+    }
+}
+
+// 2h + 1 of the child at (ix, iy)
+__device__ __forceinline__ int quadrant(int ix, int iy)
+{
+    return (iy & 1) ? ((ix & 1) ? 1 : 3) : ((ix & 1) ? 7 : 5);
+}
+
+// v 2^-s, rounded (s >= 0)
+__device__ __forceinline__ long long shift_down(long long v, int s)
+{
+    return s == 0 ? v : s > 62 ? 0ll : (v + (1ll << (s - 1))) >> s;
+}
+
+// the two words of a 57-bit integer: 28 low bits and the rest
+__device__ __forceinline__ int4 words(long long x, long long y)
+{
+    return make_int4((int)(x & 0xfffffff), (int)(x >> 28), (int)(y & 0xfffffff), (int)(y >> 28));
+}
+
+struct Sum {  // sums of weight times word, of the real and the imaginary part
+    unsigned long long xl, yl;
+    long long xh, yh;
+};
+__device__ __forceinline__ void add_term(Sum &s, unsigned c, int4 z)
+{
+    s.xl += (unsigned long long)c * (unsigned)z.x;
+    s.xh += (long long)(int)c * z.y;
+    s.yl += (unsigned long long)c * (unsigned)z.z;
+    s.yh += (long long)(int)c * z.w;
+}
+// a row's sum: the other half-warp's part of it added
+__device__ __forceinline__ Sum meet(const Sum &mine, const Sum &other)
+{
+    Sum r;
+    r.xl = mine.xl + __shfl_xor_sync(0xffffffffu, other.xl, 16);
+    r.xh = mine.xh + __shfl_xor_sync(0xffffffffu, other.xh, 16);
+    r.yl = mine.yl + __shfl_xor_sync(0xffffffffu, other.yl, 16);
+    r.yh = mine.yh + __shfl_xor_sync(0xffffffffu, other.yh, 16);
+    return r;
+}
+// (hi 2^28 + lo) 2^-s, rounded, s in 1 .. 33
+__device__ __forceinline__ long long scale_sum(long long hi, unsigned long long lo, int s)
+{
+    const long long t = hi + (long long)(lo >> 28);
+    const unsigned f = (unsigned)lo & 0xfffffffu;
+    if (s <= 28) return (t << (28 - s)) + ((f + (1u << (s - 1))) >> s);
+    return (t + (1ll << (s - 29))) >> (s - 28);
+}
+__device__ __forceinline__ int bits_of(long long x, long long y)
+{
+    const unsigned long long m = (unsigned long long)(x < 0 ? -x : x) | (unsigned long long)(y < 0 ? -y : y);
+    return 64 - __clzll((long long)m);
+}
+// x in the unit 2^sh times larger (sh < 0: smaller)
+__device__ __forceinline__ long long rescale(long long x, int sh)
+{
+    return sh > 0 ? shift_down(x, sh) : x << -sh;
+}
+
+__device__ __forceinline__ longlong2 ldcg_ll(const long long *p)
+{
+    const int4 v = __ldcg((const int4 *)p);
+    return make_longlong2((long long)(((unsigned long long)(unsigned)v.y << 32) | (unsigned)v.x),
+                          (long long)(((unsigned long long)(unsigned)v.w << 32) | (unsigned)v.z));
+}
+
+// P2M per leaf, then M2M by the warp that completes a box's last child.  Each box's multipole
+// is written as doubles (evaluation, the rows' M2P columns) and as integers: X_k = a_k
+// 2^-(k/2) in units of 2^(e - 54).  With conj(2d)^k taken exactly, 2 (2d)^-k a'_k is X_k
+// rotated (times 2, k even, or 1 +- i, k odd), and the sum over k times 2^-(l+1), rotated by
+// (2d)^l, is the parent's X_l.  Lane j of a half-warp has the rows j and P - 1 - j of the
+// triangle, P + 1 terms, a half of them each half.
+__global__ void __launch_bounds__(128)
+k_up(int64_t nleaf, const int32_t *__restrict__ leaves, const int32_t *__restrict__ ix,
+     const int32_t *__restrict__ iy, const int32_t *__restrict__ parent,
+     const int32_t *__restrict__ child0, const int32_t *__restrict__ nchild, int P, int lchunks,
+     const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
+     const double *__restrict__ rows, const double *__restrict__ binom, const double2 *__restrict__ q,
+     cx<double> *mp, long long *X, int32_t *ex, int *cnt, const int *gate, int64_t slab)
+{
+    lbf_rhs(slab, q, mp, X, ex, cnt, gate);
+    if (fmm::gate_closed(gate)) return;
+    __shared__ unsigned Cl[32 * 32];
+    __shared__ int4 Zs[4][32];
+    __shared__ double vs[4][64];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int e = threadIdx.x; e < P * P; e += blockDim.x) {
+        const int k = e / P, l = e % P;
+        Cl[k * 32 + l] = k <= l ? (unsigned)binom[l * LBF_MAX_TERMS + k] : 0u;  // C(l, k)
+    }
+    __syncthreads();
+    const int64_t t = blockIdx.x * 4ll + wid;
+    if (t >= nleaf) return;
+    const int b = leaves[t], pitch = real_pitch(P);
+    leaf_p2m(t, P, block0, items, rows, q, vs[wid], lane, 0, lchunks);
+    __syncwarp();
+    {
+        double v[2];
+        int top = -4096;
+        bool bad = false;
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int m = lane + 32 * h;
+            v[h] = m < 2 * P ? vs[wid][m] : 0.0;
+            const int E = (int)((__double_as_longlong(v[h]) >> 52) & 0x7ff);
+            bad |= E == 0x7ff;
+            if (E) top = max(top, E - (m >> 2));
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        bad = __any_sync(0xffffffffu, bad);
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int m = lane + 32 * h;
+            if (m < 2 * P) ((double *)mp)[(int64_t)b * 2 * P + m] = v[h];
+            if (m < pitch) X[(int64_t)b * pitch + m] = fixed54(__double_as_longlong(v[h]), m >> 2, top);
+        }
+        if (lane == 0) ex[b] = bad ? kBadExp : top - 1022;
+    }
+    const int hf = lane >> 4, j = lane & 15, nr = (P + 1) / 2;
+    const int r1 = j < nr ? j : 0, r2 = P - 1 - r1, n1 = r1 + 1, mid = (P + 2) / 2;
+    const int i0 = hf ? mid : 0, i1 = hf ? P + 1 : mid, row = hf ? r2 : r1;
+    const bool on = j < nr && (hf == 0 || r2 != r1);
+    for (int cur = b;;) {
+        const int p = parent[cur];
+        if (p < 0) break;
+        __threadfence();
+        __syncwarp();
+        int last = 0;
+        if (lane == 0) {
+            last = atomicAdd(&cnt[p], 1) == nchild[p] - 1;
+            if (last) cnt[p] = 0;  // ready for the next application
+            __threadfence();
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (!last) break;
+        const int nc = nchild[p], c0 = child0[p];
+        int ec = lane < nc ? __ldcg(&ex[c0 + lane]) : kZeroExp;
+        const int emax = __reduce_max_sync(0xffffffffu, ec);
+        long long sx = 0, sy = 0;
+        for (int c = 0; c < nc; c++) {
+            const int h2 = quadrant(ix[c0 + c], iy[c0 + c]);
+            if (lane < P) {
+                longlong2 v = ldcg_ll(&X[(int64_t)(c0 + c) * pitch + 2 * lane]);
+                mul_pow(v.x, v.y, (-lane * h2) & 7);
+                Zs[wid][lane] = (lane & 1) ? words(v.x, v.y) : words(2 * v.x, 2 * v.y);
+            }
+            __syncwarp();
+            Sum acc{0, 0, 0, 0}, first{0, 0, 0, 0};
+            for (int it = i0; it < i1; it++) {
+                if (it == n1) {
+                    first = acc;
+                    acc = Sum{0, 0, 0, 0};
+                }
+                const int k = it < n1 ? it : it - n1;
+                add_term(acc, Cl[k * 32 + (it < n1 ? r1 : r2)], Zs[wid][k]);
+            }
+            if (i1 <= n1) {
+                first = acc;
+                acc = Sum{0, 0, 0, 0};
+            }
+            const Sum s = meet(hf ? acc : first, hf ? first : acc);
+            long long x = scale_sum(s.xh, s.xl, row + 1), y = scale_sum(s.yh, s.yl, row + 1);
+            mul_pow(x, y, (row * h2) & 7);
+            const int sh = emax - __shfl_sync(0xffffffffu, ec, c);
+            sx += shift_down(x, sh);
+            sy += shift_down(y, sh);
+            __syncwarp();
+        }
+        const bool bad = emax >= kBadExp;
+        const int nb = __reduce_max_sync(0xffffffffu, on ? bits_of(sx, sy) : 0), sh = nb - 54;
+        if (on) {
+            const double nan = __longlong_as_double(0x7ff8000000000000ll);
+            const int E = emax - 54 + (row >> 1);
+            mp[(int64_t)p * P + row] = bad ? mk<double>(nan, nan)
+                                           : mk<double>(pack_double(sx, E), pack_double(sy, E));
+            *(longlong2 *)&X[(int64_t)p * pitch + 2 * row] = make_longlong2(rescale(sx, sh), rescale(sy, sh));
+        }
+        for (int m = 2 * P + lane; m < pitch; m += 32) X[(int64_t)p * pitch + m] = 0;
+        if (lane == 0) ex[p] = bad ? kBadExp : nb == 0 ? kZeroExp : emax + sh;
+        cur = p;
+    }
+}
+
+constexpr unsigned kL2lSpins = 1u << 24;
+
 // Every box's local expansion: its own part, and from level 3 on its parent's expansion
-// shifted down,
-//   b'_l = (2d)^-l sum_{k >= l} C(k, l) d^k b_k.
+// shifted down.  A box with children is left as integers in loc's memory, X_k = b_k 2^(k/2)
+// in units of 2^(e - 54): then d^k b_k is X_k rotated (times 1 +- i, k odd) times 2^-k, the
+// weights 2^(31-k) C(k, l) are integers below 2^31 (but for k = 0, added on its own), and the
+// sum, rotated by conj(2d)^l (and halved, l odd), is the child's X_l.  A leaf is left as
+// doubles.
 // pull: the words of k_down's chain ([1] finished warps, [2] epoch, [3] box counter, then
 // nbox words unused here and nbox epochs in which a box was finished).
 __global__ void __launch_bounds__(256)
 k_l2l(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_t *__restrict__ ix,
-      const int32_t *__restrict__ iy, const int32_t *__restrict__ parent, Own w, BoxGeo g,
-      const double *__restrict__ binom, const cx<double> *__restrict__ dtab, cx<double> *loc,
-      unsigned *pull, int *status, const int *gate, int64_t slab)
+      const int32_t *__restrict__ iy, const int32_t *__restrict__ parent,
+      const int32_t *__restrict__ nchild, Own w, BoxGeo g, const double *__restrict__ binom,
+      cx<double> *loc, int32_t *ex, unsigned *pull, int *status, const int *gate, int64_t slab)
 {
-    lbf_rhs(slab, loc, pull, gate, w.y, w.sums);
+    lbf_rhs(slab, loc, ex, pull, gate, w.y, w.sums);
     if (!w.src) lbf_rhs(slab, w.part);
     if (fmm::gate_closed(gate)) return;
-    __shared__ double Cd[32 * 32];
-    __shared__ cx<double> As[8][32];
+    __shared__ unsigned Wd[32 * 32];
+    __shared__ int4 Zs[8][32];
     const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int e = threadIdx.x; e < P * P; e += blockDim.x) {
         const int k = e / P, l = e % P;
-        Cd[e] = k >= l ? binom[k * LBF_MAX_TERMS + l] : 0.0;
+        Wd[k * 32 + l] = k >= l && k > 0 ? (unsigned)binom[k * LBF_MAX_TERMS + l] << (31 - k) : 0u;
     }
     __syncthreads();
     unsigned *done = pull + 4 + nbox;
     unsigned epoch = 0;
     if (lane == 0) epoch = *(volatile unsigned *)&pull[2];
     epoch = __shfl_sync(0xffffffffu, epoch, 0);
-    cx<double> *A = As[wid];
     // lane j of a half has the rows r1 = j and r2 = P - 1 - j of the triangle, P + 1 terms
-    // (n1 = P - r1 of them row r1's); half hf sums the terms [hf mid, hf ? P + 1 : mid)
+    // (n1 = P - r1 of them row r1's); half hf sums the terms i0 .. i1 - 1
     const int hf = lane >> 4, j = lane & 15, nr = (P + 1) / 2;
     const int r1 = j < nr ? j : 0, r2 = P - 1 - r1, n1 = P - r1, mid = (P + 2) / 2;
-    const int i0 = hf ? mid : 0, i1 = hf ? P + 1 : mid;
+    const int i0 = hf ? mid : 0, i1 = hf ? P + 1 : mid, row = hf ? r2 : r1;
+    const bool on = j < nr && (hf == 0 || r2 != r1);
     for (;;) {
         unsigned bi = 0;
         if (lane == 0) bi = atomicAdd(&pull[3], 1u);
         const int64_t b = (int64_t)__shfl_sync(0xffffffffu, bi, 0);
         if (b >= nbox) break;
-        const int lv = level[b], p = parent[b];
+        const int lv = level[b], p = parent[b], h2 = quadrant(ix[b], iy[b]);
+        const bool leaf = nchild[b] == 0;
         if (w.sums && b == 0) strength_sums(w, lane);
         const cx<double> own = own_part(w, b, P, lane, 0, 1, g.invL * fmm::pow2<double>(lv + 1), loc);
+        // its exponent, and the row of this lane
+        const int Ex = (int)((__double_as_longlong(own.x) >> 52) & 0x7ff);
+        const int Ey = (int)((__double_as_longlong(own.y) >> 52) & 0x7ff);
+        const int Em = max(Ex, Ey);
+        bool bad = __any_sync(0xffffffffu, Em == 0x7ff);
+        int e = __reduce_max_sync(0xffffffffu, Em ? Em + (lane >> 1) : -4096) - 1022;
+        const long long ox = __shfl_sync(0xffffffffu, __double_as_longlong(own.x), row);
+        const long long oy = __shfl_sync(0xffffffffu, __double_as_longlong(own.y), row);
+        long long sx = 0, sy = 0;
         if (lv >= 3) {
-            const int d = (ix[b] & 1) + 2 * (iy[b] & 1);
-            const cx<double> *dp = fmm::dpow(dtab, d), *inv = fmm::d2inv(dtab, d);
-            const cx<double> dk = dp[lane], iv = inv[hf ? r2 : r1];
             if (lane == 0) {
                 unsigned spins = 0;
                 const unsigned lim = wait_limit(status, kL2lSpins);
@@ -355,35 +485,57 @@ k_l2l(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_t *__r
                 __threadfence();
             }
             __syncwarp();
-            if (lane < P) A[lane] = fmm::cmul(fmm::ldcg_cx(&loc[(int64_t)p * P + lane]), dk);
+            const int ep = __ldcg(&ex[p]);
+            if (lane < P) {
+                longlong2 v = ldcg_ll((const long long *)&loc[(int64_t)p * P + lane]);
+                mul_pow(v.x, v.y, (lane * h2) & 7);
+                Zs[wid][lane] = words(v.x, v.y);
+            }
             __syncwarp();
-            cx<double> acc = mk<double>(0, 0), first = mk<double>(0, 0);
+            Sum acc{0, 0, 0, 0}, first{0, 0, 0, 0};
             for (int it = i0; it < i1; it++) {
                 if (it == n1) {
                     first = acc;
-                    acc = mk<double>(0, 0);
+                    acc = Sum{0, 0, 0, 0};
                 }
-                const int k = it < n1 ? r1 + it : r2 + (it - n1), l = it < n1 ? r1 : r2;
-                const cx<double> a = A[k];
-                const double c = Cd[k * P + l];
-                acc.x = fma(c, a.x, acc.x);
-                acc.y = fma(c, a.y, acc.y);
+                const int l = it < n1 ? r1 : r2, k = it < n1 ? r1 + it : r2 + (it - n1);
+                add_term(acc, Wd[k * 32 + l], Zs[wid][k]);
             }
-            if (i1 <= n1) {  // the half's terms were all row r1's
+            if (i1 <= n1) {
                 first = acc;
-                acc = mk<double>(0, 0);
+                acc = Sum{0, 0, 0, 0};
             }
-            // the first half of the warp finishes the rows r1, the second the rows r2
-            const cx<double> mine = hf ? acc : first, other = hf ? first : acc;
-            cx<double> s = mk<double>(mine.x + __shfl_xor_sync(0xffffffffu, other.x, 16),
-                                      mine.y + __shfl_xor_sync(0xffffffffu, other.y, 16));
-            const int row = hf ? r2 : r1;
-            const cx<double> o = mk<double>(__shfl_sync(0xffffffffu, own.x, row),
-                                            __shfl_sync(0xffffffffu, own.y, row));
-            s = fmm::cfma(iv, s, o);
-            if (j < nr && (hf == 0 || r2 != r1)) loc[b * P + row] = s;
-        } else if (lane < P) {
-            loc[b * P + lane] = own;
+            Sum s = meet(hf ? acc : first, hf ? first : acc);
+            if (row == 0) {  // k = 0, weight 2^31
+                const int4 z = Zs[wid][0];
+                s.xl += (unsigned long long)(unsigned)z.x << 31;
+                s.xh += (long long)z.y << 31;
+                s.yl += (unsigned long long)(unsigned)z.z << 31;
+                s.yh += (long long)z.w << 31;
+            }
+            sx = scale_sum(s.xh, s.xl, 31 + (row & 1));
+            sy = scale_sum(s.yh, s.yl, 31 + (row & 1));
+            mul_pow(sx, sy, (-row * h2) & 7);
+            bad |= ep >= kBadExp;
+            const int eb = max(e, ep);
+            sx = shift_down(sx, eb - ep);
+            sy = shift_down(sy, eb - ep);
+            e = eb;
+            __syncwarp();
+        }
+        sx += fixed54(ox, -(row >> 1), e + 1022);
+        sy += fixed54(oy, -(row >> 1), e + 1022);
+        if (leaf) {
+            const double nan = __longlong_as_double(0x7ff8000000000000ll);
+            const int E = e - 54 - (row >> 1);
+            if (on)
+                loc[b * P + row] = bad ? mk<double>(nan, nan)
+                                       : mk<double>(pack_double(sx, E), pack_double(sy, E));
+        } else {
+            const int nb = __reduce_max_sync(0xffffffffu, on ? bits_of(sx, sy) : 0), sh = nb - 54;
+            if (on)
+                *(longlong2 *)&loc[b * P + row] = make_longlong2(rescale(sx, sh), rescale(sy, sh));
+            if (lane == 0) ex[b] = bad ? kBadExp : nb == 0 ? kZeroExp : e + sh;
         }
         __threadfence();
         __syncwarp();
@@ -400,192 +552,6 @@ k_l2l(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_t *__r
     }
 }
 
-// The two passes of a small system, a thread block of four warps a leaf or box.
-//
-// Up: two chunks of a leaf's reals a warp; then the block that completes a box's last child
-// forms the box, a child a warp, the halves of a warp sharing each row's sum as in k_l2l.
-__global__ void __launch_bounds__(128)
-k_up_small(const int32_t *__restrict__ leaves, const int32_t *__restrict__ ix,
-           const int32_t *__restrict__ iy, const int32_t *__restrict__ parent,
-           const int32_t *__restrict__ child0, const int32_t *__restrict__ nchild, int P, int lchunks,
-           const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
-           const double *__restrict__ rows, const double *__restrict__ binom,
-           const cx<double> *__restrict__ dtab, const double2 *__restrict__ q, cx<double> *mp,
-           int *cnt, const int *gate, int64_t slab)
-{
-    lbf_rhs(slab, q, mp, cnt, gate);
-    if (fmm::gate_closed(gate)) return;
-    __shared__ double Cl[32 * 32];
-    __shared__ cx<double> As[4][32], part[4][32];
-    __shared__ int s_last;
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int e = threadIdx.x; e < P * P; e += blockDim.x) {
-        const int k = e / P, l = e % P;
-        Cl[e] = k <= l ? binom[l * LBF_MAX_TERMS + k] : 0.0;  // C(l, k)
-    }
-    const int64_t t = blockIdx.x;
-    const int b = leaves[t];
-    leaf_p2m(t, b, P, block0, items, rows, q, (double *)mp, lane, min(lchunks, 2 * wid),
-             min(lchunks, 2 * wid + 2));
-    const int hf = lane >> 4, j = lane & 15, nr = (P + 1) / 2;
-    const int r1 = j < nr ? j : 0, r2 = P - 1 - r1, n1 = r1 + 1, mid = (P + 2) / 2;
-    const int i0 = hf ? mid : 0, i1 = hf ? P + 1 : mid, row = hf ? r2 : r1;
-    for (int cur = b;;) {
-        const int p = parent[cur];
-        if (p < 0) break;
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int last = atomicAdd(&cnt[p], 1) == nchild[p] - 1;
-            if (last) cnt[p] = 0;  // ready for the next application
-            __threadfence();
-            s_last = last;
-        }
-        __syncthreads();
-        if (!s_last) break;
-        const int nc = nchild[p], c = child0[p] + wid;
-        if (wid < nc) {
-            const int d = (ix[c] & 1) + 2 * (iy[c] & 1);
-            if (lane < P)
-                As[wid][lane] = fmm::cmul(fmm::ldcg_cx(&mp[(int64_t)c * P + lane]), fmm::d2inv(dtab, d)[lane]);
-            const cx<double> dr = fmm::dpow(dtab, d)[row];
-            __syncwarp();
-            cx<double> acc = mk<double>(0, 0), first = mk<double>(0, 0);
-            for (int it = i0; it < i1; it++) {
-                if (it == n1) {
-                    first = acc;
-                    acc = mk<double>(0, 0);
-                }
-                const int k = it < n1 ? it : it - n1, l = it < n1 ? r1 : r2;
-                const cx<double> a = As[wid][k];
-                const double cc = Cl[k * P + l];
-                acc.x = fma(cc, a.x, acc.x);
-                acc.y = fma(cc, a.y, acc.y);
-            }
-            if (i1 <= n1) {
-                first = acc;
-                acc = mk<double>(0, 0);
-            }
-            const cx<double> mine = hf ? acc : first, other = hf ? first : acc;
-            const cx<double> s = mk<double>(mine.x + __shfl_xor_sync(0xffffffffu, other.x, 16),
-                                            mine.y + __shfl_xor_sync(0xffffffffu, other.y, 16));
-            if (j < nr && (hf == 0 || r2 != r1)) part[wid][row] = fmm::cmul(dr, s);
-        }
-        __syncthreads();
-        if (wid == 0 && lane < P) {
-            cx<double> a = part[0][lane];
-            for (int w = 1; w < nc; w++) {
-                a.x += part[w][lane].x;
-                a.y += part[w][lane].y;
-            }
-            mp[(int64_t)p * P + lane] = a;
-        }
-        cur = p;
-    }
-}
-
-// Down: as k_l2l, a box a thread block: the warps add every fourth translation, wait for the
-// parent together, and take a quarter of the shift's terms each (a half-warp an eighth).
-__global__ void __launch_bounds__(128)
-k_l2l_small(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_t *__restrict__ ix,
-            const int32_t *__restrict__ iy, const int32_t *__restrict__ parent, Own w, BoxGeo g,
-            const double *__restrict__ binom, const cx<double> *__restrict__ dtab, cx<double> *loc,
-            unsigned *pull, int *status, const int *gate, int64_t slab)
-{
-    lbf_rhs(slab, loc, pull, gate, w.y, w.sums);
-    if (!w.src) lbf_rhs(slab, w.part);
-    if (fmm::gate_closed(gate)) return;
-    __shared__ double Cd[32 * 32];
-    __shared__ cx<double> As[4][32], part[4][32], own[4][32];
-    __shared__ unsigned s_ticket, s_epoch;
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int e = threadIdx.x; e < P * P; e += blockDim.x) {
-        const int k = e / P, l = e % P;
-        Cd[e] = k >= l ? binom[k * LBF_MAX_TERMS + l] : 0.0;
-    }
-    if (threadIdx.x == 0) s_epoch = *(volatile unsigned *)&pull[2];
-    unsigned *done = pull + 4 + nbox;
-    const int hf = lane >> 4, j = lane & 15, nr = (P + 1) / 2, eighth = 2 * wid + hf;
-    const int r1 = j < nr ? j : 0, r2 = P - 1 - r1, n1 = P - r1;
-    const int i0 = (P + 1) * eighth / 8, i1 = (P + 1) * (eighth + 1) / 8;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_ticket = atomicAdd(&pull[3], 1u);
-        __syncthreads();
-        const int64_t b = (int64_t)s_ticket;
-        const unsigned epoch = s_epoch;
-        if (b >= nbox) break;
-        const int lv = level[b], p = parent[b];
-        const int d = (ix[b] & 1) + 2 * (iy[b] & 1);
-        const cx<double> dk = fmm::dpow(dtab, d)[lane], iv = fmm::d2inv(dtab, d)[lane];
-        if (w.sums && b == 0 && wid == 3) strength_sums(w, lane);
-        own[wid][lane] = own_part(w, b, P, lane, wid, 4, g.invL * fmm::pow2<double>(lv + 1), loc);
-        if (lv >= 3) {
-            if (threadIdx.x == 0) {
-                unsigned spins = 0;
-                const unsigned lim = wait_limit(status, kL2lSpins);
-                while (*(volatile unsigned *)&done[p] != epoch + 1u)
-                    if (++spins > lim) {
-                        atomicOr(status, LBF_DEV_TIMEOUT);
-                        break;
-                    }
-                __threadfence();
-            }
-            __syncthreads();
-            if (lane < P) As[wid][lane] = fmm::cmul(fmm::ldcg_cx(&loc[(int64_t)p * P + lane]), dk);
-            __syncwarp();
-            cx<double> acc = mk<double>(0, 0), first = mk<double>(0, 0);
-            for (int it = i0; it < i1; it++) {
-                if (it == n1) {
-                    first = acc;
-                    acc = mk<double>(0, 0);
-                }
-                const int k = it < n1 ? r1 + it : r2 + (it - n1), l = it < n1 ? r1 : r2;
-                const cx<double> a = As[wid][k];
-                const double c = Cd[k * P + l];
-                acc.x = fma(c, a.x, acc.x);
-                acc.y = fma(c, a.y, acc.y);
-            }
-            if (i1 <= n1) {
-                first = acc;
-                acc = mk<double>(0, 0);
-            }
-            const cx<double> mine = hf ? acc : first, other = hf ? first : acc;
-            const cx<double> s = mk<double>(mine.x + __shfl_xor_sync(0xffffffffu, other.x, 16),
-                                            mine.y + __shfl_xor_sync(0xffffffffu, other.y, 16));
-            if (j < nr && (hf == 0 || r2 != r1)) part[wid][hf ? r2 : r1] = s;
-        }
-        __syncthreads();
-        if (wid == 0) {
-            if (lane < P) {
-                cx<double> o = own[0][lane];
-                for (int w = 1; w < 4; w++) {
-                    o.x += own[w][lane].x;
-                    o.y += own[w][lane].y;
-                }
-                if (lv >= 3) {
-                    cx<double> s = part[0][lane];
-                    for (int w = 1; w < 4; w++) {
-                        s.x += part[w][lane].x;
-                        s.y += part[w][lane].y;
-                    }
-                    o = fmm::cfma(iv, s, o);
-                }
-                loc[b * P + lane] = o;
-            }
-            __threadfence();
-            __syncwarp();
-            if (lane == 0) atomicExch(&done[b], epoch + 1u);
-        }
-    }
-    if (threadIdx.x == 0 && atomicAdd(&pull[1], 1u) == gridDim.x - 1u) {
-        pull[1] = 0u;
-        pull[3] = 0u;
-        __threadfence();
-        atomicExch(&pull[2], s_epoch + 1u);
-    }
-}
-
 BoxGeo geo_of(const Tree &T)
 {
     return BoxGeo{T.xmin, T.ymin, T.L, (float)(1.0 / T.L), df64(1.0 / T.L), 1.0 / T.L};
@@ -597,15 +563,10 @@ static int l2l(lbf_plan *pl, int P, const Own &w, cx<double> *loc, int kid, cons
                cudaStream_t s)
 {
     const Tree &T = pl->tree;
-    const int64_t nsm = std::max(pl->nsm, 1);
-    if (T.nleaf < kSmallLeaves)
-        LBF_LAUNCH_P(kid, k_l2l_small, lbf_grid(pl, std::min<int64_t>(T.nbox, 8 * nsm)), 128, 0, s, T.nbox,
-                     P, T.level, T.ix, T.iy, T.parent, w, geo_of(T), pl->tab_binom,
-                     (const cx<double> *)pl->tab_dshift, loc, pl->pull, pl->dev_status, gate, pl->slab);
-    else
-        LBF_LAUNCH_P(kid, k_l2l, lbf_grid(pl, std::min<int64_t>(lbf_cdiv(T.nbox, 8), 4 * nsm)), 256, 0, s,
-                     T.nbox, P, T.level, T.ix, T.iy, T.parent, w, geo_of(T), pl->tab_binom,
-                     (const cx<double> *)pl->tab_dshift, loc, pl->pull, pl->dev_status, gate, pl->slab);
+    const int64_t grid = std::min<int64_t>(lbf_cdiv(T.nbox, 8), 6 * (int64_t)std::max(pl->nsm, 1));
+    LBF_LAUNCH_P(kid, k_l2l, lbf_grid(pl, grid), 256, 0, s, T.nbox, P, T.level, T.ix, T.iy, T.parent,
+                 T.nchild, w, geo_of(T), pl->tab_binom, loc, pl->loc_e, pl->pull, pl->dev_status, gate,
+                 pl->slab);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }
@@ -635,17 +596,10 @@ int lbf_passes_up(lbf_plan *pl, const int *gate, cudaStream_t s)
 {
     const Tree &T = pl->tree;
     const int P = pl->P, lch = (2 * P + 7) / 8;
-    const bool small = T.nleaf < kSmallLeaves;
-    if (small)
-        LBF_LAUNCH_P(LBF_KERNEL_UP, k_up_small, lbf_grid(pl, T.nleaf), 128, 0, s, T.leaves, T.ix, T.iy,
-                     T.parent, T.child0, T.nchild, P, lch, pl->rows_block0, pl->rows_items, pl->rows,
-                     pl->tab_binom, (const cx<double> *)pl->tab_dshift, pl->q, (cx<double> *)pl->mpole,
-                     pl->upcnt, gate, pl->slab);
-    else
-        LBF_LAUNCH_P(LBF_KERNEL_UP, k_up_rows, lbf_grid(pl, lbf_cdiv(T.nleaf, 4)), 128, 0, s, T.nleaf,
-                     T.leaves, T.ix, T.iy, T.parent, T.child0, T.nchild, P, lch, pl->rows_block0,
-                     pl->rows_items, pl->rows, pl->tab_binom, (const cx<double> *)pl->tab_dshift, pl->q,
-                     (cx<double> *)pl->mpole, pl->upcnt, gate, pl->slab);
+    LBF_LAUNCH_P(LBF_KERNEL_UP, k_up, lbf_grid(pl, lbf_cdiv(T.nleaf, 4)), 128, 0, s, T.nleaf, T.leaves,
+                 T.ix, T.iy, T.parent, T.child0, T.nchild, P, lch, pl->rows_block0, pl->rows_items,
+                 pl->rows, pl->tab_binom, pl->q, (cx<double> *)pl->mpole, pl->m2l_X, pl->m2l_e,
+                 pl->upcnt, gate, pl->slab);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }
@@ -657,7 +611,7 @@ int lbf_passes_apply(lbf_plan *pl, const int *gate, cudaStream_t s)
     const int P = pl->P;
     int rc = lbf_passes_up(pl, gate, s);
     if (rc) return rc;
-    rc = lbf_m2l_apply(pl, gate, s);
+    rc = lbf_m2l_apply(pl, gate, s, true);
     if (rc) return rc;
     if (pl->nbigx > 0)
         LBF_LAUNCH_P(LBF_KERNEL_DOWN, k_p2l_big, lbf_grid(pl, pl->nbigx), 128, kP2lSmem, s,
