@@ -142,7 +142,9 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
     if (o.matvec == LBF_MATVEC_FMM || o.border) {
         pl->upcnt = A.get<int32_t>(cap);
         pl->pull = A.get<uint32_t>(2 * cap + 4);
-        pl->loc_e = A.get<int32_t>(cap);
+        pl->lx_pitch = 2 * std::min(32, o.border ? 32 : P);
+        pl->loc_X = A.get<long long>(cap * pl->lx_pitch);
+        pl->loc_e = A.get<int32_t>(cap + LBF_PASS_WORDS);
     }
     if (o.matvec == LBF_MATVEC_FMM && o.fmm64) {
         pl->qdf = A.get<double2>(N);   // cx<df64>: 16 B per node
@@ -294,7 +296,8 @@ static void layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A)
     v->local = fmm ? A.get<double2>(cap * P) : nullptr;
     v->upcnt = fmm || o.border ? A.get<int32_t>(cap) : nullptr;
     v->pull = fmm || o.border ? A.get<uint32_t>(2 * cap + 4) : nullptr;
-    v->loc_e = fmm || o.border ? A.get<int32_t>(cap) : nullptr;
+    v->loc_X = fmm || o.border ? A.get<long long>(cap * pl->lx_pitch) : nullptr;
+    v->loc_e = fmm || o.border ? A.get<int32_t>(cap + LBF_PASS_WORDS) : nullptr;
     v->qdf = fmm && o.fmm64 ? (void *)A.get<double2>(N) : nullptr;
     v->q32 = f32 ? A.get<float2>(N) : nullptr;
     v->mpole32 = f32 && fmm ? A.get<float2>(cap * (o.p32 + 1)) : nullptr;
@@ -369,7 +372,7 @@ lbf_plan lbf_view_at(const lbf_plan &v, int r)
     mv(o.red); mv(o.red_count); mv(o.fvec); mv(o.yvec); mv(o.tin); mv(o.tout); mv(o.vstep);
     mv(o.bd.partial); mv(o.bd.loc); mv(o.bd.loc32); mv(o.bd.sums); mv(o.H); mv(o.gw);
     mv(o.gx); mv(o.gb); mv(o.gpart); mv(o.gs); mv(o.V); mv(o.region); mv(o.nearbuf);
-    mv(o.dpart); mv(o.dcount); mv(o.m2l_X); mv(o.m2l_e); mv(o.m2l_out); mv(o.loc_e);
+    mv(o.dpart); mv(o.dcount); mv(o.m2l_X); mv(o.m2l_e); mv(o.m2l_out); mv(o.loc_e); mv(o.loc_X);
     o.nrhs = 1;
     o.slab = 0;
     return o;
@@ -618,6 +621,14 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
     }
     if (pl->dcount) CK(cudaMemsetAsync(pl->dcount, 0, sizeof(unsigned) * lbf_cdiv(N, 32), s));
     if (pl->upcnt) CK(cudaMemsetAsync(pl->upcnt, 0, sizeof(int32_t) * cap, s));
+    if (pl->loc_X) {  // no word carries the first application's tag
+        CK(cudaMemsetAsync(pl->loc_X, 0, sizeof(long long) * cap * pl->lx_pitch, s));
+        CK(cudaMemsetAsync(pl->loc_e, 0, sizeof(int32_t) * (cap + LBF_PASS_WORDS), s));
+    }
+    if (pl->m2l_cap) {
+        CK(cudaMemsetAsync(pl->m2l_X, 0, sizeof(long long) * cap * ((2 * pl->P + 7) / 8 * 8), s));
+        CK(cudaMemsetAsync(pl->m2l_e, 0, sizeof(int32_t) * cap, s));
+    }
     if (pl->pull) CK(cudaMemsetAsync(pl->pull, 0, sizeof(uint32_t) * (2 * cap + 4), s));
     CK(cudaMemcpyAsync(pl->tab_tpow, tpow.data(), sizeof(double2) * tpow.size(), cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(pl->dev_status, 0, 2 * sizeof(int), s));

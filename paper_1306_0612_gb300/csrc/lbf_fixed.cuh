@@ -11,6 +11,22 @@ constexpr int kZeroExp = -5118;    // exponent of a box of zeros
 
 __host__ __device__ inline int real_pitch(int P) { return (2 * P + 7) / 8 * 8; }
 
+// Words of an expansion as its readers find them: the integer in 56 bits (the exponent in 24)
+// under a tag of 8 bits, the application's number.  A reader of the same launch waits on the
+// words themselves until they carry the tag, so a box is handed on with one store and one
+// load where a flag costs a fence and two trips to L2 more.  The tags go round 1 .. 255 (0:
+// words that no launch of that kind wrote) and every launch rewrites all words, so an old word
+// never carries the tag waited for.
+__device__ __forceinline__ long long tag_word(long long x, unsigned tag)
+{
+    return (long long)(((unsigned long long)x & 0xffffffffffffffull) | ((unsigned long long)tag << 56));
+}
+__device__ __forceinline__ long long untag(long long w) { return (long long)((unsigned long long)w << 8) >> 8; }
+__device__ __forceinline__ bool has_tag(long long w, unsigned tag) { return (unsigned)((unsigned long long)w >> 56) == tag; }
+__device__ __forceinline__ int tag_exp(int e, unsigned tag) { return (int)(((unsigned)e & 0xffffffu) | (tag << 24)); }
+__device__ __forceinline__ int untag_exp(int w) { return (int)((unsigned)w << 8) >> 8; }
+__device__ __forceinline__ bool exp_has_tag(int w, unsigned tag) { return (unsigned)w >> 24 == tag; }
+
 // v as an integer in units of 2^(e - 54), rounded, |v| < 2^e: its double bits with the
 // exponent lowered by `drop`; top: the largest lowered exponent field of the set (> 0)
 __device__ __forceinline__ long long fixed54(long long bits, int drop, int top)

@@ -12,6 +12,7 @@
 #define LBF_MAX_TERMS 64  // expansion terms p + 1 supported by the kernels
 #define LBF_MAX_LEVELS 31
 #define LBF_ANC_STRIDE 32
+#define LBF_PASS_WORDS 8  // of lbf_passes.cu: up ticket, warps done, application; down application
 
 // Per-process launch counter (lbf_launch_count).
 extern std::atomic<int64_t> g_lbf_launches;
@@ -189,7 +190,11 @@ struct lbf_plan {
     int32_t *m2l_vptr = nullptr, *m2l_tile0 = nullptr, *m2l_f = nullptr, *m2l_e = nullptr;
     uint4 *m2l_img = nullptr;
     long long *m2l_X = nullptr;
-    int32_t *loc_e = nullptr;   // exponents of the integer local expansions (lbf_passes.cu)
+    // integer local expansions (lbf_passes.cu): lx_pitch reals a box, exponents, and after
+    // them the passes' words (kPassWords)
+    long long *loc_X = nullptr;
+    int32_t *loc_e = nullptr;
+    int lx_pitch = 0;
     double *m2l_out = nullptr;
     // stored leaf rows of the accurate forward operator (lbf_rows.cu; rows null: not stored)
     // direct sums: partial sums of the runs of sources, finished runs per 32 nodes

@@ -96,9 +96,9 @@ __global__ void k_m2l_fix(int64_t nbox, int P, const cx<double> *__restrict__ mp
 #pragma unroll
     for (int h = 0; h < 2; h++) {
         const int m = lane + 32 * h;
-        if (m < pitch) X[b * pitch + m] = fixed54(v[h], m >> 2, top);
+        if (m < pitch) X[b * pitch + m] = tag_word(fixed54(v[h], m >> 2, top), 0);
     }
-    if (lane == 0) ex[b] = bad ? kBadExp : top - 1022;
+    if (lane == 0) ex[b] = tag_exp(bad ? kBadExp : top - 1022, 0);
 }
 
 // digit images (the rows of the digits one after another) and row exponents of the
@@ -308,7 +308,7 @@ k_m2l_tc(int P, const int32_t *__restrict__ tile0, const int2 *__restrict__ pair
                 unsigned lo[8], hi[8];
 #pragma unroll
                 for (int i = 0; i < 4; i++) {
-                    const unsigned long long a = digits(x[h][i].x), b = digits(x[h][i].y);
+                    const unsigned long long a = digits(untag(x[h][i].x)), b = digits(untag(x[h][i].y));
                     lo[2 * i] = (unsigned)a;
                     hi[2 * i] = (unsigned)(a >> 32);
                     lo[2 * i + 1] = (unsigned)b;
@@ -356,7 +356,7 @@ k_m2l_tc(int P, const int32_t *__restrict__ tile0, const int2 *__restrict__ pair
             const unsigned n = (unsigned)(t - t0);
             while (t >= s_tile0[o + 1]) o++;
             const int2 pr = pairs[(int64_t)t * kRowsT + quarter * 32 + lane];
-            const int e = pr.x >= 0 ? ex[pr.x] : 0;
+            const int e = pr.x >= 0 ? untag_exp(ex[pr.x]) : 0;
             const int32_t *f = fx + o * 64;
             double *dst = out + (int64_t)pr.y * 2 * P;
             wait(mm, n & 1);
