@@ -57,4 +57,71 @@ __device__ __forceinline__ double pack_double(long long w, int E)
     return __longlong_as_double((long long)(bits | (w < 0 ? 0x8000000000000000ull : 0ull)));
 }
 
+// Dot products on the integer pipes.  A 32 x 32 -> 64 bit multiply-add leaves a scheduler every
+// 4 cycles, a double one every 64; an integer x of 54 bits (|x| <= 2^53) goes as two words,
+// x = hi 2^27 + lo, |hi| <= 2^26, |lo| <= 2^26, and a product as the three of them that reach the
+// leading 54 of its 106 bits (measured 2.16e12 such products a second, 0.49e12 double).
+__device__ __forceinline__ int2 split27(long long x)
+{
+    const int lo = (int)((unsigned)x << 5) >> 5;
+    return make_int2(lo, (int)((x - lo) >> 27));
+}
+struct Dot {  // sum = h 2^54 + m 2^27, of 768 products at most
+    long long h, m;
+};
+__device__ __forceinline__ void dot_add(Dot &d, int2 e, int2 x)
+{
+    d.h += (long long)e.y * x.y;
+    d.m += (long long)e.y * x.x;
+    d.m += (long long)e.x * x.y;
+}
+// asks for the tiles at p (a multiple of 256 bytes) to be brought to L2, by one lane
+__device__ __forceinline__ void prefetch_tiles(const double *p, int tiles, int lane)
+{
+    if (lane == 0 && tiles > 0)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(tiles * 256) : "memory");
+}
+__device__ __forceinline__ int2 shfl_word(int2 v, int src)
+{
+    return make_int2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+__device__ __forceinline__ long long shfl_xor_ll(long long v, int mask)
+{
+    return (long long)__shfl_xor_sync(0xffffffffu, (unsigned long long)v, mask);
+}
+// a lane keeps one of two sums (the second: `second`) and adds its partner's part of it
+__device__ __forceinline__ Dot dot_meet(const Dot &x, const Dot &y, bool second, int bit)
+{
+    const Dot keep = second ? y : x, send = second ? x : y;
+    return Dot{keep.h + shfl_xor_ll(send.h, bit), keep.m + shfl_xor_ll(send.m, bit)};
+}
+// d 2^E as a double
+__device__ __forceinline__ double dot_double(Dot d, int E)
+{
+    const long long t = d.h + (d.m >> 27);
+    const int f = (int)(d.m & 0x7ffffff);
+    const int sh = min(27, __clzll(t < 0 ? ~t : t) - 2);  // room left of t's bits
+    return pack_double((long long)((unsigned long long)t << sh) + (f >> (27 - sh)), E + 54 - sh);
+}
+// the words of v, its exponent field raised by `up`, in a sum whose largest raised field is top
+__device__ __forceinline__ int2 dot_word(double v, int up, int top)
+{
+    return split27(fixed54(__double_as_longlong(v), -up, top + 1));
+}
+__device__ __forceinline__ int exp_field(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff); }
+
+// f<NG>() for the number of row groups of a block, 1 to 8: the loops over tiles have a copy
+// each, and nothing else does (with whole kernels copied the warps waited for instructions)
+#define LBF_GROUPS(ng, CALL)    \
+    switch (ng) {               \
+    case 1: CALL(1); break;     \
+    case 2: CALL(2); break;     \
+    case 3: CALL(3); break;     \
+    case 4: CALL(4); break;     \
+    case 5: CALL(5); break;     \
+    case 6: CALL(6); break;     \
+    case 7: CALL(7); break;     \
+    default: CALL(8); break;    \
+    }
+
 }  // namespace

@@ -209,6 +209,7 @@ struct lbf_plan {
     // columns (rptr null: not stored), a value per column
     int32_t *rows_block0 = nullptr, *rows_rptr = nullptr, *rows_rbase = nullptr;
     double *rows_z = nullptr;
+    int32_t *rows_e = nullptr;  // exponent field of each node's largest near entry
     // boxes whose X lists are not near columns (nbigx < 0: the passes of lbf_passes.cu are off)
     int64_t nbigx = -1, bigx_cap = 0;
     int32_t *bigx = nullptr;
@@ -218,6 +219,7 @@ struct lbf_plan {
     double *bsig = nullptr;     // scalar beta . sigma
     double *red = nullptr;      // reduction partials
     unsigned int *red_count = nullptr;
+    int32_t *sigma_e = nullptr;  // largest exponent field of the density: being formed, of the last pass
     // border
     Border bd;                  // E y by island expansions (E itself is never formed)
     double *Sinv = nullptr;     // M x M inverse Schur complement, or (lu) its LU factors

@@ -42,49 +42,88 @@ namespace {
 constexpr int kP2lSmem = 4 * 32 * 33 * 16;
 constexpr int kGroups = 8;  // row groups of a block at most (lbf_rows.cu)
 
-// P2M of leaf t by a warp, the chunks cbeg .. cend - 1 of eight reals: sum_i q_i u_i^l over the
-// leaf's row blocks, four chunks at a time.  Column 2 l of a row holds -(1/pi) Im u^l, column 2 l + 1 -(1/pi) Re u^l:
-// an even lane adds their parts of both reals of coefficient l, an odd lane likewise, and
-// one exchange leaves the real part on the even lane, the imaginary part on the odd one.
-__device__ __forceinline__ void leaf_p2m(int64_t t, int P,
+// re[h], im[h] += the tiles of chunk h (of n, at most 4) times the rows' values
+template <int NG>
+__device__ __forceinline__ void p2m_chunks(const double *__restrict__ t, const int2 *cr, const int2 *ci,
+                                           int n, Dot *re, Dot *im)
+{
+#pragma unroll
+    for (int h = 0; h < 4; h++) {
+        const double *th = t + 32 * NG * min(h, n - 1);  // (beyond n: a sum nobody takes)
+#pragma unroll
+        for (int g = 0; g < NG; g++) {
+            const int2 e = *(const int2 *)&th[32 * g];
+            dot_add(re[h], e, cr[g]);
+            dot_add(im[h], e, ci[g]);
+        }
+    }
+}
+
+// P2M of leaf t by a warp: a_l = sum_i q_i u_i^l, the reals left in a[2 P].  Column 2 l of a row holds -(1/pi) Im u^l, column 2 l + 1 -(1/pi) Re u^l,
+// both times 2^-(l/2): an even lane adds their parts of both reals of coefficient l, an odd lane
+// likewise, and one exchange leaves the real part on the even lane, the imaginary part on the
+// odd one.  The charges are integers in units of the leaf's largest (up bits more for a leaf
+// of many nodes); sum: room for the 2 P sums of a leaf of several row blocks.
+__device__ __forceinline__ void leaf_p2m(int64_t t, int P, int lchunks,
                                          const int32_t *__restrict__ block0,
                                          const RowItem *__restrict__ items,
                                          const double *__restrict__ rows,
-                                         const double2 *__restrict__ q, double *a, int lane,
-                                         int cbeg, int cend)
+                                         const double2 *__restrict__ q, double *a, Dot *sum, int lane)
 {
     const int k0 = block0[t], k1 = block0[t + 1];
     const bool odd = (lane & 1) != 0, u = (lane & 16) != 0, w = (lane & 8) != 0;
-    for (int c = cbeg; c < cend; c += 4) {
-        double re[4] = {0.0, 0.0, 0.0, 0.0}, im[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int k = k0; k < k1; k++) {
-            const RowItem it = items[k];
-            const int ng = (it.nrow + 3) / 4;
-            const double *tl = rows + ((int64_t)it.tile + (int64_t)(it.nchunk + c) * ng) * 32 + lane;
+    int top = 0, n = 0;
+    bool bad = false;
+    for (int k = k0; k < k1; k++) {
+        const RowItem it = items[k];
+        const int row0 = it.row0, nrow = it.nrow, ng = (nrow + 3) / 4;  // 32 rows at most
+        prefetch_tiles(rows + ((int64_t)it.tile + (int64_t)it.nchunk * ng) * 32, lchunks * ng, lane);
+        const double2 qq = lane < nrow ? q[row0 + lane] : make_double2(0.0, 0.0);
+        const int E = max(exp_field(qq.x), exp_field(qq.y));
+        bad |= E == 0x7ff;
+        top = max(top, E);
+        n += nrow;
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    bad = __any_sync(0xffffffffu, bad);
+    const int up = n > 128 ? 25 - __clz(n) : 0;  // n 2^-up <= 128
+    for (int k = k0; k < k1; k++) {
+        const RowItem it = items[k];
+        const int ng = (it.nrow + 3) / 4;
+        // a charge a lane, then the rows of each lane's sums: (im, -re) of q for the columns of
+        // Im u^l, (-re, -im) for those of Re u^l
+        const double2 qq = lane < it.nrow ? q[it.row0 + lane] : make_double2(0.0, 0.0);
+        const int2 qx = dot_word(-qq.x, 0, top + up), qy = dot_word(qq.y, 0, top + up);
+        int2 cr[kGroups], ci[kGroups];
 #pragma unroll
-            for (int g = 0; g < kGroups; g++)
-                if (g < ng) {
-                    const int r = 4 * g + (lane >> 3);
-                    const double2 qq = r < it.nrow ? q[it.row0 + r] : make_double2(0.0, 0.0);
-                    const double cr = odd ? -qq.x : qq.y, ci = odd ? -qq.y : -qq.x;
-#pragma unroll
-                    for (int h = 0; h < 4; h++)
-                        if (c + h < cend) {
-                            const double e = tl[32 * (h * ng + g)];
-                            re[h] = fma(e, cr, re[h]);
-                            im[h] = fma(e, ci, im[h]);
-                        }
-                }
+        for (int g = 0; g < kGroups; g++) {
+            const int2 x = shfl_word(qx, 4 * g + (lane >> 3)), y = shfl_word(qy, 4 * g + (lane >> 3));
+            cr[g] = odd ? x : y;
+            ci[g] = odd ? make_int2(-y.x, -y.y) : x;
         }
-        double s[4];
+        const double *tl = rows + ((int64_t)it.tile + (int64_t)it.nchunk * ng) * 32 + lane;
+        for (int c = 0; c < lchunks; c += 4, tl += 128 * ng) {
+            Dot re[4], im[4];
 #pragma unroll
-        for (int h = 0; h < 4; h++)
-            s[h] = (odd ? im[h] : re[h]) + __shfl_xor_sync(0xffffffffu, odd ? re[h] : im[h], 1);
-        const double b0 = (u ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, u ? s[0] : s[2], 16);
-        const double b1 = (u ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, u ? s[1] : s[3], 16);
-        const double v = (w ? b1 : b0) + __shfl_xor_sync(0xffffffffu, w ? b0 : b1, 8);
-        const int h = (u ? 2 : 0) + (w ? 1 : 0), m = 8 * (c + h) + (lane & 7);
-        if (c + h < cend && m < 2 * P) a[m] = v * LBF_PI;
+            for (int h = 0; h < 4; h++) re[h] = im[h] = Dot{0, 0};
+#define LBF_DOT(NG) p2m_chunks<NG>(tl, cr, ci, lchunks - c, re, im)
+            LBF_GROUPS(ng, LBF_DOT)
+#undef LBF_DOT
+            Dot s[4];
+#pragma unroll
+            for (int h = 0; h < 4; h++) s[h] = dot_meet(re[h], im[h], odd, 1);
+            Dot v = dot_meet(dot_meet(s[0], s[2], u, 16), dot_meet(s[1], s[3], u, 16), w, 8);
+            const int h = (u ? 2 : 0) + (w ? 1 : 0), m = 8 * (c + h) + (lane & 7);
+            if (c + h < lchunks && m < 2 * P) {
+                if (k > k0) {
+                    v.h += sum[m].h;
+                    v.m += sum[m].m;
+                }
+                if (k + 1 < k1) sum[m] = v;
+                else a[m] = bad ? __longlong_as_double(0x7ff8000000000000ll)
+                                : dot_double(v, top + up - 1129 + (m >> 2)) * LBF_PI;
+            }
+        }
     }
 }
 
@@ -355,7 +394,7 @@ constexpr unsigned kPassSpins = 1u << 22;
 // rotated (times 2, k even, or 1 +- i, k odd), and the sum over k times 2^-(l+1), rotated by
 // (2d)^l, is the parent's X_l.  Lane j of a half-warp has the rows j and P - 1 - j of the
 // triangle, P + 1 terms, a half of them each half.
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 4)
 k_up(int64_t nleaf, int64_t nbox, const int32_t *__restrict__ leaves, const int32_t *__restrict__ ix,
      const int32_t *__restrict__ iy, const int32_t *__restrict__ child0,
      const int32_t *__restrict__ nchild, int P, int lchunks, const int32_t *__restrict__ block0,
@@ -368,6 +407,7 @@ k_up(int64_t nleaf, int64_t nbox, const int32_t *__restrict__ leaves, const int3
     __shared__ unsigned Cl[32 * 32];
     __shared__ int4 Zs[4][32];
     __shared__ double vs[4][64];
+    __shared__ Dot sums[4][64];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int e = threadIdx.x; e < P * P; e += blockDim.x) {
         const int k = e / P, l = e % P;
@@ -388,7 +428,7 @@ k_up(int64_t nleaf, int64_t nbox, const int32_t *__restrict__ leaves, const int3
         if (t >= nleaf + nbox) break;
         if (t < nleaf) {
             const int b = leaves[t];
-            leaf_p2m(t, P, block0, items, rows, q, vs[wid], lane, 0, lchunks);
+            leaf_p2m(t, P, lchunks, block0, items, rows, q, vs[wid], sums[wid], lane);
             __syncwarp();
             double v[2];
             int top = -4096;

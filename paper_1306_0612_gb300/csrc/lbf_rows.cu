@@ -25,14 +25,28 @@
 // such boxes a leaf, but up to 22, and a chain of P dependent steps for each, run by the
 // leaf's warp, held the launch at 181,783 nodes to 250 us.
 //
+// On the integer pipes: a double multiply-add leaves a scheduler every 64 cycles, the three
+// 32 x 32 -> 64 bit products that stand for one every 17 (lbf_fixed.cuh).  An entry is an integer
+// of 54 bits below its row's largest near entry (rexp), the density below its largest, the
+// local columns and the expansion below fixed sizes (|u_i^l| 2^-(l/2) < 3/2); the sums are exact
+// but for the products' last 52 bits.  Errors of whole applications against 64 bits are what they
+// were with double entries, to three digits, at orders 22 to 31.  The multipole columns, few and in units
+// of their own, stay double.
+//
 // Layout: a leaf's rows are cut into blocks of at most kGroups groups of four rows, its
 // columns into chunks of eight; a tile is one group x one chunk, 32 doubles, row-major,
 // so lane = 8 (row mod 4) + (column mod 8) and a warp's load is 256 contiguous bytes.  A
-// block's tiles are stored chunk by chunk: the near nodes and the W multipoles' reals, then
+// block's tiles are stored chunk by chunk: the near nodes, the W multipoles' reals, then
 // the 2 P reals of the local expansion.  Each lane holds one sum per group; eight lanes share a row, and a butterfly
 // that halves the groups at each step adds them in 7 additions for 8 groups (lanes on
 // rows alone would leave 19 % of the lanes idle at 26 nodes a leaf, lanes on columns
 // alone would add 31 shuffled sums to 4 x 26 multiply-adds).
+//
+// Measured, rows of one application at 16.8 million nodes, 416,768 and 8192: 6.5 ms, 127 us
+// and 14 us (double entries 7.4 ms, 201 us, 22 us); transposed, 131,072 nodes, 89 and 97 us
+// (147 and 137).  Bound by the latency of the tiles' loads, 3.9 of 6.7 TB/s at the large end: the
+// next eight chunks are asked for ahead, four are read at once; more warps with fewer loads
+// each were slower (6.9 ms with two chunks at once, 8.8 with 24 warps an SM).
 //
 // The transposed rows (K^T tau)_i read the same tiles: near pairs are symmetric (b's columns
 // hold leaf t's nodes exactly when t's hold b's), so each leaf forms z = G_b^T tau_b over its
@@ -41,6 +55,7 @@
 // The far field is Im(w_i Phi(xi_i)): the same local and M2P columns with two sums a row.
 #include <algorithm>
 
+#include "lbf_fixed.cuh"
 #include "lbf_fmm_tpl.cuh"
 
 using fmm::BoxGeo;
@@ -55,6 +70,12 @@ constexpr int kGroups = 8, kGroupsSmall = 2;
 // (8192 nodes: 458 us an application with whole leaves a warp, 408 shared; at 7130 leaves
 // the two are within 1 %, at 16,150 sharing costs 4 % of a solve)
 constexpr int64_t kSmallLeaves = 4864;
+constexpr int kLocalTop = 1021;  // exponent field of the local columns' largest: [1/4, 1/2)
+constexpr int kRowBlocks = 4;    // thread blocks an SM
+constexpr int kRun = 4;          // chunks read at a time (2 or 4)
+constexpr int kAhead = 8;        // chunks asked for before they are read
+constexpr int kDotChunks = 64;   // chunks a Dot takes at most between two conversions (a multiple of 4)
+static_assert(kDotChunks % 4 == 0, "xs is filled by four chunks");
 
 // the column ranges of leaf b, in order: U(b), the small boxes of W(b), the X lists of
 // b and its ancestors that are small.  f(first node, end)
@@ -101,8 +122,7 @@ __global__ void k_rows_count(int64_t nleaf, const int32_t *__restrict__ leaves, 
     unsigned long long nt = 0, nc = 0;
     if (t < nleaf) {
         const int b = leaves[t];
-        const long long cols = near_nodes(T, b, thr) + 2ll * P * big_boxes(T, b, thr);
-        const long long ch = (cols + 7) / 8, g = (T.end[b] - T.begin[b] + 3) / 4;
+        const long long ch = (near_nodes(T, b, thr) + 7) / 8 + (2ll * P * big_boxes(T, b, thr) + 7) / 8, g = (T.end[b] - T.begin[b] + 3) / 4;
         nc = (unsigned long long)ch;
         nt = (unsigned long long)(g * (ch + lchunks));
         chunks[t] = (int32_t)ch;
@@ -146,8 +166,9 @@ __global__ void k_rows_items(int64_t nleaf, const int32_t *__restrict__ leaves, 
     }
 }
 
-// each leaf's columns, a warp per leaf: node j, or -1 - m for the real m of the multipoles;
-// the last chunk is filled up with the leaf's first node (zero entries)
+// each leaf's columns, a warp per leaf: the near nodes, then from the next chunk on -1 - m for
+// the real m of the multipoles; both are filled up to a chunk with the leaf's first node (zero
+// entries)
 __global__ void k_rows_cols(int64_t nleaf, const int32_t *__restrict__ leaves, TreeLists T, int thr,
                             int P,
                             const int32_t *__restrict__ chunk0, int32_t *__restrict__ cols)
@@ -162,6 +183,8 @@ __global__ void k_rows_cols(int64_t nleaf, const int32_t *__restrict__ leaves, T
         for (int j = s + lane; j < e; j += 32) c[m + j - s] = j;
         m += e - s;
     });
+    if (m + lane < (m + 7) / 8 * 8) c[m + lane] = T.begin[b];
+    m = (m + 7) / 8 * 8;
     for (int q = T.wptr[b]; q < T.wptr[b + 1]; q++) {
         const int s = T.widx[q];
         if (T.end[s] - T.begin[s] <= thr) continue;
@@ -205,26 +228,33 @@ __global__ void k_rows_rev_sort(int64_t nleaf, const int32_t *__restrict__ ptr, 
     }
 }
 
-// the entries, a warp per row block
+// the entries, a warp per row block: the near ones as doubles first, turned into integers in
+// the unit of their row's largest once that is known
 __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, TreeLists T, int thr,
                             BoxGeo g, int P, int lchunks, const int32_t *__restrict__ cols,
                             const double2 *__restrict__ xi, const double2 *__restrict__ w,
-                            const double *__restrict__ dself, double *__restrict__ rows)
+                            const double *__restrict__ dself, double *__restrict__ rows,
+                            int32_t *__restrict__ rexp)
 {
     const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (k >= nitem) return;
     const RowItem it = items[k];
     const int ng = (it.nrow + 3) / 4;
-    const int ncol = it.ncol;
-    const int nend = ncol + 2 * P * big_boxes(T, it.box, thr);
+    const int ncol = it.ncol, nn = (ncol + 7) / 8;
+    const int nend = 8 * nn + 2 * P * big_boxes(T, it.box, thr);
     double *t = rows + (int64_t)it.tile * 32 + lane;
-    for (int c = 0; c < it.nchunk; c++) {
+    int top[kGroups];
+#pragma unroll
+    for (int q = 0; q < kGroups; q++) top[q] = 0;
+    for (int c = 0; c < nn; c++, t += 32 * ng) {
         const int m = 8 * c + (lane & 7);
         const bool node = m < ncol;
         const int j = node ? cols[(int64_t)it.chunk * 8 + m] : it.row0;
         const double2 zj = xi[j], wj = w[j];
-        for (int q = 0; q < ng; q++, t += 32) {
+#pragma unroll
+        for (int q = 0; q < kGroups; q++) {
+            if (q >= ng) break;
             const int r = 4 * q + (lane >> 3), i = it.row0 + r;
             double e = 0.0;
             if (r < it.nrow && node) {
@@ -241,14 +271,30 @@ __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, Tr
                     e = fma(wj.y, dr, -wj.x * di) * id * (1.0 / LBF_PI);
                 }
             }
-            if (node || m >= nend || r >= it.nrow) *t = e;
+            t[32 * q] = e;
+            top[q] = max(top[q], exp_field(e));
         }
     }
+#pragma unroll
+    for (int q = 0; q < kGroups; q++) {
+        if (q >= ng) break;
+        for (int o = 4; o > 0; o >>= 1) top[q] = max(top[q], __shfl_xor_sync(0xffffffffu, top[q], o));
+        const int r = 4 * q + (lane >> 3);
+        if ((lane & 7) == 0 && r < it.nrow) rexp[it.row0 + r] = top[q];
+    }
+    t = rows + (int64_t)it.tile * 32 + lane;
+    for (int c = 0; c < nn; c++, t += 32 * ng)
+#pragma unroll
+        for (int q = 0; q < kGroups; q++)
+            if (q < ng) *(int2 *)&t[32 * q] = dot_word(t[32 * q], 0, top[q]);
+    for (int c = nn; c < it.nchunk; c++, t += 32 * ng)
+        for (int q = 0; q < ng; q++)
+            if (8 * c + (lane & 7) >= nend || 4 * q + (lane >> 3) >= it.nrow) t[32 * q] = 0.0;
     const int b = it.box;
     // the M2P columns: powers of rho_i, a lane per row
-    if (lane < it.nrow && nend > ncol) {
+    if (lane < it.nrow && nend > 8 * nn) {
         const double2 zi = xi[it.row0 + lane];
-        int m = ncol;
+        int m = 8 * nn;
         for (int q = T.wptr[b]; q < T.wptr[b + 1]; q++) {
             const int s = T.widx[q];
             if (T.end[s] - T.begin[s] <= thr) continue;
@@ -265,7 +311,7 @@ __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, Tr
             }
         }
     }
-    // the local expansion's columns: powers of u_i, a lane per row
+    // the local expansion's columns: powers of u_i, times 2^-(l/2) below 1/2, a lane per row
     double cxd, cyd, r;
     box_centre(g, T.level[b], T.ix[b], T.iy[b], cxd, cyd, r);
     const double ir = 1.0 / r;
@@ -276,9 +322,12 @@ __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, Tr
     double *base = rows + ((int64_t)it.tile + (int64_t)it.nchunk * ng) * 32;
     if (lane < 4 * ng)
         for (int l = 0; l < 4 * lchunks; l++) {
-            double2 e = make_double2(0.0, 0.0);
-            if (l < P) e = make_double2(p.y, p.x);  // times (b_l.x, b_l.y)
-            *(double2 *)(base + ((int64_t)(l >> 2) * ng + (lane >> 2)) * 32 + (lane & 3) * 8 +
+            int4 e = make_int4(0, 0, 0, 0);
+            if (l < P) {  // times (b_l.x, b_l.y)
+                const int2 ey = dot_word(p.y, -(l >> 1), kLocalTop), ex = dot_word(p.x, -(l >> 1), kLocalTop);
+                e = make_int4(ey.x, ey.y, ex.x, ex.y);
+            }
+            *(int4 *)(base + ((int64_t)(l >> 2) * ng + (lane >> 2)) * 32 + (lane & 3) * 8 +
                          2 * (l & 3)) = e;
             p = cmul(p, u);
         }
@@ -296,128 +345,200 @@ __device__ __forceinline__ double local_real(const cx<df64> *loc, int64_t at)
     return (double)v.x + (double)v.y;
 }
 
-// The sums of a block of NG row groups over its column chunks k0 .. k1 - 1 (near chunks,
-// then the local expansion's); lane's result (after the butterfly) and its row.  The
-// columns' values are fetched 32 at a time, a column a lane, one step ahead of their tiles,
-// and handed to the row lanes by shuffles: the chain index -> density -> multiply-add is
-// then two loads per 4 NG tiles (a fetch per chunk left a small system waiting on it).
-template <int NG, typename R>
-__device__ __forceinline__ double block_rows(const RowItem &it, const double *__restrict__ rows,
-                                             const int32_t *__restrict__ cols,
-                                             const double *__restrict__ sigma,
-                                             const cx<R> *__restrict__ loc,
-                                             const cx<R> *__restrict__ mp, int P, int k0, int k1,
-                                             int lane, int &row)
+// Add the eight lanes of a row over G groups: at each step a lane keeps one half of its groups
+// and sends the other half to its partner; once one is left, plain sums.  Returns the lane's
+// group (G: another lane has this row).
+template <int G, class F> __device__ __forceinline__ int fold_rows(int lane, F add)
 {
-    constexpr int NP = NG <= 1 ? 1 : NG <= 2 ? 2 : NG <= 4 ? 4 : 8;  // power of two >= NG
-    double acc[NP];
-#pragma unroll
-    for (int q = 0; q < NP; q++) acc[q] = 0.0;
-    const double *t = rows + ((int64_t)it.tile + (int64_t)k0 * NG) * 32 + lane;
-    const int near = 8 * it.nchunk, end = 8 * k1;
-    const int32_t *c = cols + (int64_t)it.chunk * 8;
-    const int64_t lb = (int64_t)it.box * 2 * P;
-    auto index = [&](int m) { return m < near && m < end ? c[m] : 0; };
-    auto value = [&](int m, int j) {
-        if (m < near) return j >= 0 ? sigma[j] : local_real(mp, -1 - j);
-        return m < near + 2 * P ? local_real(loc, lb + m - near) : 0.0;
-    };
-    int m = 8 * k0 + lane;
-    double s = m < end ? value(m, index(m)) : 0.0;
-    int jn = index(m + 32);
-    for (int k = k0; k < k1; k += 4) {
-        const double sc = s;
-        m += 32;
-        s = m < end ? value(m, jn) : 0.0;
-        jn = index(m + 32);
-#pragma unroll
-        for (int h = 0; h < 4; h++) {
-            if (k + h < k1) {
-                double e[NG];
-#pragma unroll
-                for (int q = 0; q < NG; q++) e[q] = t[32 * (h * NG + q)];
-                const double sh = __shfl_sync(0xffffffffu, sc, 8 * h + (lane & 7));
-#pragma unroll
-                for (int q = 0; q < NG; q++) acc[q] = fma(e[q], sh, acc[q]);
-            }
-        }
-        t += 32 * 4 * NG;
-    }
-    // add the eight lanes of a row: at each step a lane keeps one half of its groups and
-    // sends the other half to its partner; once one is left, plain sums
     int grp = 0;
 #pragma unroll
-    for (int bit = 4, h = NP / 2; bit > 0; bit >>= 1, h >>= 1) {
+    for (int bit = 4, h = G / 2; bit > 0; bit >>= 1, h >>= 1) {
         const bool up = (lane & bit) != 0;
         if (h >= 1) {
 #pragma unroll
-            for (int q = 0; q < (h >= 1 ? h : 1); q++) {
-                const double keep = up ? acc[q + h] : acc[q], send = up ? acc[q] : acc[q + h];
-                acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
-            }
+            for (int q = 0; q < (h >= 1 ? h : 1); q++) add(q, q + h, up, bit);
             grp += up ? h : 0;
         } else {
-            acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], bit);
-            if (up) grp = NG;  // another lane writes this row
+            add(0, 0, up, bit);
+            if (up) grp = G;
         }
     }
-    row = grp < NG ? 4 * grp + (lane >> 3) : it.nrow;
-    return acc[0];
+    return grp;
+}
+// the largest exponent field of a leaf's b_l 2^(l/2); bad: one is not finite
+template <typename R>
+__device__ __forceinline__ int local_top(const cx<R> *loc, int64_t lb, int P, int lane, bool &bad)
+{
+    int top = 0;
+    bad = false;
+    for (int m = lane; m < 2 * P; m += 32) {
+        const int E = exp_field(local_real(loc, lb + m));
+        bad |= E == 0x7ff;
+        if (E) top = max(top, E + (m >> 2));
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    return __reduce_max_sync(0xffffffffu, top);
 }
 
-// v of a block's rows: a warp per block, or (split) the four warps of a thread block, each
-// over a quarter of the columns, the quarters added in order.
-template <typename R>
-__global__ void __launch_bounds__(128)
-k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__restrict__ rows,
-             const int32_t *__restrict__ cols, const double *__restrict__ sigma,
-             const cx<R> *__restrict__ loc, const cx<R> *__restrict__ mp, int P, int lchunks,
-             const double *__restrict__ bsig, double *__restrict__ v, const int *gate, int split,
-             int64_t slab)
+// acc += the n chunks of x (eight columns each, zeros up to a multiple of four) times their
+// tiles of NG row groups; the tiles of kRun chunks are all asked for before the first is used
+template <int NG>
+__device__ __forceinline__ void dot_chunks(const double *__restrict__ t, const int2 *x, int n, int lane,
+                                           Dot *acc)
 {
-    lbf_rhs(slab, sigma, loc, mp, bsig, v, gate);
+    for (int k = 0; k < n; k += kRun, x += 8 * kRun) {
+        prefetch_tiles(t - lane + 32 * NG * (k + kAhead), NG * min(kRun, n - k - kAhead), lane);
+        int2 e[kRun * NG];
+#pragma unroll
+        for (int h = 0; h < kRun; h++) {
+            const double *th = t + 32 * NG * min(k + h, n - 1);
+#pragma unroll
+            for (int q = 0; q < NG; q++) e[h * NG + q] = *(const int2 *)&th[32 * q];
+        }
+#pragma unroll
+        for (int h = 0; h < kRun; h++) {
+            const int2 xk = x[8 * h];
+#pragma unroll
+            for (int q = 0; q < NG; q++) dot_add(acc[q], e[h * NG + q], xk);
+        }
+    }
+}
+
+// The sum of one row of a block of at most G row groups over its column chunks k0 .. k1 - 1
+// (near chunks, multipole chunks, then the local expansion's), and that row.  The columns'
+// values of a run of chunks are made integers first, a column a lane, and left in xs.
+template <int G, typename R>
+__device__ __forceinline__ double block_rows(const RowItem &it, const double *__restrict__ rows,
+                                             const int32_t *__restrict__ rexp,
+                                             const int32_t *__restrict__ cols,
+                                             const double *__restrict__ sigma, int sexp,
+                                             const cx<R> *__restrict__ loc,
+                                             const cx<R> *__restrict__ mp, int P, int k0, int k1,
+                                             int2 *xs, int lane, int &row)
+{
+    const int ng = (it.nrow + 3) / 4;
+    const double *t = rows + ((int64_t)it.tile + (int64_t)k0 * ng) * 32 + lane;
+    const int32_t *cl = cols + (int64_t)it.chunk * 8;
+    const int64_t lb = (int64_t)it.box * 2 * P;
+    const int nn = (it.ncol + 7) / 8;
+    const int grp = fold_rows<G>(lane, [](int, int, bool, int) {});
+    row = grp < ng ? 4 * grp + (lane >> 3) : it.nrow;
+    prefetch_tiles(t - lane, ng * min(k1 - k0, kAhead), lane);
+    double s = 0.0;
+    int k = k0;
+    while (k < k1) {
+        if (k >= nn && k < it.nchunk) {
+            // multipoles of W boxes: few, and in units of their own
+            double d[G];
+#pragma unroll
+            for (int q = 0; q < G; q++) d[q] = 0.0;
+            for (const int ke = min(k1, it.nchunk); k < ke; k++, t += 32 * ng) {
+                const int j = cl[8 * k + (lane & 7)];
+                const double x = j < 0 ? local_real(mp, -1 - j) : 0.0;
+#pragma unroll
+                for (int q = 0; q < G; q++)
+                    if (q < ng) d[q] = fma(t[32 * q], x, d[q]);
+            }
+            fold_rows<G>(lane, [&](int a, int b, bool up, int bit) {
+                const double keep = up ? d[b] : d[a], send = up ? d[a] : d[b];
+                d[a] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+            });
+            s += d[0];
+            continue;
+        }
+        // near nodes, in units of the density's largest and the row's largest; the local
+        // expansion, in those of its largest b_l 2^(l/2)
+        const bool far = k >= nn;
+        const int n = min((far ? k1 : min(k1, nn)) - k, kDotChunks);
+        bool bad = false;
+        if (k > k0) prefetch_tiles(t - lane, ng * min(n, kAhead), lane);
+        const int top = far ? local_top(loc, lb, P, lane, bad) : sexp;
+        const int off = 8 * (far ? it.nchunk : 0), end = far ? off + 2 * P : it.ncol;
+        __syncwarp();
+#pragma unroll 2
+        for (int m = 8 * k + lane; m < 8 * (k + (n + 3) / 4 * 4); m += 32) {
+            double v = 0.0;
+            if (m < min(end, 8 * (k + n))) v = far ? local_real(loc, lb + m - off) : sigma[cl[m]];
+            xs[m - 8 * k] = dot_word(v, far ? (m - off) >> 2 : 0, top);
+        }
+        __syncwarp();
+        Dot acc[G];
+#pragma unroll
+        for (int q = 0; q < G; q++) acc[q] = Dot{0, 0};
+#define LBF_DOT(NG) dot_chunks<(NG <= G ? NG : G)>(t, xs + (lane & 7), n, lane, acc)
+        if (G <= 2) {
+            if (ng == 1) LBF_DOT(1);
+            else LBF_DOT(2);
+        } else {
+            LBF_GROUPS(ng, LBF_DOT)
+        }
+#undef LBF_DOT
+        k += n;
+        t += (int64_t)32 * n * ng;
+        fold_rows<G>(lane, [&](int a, int b, bool up, int bit) { acc[a] = dot_meet(acc[a], acc[b], up, bit); });
+        if (row < it.nrow)
+            s += bad ? __longlong_as_double(0x7ff8000000000000ll)
+                     : dot_double(acc[0], top + (far ? -1129 : rexp[it.row0 + row] - 2150));
+    }
+    return s;
+}
+
+// v of a block's rows: a warp per block, or (SPLIT, blocks of kGroupsSmall groups) the four
+// warps of a thread block, each over a quarter of the columns, the quarters added in order.
+template <typename R, bool SPLIT>
+__global__ void __launch_bounds__(128, kRowBlocks)
+k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__restrict__ rows,
+             const int32_t *__restrict__ rexp, const int32_t *__restrict__ cols,
+             const double *__restrict__ sigma, const int32_t *__restrict__ sexp,
+             const cx<R> *__restrict__ loc, const cx<R> *__restrict__ mp, int P, int lchunks,
+             const double *__restrict__ bsig, double *__restrict__ v, const int *gate, int64_t slab)
+{
+    lbf_rhs(slab, sigma, sexp, loc, mp, bsig, v, gate);
     if (fmm::gate_closed(gate)) return;
     __shared__ double part[4][32];
+    __shared__ int2 xs[4][8 * kDotChunks];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t k = split ? (int64_t)blockIdx.x : blockIdx.x * (int64_t)(blockDim.x >> 5) + wid;
+    const int64_t k = SPLIT ? (int64_t)blockIdx.x : blockIdx.x * (int64_t)(blockDim.x >> 5) + wid;
     if (k >= nitem) return;
     const int4 i0 = ((const int4 *)items)[2 * k], i1 = ((const int4 *)items)[2 * k + 1];
     const RowItem it{i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
     const int nk = it.nchunk + lchunks;
-    const int k0 = split ? nk * wid / 4 : 0, k1 = split ? nk * (wid + 1) / 4 : nk;
+    const int k0 = SPLIT ? nk * wid / 4 : 0, k1 = SPLIT ? nk * (wid + 1) / 4 : nk;
+    const int se = sexp[1];
     int row;
-    double s;
-    switch ((it.nrow + 3) / 4) {
-#define LBF_ROWS(NG) \
-    case NG: s = block_rows<NG>(it, rows, cols, sigma, loc, mp, P, k0, k1, lane, row); break
-        LBF_ROWS(1);
-        LBF_ROWS(2);
-        LBF_ROWS(3);
-        LBF_ROWS(4);
-        LBF_ROWS(5);
-        LBF_ROWS(6);
-        LBF_ROWS(7);
-    default: s = block_rows<8>(it, rows, cols, sigma, loc, mp, P, k0, k1, lane, row); break;
-#undef LBF_ROWS
-    }
-    if (split) {
+    double s = block_rows<SPLIT ? kGroupsSmall : kGroups>(it, rows, rexp, cols, sigma, se, loc, mp, P, k0,
+                                                          k1, xs[wid], lane, row);
+    if (SPLIT) {
         part[wid][lane] = s;
         __syncthreads();
         if (wid != 0) return;
         s = part[0][lane] + part[1][lane] + part[2][lane] + part[3][lane];
     }
-    if (row < it.nrow) v[it.row0 + row] = s + 2.0 * *bsig;
+    if (row < it.nrow)
+        v[it.row0 + row] = se == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : s + 2.0 * *bsig;
 }
 
-// z = G^T tau over each leaf's columns, a thread block of four warps per leaf, a quarter of
-// the columns a warp (no sums between warps; a warp per leaf left the leaf with the most
+// a[h] += the tiles of chunk h (of n, at most 4) times the rows' values
+template <int NG>
+__device__ __forceinline__ void dot_rows(const double *__restrict__ t, const int2 *x, int n, Dot *a)
+{
+#pragma unroll
+    for (int h = 0; h < 4; h++) {
+        const double *th = t + 32 * NG * min(h, n - 1);  // (beyond n: a sum nobody takes)
+#pragma unroll
+        for (int q = 0; q < NG; q++) dot_add(a[h], *(const int2 *)&th[32 * q], x[q]);
+    }
+}
+
+// z = G^T tau over each leaf's columns, thread blocks of four warps per leaf, a part of the
+// columns a warp (no sums between warps; a warp per leaf left the leaf with the most
 // columns, 1500 of a mean of 200, running alone: 582 us at 131,072 nodes).  Four chunks at a
 // time: a lane sums its rows' parts of a column of each, and the four lanes of a column are
 // added in 3 additions.
 __global__ void __launch_bounds__(128)
 k_rows_t(const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
-         const double *__restrict__ rows, const double *__restrict__ tau, double *__restrict__ z,
-         const int *gate)
+         const double *__restrict__ rows, const int32_t *__restrict__ rexp,
+         const double *__restrict__ tau, double *__restrict__ z, const int *gate)
 {
     if (fmm::gate_closed(gate)) return;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -427,34 +548,34 @@ k_rows_t(const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
     for (int k = b0; k < b1; k++) {
         const RowItem it = items[k];
         const int ng = (it.nrow + 3) / 4, nk = (it.ncol + 7) / 8;
-        const int k0 = nk * wid / 4, k1 = nk * (wid + 1) / 4;
-        double tv[kGroups];
+        const int nw = 4 * gridDim.y, iw = 4 * blockIdx.y + wid;
+        const int k0 = (int)((int64_t)nk * iw / nw), k1 = (int)((int64_t)nk * (iw + 1) / nw);
+        if (k0 == k1) continue;
+        // tau_r in the unit of its row's entries, as an integer in that of the block's largest,
+        // a lane a row; then the rows of each lane's sums
+        const double tr = lane < it.nrow ? tau[it.row0 + lane] : 0.0;
+        const int re = lane < it.nrow ? rexp[it.row0 + lane] : 0, E = exp_field(tr);
+        const bool bad = __any_sync(0xffffffffu, E == 0x7ff);
+        const int top = __reduce_max_sync(0xffffffffu, E ? E + re : 0);
+        const int2 x = dot_word(tr, re, top);
+        int2 tv[kGroups];
 #pragma unroll
-        for (int q = 0; q < kGroups; q++) {
-            const int r = 4 * q + (lane >> 3);
-            tv[q] = r < it.nrow ? tau[it.row0 + r] : 0.0;
-        }
+        for (int q = 0; q < kGroups; q++) tv[q] = shfl_word(x, 4 * q + (lane >> 3));
         const double *tl = rows + ((int64_t)it.tile + (int64_t)k0 * ng) * 32 + lane;
+        prefetch_tiles(tl - lane, ng * min(k1 - k0, 2 * kAhead), lane);
         for (int c = k0; c < k1; c += 4, tl += 128 * ng) {
-            double a[4];
+            prefetch_tiles(tl - lane + (int64_t)64 * kAhead * ng, ng * min(4, k1 - c - 2 * kAhead), lane);
+            Dot a[4];
 #pragma unroll
-            for (int h = 0; h < 4; h++) {
-                double e[kGroups];
-                const bool on = c + h < k1;
-#pragma unroll
-                for (int q = 0; q < kGroups; q++) e[q] = on && q < ng ? tl[32 * (h * ng + q)] : 0.0;
-                double s = 0.0;
-#pragma unroll
-                for (int q = 0; q < kGroups; q++)
-                    if (q < ng) s = fma(e[q], tv[q], s);
-                a[h] = s;
-            }
-            const double s0 = (u ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, u ? a[0] : a[2], 16);
-            const double s1 = (u ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, u ? a[1] : a[3], 16);
-            const double s = (w ? s1 : s0) + __shfl_xor_sync(0xffffffffu, w ? s0 : s1, 8);
+            for (int h = 0; h < 4; h++) a[h] = Dot{0, 0};
+#define LBF_DOT(NG) dot_rows<NG>(tl, tv, k1 - c, a)
+            LBF_GROUPS(ng, LBF_DOT)
+#undef LBF_DOT
+            const Dot d = dot_meet(dot_meet(a[0], a[2], u, 16), dot_meet(a[1], a[3], u, 16), w, 8);
             const int h = (u ? 2 : 0) + (w ? 1 : 0);  // the chunk this lane's sum belongs to
             if (c + h < k1) {
                 double *o = z + ((int64_t)it.chunk + c + h) * 8 + (lane & 7);
+                const double s = bad ? __longlong_as_double(0x7ff8000000000000ll) : dot_double(d, top - 2150);
                 *o = k == b0 ? s : *o + s;
             }
         }
@@ -479,58 +600,74 @@ k_rows_t_out(int64_t nitem, const RowItem *__restrict__ items, const double *__r
     if (k >= nitem) return;
     const RowItem it = items[k];
     const int ng = (it.nrow + 3) / 4;
-    double ai[kGroups], ar[kGroups];
-#pragma unroll
-    for (int q = 0; q < kGroups; q++) ai[q] = ar[q] = 0.0;
-    const int c0 = it.ncol >> 3, near = 8 * it.nchunk, par = lane & 1;
-    const double *t = rows + ((int64_t)it.tile + (int64_t)c0 * ng) * 32 + lane;
+    // columns 2 l and 2 l + 1 hold -(1/pi) (Im, Re) of a power, to be met by (x, y) of the
+    // coefficient for the imaginary part of the sum and by (-y, x) for the real part
+    const int nn = (it.ncol + 7) / 8, par = lane & 1;
+    const double *t = rows + ((int64_t)it.tile + (int64_t)nn * ng) * 32 + lane;
     const int64_t lb = (int64_t)it.box * 2 * P;
-    for (int c = c0; c < it.nchunk + lchunks; c++, t += 32 * ng) {
-        // the real of this lane's column, and the other real of its coefficient: columns
-        // 2 l and 2 l + 1 hold -(1/pi) (Im, Re) of a power, to be met by (x, y) for the
-        // imaginary part of the sum and by (-y, x) for the real part
-        const int m = 8 * c + (lane & 7);
-        double si = 0.0, sr = 0.0;
-        if (m < near) {
-            const int j = cols[(int64_t)it.chunk * 8 + m];
-            if (m >= it.ncol && j < 0) {
-                const int e = -1 - j, odd = e & 1;
+    double fi = 0.0, fr = 0.0;
+    if (nn < it.nchunk) {
+        double ai[kGroups], ar[kGroups];
+#pragma unroll
+        for (int q = 0; q < kGroups; q++) ai[q] = ar[q] = 0.0;
+        for (int c = nn; c < it.nchunk; c++, t += 32 * ng) {
+            const int j = cols[(int64_t)it.chunk * 8 + 8 * c + (lane & 7)];
+            double si = 0.0, sr = 0.0;
+            if (j < 0) {
+                const int e = -1 - j;
                 si = local_real(mp, e);
-                sr = odd ? local_real(mp, e - 1) : -local_real(mp, e + 1);
+                sr = (e & 1) ? local_real(mp, e - 1) : -local_real(mp, e + 1);
             }
-        } else if (m < near + 2 * P) {
-            const int64_t e = lb + m - near;
-            si = local_real(loc, e);
-            sr = par ? local_real(loc, e - 1) : -local_real(loc, e + 1);
+#pragma unroll
+            for (int q = 0; q < kGroups; q++)
+                if (q < ng) {
+                    const double e = t[32 * q];
+                    ai[q] = fma(e, si, ai[q]);
+                    ar[q] = fma(e, sr, ar[q]);
+                }
         }
+        fold_rows<kGroups>(lane, [&](int a, int b, bool up, int bit) {
+            const double ki = up ? ai[b] : ai[a], sdi = up ? ai[a] : ai[b];
+            const double kr = up ? ar[b] : ar[a], sdr = up ? ar[a] : ar[b];
+            ai[a] = ki + __shfl_xor_sync(0xffffffffu, sdi, bit);
+            ar[a] = kr + __shfl_xor_sync(0xffffffffu, sdr, bit);
+        });
+        fi = ai[0];
+        fr = ar[0];
+    }
+    // the local expansion, in units of its largest b_l 2^(l/2)
+    bool bad;
+    const int top = local_top(loc, lb, P, lane, bad);
+    Dot di[kGroups], dr[kGroups];
+#pragma unroll
+    for (int q = 0; q < kGroups; q++) di[q] = dr[q] = Dot{0, 0};
+    for (int c = 0; c < lchunks; c++, t += 32 * ng) {
+        const int m = 8 * c + (lane & 7);
+        const int2 xi = m < 2 * P ? dot_word(local_real(loc, lb + m), m >> 2, top) : make_int2(0, 0);
+        int2 xr = make_int2(__shfl_xor_sync(0xffffffffu, xi.x, 1), __shfl_xor_sync(0xffffffffu, xi.y, 1));
+        if (!par) xr = make_int2(-xr.x, -xr.y);
 #pragma unroll
         for (int q = 0; q < kGroups; q++)
             if (q < ng) {
-                const double e = t[32 * q];
-                ai[q] = fma(e, si, ai[q]);
-                ar[q] = fma(e, sr, ar[q]);
+                const int2 e = *(const int2 *)&t[32 * q];
+                dot_add(di[q], e, xi);
+                dot_add(dr[q], e, xr);
             }
     }
-    int grp = 0;
-#pragma unroll
-    for (int bit = 4; bit > 0; bit >>= 1) {
-        const bool up = (lane & bit) != 0;
-#pragma unroll
-        for (int q = 0; q < bit; q++) {
-            const double ki = up ? ai[q + bit] : ai[q], sdi = up ? ai[q] : ai[q + bit];
-            const double kr = up ? ar[q + bit] : ar[q], sdr = up ? ar[q] : ar[q + bit];
-            ai[q] = ki + __shfl_xor_sync(0xffffffffu, sdi, bit);
-            ar[q] = kr + __shfl_xor_sync(0xffffffffu, sdr, bit);
-        }
-        grp += up ? bit : 0;
-    }
+    const int grp = fold_rows<kGroups>(lane, [&](int a, int b, bool up, int bit) {
+        di[a] = dot_meet(di[a], di[b], up, bit);
+        dr[a] = dot_meet(dr[a], dr[b], up, bit);
+    });
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    fi += bad ? nan : dot_double(di[0], top - 1129);
+    fr += bad ? nan : dot_double(dr[0], top - 1129);
     const int row = 4 * grp + (lane >> 3);
     if (row >= it.nrow) return;
     const int i = it.row0 + row, at = i - begin[it.box];
     double s = 0.0;
     for (int e = rptr[it.leaf]; e < rptr[it.leaf + 1]; e++) s += z[(int64_t)rbase[e] + at];
     const double2 ww = w[i];
-    v[i] = s - fma(ww.x, ai[0], ww.y * ar[0]) + 2.0 * (beta[i] * *bsig);
+    v[i] = s - fma(ww.x, fi, ww.y * fr) + 2.0 * (beta[i] * *bsig);
 }
 
 TreeLists lists_of(const Tree &T)
@@ -574,6 +711,7 @@ void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap)
     pl->rows_rptr = A.get<int32_t>(cap + 1);
     pl->rows_rbase = A.get<int32_t>(pl->rows_rev_cap);
     pl->rows_z = A.get<double>(8 * chunks);
+    pl->rows_e = A.get<int32_t>(N);
     pl->bigx_cap = cap / 8 + 16;
     pl->bigx = A.get<int32_t>(pl->bigx_cap);
     pl->rows = A.get<double>(32 * tiles);
@@ -638,7 +776,7 @@ int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scrat
     LBF_LAUNCH(k_rows_cols, lbf_cdiv(nl, 4), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, P, chunks,
                pl->rows_cols);
     LBF_LAUNCH(k_rows_fill, lbf_cdiv((int64_t)nitem, 4), 128, 0, s, (int64_t)nitem, pl->rows_items, tl,
-               pl->rows_thr, geo_of(T), P, lch, pl->rows_cols, pl->xi, pl->w, pl->dself, pl->rows);
+               pl->rows_thr, geo_of(T), P, lch, pl->rows_cols, pl->xi, pl->w, pl->dself, pl->rows, pl->rows_e);
     // the transposed rows' lists
     LBF_LAUNCH(k_rows_rev, lbf_cdiv(nl, 128), 128, 0, s, nl, T.leaves, tl, pl->rows_thr, chunks, leaf,
                pl->rows_rptr, (const int32_t *)nullptr, (int32_t *)nullptr);
@@ -664,14 +802,15 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
 {
     const int64_t n = pl->rows_nitem;
     const dim3 grid = lbf_grid(pl, pl->rows_split ? n : lbf_cdiv(n, 4));
-    if (df)
-        LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_apply<df64>, grid, 128, 0, s, n, pl->rows_items, pl->rows,
-                     pl->rows_cols, sigma, (const cx<df64> *)pl->local, (const cx<df64> *)pl->mpole,
-                     pl->P, local_chunks(pl->P), pl->bsig, v, gate, pl->rows_split, pl->slab);
-    else
-        LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_apply<double>, grid, 128, 0, s, n, pl->rows_items,
-                     pl->rows, pl->rows_cols, sigma, (const cx<double> *)pl->local,
-                     (const cx<double> *)pl->mpole, pl->P, local_chunks(pl->P), pl->bsig, v, gate, pl->rows_split, pl->slab);
+#define LBF_ROWS(R, SPLIT)                                                                         \
+    LBF_LAUNCH_P(LBF_KERNEL_LEAF, (k_rows_apply<R, SPLIT>), grid, 128, 0, s, n, pl->rows_items, pl->rows, \
+                 pl->rows_e, pl->rows_cols, sigma, pl->sigma_e, (const cx<R> *)pl->local,          \
+                 (const cx<R> *)pl->mpole, pl->P, local_chunks(pl->P), pl->bsig, v, gate, pl->slab)
+    if (df && pl->rows_split) LBF_ROWS(df64, true);
+    else if (df) LBF_ROWS(df64, false);
+    else if (pl->rows_split) LBF_ROWS(double, true);
+    else LBF_ROWS(double, false);
+#undef LBF_ROWS
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }
@@ -681,8 +820,8 @@ int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate
 {
     const Tree &T = pl->tree;
     const int64_t n = pl->rows_nitem;
-    LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t, T.nleaf, 128, 0, s, pl->rows_block0, pl->rows_items,
-                 pl->rows, tau, pl->rows_z, gate);
+    LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t, dim3((unsigned)T.nleaf, pl->rows_split ? 4 : 1), 128, 0, s, pl->rows_block0, pl->rows_items,
+                 pl->rows, pl->rows_e, tau, pl->rows_z, gate);
     const int lch = local_chunks(pl->P);
     if (df)
         LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t_out<df64>, lbf_cdiv(n, 4), 128, 0, s, n, pl->rows_items,

@@ -114,3 +114,24 @@ def test_stored_multiplier_block_both_ways(M, nodes):
     tau = rng.standard_normal(g.N)
     L.lbf_apply(plan, L.LBF_OP_FULL | L.LBF_OP_TRANSPOSE, dev(np.concatenate([tau, np.zeros(g.M)])), o)
     assert rel_l2(host(o)[g.N:], E.T @ tau) < 1e-13 * np.sqrt(g.N)
+
+
+@pytest.mark.parametrize("op", [L.LBF_OP_K_ONLY, L.LBF_OP_K_ONLY | L.LBF_OP_TRANSPOSE])
+@pytest.mark.parametrize("leaf", [8, 300])
+def test_integer_rows_keep_scale_and_non_finite_values(leaf, op):
+    """The densities' integers are relative to the largest: a power of two comes out exactly
+    (no step rounds differently), and a value that is not finite reaches every row (through
+    the sum over all nodes that each row holds)."""
+    g = wl.star_caps(11, 5, np.array([64, 37, 201, 90, 333]))
+    plan = plan_for(g, leaf_size=leaf, p=30, border=0)
+    v = dev(np.random.default_rng(leaf).standard_normal(g.N))
+    o, p = zeros(g.N), zeros(g.N)
+    L.lbf_apply(plan, op, v, o)
+    for k in (-800, -1, 800):
+        L.lbf_apply(plan, op, v * 2.0 ** k, p)
+        assert torch.equal(p * 2.0 ** -k, o)
+    for bad in (float("nan"), float("inf")):
+        w = v.clone()
+        w[g.N // 2] = bad
+        L.lbf_apply(plan, op, w, p)
+        assert not torch.isfinite(p).any()
