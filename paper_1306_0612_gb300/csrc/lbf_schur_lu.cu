@@ -49,6 +49,7 @@ namespace {
 constexpr int kLuNb = 64;          // panel width
 constexpr int kLuThreads = 256;
 constexpr int kLuTs = 64;          // row block of the triangular solves, GEMM tile
+constexpr int kTrsvThreads = 8 * kLuTs;
 constexpr int kLuPad = 65;         // shared-memory row stride of 64-wide tiles
 constexpr unsigned kLuSpins = 1u << 24;
 constexpr int kLuMaxPanelBlocks = 1024;
@@ -682,40 +683,74 @@ __global__ void k_lu_scatter(int M, const int *__restrict__ perm, const float2 *
     y[trans ? perm[i] : i] = v;
 }
 
-// Triangular solve T x = x (in place, double-float), T from the factors:
+// one element of a triangular solve's solution as its readers find it: the two floats, each in
+// a word of 64 bits under the launch's tag, so that a word that carries the tag is complete
+__device__ __forceinline__ void put_tagged(longlong2 *p, float2 v, unsigned tag)
+{
+    const unsigned long long t = (unsigned long long)tag << 32;
+    const unsigned long long a = t | __float_as_uint(v.x), b = t | __float_as_uint(v.y);
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
+}
+__device__ __forceinline__ float2 wait_tagged(const longlong2 *p, unsigned tag, unsigned lim, int *status)
+{
+    unsigned long long a, b;
+    for (unsigned it = 0;; it++) {
+        asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+        if ((unsigned)(a >> 32) == tag && (unsigned)(b >> 32) == tag) break;
+        if (it > lim) {
+            atomicOr(status, LBF_DEV_TIMEOUT);
+            break;
+        }
+    }
+    return make_float2(__uint_as_float((unsigned)a), __uint_as_float((unsigned)b));
+}
+// the sum over the eight lanes 8 i .. 8 i + 7, on each of them
+__device__ __forceinline__ df64 sum8(df64 a)
+{
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1)
+        a = a + df64(__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o), 0);
+    return a;
+}
+
+// Triangular solve T x = x (in place, double-float; xd: the solution in double too), T from the
+// factors:
 //   mode 0: L (unit lower)   mode 1: U (upper)   mode 2: U^T (lower)   mode 3: L^T (unit upper).
 // Row blocks of kLuTs rows are taken from a ticket counter in solve order (increasing
-// for lower, decreasing for upper).  A block first prefetches its diagonal block's
-// inverse (shared memory) and the off-diagonal tile it will need last (registers),
-// then waits (bounded) for each block it depends on, in solve order, subtracting that
-// block's part as it arrives, and finally multiplies by the diagonal inverse and
-// publishes its rows by a flag word.  Every block it waits for took its ticket
-// earlier and is running, so every wait ends.
-// sw: [0] ticket, [1] finished blocks, [2] epoch, then one flag per row block; the last
-// block to finish resets the counters and advances the epoch.
-__global__ void __launch_bounds__(kLuThreads)
+// for lower, decreasing for upper).  A block subtracts the part of each block it depends on as
+// that arrives, in solve order, the tile of the next one already on its way, and finally
+// multiplies by the diagonal block's inverse (shared memory) and publishes its rows in xw.
+// Every block it waits for took its ticket earlier and is running, so every wait ends
+// (bounded all the same).
+// Bound by the chain of M / 64 blocks: a step is a trip of the last rows through L2 and two
+// 64 x 64 products.  Readers wait on the rows themselves (put_tagged: no fence, no flag), a
+// product is eight terms a thread and three shuffled additions: 2.1 us a step, 0.55 ms a solve at
+// M = 16,384 (6.1 us and 1.56 ms with flags, 16 terms a thread and sums through shared memory).
+// sw: [0] ticket, [1] finished blocks, [2] epoch; the last block to finish resets the counters
+// and advances the epoch.
+__global__ void __launch_bounds__(kTrsvThreads)
 k_lu_trsv(int M, int mode, const float2 *__restrict__ A, const float2 *__restrict__ dinv,
-          float2 *x, unsigned *sw, int *status, const int *gate)
+          float2 *x, double *xd, longlong2 *xw, unsigned *sw, int *status, const int *gate)
 {
     if (gate_shut(gate)) return;
     extern __shared__ __align__(16) float2 vsm[];
     float2 *T = vsm;                      // kLuTs x kLuPad: the diagonal block's inverse (as T)
-    float2 *part = vsm + kLuTs * kLuPad;  // 4 x kLuTs partial sums
-    __shared__ float2 xs[kLuTs], rv[kLuTs];
-    __shared__ unsigned s_t, s_epoch;
+    float2 *part = vsm + kLuTs * kLuPad;  // 8 x kLuTs partial sums (transposed modes)
+    __shared__ float2 xs[2][kLuTs], rv[kLuTs];
+    __shared__ unsigned s_t;
     const bool lower = mode == 0 || mode == 2, trans = mode >= 2;
     const int nB = (M + kLuTs - 1) / kLuTs, tid = threadIdx.x;
-    unsigned *flag = sw + 3;
-    if (tid == 0) s_epoch = *(volatile unsigned *)&sw[2];
-    __syncthreads();
-    const unsigned epoch = s_epoch;
-    // this thread's (row, quarter) of a tile product
-    const int r = trans ? (tid & 63) : (tid >> 2), q = trans ? (tid >> 6) : (tid & 3);
+    const unsigned epoch = *(volatile unsigned *)&sw[2], tag = epoch + 1u;
+    const unsigned lim = wait_limit(status, kLuSpins);
+    // this thread's row and its eight columns c0 + dc k of a tile product: a row's columns over
+    // eight lanes, or (transposed: A is read along its rows) over eight groups of 64 threads
+    const int r = trans ? (tid & 63) : (tid >> 3), q = trans ? (tid >> 6) : (tid & 7);
+    const int c0 = trans ? 8 * q : q, dc = trans ? 1 : 8;
+    const int row = tid >> 3, l8 = tid & 7;  // row and lane of the sums over eight lanes
     for (;;) {
         if (tid == 0) s_t = atomicAdd(&sw[0], 1u);
         __syncthreads();
         const unsigned t = s_t;
-        __syncthreads();
         if (t >= (unsigned)nB) break;
         const int b = lower ? (int)t : nB - 1 - (int)t;
         const int rb = b * kLuTs, nr = min(kLuTs, M - rb);
@@ -727,73 +762,60 @@ k_lu_trsv(int M, int mode, const float2 *__restrict__ A, const float2 *__restric
                 T[(trans ? cc : rr) * kLuPad + (trans ? rr : cc)] = D[e];
             }
         }
+        const float2 rhs = row < nr ? x[rb + row] : make_float2(0.f, 0.f);
         const int nj = lower ? b : nB - 1 - b;
-        // prefetch of the last off-diagonal tile (the one on the critical path)
-        float2 pre[16];
-        if (nj > 0) {
-            const int j = lower ? b - 1 : b + 1, cb = j * kLuTs, nc = min(kLuTs, M - cb);
+        float2 tile[8], next[8];
+        auto fetch = [&](int jj, float2 *to) {
+            const int j = lower ? jj : nB - 1 - jj, cb = j * kLuTs, nc = min(kLuTs, M - cb);
 #pragma unroll
-            for (int k = 0; k < 16; k++) {
-                const int c = q * 16 + k;
-                pre[k] = make_float2(0.f, 0.f);
+            for (int k = 0; k < 8; k++) {
+                const int c = c0 + dc * k;
+                to[k] = make_float2(0.f, 0.f);
                 if (r < nr && c < nc)
-                    pre[k] = trans ? A[(int64_t)(cb + c) * M + rb + r] : A[(int64_t)(rb + r) * M + cb + c];
+                    to[k] = trans ? A[(int64_t)(cb + c) * M + rb + r] : A[(int64_t)(rb + r) * M + cb + c];
             }
-        }
-        df64 accp(0.f);
+        };
+        if (nj > 0) fetch(0, tile);
+        df64 acc0(0.f), acc1(0.f);
         for (int jj = 0; jj < nj; jj++) {
-            const int j = lower ? jj : nB - 1 - jj;
-            block_wait_flag(&flag[j], epoch + 1u, status, kLuSpins);
-            const int cb = j * kLuTs, nc = min(kLuTs, M - cb);
-            if (tid < nc) xs[tid] = __ldcg(&x[cb + tid]);
+            if (jj + 1 < nj) fetch(jj + 1, next);
+            const int j = lower ? jj : nB - 1 - jj, cb = j * kLuTs, nc = min(kLuTs, M - cb);
+            float2 *xj = xs[jj & 1];  // (the other half is still read by the step before)
+            if (tid < kLuTs) xj[tid] = tid < nc ? wait_tagged(&xw[cb + tid], tag, lim, status) : make_float2(0.f, 0.f);
             __syncthreads();
-            if (r < nr) {
-                if (jj == nj - 1) {
 #pragma unroll
-                    for (int k = 0; k < 16; k++)
-                        if (q * 16 + k < nc) accp = df_fma(ld(pre[k]), ld(xs[q * 16 + k]), accp);
-                } else {
-                    const int c1 = min(nc, q * 16 + 16);
-                    if (!trans) {
-                        const float2 *row = A + (int64_t)(rb + r) * M + cb;
-                        for (int c = q * 16; c < c1; c++) accp = df_fma(ld(row[c]), ld(xs[c]), accp);
-                    } else {
-                        for (int c = q * 16; c < c1; c++)
-                            accp = df_fma(ld(A[(int64_t)(cb + c) * M + rb + r]), ld(xs[c]), accp);
-                    }
-                }
+            for (int k = 0; k < 8; k += 2) {
+                acc0 = df_fma(ld(tile[k]), ld(xj[c0 + dc * k]), acc0);
+                acc1 = df_fma(ld(tile[k + 1]), ld(xj[c0 + dc * (k + 1)]), acc1);
             }
-            __syncthreads();  // xs is refilled next
-        }
-        part[q * kLuTs + r] = pk(accp);
-        __syncthreads();
-        if (tid < kLuTs) {
-            df64 v(0.f);
-            if (tid < nr)
-                v = ld(__ldcg(&x[rb + tid])) - (((ld(part[tid]) + ld(part[kLuTs + tid])) +
-                                                 ld(part[2 * kLuTs + tid])) + ld(part[3 * kLuTs + tid]));
-            rv[tid] = pk(v);
-        }
-        __syncthreads();
-        {
-            df64 a(0.f);
 #pragma unroll
-            for (int k = 0; k < 16; k++) {
-                const int c = q * 16 + k;
-                a = df_fma(ld(T[r * kLuPad + c]), ld(rv[c]), a);
-            }
+            for (int k = 0; k < 8; k++) tile[k] = next[k];
+        }
+        df64 a = acc0 + acc1;
+        if (trans) {
             part[q * kLuTs + r] = pk(a);
+            __syncthreads();
+            a = ld(part[l8 * kLuTs + row]);
         }
-        __syncthreads();
-        if (tid < nr)
-            x[rb + tid] = pk(((ld(part[tid]) + ld(part[kLuTs + tid])) + ld(part[2 * kLuTs + tid])) +
-                             ld(part[3 * kLuTs + tid]));
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) atomicExch(&flag[b], epoch + 1u);
+        a = ld(rhs) - sum8(a);
+        if (l8 == 0) rv[row] = pk(a);
+        __syncthreads();  // (and T is complete)
+        acc0 = acc1 = df64(0.f);
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+            const int c = l8 + 8 * k;
+            acc0 = df_fma(ld(T[row * kLuPad + c]), ld(rv[c]), acc0);
+            acc1 = df_fma(ld(T[row * kLuPad + c + 8]), ld(rv[c + 8]), acc1);
+        }
+        a = sum8(acc0 + acc1);
+        if (l8 == 0 && row < nr) {
+            put_tagged(&xw[rb + row], pk(a), tag);
+            x[rb + row] = pk(a);
+            if (xd) xd[rb + row] = (double)a.hi + (double)a.lo;
+        }
+        __syncthreads();  // the shared arrays are refilled next
     }
     if (tid == 0) {
-        __threadfence();
         if (atomicAdd(&sw[1], 1u) == gridDim.x - 1) {
             sw[0] = 0u;
             sw[1] = 0u;
@@ -804,25 +826,34 @@ k_lu_trsv(int M, int mode, const float2 *__restrict__ A, const float2 *__restric
 }
 
 // r = f - S z_nat (forward) or r = f - S^T z_nat (transposed) in double, where z holds
-// the double-float solve in the triangular solves' order (z_nat = z forward; z_nat[perm[k]]
-// = z[k] transposed): the residual of one refinement step against the double S.
+// the solution in the triangular solves' order (z_nat = z forward; z_nat[perm[k]] = z[k]
+// transposed): the residual of one refinement step against the double S.  z is in double
+// already: its two floats joined here were three double instructions beside the one
+// multiply-add (2.0 ms at M = 16,384, 0.5 without).
 __global__ void k_lu_resid(int M, const double *__restrict__ S, const int *__restrict__ perm,
-                           const float2 *__restrict__ z, const double *__restrict__ f,
+                           const double *__restrict__ z, const double *__restrict__ f,
                            double *__restrict__ r, int trans, const int *gate)
 {
     if (gate_shut(gate)) return;
     if (!trans) {  // a warp per row
         const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
         if (i >= M) return;
-        double acc = 0.0;
-        for (int m = lane; m < M; m += 32) acc = fma(S[(int64_t)i * M + m], (double)z[m].x + (double)z[m].y, acc);
+        const double *row = S + (int64_t)i * M;
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+        int m = lane;
+        for (; m + 96 < M; m += 128) {
+#pragma unroll
+            for (int k = 0; k < 4; k++) a[k] = fma(row[m + 32 * k], z[m + 32 * k], a[k]);
+        }
+        for (; m < M; m += 32) a[0] = fma(row[m], z[m], a[0]);
+        double acc = (a[0] + a[1]) + (a[2] + a[3]);
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) r[i] = f[i] - acc;
     } else {  // a thread per column of S, coalesced over the rows
         const int i = blockIdx.x * blockDim.x + threadIdx.x;
         if (i >= M) return;
         double acc = 0.0;
-        for (int k = 0; k < M; k++) acc = fma(S[(int64_t)perm[k] * M + i], (double)z[k].x + (double)z[k].y, acc);
+        for (int k = 0; k < M; k++) acc = fma(S[(int64_t)perm[k] * M + i], z[k], acc);
         r[i] = f[i] - acc;
     }
 }
@@ -855,7 +886,8 @@ size_t lbf_lu_scratch_bytes(int M)
            sizeof(int) * (size_t)(oz_col_blocks(M) * kTcN) + 8 * 256;
 }
 
-int lbf_lu_sync_words(int M) { return 3 + (M + kLuTs - 1) / kLuTs; }
+// ticket, finished blocks and epoch of the triangular solves, then (from word 4) the rows' words
+int lbf_lu_sync_words(int M) { return 4 + 4 * M; }
 
 int64_t lbf_lu_dinv_entries(int M) { return 2 * (int64_t)((M + kLuTs - 1) / kLuTs) * kLuTs * kLuTs; }
 
@@ -961,20 +993,22 @@ int lbf_schur_lu_apply(lbf_plan *pl, const double *f, double alpha, double *y, i
                        const int *gate, cudaStream_t s, int accurate)
 {
     const int M = pl->M;
-    const size_t smem = sizeof(float2) * (kLuTs * kLuPad + 4 * kLuTs);  // < 48 KB
+    const size_t smem = sizeof(float2) * (kLuTs * kLuPad + 8 * kLuTs);  // < 48 KB
     const int nB = (M + kLuTs - 1) / kLuTs;
     const int grid = std::min(nB, 2 * std::max(1, pl->nsm));
     const float2 *A = (const float2 *)pl->Sinv;
-    auto solve = [&](const double *rhs, float2 *z) -> int {
+    double *zd = (double *)pl->lu_z2;  // the first solution in double, until the second solve
+    auto solve = [&](const double *rhs, float2 *z, double *xd) -> int {
         LBF_LAUNCH(k_lu_gather, lbf_cdiv(M, 256), 256, 0, s, M, pl->lu_perm, rhs, z, trans, gate);
-        LBF_LAUNCH_P(LBF_KERNEL_LU_SOLVE, k_lu_trsv, grid, kLuThreads, smem, s, M, trans ? 2 : 0, A,
-                     pl->lu_dinv, z, pl->lu_sync, pl->dev_status, gate);
-        LBF_LAUNCH_P(LBF_KERNEL_LU_SOLVE, k_lu_trsv, grid, kLuThreads, smem, s, M, trans ? 3 : 1, A,
-                     pl->lu_dinv, z, pl->lu_sync, pl->dev_status, gate);
+        LBF_LAUNCH_P(LBF_KERNEL_LU_SOLVE, k_lu_trsv, grid, kTrsvThreads, smem, s, M, trans ? 2 : 0, A,
+                     pl->lu_dinv, z, (double *)nullptr, (longlong2 *)(pl->lu_sync + 4), pl->lu_sync, pl->dev_status,
+                     gate);
+        LBF_LAUNCH_P(LBF_KERNEL_LU_SOLVE, k_lu_trsv, grid, kTrsvThreads, smem, s, M, trans ? 3 : 1, A,
+                     pl->lu_dinv, z, xd, (longlong2 *)(pl->lu_sync + 4), pl->lu_sync, pl->dev_status, gate);
         LBF_CHECK_LAUNCH();
         return LBF_OK;
     };
-    int rc = solve(f, pl->lu_z);
+    int rc = solve(f, pl->lu_z, accurate ? zd : nullptr);
     if (rc) return rc;
     if (!accurate) {
         LBF_LAUNCH(k_lu_scatter, lbf_cdiv(M, 256), 256, 0, s, M, pl->lu_perm, pl->lu_z, alpha, y, trans,
@@ -982,12 +1016,12 @@ int lbf_schur_lu_apply(lbf_plan *pl, const double *f, double alpha, double *y, i
         LBF_CHECK_LAUNCH();
         return LBF_OK;
     }
-    if (trans) LBF_LAUNCH(k_lu_resid, lbf_cdiv(M, 128), 128, 0, s, M, pl->lu_S, pl->lu_perm, pl->lu_z, f,
+    if (trans) LBF_LAUNCH(k_lu_resid, lbf_cdiv(M, 128), 128, 0, s, M, pl->lu_S, pl->lu_perm, zd, f,
                           pl->lu_r, 1, gate);
     else LBF_LAUNCH(k_lu_resid, lbf_cdiv((int64_t)M * 32, 256), 256, 0, s, M, pl->lu_S, pl->lu_perm,
-                    pl->lu_z, f, pl->lu_r, 0, gate);
+                    zd, f, pl->lu_r, 0, gate);
     LBF_CHECK_LAUNCH();
-    if ((rc = solve(pl->lu_r, pl->lu_z2))) return rc;
+    if ((rc = solve(pl->lu_r, pl->lu_z2, nullptr))) return rc;
     LBF_LAUNCH(k_lu_scatter2, lbf_cdiv(M, 256), 256, 0, s, M, pl->lu_perm, pl->lu_z, pl->lu_z2, alpha, y,
                trans, gate);
     LBF_CHECK_LAUNCH();

@@ -52,26 +52,3 @@ static __device__ __noinline__ bool grid_barrier(GridBarrier *bar, unsigned nb, 
     __syncthreads();
     return ok != 0;
 }
-
-// thread 0 waits until *flag == want (another block of the same launch sets it);
-// false (status set) on time-out; the whole block returns the same value
-static __device__ __noinline__ bool block_wait_flag(const unsigned *flag, unsigned want, int *status,
-                                            unsigned dflt_spins)
-{
-    __shared__ int ok;
-    if (threadIdx.x == 0) {
-        ok = 1;
-        const unsigned lim = wait_limit(status, dflt_spins);
-        unsigned it = 0;
-        while (*(const volatile unsigned *)flag != want) {
-            if (++it > lim) {
-                atomicOr(status, LBF_DEV_TIMEOUT);
-                ok = 0;
-                break;
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return ok != 0;
-}
