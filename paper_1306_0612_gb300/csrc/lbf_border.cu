@@ -1222,6 +1222,7 @@ int lbf_mp_apply(lbf_plan *pl, const double *y, const double *x, const double *v
             LBF_LAUNCH(k_mp_near<double>, lbf_grid(pl, lbf_cdiv(B.nchunks, 8)), 256, 0, s, B.nchunks,
                        B.chunk_leaf, B.chunk_k, B.near_ptr, B.near_src, T.begin, T.end, pl->xi,
                        B.xc, y, B.nodebase, B.partial, gate, pl->slab);
+        if (pl->rows) return lbf_rows_mp(pl, y, x, v, sc, out, gate, s);
         LBF_LAUNCH_P(LBF_KERNEL_ESUM, k_mp_eval<double>, lbf_grid(pl, lbf_cdiv(pl->N, 256)), 256, 0,
                      s, pl->N, B.Pe, pl->xi, B.leaf_of, T.level, T.ix, T.iy, g,
                      (const cz<double> *)B.loc, B.near_ptr, B.near_src, B.glob, B.nglob_h, B.xc, y,

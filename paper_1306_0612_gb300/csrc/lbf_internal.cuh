@@ -213,6 +213,7 @@ struct lbf_plan {
     // boxes whose X lists are not near columns (nbigx < 0: the passes of lbf_passes.cu are off)
     int64_t nbigx = -1, bigx_cap = 0;
     int32_t *bigx = nullptr;
+    int rows_lch = 0;           // local chunks stored
     int rows_split = 0;         // a small system: four warps share a block's columns
     int rows_thr = 0;           // boxes of at most this many nodes enter W and X lists as pairs
     double *v = nullptr;        // (I + K - I) sigma = K sigma, doubled scaling
@@ -226,7 +227,7 @@ struct lbf_plan {
     int lu = 0;                 // S^-1 by the double-float LU factors (lbf_schur_lu.cu)
     int *lu_piv = nullptr, *lu_perm = nullptr;  // row interchanges, final row order (M each)
     float2 *lu_z = nullptr;     // M-vector of the triangular solves (double-float)
-    unsigned *lu_sync = nullptr;  // ticket, finished blocks, epoch, row-block flags
+    unsigned *lu_sync = nullptr;  // ticket, finished blocks, epoch, the rows' words
     float2 *lu_dinv = nullptr;    // inverses of the 64 x 64 diagonal blocks of L and U
     double *lu_S = nullptr;       // S itself (double), for the refinement step of accurate applies
     double *lu_r = nullptr;       // M: that step's residual
@@ -392,6 +393,8 @@ static inline int lbf_direct_runs(int64_t N)
 }
 // ---- stored leaf rows (lbf_rows.cu) ----------------------------------------------
 void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap);
+int lbf_rows_mp(lbf_plan *pl, const double *y, const double *x, const double *v, double sc, double *out,
+                const int *gate, cudaStream_t s);
 int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratch_len,
                    int32_t *leaf);
 // df: the expansions are double-float

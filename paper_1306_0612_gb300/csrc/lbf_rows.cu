@@ -322,13 +322,10 @@ __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, Tr
     double *base = rows + ((int64_t)it.tile + (int64_t)it.nchunk * ng) * 32;
     if (lane < 4 * ng)
         for (int l = 0; l < 4 * lchunks; l++) {
-            int4 e = make_int4(0, 0, 0, 0);
-            if (l < P) {  // times (b_l.x, b_l.y)
-                const int2 ey = dot_word(p.y, -(l >> 1), kLocalTop), ex = dot_word(p.x, -(l >> 1), kLocalTop);
-                e = make_int4(ey.x, ey.y, ex.x, ex.y);
-            }
-            *(int4 *)(base + ((int64_t)(l >> 2) * ng + (lane >> 2)) * 32 + (lane & 3) * 8 +
-                         2 * (l & 3)) = e;
+            // times (b_l.x, b_l.y)
+            const int2 ey = dot_word(p.y, -(l >> 1), kLocalTop), ex = dot_word(p.x, -(l >> 1), kLocalTop);
+            *(int4 *)(base + ((int64_t)(l >> 2) * ng + (lane >> 2)) * 32 + (lane & 3) * 8 + 2 * (l & 3)) =
+                make_int4(ey.x, ey.y, ex.x, ex.y);
             p = cmul(p, u);
         }
 }
@@ -670,6 +667,64 @@ k_rows_t_out(int64_t nitem, const RowItem *__restrict__ items, const double *__r
     v[i] = s - fma(ww.x, fi, ww.y * fr) + 2.0 * (beta[i] * *bsig);
 }
 
+// out_i = x_i + v_i + s (E y)_i (v nullable): the multiplier potential's local expansions loc
+// (P terms) through the stored columns, a warp per row block, Re(b_l u^l) as -pi times column
+// 2 l against -Im b_l and column 2 l + 1 against Re b_l; then the node's direct centres
+// (partial), the centres summed directly everywhere and the constants.
+// Bound by the columns' bytes: 1.9 ms at 16.8 million nodes, 4.2 as a Horner chain a node
+// (four double multiply-adds a term).
+__global__ void __launch_bounds__(128, 4)
+k_rows_mp(int64_t nitem, const RowItem *__restrict__ items, const double *__restrict__ rows, int P,
+          const cx<double> *__restrict__ loc, const double2 *__restrict__ xi,
+          const int32_t *__restrict__ glob, int nglob, const double2 *__restrict__ xc,
+          const double *__restrict__ y, const double *__restrict__ ell, const double *__restrict__ sums,
+          const double *__restrict__ x, const double *__restrict__ v, double sc, double *__restrict__ out,
+          const int *gate, const int32_t *__restrict__ nodebase, const double *__restrict__ partial,
+          int64_t slab)
+{
+    lbf_rhs(slab, loc, y, sums, x, v, out, gate, partial);
+    if (fmm::gate_closed(gate)) return;
+    __shared__ int2 xs[4][64];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t k = blockIdx.x * (int64_t)(blockDim.x >> 5) + wid;
+    if (k >= nitem) return;
+    const RowItem it = items[k];
+    const int ng = (it.nrow + 3) / 4, n = (2 * P + 7) / 8;
+    const double *t = rows + ((int64_t)it.tile + (int64_t)it.nchunk * ng) * 32 + lane;
+    prefetch_tiles(t - lane, ng * n, lane);
+    const int64_t lb = (int64_t)it.box * 2 * P;
+    bool bad;
+    const int top = local_top(loc, lb, P, lane, bad);
+    for (int m = lane; m < 64; m += 32) {
+        double b = 0.0;
+        if (m < 2 * P) b = (m & 1) ? local_real(loc, lb + m - 1) : -local_real(loc, lb + m + 1);
+        xs[wid][m] = dot_word(b, m >> 2, top);
+    }
+    __syncwarp();
+    Dot acc[kGroups];
+#pragma unroll
+    for (int q = 0; q < kGroups; q++) acc[q] = Dot{0, 0};
+#define LBF_DOT(NG) dot_chunks<NG>(t, xs[wid] + (lane & 7), n, lane, acc)
+    LBF_GROUPS(ng, LBF_DOT)
+#undef LBF_DOT
+    const int grp = fold_rows<kGroups>(lane, [&](int a, int b, bool up, int bit) { acc[a] = dot_meet(acc[a], acc[b], up, bit); });
+    const int row = 4 * grp + (lane >> 3);
+    if (row >= it.nrow) return;
+    const int i = it.row0 + row;
+    double lsum = bad ? __longlong_as_double(0x7ff8000000000000ll) : -LBF_PI * dot_double(acc[0], top - 1129);
+    for (int q = nodebase[i]; q < nodebase[i + 1]; q++) lsum += partial[q];
+    if (nglob) {
+        const double2 zi = xi[i];
+        for (int q = 0; q < nglob; q++) {
+            const int m = glob[q];
+            const double ex = zi.x - xc[m].x, ey = zi.y - xc[m].y;
+            lsum += y[m] * 0.5 * log(ex * ex + ey * ey);
+        }
+    }
+    const double phi = ((ell[i] - LBF_LN2) * sums[0] + sums[1] - 2.0 * lsum) * (1.0 / (2.0 * LBF_PI));
+    out[i] = x[i] + (v ? v[i] : 0.0) + sc * phi;
+}
+
 TreeLists lists_of(const Tree &T)
 {
     return TreeLists{T.level, T.ix,    T.iy,    T.parent, T.begin, T.end,
@@ -693,7 +748,10 @@ void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap)
 {
     pl->rows = nullptr;
     if (o.matvec != LBF_MATVEC_FMM) return;
-    const int64_t cols = (N <= 1 << 18 ? 10 : 4) * (int64_t)o.leaf_size + 2 * (o.p + 1) + 48;
+    // local columns for the density's expansions and, where E y is one, the multipliers'
+    const int Pl = std::max(o.p + 1, pl->bd.p2l_exp_cap ? pl->bd.Pe : 0);
+    pl->rows_lch = local_chunks(Pl);
+    const int64_t cols = (N <= 1 << 18 ? 10 : 4) * (int64_t)o.leaf_size + 2 * Pl + 48;
     // a chunk of columns serves every row group of its leaf (leaves hold about half of leaf_size)
     const int64_t tiles = (N * cols) / 32 + 4096;
     const int64_t chunks = tiles / std::max(1, o.leaf_size / 10) + 4096;
@@ -729,7 +787,7 @@ int lbf_rows_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scrat
     if (!pl->rows) return LBF_OK;
     Tree &T = pl->tree;
     const int64_t nl = T.nleaf;
-    const int P = pl->P, lch = local_chunks(P);
+    const int P = pl->P, lch = pl->rows_lch;
         // (in a small system W and X boxes of up to 512 nodes are pairs while there is room: their
     // few P2L and M2P are dependent steps that the whole application waits for; with boxes of up
     // to 2048 the longest rows hold it up instead, 85 against 22 us for the rows of 8192 nodes)
@@ -811,6 +869,19 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
     else if (pl->rows_split) LBF_ROWS(double, true);
     else LBF_ROWS(double, false);
 #undef LBF_ROWS
+    LBF_CHECK_LAUNCH();
+    return LBF_OK;
+}
+
+// out = x + v + sc E y from the multiplier potential's local expansions (B.loc, Pe terms)
+int lbf_rows_mp(lbf_plan *pl, const double *y, const double *x, const double *v, double sc, double *out,
+                const int *gate, cudaStream_t s)
+{
+    const Border &B = pl->bd;
+    const int64_t n = pl->rows_nitem;
+    LBF_LAUNCH_P(LBF_KERNEL_ESUM, k_rows_mp, lbf_grid(pl, lbf_cdiv(n, 4)), 128, 0, s, n, pl->rows_items,
+                 pl->rows, B.Pe, (const cx<double> *)B.loc, pl->xi, B.glob, B.nglob_h, B.xc, y, B.ell,
+                 B.sums, x, v, sc, out, gate, B.nodebase, B.partial, pl->slab);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }
