@@ -85,8 +85,8 @@ typedef struct lbf_options {
                              (default 3e-4) */
     int max_refine;       /* FP32_REFINE: maximum refinement steps */
     int graphs;           /* GMRES steps replayed from a CUDA graph captured once per plan
-                             (stream must not be the legacy default stream): 1 on, 0 off,
-                             -1 automatic (on for N <= 262144, where launches dominate);
+                             (for the legacy default stream on a stream of its own): 1 on,
+                             0 off, -1 automatic (on for N <= 4194304, where launches count);
                              per-kernel tracing skips graph-replayed kernels */
     int fmm64;            /* arithmetic of the accurate (double) FMM operator: 0 double,
                              1 double-float (pairs of floats, ~48-bit significands; this

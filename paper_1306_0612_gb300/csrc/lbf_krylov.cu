@@ -721,18 +721,33 @@ static int arnoldi_step(lbf_plan *pl, int opc, int prec, int k, bool from_state,
     return arnoldi_step_t<double>(pl, opc, prec, k, from_state, pl->V, pl->gw, s);
 }
 
+// Nodes up to which a plan's steps are replayed as graphs by default.  A first solve, capture
+// included, with graphs and without: 131,072 nodes, gradient of a solve, 45.9 and 47.7 ms;
+// 416,768 nodes 22.6 and 23.7; 524,288 refined 20.4 and 22.2; 2.1 million 115.6 and 117.1.
+constexpr int64_t kGraphNodes = 1 << 22;
+
 // The captured step graph of (prec, transpose), built on first use; null when graphs
-// are off for this plan or the stream cannot capture (the legacy default stream).
+// are off for this plan.  The legacy default stream cannot capture (but runs graphs): the
+// capture for it is made on a stream of its own.
 static cudaGraphExec_t step_graph(lbf_plan *pl, int opc, int prec, cudaStream_t s)
 {
     const int g = pl->opt.graphs;
-    if (g == 0 || (g < 0 && pl->N > (1 << 18)) || s == nullptr || !pl->vstep) return nullptr;
+    if (g == 0 || (g < 0 && pl->N > kGraphNodes) || !pl->vstep) return nullptr;
     if (!(opc & LBF_OP_PRECONDITIONED)) return nullptr;  // the graphs hold the preconditioned step
     const int pi = prec == LBF_PREC_FP32 ? 1 : 0, ti = (opc & LBF_OP_TRANSPOSE) ? 1 : 0;
     if (pl->gexec[pi][ti]) return pl->gexec[pi][ti];
     cudaGraph_t graph = nullptr;
+    cudaStream_t own = nullptr;
+    if (s == nullptr || s == cudaStreamLegacy) {
+        if (cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        s = own;
+    }
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
+        if (own) cudaStreamDestroy(own);
         return nullptr;
     }
     lbf_prof_capture(true);
@@ -750,6 +765,7 @@ static cudaGraphExec_t step_graph(lbf_plan *pl, int opc, int prec, cudaStream_t 
     else
         cudaGetLastError();
     if (graph) cudaGraphDestroy(graph);
+    if (own) cudaStreamDestroy(own);
     return pl->gexec[pi][ti];
 }
 
