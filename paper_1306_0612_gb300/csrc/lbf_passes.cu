@@ -24,10 +24,11 @@
 //
 // Both passes are one launch each whose warps wait on the expansions themselves: every word
 // carries the launch's tag (lbf_fixed.cuh), so a level costs one trip through L2 and no fence.
-// Measured, microseconds at 8192 nodes and at 16.8 million: up 65 and 6300 (double shifts
-// 8000 at the latter; integer shifts with arrival counters 91 and 6100), a chain 26 and 3010
-// (5400; with flags 70 and 3600).  What is left is bound by the integer pipes at the large
-// end, by the depth of the tree at the small one.
+// Measured, microseconds at 8192 nodes and at 16.8 million: up 50 and 3300 (double shifts
+// and P2M 8000 at the latter; integer shifts with arrival counters 91 and 6100, P2M still
+// double), a chain 26 and 3010 (5400; with flags 70 and 3600).  What is left is bound by the
+// dependent loads of a box (a third fewer instructions for its sums changed nothing) and by
+// the depth of the tree.
 #include <algorithm>
 
 #include "lbf_fixed.cuh"
@@ -400,7 +401,7 @@ k_up(int64_t nleaf, int64_t nbox, const int32_t *__restrict__ leaves, const int3
      const int32_t *__restrict__ nchild, int P, int lchunks, const int32_t *__restrict__ block0,
      const RowItem *__restrict__ items, const double *__restrict__ rows,
      const double *__restrict__ binom, const double2 *__restrict__ q, cx<double> *mp, long long *X,
-     int32_t *ex, unsigned *words_, int *status, const int *gate, int64_t slab)
+     int32_t *ex, unsigned *words_, int run, int *status, const int *gate, int64_t slab)
 {
     lbf_rhs(slab, q, mp, X, ex, words_, gate);
     if (fmm::gate_closed(gate)) return;
@@ -423,81 +424,83 @@ k_up(int64_t nleaf, int64_t nbox, const int32_t *__restrict__ leaves, const int3
     const bool on = j < nr && (hf == 0 || r2 != r1);
     for (;;) {
         unsigned ti = 0;
-        if (lane == 0) ti = atomicAdd(&words_[0], 1u);
-        const int64_t t = (int64_t)__shfl_sync(0xffffffffu, ti, 0);
-        if (t >= nleaf + nbox) break;
-        if (t < nleaf) {
-            const int b = leaves[t];
-            leaf_p2m(t, P, lchunks, block0, items, rows, q, vs[wid], sums[wid], lane);
-            __syncwarp();
-            double v[2];
-            int top = -4096;
-            bool bad = false;
+        if (lane == 0) ti = atomicAdd(&words_[0], (unsigned)run);
+        const int64_t t0 = (int64_t)__shfl_sync(0xffffffffu, ti, 0);
+        if (t0 >= nleaf + nbox) break;
+        for (int64_t t = t0; t < min(t0 + run, nleaf + nbox); t++) {
+            if (t < nleaf) {
+                const int b = leaves[t];
+                leaf_p2m(t, P, lchunks, block0, items, rows, q, vs[wid], sums[wid], lane);
+                __syncwarp();
+                double v[2];
+                int top = -4096;
+                bool bad = false;
 #pragma unroll
-            for (int h = 0; h < 2; h++) {  // lane: coefficient
-                const int m = 2 * lane + h;
-                v[h] = m < 2 * P ? vs[wid][m] : 0.0;
-                const int E = (int)((__double_as_longlong(v[h]) >> 52) & 0x7ff);
-                bad |= E == 0x7ff;
-                if (E) top = max(top, E - (lane >> 1));
+                for (int h = 0; h < 2; h++) {  // lane: coefficient
+                    const int m = 2 * lane + h;
+                    v[h] = m < 2 * P ? vs[wid][m] : 0.0;
+                    const int E = (int)((__double_as_longlong(v[h]) >> 52) & 0x7ff);
+                    bad |= E == 0x7ff;
+                    if (E) top = max(top, E - (lane >> 1));
+                }
+                top = __reduce_max_sync(0xffffffffu, top);
+                bad = __any_sync(0xffffffffu, bad);
+                if (2 * lane < pitch)
+                    st_words(&X[(int64_t)b * pitch + 2 * lane],
+                             tag_word(fixed54(__double_as_longlong(v[0]), lane >> 1, top), tag),
+                             tag_word(fixed54(__double_as_longlong(v[1]), lane >> 1, top), tag));
+                if (lane == 0) st_word(&ex[b], tag_exp(bad ? kBadExp : top - 1022, tag));
+                if (lane < P) mp[(int64_t)b * P + lane] = mk<double>(v[0], v[1]);
+                __syncwarp();
+                continue;
             }
-            top = __reduce_max_sync(0xffffffffu, top);
-            bad = __any_sync(0xffffffffu, bad);
-            if (2 * lane < pitch)
-                st_words(&X[(int64_t)b * pitch + 2 * lane],
-                         tag_word(fixed54(__double_as_longlong(v[0]), lane >> 1, top), tag),
-                         tag_word(fixed54(__double_as_longlong(v[1]), lane >> 1, top), tag));
-            if (lane == 0) st_word(&ex[b], tag_exp(bad ? kBadExp : top - 1022, tag));
-            if (lane < P) mp[(int64_t)b * P + lane] = mk<double>(v[0], v[1]);
-            __syncwarp();
-            continue;
-        }
-        const int64_t p = nbox - 1 - (t - nleaf);
-        const int nc = nchild[p], c0 = child0[p];
-        if (nc == 0) continue;
-        long long sx = 0, sy = 0;
-        int emax = -(1 << 22);
-        for (int c = 0; c < nc; c++) {
-            const int h2 = quadrant(ix[c0 + c], iy[c0 + c]);
-            int ec;
-            longlong2 v = wait_words(X + (int64_t)(c0 + c) * pitch, ex + c0 + c, P, lane, tag, lim, status, ec);
-            mul_pow(v.x, v.y, (-lane * h2) & 7);
-            Zs[wid][lane] = (lane & 1) ? words(v.x, v.y) : words(2 * v.x, 2 * v.y);
-            __syncwarp();
-            Sum acc{0, 0, 0, 0}, first{0, 0, 0, 0};
+            const int64_t p = nbox - 1 - (t - nleaf);
+            const int nc = nchild[p], c0 = child0[p];
+            if (nc == 0) continue;
+            long long sx = 0, sy = 0;
+            int emax = -(1 << 22);
+            for (int c = 0; c < nc; c++) {
+                const int h2 = quadrant(ix[c0 + c], iy[c0 + c]);
+                int ec;
+                longlong2 v = wait_words(X + (int64_t)(c0 + c) * pitch, ex + c0 + c, P, lane, tag, lim, status, ec);
+                mul_pow(v.x, v.y, (-lane * h2) & 7);
+                Zs[wid][lane] = (lane & 1) ? words(v.x, v.y) : words(2 * v.x, 2 * v.y);
+                __syncwarp();
+                Sum acc{0, 0, 0, 0}, first{0, 0, 0, 0};
 #pragma unroll 4
-            for (int it = i0; it < i1; it++) {
-                if (it == n1) {
+                for (int it = i0; it < i1; it++) {
+                    if (it == n1) {
+                        first = acc;
+                        acc = Sum{0, 0, 0, 0};
+                    }
+                    const int k = it < n1 ? it : it - n1;
+                    add_term(acc, Cl[k * 32 + (it < n1 ? r1 : r2)], Zs[wid][k]);
+                }
+                if (i1 <= n1) {
                     first = acc;
                     acc = Sum{0, 0, 0, 0};
                 }
-                const int k = it < n1 ? it : it - n1;
-                add_term(acc, Cl[k * 32 + (it < n1 ? r1 : r2)], Zs[wid][k]);
+                const Sum s = meet(hf ? acc : first, hf ? first : acc);
+                long long x = scale_sum(s.xh, s.xl, row + 1), y = scale_sum(s.yh, s.yl, row + 1);
+                mul_pow(x, y, (row * h2) & 7);
+                // to the larger unit of the children so far and this one
+                const int em = max(emax, ec);
+                sx = shift_down(sx, em - emax) + shift_down(x, em - ec);
+                sy = shift_down(sy, em - emax) + shift_down(y, em - ec);
+                emax = em;
+                __syncwarp();
             }
-            if (i1 <= n1) {
-                first = acc;
-                acc = Sum{0, 0, 0, 0};
+            const bool bad = emax >= kBadExp;
+            const int nb = __reduce_max_sync(0xffffffffu, on ? bits_of(sx, sy) : 0), sh = nb - 54;
+            if (on)
+                st_words(&X[p * pitch + 2 * row], tag_word(rescale(sx, sh), tag), tag_word(rescale(sy, sh), tag));
+            if (lane == 0) st_word(&ex[p], tag_exp(bad ? kBadExp : nb == 0 ? kZeroExp : emax + sh, tag));
+            for (int m = 2 * P + lane; m < pitch; m += 32) X[p * pitch + m] = 0;
+            if (on) {
+                const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                const int E = emax - 54 + (row >> 1);
+                mp[p * P + row] = bad ? mk<double>(nan, nan) : mk<double>(pack_double(sx, E), pack_double(sy, E));
             }
-            const Sum s = meet(hf ? acc : first, hf ? first : acc);
-            long long x = scale_sum(s.xh, s.xl, row + 1), y = scale_sum(s.yh, s.yl, row + 1);
-            mul_pow(x, y, (row * h2) & 7);
-            // to the larger unit of the children so far and this one
-            const int em = max(emax, ec);
-            sx = shift_down(sx, em - emax) + shift_down(x, em - ec);
-            sy = shift_down(sy, em - emax) + shift_down(y, em - ec);
-            emax = em;
-            __syncwarp();
-        }
-        const bool bad = emax >= kBadExp;
-        const int nb = __reduce_max_sync(0xffffffffu, on ? bits_of(sx, sy) : 0), sh = nb - 54;
-        if (on)
-            st_words(&X[p * pitch + 2 * row], tag_word(rescale(sx, sh), tag), tag_word(rescale(sy, sh), tag));
-        if (lane == 0) st_word(&ex[p], tag_exp(bad ? kBadExp : nb == 0 ? kZeroExp : emax + sh, tag));
-        for (int m = 2 * P + lane; m < pitch; m += 32) X[p * pitch + m] = 0;
-        if (on) {
-            const double nan = __longlong_as_double(0x7ff8000000000000ll);
-            const int E = emax - 54 + (row >> 1);
-            mp[p * P + row] = bad ? mk<double>(nan, nan) : mk<double>(pack_double(sx, E), pack_double(sy, E));
         }
     }
     // the last warp to finish readies the counters for the next application
@@ -669,6 +672,12 @@ int lbf_passes_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch)
     return LBF_OK;
 }
 
+// leaves and boxes a warp of k_up takes at a time, of n in all: several where every warp has
+// many turns (16.8 million nodes, 8: 3.3 ms, 1: 3.6), one where the chain of a small tree
+// counts.  (Boxes of k_l2l one by one: their parents are near in the order, and eight at a time
+// held a level up, 29 ms against 3.)
+static int run_of(int64_t n, int64_t warps) { return (int)std::max<int64_t>(1, std::min<int64_t>(8, n / (8 * warps))); }
+
 // multipoles of the charges pl->q
 int lbf_passes_up(lbf_plan *pl, const int *gate, cudaStream_t s)
 {
@@ -677,8 +686,8 @@ int lbf_passes_up(lbf_plan *pl, const int *gate, cudaStream_t s)
     const int64_t grid = std::min<int64_t>(lbf_cdiv(T.nleaf + T.nbox, 4), 8 * (int64_t)std::max(pl->nsm, 1));
     LBF_LAUNCH_P(LBF_KERNEL_UP, k_up, lbf_grid(pl, grid), 128, 0, s, T.nleaf, T.nbox, T.leaves, T.ix, T.iy,
                  T.child0, T.nchild, P, lch, pl->rows_block0, pl->rows_items, pl->rows, pl->tab_binom,
-                 pl->q, (cx<double> *)pl->mpole, pl->m2l_X, pl->m2l_e, pass_words(pl), pl->dev_status, gate,
-                 pl->slab);
+                 pl->q, (cx<double> *)pl->mpole, pl->m2l_X, pl->m2l_e, pass_words(pl),
+                 run_of(T.nleaf + T.nbox, 4 * grid), pl->dev_status, gate, pl->slab);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }

@@ -70,6 +70,9 @@ constexpr int kGroups = 8, kGroupsSmall = 2;
 // (8192 nodes: 458 us an application with whole leaves a warp, 408 shared; at 7130 leaves
 // the two are within 1 %, at 16,150 sharing costs 4 % of a solve)
 constexpr int64_t kSmallLeaves = 4864;
+// (several right-hand sides in lockstep share no columns once their blocks make this many warps
+// an SM, four times what is resident: 16 of 10,000 nodes 135 us, shared 150)
+constexpr int64_t kFullWarps = 64;
 constexpr int kLocalTop = 1021;  // exponent field of the local columns' largest: [1/4, 1/2)
 constexpr int kRowBlocks = 4;    // thread blocks an SM
 constexpr int kRun = 4;          // chunks read at a time (2 or 4)
@@ -251,7 +254,7 @@ __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, Tr
         const int m = 8 * c + (lane & 7);
         const bool node = m < ncol;
         const int j = node ? cols[(int64_t)it.chunk * 8 + m] : it.row0;
-        const double2 zj = xi[j], wj = w[j];
+        const double2 zj = xi[j], w1 = w[j], wj = make_double2(w1.x * (1.0 / LBF_PI), w1.y * (1.0 / LBF_PI));
 #pragma unroll
         for (int q = 0; q < kGroups; q++) {
             if (q >= ng) break;
@@ -265,10 +268,10 @@ __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, Tr
                     const double dr = zj.x - zi.x, di = zj.y - zi.y;
                     const double d2 = fma(dr, dr, di * di);
                     // coincident nodes add nothing; outside rcp_near's range, a division
-                    const double id = d2 > 0x1p-120 && d2 < 0x1p120 ? fmm::rcp_near(d2)
-                                      : d2 > 0.0                    ? 1.0 / d2
-                                                                    : 0.0;
-                    e = fma(wj.y, dr, -wj.x * di) * id * (1.0 / LBF_PI);
+                    const double id = abs(exp_field(d2) - 1023) < 120 ? fmm::rcp_near(d2)
+                                      : d2 > 0.0                      ? 1.0 / d2
+                                                                      : 0.0;
+                    e = fma(wj.y, dr, -wj.x * di) * id;
                 }
             }
             t[32 * q] = e;
@@ -859,14 +862,16 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
                    bool df)
 {
     const int64_t n = pl->rows_nitem;
-    const dim3 grid = lbf_grid(pl, pl->rows_split ? n : lbf_cdiv(n, 4));
+    // several right-hand sides fill the chip without sharing a block's columns
+    const bool split = pl->rows_split && (pl->nrhs == 1 || n * pl->nrhs < kFullWarps * (int64_t)std::max(pl->nsm, 1));
+    const dim3 grid = lbf_grid(pl, split ? n : lbf_cdiv(n, 4));
 #define LBF_ROWS(R, SPLIT)                                                                         \
     LBF_LAUNCH_P(LBF_KERNEL_LEAF, (k_rows_apply<R, SPLIT>), grid, 128, 0, s, n, pl->rows_items, pl->rows, \
                  pl->rows_e, pl->rows_cols, sigma, pl->sigma_e, (const cx<R> *)pl->local,          \
                  (const cx<R> *)pl->mpole, pl->P, local_chunks(pl->P), pl->bsig, v, gate, pl->slab)
-    if (df && pl->rows_split) LBF_ROWS(df64, true);
+    if (df && split) LBF_ROWS(df64, true);
     else if (df) LBF_ROWS(df64, false);
-    else if (pl->rows_split) LBF_ROWS(double, true);
+    else if (split) LBF_ROWS(double, true);
     else LBF_ROWS(double, false);
 #undef LBF_ROWS
     LBF_CHECK_LAUNCH();

@@ -135,3 +135,29 @@ def test_integer_rows_keep_scale_and_non_finite_values(leaf, op):
         w[g.N // 2] = bad
         L.lbf_apply(plan, op, w, p)
         assert not torch.isfinite(p).any()
+
+
+def test_passes_where_a_warp_takes_several_leaves():
+    """More than 16 leaves and boxes for every warp of the upward pass: sampled rows."""
+    g = wl.star_caps(5, 1024, 400)
+    plan = plan_for(g, leaf_size=8, p=26, border=0)
+    assert L.lbf_plan_info(plan)["nleaf"] > 80000
+    v = np.random.default_rng(6).standard_normal(g.N)
+    o = zeros(g.N)
+    L.lbf_apply(plan, L.LBF_OP_K_ONLY, dev(v), o)
+    rows = np.random.default_rng(7).choice(g.N, 60, replace=False)
+    assert rel_l2(host(o)[rows], oracle.apply_rows(g, np.concatenate([v, np.zeros(g.M)]), rows, 0)) < TOL
+
+
+@pytest.mark.parametrize("p", [22, 35])  # fewer, more local columns than the multipliers' terms
+@pytest.mark.parametrize("leaf", [3, 48, 200])
+def test_multiplier_potential_through_the_local_columns(leaf, p):
+    """E y of 600 islands (too many for a stored E) at sampled nodes; the expansions' 32 terms
+    are worth 1e-12."""
+    g = wl.star_caps(7, 600, 33)
+    plan = plan_for(g, leaf_size=leaf, p=p)
+    v = np.concatenate([np.zeros(g.N), np.random.default_rng(leaf).standard_normal(g.M)])
+    o = zeros(g.N + g.M)
+    L.lbf_apply(plan, L.LBF_OP_FULL, dev(v), o)
+    rows = np.random.default_rng(8).choice(g.N, 100, replace=False)
+    assert rel_l2(host(o)[rows], oracle.apply_rows(g, v, rows, 0)) < TOL
