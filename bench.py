@@ -239,7 +239,8 @@ def run_reference(args):
 # and 39, 1.72 s.)
 C4_INNER_TOL = 1e-5
 
-FMM_SOURCES = ("lbf_fmm_tpl.cuh", "lbf_fmm.cu", "lbf_tree.cu", "lbf_df64.cuh", "lbf_internal.cuh")
+FMM_SOURCES = ("lbf_fmm_tpl.cuh", "lbf_fmm.cu", "lbf_tree.cu", "lbf_df64.cuh", "lbf_internal.cuh",
+               "lbf_rows.cu", "lbf_m2l.cu", "lbf_passes.cu", "lbf_fixed.cuh", "lbf_tc.cuh")
 
 
 def src_hash():
@@ -296,19 +297,23 @@ def peak_fractions(line):
         s, rf = line["solve"], line["roofline"]
         c, bc, N = s["counts"], s["border_counts"], s["counts"]["N"]
         P = s["tree"]["p"] + 1
-        if rf.get("unit") != "TFLOP/s" or not line["matvec"].get("fp64"):
+        if rf.get("unit") not in ("TFLOP/s", "GB/s") or not line["matvec"].get("fp64"):
             return None
         w = {k: kernel_work(k, c, bc, P, 0, N)[0] for k in ("up", "down", "leaf", "esum")}
         k_apply = w["up"] + w["down"] + w["leaf"]
         mv_ms = line["matvec"]["fp64"]["ms"]
         work = s["fp64_applies"] * (k_apply + (w["esum"] or 0))
-        peak = rf["peak"]
+        stored = rf["unit"] == "GB/s"  # passes over stored parts, bound by memory
+        peak = FP64_PEAK_TFLOPS if stored else rf["peak"]
+        src = ("nominal FP64; above 1 because the flops are those of forming every pair and translation, "
+               "most of which a plan stores or sums on the integer pipes and the tensor cores"
+               if stored else rf.get("peak_source"))
 
         def rate(flop, ms):
             a = flop / (ms * 1e-3) / 1e12
             return {"gflop": flop / 1e9, "ms": ms, "achieved": a, "frac": a / peak}
 
-        return {"unit": "TFLOP/s", "peak": peak, "peak_source": rf.get("peak_source"),
+        return {"unit": "TFLOP/s", "peak": peak, "peak_source": src,
                 "matvec": rate(k_apply, mv_ms), "solve": rate(work, s["solve_ms"])}
     except (KeyError, TypeError, AttributeError, ZeroDivisionError):
         return None
@@ -423,11 +428,27 @@ def roofline_of(L, prof, plan, opt, g, n64, n32, fmm64):
     work, unit = kernel_work(dom, counts, bcounts, P, P32, g.N)
     if work is None:
         return None, counts, bcounts, info
-    per_launch_ms = prof[dom]["ms"] / prof[dom]["launches"]
     f32 = dom.endswith("32")
-    # leaf, up and down run once per application; esum once per FULL/PRECONDITIONED one
+    # per application: the upward pass is one launch of it, the others one to three
+    apps = prof.get("up32" if f32 else "up", prof[dom])["launches"]
+    per_launch_ms = prof[dom]["ms"] / apps
+    bound, scale = "alu", 1e12
+    if not f32 and per_launch_ms * 1e-3 * FP64_PEAK_TFLOPS * 1e12 < work:
+        # faster than the double pipe could be: the pass reads stored parts (8 bytes a row
+        # entry, 16 a coefficient) and sums them on the integer pipes and the tensor cores, so
+        # its rate is that of these bytes
+        bound, scale, unit = "hbm", 1e9, "GB/s"
+        Pe = bcounts["terms"] if bcounts else 0
+        work = {"leaf": 8 * (counts["p2p_pairs"] + 2 * P * g.N),
+                "up": 8 * 2 * P * g.N + 16 * P * counts["m2m"],
+                "down": 16 * P * (counts["m2l"] + 2 * counts["l2l"]),
+                "esum": 8 * 2 * Pe * g.N + 16 * Pe * ((bcounts or {}).get("p2l_pairs", 0) + 2 * counts["l2l"])}[dom]
     rate = work / (per_launch_ms / 1e3)
-    if f32:
+    if bound == "hbm":
+        mp = os.path.join(ROOT, "MEASURED_PEAKS.json")
+        peak, src_p = ((json.load(open(mp))["hbm_gbs"], "measured copy bandwidth") if os.path.exists(mp)
+                       else (6800.0, "copy bandwidth of one earlier measurement"))
+    elif f32:
         peak, src_p = FP32_PEAK_TFLOPS, "FP32: 152 SMs x 128 lanes x 2 flops x 2.07 GHz"
     else:
         peak = FP64_PEAK_TFLOPS
@@ -436,8 +457,8 @@ def roofline_of(L, prof, plan, opt, g, n64, n32, fmm64):
         if fmm64 and dom in ("up", "down", "leaf"):
             src_p += ("; this kernel runs double-float arithmetic on the FP32 pipes, whose own "
                       f"ceiling is {FP32_PEAK_TFLOPS / DF64_FLOPS_PER_FLOP:.2f} TFLOP/s of double flops")
-    ach = rate / 1e12
-    return ({"bound": "alu", "kernel": dom, "achieved": ach, "peak": peak, "unit": unit,
+    ach = rate / scale
+    return ({"bound": bound, "kernel": dom, "achieved": ach, "peak": peak, "unit": unit,
              "frac": ach / peak,
              "traffic": traffic_for(dom + ("_df64" if fmm64 and not f32 else ""),
                                     opt.p32 if f32 else info["p"], opt.leaf_size),
