@@ -873,8 +873,8 @@ int lbf_debug_inject(lbf_plan *pl, int what, unsigned polls, lbf_stream_t stream
     if (what != LBF_INJECT_CHAIN || !pl) return LBF_EINVAL;
     if (!pl->pull || pl->opt.matvec != LBF_MATVEC_FMM || pl->tree.nlev <= 3) return LBF_ENOTBUILT;
     // the poll limit, and the second phase of the next chain starting at the first box of
-    // level 3: levels 0..2 are never marked done in that epoch, so their children's
-    // parent waits run out; the chain's last warp resets the counters as always
+    // level 3: levels 0..2 are never marked done in that epoch (their words never written
+    // under its tag), so their children's parent waits run out; the chain's last warp resets the counters as always
     const int lim = (int)polls;
     const unsigned first = (unsigned)pl->tree.lev_start[3];
     LBF_CUDA(cudaMemcpyAsync(pl->dev_status + 1, &lim, sizeof(int), cudaMemcpyHostToDevice, s));
