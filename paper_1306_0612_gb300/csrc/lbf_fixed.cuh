@@ -15,8 +15,9 @@ __host__ __device__ inline int real_pitch(int P) { return (2 * P + 7) / 8 * 8; }
 // under a tag of 8 bits, the application's number.  A reader of the same launch waits on the
 // words themselves until they carry the tag, so a box is handed on with one store and one
 // load where a flag costs a fence and two trips to L2 more.  The tags go round 1 .. 255 (0:
-// words that no launch of that kind wrote) and every launch rewrites all words, so an old word
-// never carries the tag waited for.
+// words that no launch wrote) and every launch writes all words of the boxes it hands on, zeros
+// past its own order (launches of several orders share the words and the count of launches), so
+// an old word never carries the tag waited for.
 __device__ __forceinline__ long long tag_word(long long x, unsigned tag)
 {
     return (long long)(((unsigned long long)x & 0xffffffffffffffull) | ((unsigned long long)tag << 56));
