@@ -209,7 +209,7 @@ struct lbf_plan {
     // columns (rptr null: not stored), a value per column
     int32_t *rows_block0 = nullptr, *rows_rptr = nullptr, *rows_rbase = nullptr;
     double *rows_z = nullptr;
-    int32_t *rows_e = nullptr;  // exponent field of each node's largest near entry
+    int32_t *rows_e = nullptr;  // exponent field of each node's largest finite near entry, kBadRow: not all are
     // boxes whose X lists are not near columns (nbigx < 0: the passes of lbf_passes.cu are off)
     int64_t nbigx = -1, bigx_cap = 0;
     int32_t *bigx = nullptr;
