@@ -177,8 +177,7 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
     pl->v = A.get<double>(N);
     pl->bsig = A.get<double>(4);
     pl->red = A.get<double>(1024);
-    pl->red_count = A.get<unsigned>(8);
-    pl->sigma_e = (int32_t *)(pl->red_count + 4);
+    pl->red_count = A.get<unsigned>(4);
     pl->dev_status = A.get<int>(2);  // [0] error bits, [1] poll limit of device waits (0: default)
     pl->fvec = A.get<double>(M);
     pl->yvec = A.get<double>(M);
@@ -309,8 +308,7 @@ static void layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A)
     v->v = A.get<double>(N);
     v->bsig = A.get<double>(4);
     v->red = A.get<double>(1024);
-    v->red_count = A.get<unsigned>(8);
-    v->sigma_e = (int32_t *)(v->red_count + 4);
+    v->red_count = A.get<unsigned>(4);
     v->fvec = A.get<double>(M);
     v->yvec = A.get<double>(M);
     v->tin = A.get<double>(n);
@@ -371,7 +369,7 @@ lbf_plan lbf_view_at(const lbf_plan &v, int r)
     };
     mv(o.q); mv(o.mpole); mv(o.local); mv(o.upcnt); mv(o.pull); mv(o.qdf); mv(o.q32);
     mv(o.mpole32); mv(o.local32); mv(o.imean); mv(o.gr); mv(o.gd); mv(o.v); mv(o.bsig);
-    mv(o.red); mv(o.red_count); mv(o.sigma_e); mv(o.fvec); mv(o.yvec); mv(o.tin); mv(o.tout); mv(o.vstep);
+    mv(o.red); mv(o.red_count); mv(o.fvec); mv(o.yvec); mv(o.tin); mv(o.tout); mv(o.vstep);
     mv(o.bd.partial); mv(o.bd.loc); mv(o.bd.loc32); mv(o.bd.sums); mv(o.H); mv(o.gw);
     mv(o.gx); mv(o.gb); mv(o.gpart); mv(o.gs); mv(o.V); mv(o.region); mv(o.nearbuf);
     mv(o.dpart); mv(o.dcount); mv(o.m2l_X); mv(o.m2l_e); mv(o.m2l_out); mv(o.loc_e); mv(o.loc_X);
@@ -639,7 +637,7 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
         CK(cudaMemcpyAsync(pl->dev_status + 1, &lim, sizeof(int), cudaMemcpyHostToDevice, s));
         CK(cudaStreamSynchronize(s));
     }
-    CK(cudaMemsetAsync(pl->red_count, 0, 8 * sizeof(unsigned), s));
+    CK(cudaMemsetAsync(pl->red_count, 0, 4 * sizeof(unsigned), s));
     CK(cudaMemsetAsync(pl->bsig, 0, 4 * sizeof(double), s));
     // plan-creation temporaries overlay the region of the GMRES basis
     Temps tt = temps(pl, pl->region, N, M, cap);

@@ -40,18 +40,16 @@ __global__ void k_prep(int64_t N, const double *__restrict__ sigma, const double
                        double *__restrict__ part, unsigned *__restrict__ count,
                        double *__restrict__ out, const int *gate,
                        const int32_t *__restrict__ isl, const double *__restrict__ mean,
-                       int32_t *__restrict__ sexp, int64_t slab)
+                       int64_t slab)
 {
-    lbf_rhs(slab, sigma, q, q32, qdf, part, count, out, gate, mean, sexp);
+    lbf_rhs(slab, sigma, q, q32, qdf, part, count, out, gate, mean);
     if (fmm::gate_closed(gate)) return;
     __shared__ double sh[32];
     __shared__ bool last;
     double acc = 0.0;
-    int top = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
          i += (int64_t)gridDim.x * blockDim.x) {
         double s = sigma[i];
-        top = max(top, (int)((__double_as_longlong(s) >> 52) & 0x7ff));
         const double sc = isl ? s - mean[isl[i]] : s;  // the charges of sigma less its island means
         double2 qq = make_double2(sc, 0.0);
         if (w) {
@@ -66,8 +64,6 @@ __global__ void k_prep(int64_t N, const double *__restrict__ sigma, const double
     acc = warp_sum(acc);
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (lane == 0) sh[wid] = acc;
-    top = __reduce_max_sync(0xffffffffu, top);
-    if (lane == 0) atomicMax(&sexp[0], top);
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
@@ -91,7 +87,6 @@ __global__ void k_prep(int64_t N, const double *__restrict__ sigma, const double
         for (int k = 0; k < (int)(blockDim.x >> 5); k++) u += sh[k];
         *out = u;
         *count = 0u;
-        sexp[1] = atomicExch(&sexp[0], 0);
     }
 }
 
@@ -528,7 +523,7 @@ static int prep(lbf_plan *pl, const double *sigma, Arith ar, bool weighted, cons
                ar == Arith::DF64 ? (cx<df64> *)pl->qdf : (cx<df64> *)nullptr, pl->red,
                pl->red_count, pl->bsig, gate,
                split ? (const int32_t *)pl->isl : (const int32_t *)nullptr,
-               split ? (const double *)pl->imean : (const double *)nullptr, pl->sigma_e, pl->slab);
+               split ? (const double *)pl->imean : (const double *)nullptr, pl->slab);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }

@@ -220,7 +220,6 @@ struct lbf_plan {
     double *bsig = nullptr;     // scalar beta . sigma
     double *red = nullptr;      // reduction partials
     unsigned int *red_count = nullptr;
-    int32_t *sigma_e = nullptr;  // largest exponent field of the density: being formed, of the last pass
     // border
     Border bd;                  // E y by island expansions (E itself is never formed)
     double *Sinv = nullptr;     // M x M inverse Schur complement, or (lu) its LU factors

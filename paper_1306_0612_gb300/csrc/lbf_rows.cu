@@ -27,8 +27,8 @@
 //
 // On the integer pipes: a double multiply-add leaves a scheduler every 64 cycles, the three
 // 32 x 32 -> 64 bit products that stand for one every 17 (lbf_fixed.cuh).  An entry is an integer
-// of 54 bits below its row's largest near entry (rexp), the density below its largest, the
-// local columns and the expansion below fixed sizes (|u_i^l| 2^-(l/2) < 3/2); the sums are exact
+// of 54 bits below its row's largest near entry (rexp), the density below the largest of the run
+// of up to 512 columns it is summed with, the local columns and the expansion below fixed sizes (|u_i^l| 2^-(l/2) < 3/2); the sums are exact
 // but for the products' last 52 bits.  Errors of whole applications against 64 bits are what they
 // were with double entries, to three digits, at orders 22 to 31.  The multipole columns, few and in units
 // of their own, stay double.
@@ -418,7 +418,7 @@ template <int G, typename R>
 __device__ __forceinline__ double block_rows(const RowItem &it, const double *__restrict__ rows,
                                              const int32_t *__restrict__ rexp,
                                              const int32_t *__restrict__ cols,
-                                             const double *__restrict__ sigma, int sexp,
+                                             const double *__restrict__ sigma,
                                              const cx<R> *__restrict__ loc,
                                              const cx<R> *__restrict__ mp, int P, int k0, int k1,
                                              int2 *xs, int lane, int &row)
@@ -453,20 +453,29 @@ __device__ __forceinline__ double block_rows(const RowItem &it, const double *__
             s += d[0];
             continue;
         }
-        // near nodes, in units of the density's largest and the row's largest; the local
-        // expansion, in those of its largest b_l 2^(l/2)
+        // near nodes, in units of the run's largest density and the row's largest entry; the
+        // local expansion, in those of the run's largest b_l 2^(l/2)
         const bool far = k >= nn;
         const int n = min((far ? k1 : min(k1, nn)) - k, kDotChunks);
-        bool bad = false;
         if (k > k0) prefetch_tiles(t - lane, ng * min(n, kAhead), lane);
-        const int top = far ? local_top(loc, lb, P, lane, bad) : sexp;
-        const int off = 8 * (far ? it.nchunk : 0), end = far ? off + 2 * P : it.ncol;
+        const int off = 8 * (far ? it.nchunk : 0), end = min(far ? off + 2 * P : it.ncol, 8 * (k + n));
+        const int m1 = 8 * (k + (n + 3) / 4 * 4);
+        int top = 0;
         __syncwarp();
 #pragma unroll 2
-        for (int m = 8 * k + lane; m < 8 * (k + (n + 3) / 4 * 4); m += 32) {
+        for (int m = 8 * k + lane; m < m1; m += 32) {
             double v = 0.0;
-            if (m < min(end, 8 * (k + n))) v = far ? local_real(loc, lb + m - off) : sigma[cl[m]];
-            xs[m - 8 * k] = dot_word(v, far ? (m - off) >> 2 : 0, top);
+            if (m < end) v = far ? local_real(loc, lb + m - off) : sigma[cl[m]];
+            const int E = exp_field(v);
+            if (E) top = max(top, E == 0x7ff ? kBadExp : E + (far ? (m - off) >> 2 : 0));
+            xs[m - 8 * k] = make_int2(__double2loint(v), __double2hiint(v));  // a lane's own until they are words
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        const bool bad = top >= kBadExp;
+#pragma unroll 2
+        for (int m = 8 * k + lane; m < m1; m += 32) {
+            const int2 b = xs[m - 8 * k];
+            xs[m - 8 * k] = dot_word(__hiloint2double(b.y, b.x), far ? (m - off) >> 2 : 0, top);
         }
         __syncwarp();
         Dot acc[G];
@@ -498,11 +507,11 @@ template <typename R, bool SPLIT>
 __global__ void __launch_bounds__(128, kRowBlocks)
 k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__restrict__ rows,
              const int32_t *__restrict__ rexp, const int32_t *__restrict__ cols,
-             const double *__restrict__ sigma, const int32_t *__restrict__ sexp,
+             const double *__restrict__ sigma,
              const cx<R> *__restrict__ loc, const cx<R> *__restrict__ mp, int P, int lchunks,
              const double *__restrict__ bsig, double *__restrict__ v, const int *gate, int64_t slab)
 {
-    lbf_rhs(slab, sigma, sexp, loc, mp, bsig, v, gate);
+    lbf_rhs(slab, sigma, loc, mp, bsig, v, gate);
     if (fmm::gate_closed(gate)) return;
     __shared__ double part[4][32];
     __shared__ int2 xs[4][8 * kDotChunks];
@@ -513,18 +522,16 @@ k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__r
     const RowItem it{i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
     const int nk = it.nchunk + lchunks;
     const int k0 = SPLIT ? nk * wid / 4 : 0, k1 = SPLIT ? nk * (wid + 1) / 4 : nk;
-    const int se = sexp[1];
     int row;
-    double s = block_rows<SPLIT ? kGroupsSmall : kGroups>(it, rows, rexp, cols, sigma, se, loc, mp, P, k0,
-                                                          k1, xs[wid], lane, row);
+    double s = block_rows<SPLIT ? kGroupsSmall : kGroups>(it, rows, rexp, cols, sigma, loc, mp, P, k0, k1,
+                                                          xs[wid], lane, row);
     if (SPLIT) {
         part[wid][lane] = s;
         __syncthreads();
         if (wid != 0) return;
         s = part[0][lane] + part[1][lane] + part[2][lane] + part[3][lane];
     }
-    if (row < it.nrow)
-        v[it.row0 + row] = se == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : s + 2.0 * *bsig;
+    if (row < it.nrow) v[it.row0 + row] = s + 2.0 * *bsig;
 }
 
 // a[h] += the tiles of chunk h (of n, at most 4) times the rows' values
@@ -878,7 +885,7 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
     const dim3 grid = lbf_grid(pl, split ? n : lbf_cdiv(n, 4));
 #define LBF_ROWS(R, SPLIT)                                                                         \
     LBF_LAUNCH_P(LBF_KERNEL_LEAF, (k_rows_apply<R, SPLIT>), grid, 128, 0, s, n, pl->rows_items, pl->rows, \
-                 pl->rows_e, pl->rows_cols, sigma, pl->sigma_e, (const cx<R> *)pl->local,          \
+                 pl->rows_e, pl->rows_cols, sigma, (const cx<R> *)pl->local,                       \
                  (const cx<R> *)pl->mpole, pl->P, local_chunks(pl->P), pl->bsig, v, gate, pl->slab)
     if (df && split) LBF_ROWS(df64, true);
     else if (df) LBF_ROWS(df64, false);
