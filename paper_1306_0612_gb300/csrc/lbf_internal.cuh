@@ -122,7 +122,8 @@ struct Border {
 
 // A block of stored leaf rows (lbf_rows.cu): nrow rows of leaf `box` from node row0 on,
 // nchunk chunks of eight near columns from chunk `chunk` on (the first ncol columns are
-// nodes), tiles from `tile` on; leaf: the box's index among the leaves
+// nodes), tiles from `tile` on; leaf: the box's index among the leaves, ~ of it where the near
+// tiles hold doubles
 struct __align__(16) RowItem {
     int32_t box, row0, nrow, tile, chunk, nchunk, ncol, leaf;
 };
@@ -209,7 +210,7 @@ struct lbf_plan {
     // columns (rptr null: not stored), a value per column
     int32_t *rows_block0 = nullptr, *rows_rptr = nullptr, *rows_rbase = nullptr;
     double *rows_z = nullptr;
-    int32_t *rows_e = nullptr;  // exponent field of each node's largest finite near entry, kBadRow: not all are
+    int32_t *rows_e = nullptr;  // exponent field of each node's largest near entry
     // boxes whose X lists are not near columns (nbigx < 0: the passes of lbf_passes.cu are off)
     int64_t nbigx = -1, bigx_cap = 0;
     int32_t *bigx = nullptr;

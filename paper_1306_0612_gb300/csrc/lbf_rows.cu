@@ -77,7 +77,13 @@ constexpr int kLocalTop = 1021;  // exponent field of the local columns' largest
 constexpr int kRowBlocks = 4;    // thread blocks an SM
 constexpr int kRun = 4;          // chunks read at a time (2 or 4)
 constexpr int kAhead = 8;        // chunks asked for before they are read
-constexpr int kBadRow = 0x800;   // in a row's exponent field: an entry is not finite
+// A block with a near entry of 1/2 or more, or one that is not finite, keeps its near entries as
+// doubles.  Entries above 1/pi are curves closer than their node spacing; the integers would
+// take from the row's other entries what such an entry needs, and in transposed sums, which have
+// one unit for a block's rows, from all of the block's columns (median error of transposed rows
+// beside two islands that touch, in units of 2^-53 of their terms: 0.9 with entries up to 0.3, 48
+// with 32, 409 with 3200; 18 to 20 with pairs formed on the fly, 1 to 2 as doubles).
+constexpr int kWideTop = 1021;  // largest exponent field of an integer block's entries
 constexpr int kDotChunks = 64;   // chunks a Dot takes at most between two conversions (a multiple of 4)
 static_assert(kDotChunks % 4 == 0, "xs is filled by four chunks");
 
@@ -233,9 +239,9 @@ __global__ void k_rows_rev_sort(int64_t nleaf, const int32_t *__restrict__ ptr, 
 }
 
 // the entries, a warp per row block: the near ones as doubles first, turned into integers in
-// the unit of their row's largest once that is known.  An entry that is not finite (the self
-// term 0/0 of a node where the parametrisation stops) is left zero and its row marked
-__global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, TreeLists T, int thr,
+// the unit of their row's largest once that is known (unless one is too large for that, or not
+// finite: the self term 0/0 of a node where the parametrisation stops)
+__global__ void k_rows_fill(int64_t nitem, RowItem *__restrict__ items, TreeLists T, int thr,
                             BoxGeo g, int P, int lchunks, const int32_t *__restrict__ cols,
                             const double2 *__restrict__ xi, const double2 *__restrict__ w,
                             const double *__restrict__ dself, double *__restrict__ rows,
@@ -249,7 +255,7 @@ __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, Tr
     const int ncol = it.ncol, nn = (ncol + 7) / 8;
     const int nend = 8 * nn + 2 * P * big_boxes(T, it.box, thr);
     double *t = rows + (int64_t)it.tile * 32 + lane;
-    int top[kGroups], bad = 0;  // bad: bit q for the lane's row of group q
+    int top[kGroups];
 #pragma unroll
     for (int q = 0; q < kGroups; q++) top[q] = 0;
     for (int c = 0; c < nn; c++, t += 32 * ng) {
@@ -276,27 +282,27 @@ __global__ void k_rows_fill(int64_t nitem, const RowItem *__restrict__ items, Tr
                     e = fma(wj.y, dr, -wj.x * di) * id;
                 }
             }
-            if (exp_field(e) == 0x7ff) {
-                e = 0.0;
-                bad |= 1 << q;
-            }
             t[32 * q] = e;
             top[q] = max(top[q], exp_field(e));
         }
     }
-    for (int o = 4; o > 0; o >>= 1) bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+    int most = 0;
+#pragma unroll
+    for (int q = 0; q < kGroups; q++) most = max(most, top[q]);
+    const bool wide = __any_sync(0xffffffffu, most > kWideTop);
 #pragma unroll
     for (int q = 0; q < kGroups; q++) {
         if (q >= ng) break;
         for (int o = 4; o > 0; o >>= 1) top[q] = max(top[q], __shfl_xor_sync(0xffffffffu, top[q], o));
         const int r = 4 * q + (lane >> 3);
-        if ((lane & 7) == 0 && r < it.nrow) rexp[it.row0 + r] = top[q] | ((bad >> q & 1) ? kBadRow : 0);
+        if ((lane & 7) == 0 && r < it.nrow) rexp[it.row0 + r] = top[q];
     }
+    if (wide && lane == 0) items[k].leaf = ~it.leaf;
     t = rows + (int64_t)it.tile * 32 + lane;
     for (int c = 0; c < nn; c++, t += 32 * ng)
 #pragma unroll
         for (int q = 0; q < kGroups; q++)
-            if (q < ng) *(int2 *)&t[32 * q] = dot_word(t[32 * q], 0, top[q]);
+            if (q < ng && !wide) *(int2 *)&t[32 * q] = dot_word(t[32 * q], 0, top[q]);
     for (int c = nn; c < it.nchunk; c++, t += 32 * ng)
         for (int q = 0; q < ng; q++)
             if (8 * c + (lane & 7) >= nend || 4 * q + (lane >> 3) >= it.nrow) t[32 * q] = 0.0;
@@ -428,20 +434,21 @@ __device__ __forceinline__ double block_rows(const RowItem &it, const double *__
     const int32_t *cl = cols + (int64_t)it.chunk * 8;
     const int64_t lb = (int64_t)it.box * 2 * P;
     const int nn = (it.ncol + 7) / 8;
+    const bool wide = it.leaf < 0;
     const int grp = fold_rows<G>(lane, [](int, int, bool, int) {});
     row = grp < ng ? 4 * grp + (lane >> 3) : it.nrow;
     prefetch_tiles(t - lane, ng * min(k1 - k0, kAhead), lane);
     double s = 0.0;
     int k = k0;
     while (k < k1) {
-        if (k >= nn && k < it.nchunk) {
-            // multipoles of W boxes: few, and in units of their own
+        if (k < it.nchunk && (wide || k >= nn)) {
+            // multipoles of W boxes: few, and in units of their own; near entries kept as doubles
             double d[G];
 #pragma unroll
             for (int q = 0; q < G; q++) d[q] = 0.0;
             for (const int ke = min(k1, it.nchunk); k < ke; k++, t += 32 * ng) {
-                const int j = cl[8 * k + (lane & 7)];
-                const double x = j < 0 ? local_real(mp, -1 - j) : 0.0;
+                const int m = 8 * k + (lane & 7), j = cl[m];
+                const double x = m < it.ncol ? sigma[j] : j < 0 ? local_real(mp, -1 - j) : 0.0;
 #pragma unroll
                 for (int q = 0; q < G; q++)
                     if (q < ng) d[q] = fma(t[32 * q], x, d[q]);
@@ -492,11 +499,9 @@ __device__ __forceinline__ double block_rows(const RowItem &it, const double *__
         k += n;
         t += (int64_t)32 * n * ng;
         fold_rows<G>(lane, [&](int a, int b, bool up, int bit) { acc[a] = dot_meet(acc[a], acc[b], up, bit); });
-        if (row < it.nrow) {
-            const int re = far ? 0 : rexp[it.row0 + row];
-            s += bad || (re & kBadRow) ? __longlong_as_double(0x7ff8000000000000ll)
-                                       : dot_double(acc[0], top + (far ? -1129 : re - 2150));
-        }
+        if (row < it.nrow)
+            s += bad ? __longlong_as_double(0x7ff8000000000000ll)
+                     : dot_double(acc[0], top + (far ? -1129 : rexp[it.row0 + row] - 2150));
     }
     return s;
 }
@@ -570,7 +575,21 @@ k_rows_t(const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
         // tau_r in the unit of its row's entries, as an integer in that of the block's largest,
         // a lane a row; then the rows of each lane's sums
         const double tr = lane < it.nrow ? tau[it.row0 + lane] : 0.0;
-        const int re = lane < it.nrow ? rexp[it.row0 + lane] & ~kBadRow : 0, E = exp_field(tr);
+        if (it.leaf < 0) {  // near entries kept as doubles
+            const double *tl = rows + ((int64_t)it.tile + (int64_t)k0 * ng) * 32 + lane;
+            for (int c = k0; c < k1; c++, tl += 32 * ng) {
+                double s = 0.0;
+                for (int q = 0; q < ng; q++)
+                    s = fma(tl[32 * q], __shfl_sync(0xffffffffu, tr, 4 * q + (lane >> 3)), s);
+                s += __shfl_xor_sync(0xffffffffu, s, 8);
+                s += __shfl_xor_sync(0xffffffffu, s, 16);
+                double *o = z + ((int64_t)it.chunk + c) * 8 + lane;
+                if (lane < 8) *o = k == b0 ? s : *o + s;
+            }
+            __syncwarp();  // (another lane may add to these columns in the next block)
+            continue;
+        }
+        const int re = lane < it.nrow ? rexp[it.row0 + lane] : 0, E = exp_field(tr);
         const bool bad = __any_sync(0xffffffffu, E == 0x7ff);
         const int top = __reduce_max_sync(0xffffffffu, E ? E + re : 0);
         const int2 x = dot_word(tr, re, top);
@@ -595,11 +614,12 @@ k_rows_t(const int32_t *__restrict__ block0, const RowItem *__restrict__ items,
                 *o = k == b0 ? s : *o + s;
             }
         }
+        __syncwarp();
     }
 }
 
-// v_i = Im(w_i Phi_far)/pi + 2 beta_i sum tau + the node's entries of the z vectors (and a self
-// term that is not finite, which they leave out), a warp per row block
+// v_i = Im(w_i Phi_far)/pi + 2 beta_i sum tau + the node's entries of the z vectors, a warp
+// per row block
 template <typename R>
 __global__ void __launch_bounds__(128)
 k_rows_t_out(int64_t nitem, const RowItem *__restrict__ items, const double *__restrict__ rows,
@@ -607,8 +627,7 @@ k_rows_t_out(int64_t nitem, const RowItem *__restrict__ items, const double *__r
              const int32_t *__restrict__ rptr, const int32_t *__restrict__ rbase,
              const int32_t *__restrict__ begin, const cx<R> *__restrict__ loc,
              const cx<R> *__restrict__ mp, int P, int lchunks, const double2 *__restrict__ w,
-             const double *__restrict__ beta, const double *__restrict__ dself,
-             const double *__restrict__ tau, const double *__restrict__ bsig,
+             const double *__restrict__ beta, const double *__restrict__ bsig,
              double *__restrict__ v, const int *gate)
 {
     if (fmm::gate_closed(gate)) return;
@@ -680,10 +699,9 @@ k_rows_t_out(int64_t nitem, const RowItem *__restrict__ items, const double *__r
     fr += bad ? nan : dot_double(dr[0], top - 1129);
     const int row = 4 * grp + (lane >> 3);
     if (row >= it.nrow) return;
-    const int i = it.row0 + row, at = i - begin[it.box];
+    const int i = it.row0 + row, at = i - begin[it.box], leaf = it.leaf < 0 ? ~it.leaf : it.leaf;
     double s = 0.0;
-    for (int e = rptr[it.leaf]; e < rptr[it.leaf + 1]; e++) s += z[(int64_t)rbase[e] + at];
-    if (exp_field(dself[i]) == 0x7ff) s += 2.0 * dself[i] * tau[i];
+    for (int e = rptr[leaf]; e < rptr[leaf + 1]; e++) s += z[(int64_t)rbase[e] + at];
     const double2 ww = w[i];
     v[i] = s - fma(ww.x, fi, ww.y * fr) + 2.0 * (beta[i] * *bsig);
 }
@@ -921,13 +939,12 @@ int lbf_rows_apply_t(lbf_plan *pl, const double *tau, double *v, const int *gate
         LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t_out<df64>, lbf_cdiv(n, 4), 128, 0, s, n, pl->rows_items,
                      pl->rows, pl->rows_cols, pl->rows_z, pl->rows_rptr, pl->rows_rbase, T.begin,
                      (const cx<df64> *)pl->local, (const cx<df64> *)pl->mpole, pl->P, lch, pl->w,
-                     pl->beta, pl->dself, tau, pl->bsig, v, gate);
+                     pl->beta, pl->bsig, v, gate);
     else
         LBF_LAUNCH_P(LBF_KERNEL_LEAF, k_rows_t_out<double>, lbf_cdiv(n, 4), 128, 0, s, n,
                      pl->rows_items, pl->rows, pl->rows_cols, pl->rows_z, pl->rows_rptr,
                      pl->rows_rbase, T.begin, (const cx<double> *)pl->local,
-                     (const cx<double> *)pl->mpole, pl->P, lch, pl->w, pl->beta, pl->dself, tau, pl->bsig,
-                     v, gate);
+                     (const cx<double> *)pl->mpole, pl->P, lch, pl->w, pl->beta, pl->bsig, v, gate);
     LBF_CHECK_LAUNCH();
     return LBF_OK;
 }

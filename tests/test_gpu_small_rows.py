@@ -72,3 +72,32 @@ def test_a_far_large_density_costs_small_rows_nothing(fmm64, leaf, nodes):
     rows = np.unique(np.concatenate([rows, [int(ptr[2]) + nodes // 2]]))
     err = np.abs(out[2] - out[0] - out[1])[rows]
     assert np.all(err <= 27 * 30 * EPS * row_sizes(ptr, z, big + small, rows))
+
+
+@pytest.mark.parametrize("gap", [1.0, 0.1, 1e-3, 1e-6])
+@pytest.mark.parametrize("fmm64", [0, 1])
+def test_transposed_rows_beside_islands_that_touch(fmm64, gap):
+    """Transposed rows of islands from a node spacing to a millionth of one apart, all pairs near
+    (one leaf), against the direct sums: every node but the two that meet has the error that
+    coordinates rounded to 2^-53 of the box's half-width (0.68) make at the node spacing, however
+    large the entries of the rows that meet."""
+    nodes = 200
+    ptr, z, centres = circles([(0, 64), (1.0, nodes), (0, nodes)], gap)
+    N = int(ptr[-1])
+    v = np.random.default_rng(5).standard_normal(N)
+    out = []
+    for matvec in (L.LBF_MATVEC_FMM, L.LBF_MATVEC_DIRECT):
+        plan = plan_of(ptr, z, centres, leaf_size=1024, p=26, fmm64=fmm64, matvec=matvec)
+        o = zeros(N)
+        L.lbf_apply(plan, L.LBF_OP_K_ONLY | L.LBF_OP_TRANSPOSE, dev(v), o)
+        assert L.lbf_sync_status(plan) == L.LBF_OK
+        out.append(host(o))
+    rest = np.ones(N, dtype=bool)
+    rest[[int(ptr[1]), int(ptr[2]) + nodes // 2]] = False
+    xi, d = (a[:, 0] + 1j * a[:, 1] for a in z[:2])
+    w = d * np.repeat(2 * np.pi / np.diff(ptr), np.diff(ptr))
+    dz = xi[:, None] - xi[None, :] + np.eye(N)
+    k = np.abs((w[:, None] / dz).imag) / np.pi * (1 - np.eye(N))
+    size = np.abs(v) + k @ np.abs(v)
+    bound = 4 * 0.68 / (2 * np.pi * 0.1 / nodes) * EPS * size
+    assert np.all(np.abs(out[0] - out[1])[rest] <= bound[rest])
