@@ -15,15 +15,18 @@
 //   * an integer is seven balanced base-256 digits, each exact in bf16; a product of two
 //     digits is at most 2^14, a sum of 64 of them over at most seven digit pairs stays below
 //     2^23: exact in the float accumulators of tcgen05.mma;
-//   * the digit pairs with s + t <= 6 (28 of 49) go into seven TMEM accumulators, one per
-//     s + t; the dropped ones are below 2^-56 of the product of the two maxima, where a
-//     double evaluation rounds each of its terms at 2^-53;
+//   * the digit pairs with s + t <= 7 (34 of 49) go into eight TMEM accumulators, one per
+//     s + t.  A dropped pair is at most 2^-62 of 2^108, all of them over 64 columns below 2^-53
+//     of the product of the two maxima, 2^-59 as digits fall.  (Without s + t = 7, up to
+//     2^-45 and 2^-51.4: measured on translations of forty charges over all offsets, in units of
+//     2^-53 of their absolute sum, 0.63, with it 0.13, as a double evaluation, which rounds each
+//     of its terms, 0.40);
 //   * the accumulators are combined as integers and packed into doubles without an
 //     instruction on the double pipe.
 //
-// Work: 28 products of 128 x N x K a tile of 128 translations (N, K = 2 P rounded up to 16).
+// Work: 34 products of 128 x N x K a tile of 128 translations (N, K = 2 P rounded up to 16).
 // The matrix's digits stand one after another along N, so digit s of the rows meets digits
-// 0 .. 6 - s of the matrix in one or two MMAs of up to 256 columns, ten a K step of 16 (one
+// 0 .. 7 - s of the matrix in one or two MMAs of up to 256 columns, twelve a K step of 16 (one
 // digit pair an MMA re-read the 4 KB of rows for every 64 columns).  k_m2l_tc is persistent,
 // one CTA an SM: eight warps expand the gathered rows' digits into shared memory (112 KB; the
 // next tile's integers are fetched before the wait for the MMAs) and one of their threads
@@ -32,7 +35,7 @@
 // target's warp in k_down then adds its translations in list order (two additions a
 // coefficient).
 //
-// Chosen for P <= 32 (K = 64: one accumulator set fills 448 of TMEM's 512 columns); longer
+// Chosen for P <= 32 (K = 64: one accumulator set fills TMEM's 512 columns); longer
 // expansions keep the double loop in k_down.
 #include <algorithm>
 
@@ -45,6 +48,7 @@ using fmm::cx;
 namespace {
 
 constexpr int kSl = 7;                  // digits of an operand
+constexpr int kAcc = 8;                 // sums of digit products, by the digits' places
 constexpr int kRowsT = 128;             // translations a tile
 constexpr int kABytes = kRowsT * 64 * 2;  // one digit of a tile's rows
 constexpr int kBBytes = 64 * 64 * 2;      // room for one digit of a translation matrix
@@ -330,16 +334,19 @@ k_m2l_tc(int P, const int32_t *__restrict__ tile0, const int2 *__restrict__ pair
                 if (load) wait(mb, nb++ & 1);
                 if (n > 0) wait(mf, (n - 1) & 1);  // the accumulators have been read
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                // digit s of the rows by digits 0 .. 6 - s of the matrix into sums s .. 6
-                for (int s = 0; s < kSl; s++)
-                    for (int c = 0; c < (kSl - s) * N; c += 256) {
-                        const int w = min(256, (kSl - s) * N - c);
-                        const uint32_t idesc = tc_idesc(kRowsT, w);
-                        for (int k = 0; k < nk; k++)
-                            tc_mma(tmem + (uint32_t)(s * N + c), dA + (uint64_t)((s * kABytes + k * 256) >> 4),
-                                   dB + (uint64_t)((c * 128 + k * 256) >> 4), idesc,
-                                   (s > 0 || k > 0) ? 1u : 0u);
-                    }
+                // digit s of the rows by digits 0 .. 7 - s of the matrix into sums s .. 7 (sum 7
+                // begins with s = 1, the others with s = 0)
+                auto mul = [&](int s, int c, int w, bool first) {
+                    const uint32_t idesc = tc_idesc(kRowsT, w);
+                    for (int k = 0; k < nk; k++)
+                        tc_mma(tmem + (uint32_t)(s * N + c), dA + (uint64_t)((s * kABytes + k * 256) >> 4),
+                               dB + (uint64_t)((c * 128 + k * 256) >> 4), idesc, !first || k > 0 ? 1u : 0u);
+                };
+                for (int s = 0; s < kSl; s++) {
+                    const int cols = (s == 0 ? kSl : s == 1 ? kSl - 1 : kAcc - s) * N;
+                    for (int c = 0; c < cols; c += 256) mul(s, c, min(256, cols - c), s == 0);
+                    if (s == 1) mul(1, cols, N, true);
+                }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                              :: "r"(mm) : "memory");
             }
@@ -363,12 +370,12 @@ k_m2l_tc(int P, const int32_t *__restrict__ tile0, const int2 *__restrict__ pair
             __syncwarp();
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             for (int c = h0; c < h0 + N / 2; c += 8) {
-                float a[kSl][8];
+                float a[kAcc][8];
 #pragma unroll
-                for (int g = 0; g < kSl; g++) tc_ld8(trow + (uint32_t)(g * N + c), a[g]);
+                for (int g = 0; g < kAcc; g++) tc_ld8(trow + (uint32_t)(g * N + c), a[g]);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                for (int g = 0; g < kSl; g++)
+                for (int g = 0; g < kAcc; g++)
 #pragma unroll
                     for (int i = 0; i < 8; i++) asm volatile("" : "+f"(a[g][i]));  // not before the wait
                 if (c + 8 >= h0 + N / 2) {
@@ -381,13 +388,14 @@ k_m2l_tc(int P, const int32_t *__restrict__ tile0, const int2 *__restrict__ pair
                     double v[8];
 #pragma unroll
                     for (int i = 0; i < 8; i++) {
-                        int d[kSl];
+                        int d[kAcc];
 #pragma unroll
-                        for (int g = 0; g < kSl; g++) d[g] = __float2int_rn(a[g][i]);
+                        for (int g = 0; g < kAcc; g++) d[g] = __float2int_rn(a[g][i]);
                         // sum_g d_g 256^(6 - g) in units of 16
                         const long long w = (long long)(d[0] * 256 + d[1]) * (1ll << 36) +
                                             (long long)(d[2] * 256 + d[3]) * (1ll << 20) +
-                                            (long long)(d[4] * 256 + d[5]) * 16ll + ((d[6] + 8) >> 4);
+                                            (long long)(d[4] * 256 + d[5]) * 16ll +
+                                            ((d[6] + ((d[7] + 128) >> 8) + 8) >> 4);
                         v[i] = pack_double(w, e + f[c + i] - 56);
                     }
                     if (e == kBadExp)  // an infinity or NaN in the multipole
