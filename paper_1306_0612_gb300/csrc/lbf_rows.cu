@@ -70,9 +70,8 @@ constexpr int kGroups = 8, kGroupsSmall = 2;
 // (8192 nodes: 458 us an application with whole leaves a warp, 408 shared; at 7130 leaves
 // the two are within 1 %, at 16,150 sharing costs 4 % of a solve)
 constexpr int64_t kSmallLeaves = 4864;
-// (several right-hand sides in lockstep take the quarters in turn once their blocks make this
-// many warps an SM, four times what is resident: 16 of 10,000 nodes 135 us, shared 150)
-constexpr int64_t kFullWarps = 64;
+// (several right-hand sides in lockstep share columns too, so that their sums are those of a
+// separate solve: 16 of 10,000 nodes 134 us, 157 with the quarters taken in turn by one warp)
 constexpr int kLocalTop = 1021;  // exponent field of the local columns' largest: [1/4, 1/2)
 constexpr int kRowBlocks = 4;    // thread blocks an SM
 constexpr int kRun = 4;          // chunks read at a time (2 or 4)
@@ -506,11 +505,9 @@ __device__ __forceinline__ double block_rows(const RowItem &it, const double *__
     return s;
 }
 
-// v of a block's rows: a warp per block (kWhole), or, blocks of kGroupsSmall groups, the sums of
-// the four quarters of its columns added in order: by the four warps of a thread block, a
-// quarter each (kWarps), or one after another by one warp (kTurns), the same sums bit for bit.
-enum Share { kWhole, kWarps, kTurns };
-template <typename R, Share SHARE>
+// v of a block's rows: a warp per block, or (SPLIT, blocks of kGroupsSmall groups) the four
+// warps of a thread block, each over a quarter of the columns, the quarters added in order.
+template <typename R, bool SPLIT>
 __global__ void __launch_bounds__(128, kRowBlocks)
 k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__restrict__ rows,
              const int32_t *__restrict__ rexp, const int32_t *__restrict__ cols,
@@ -520,31 +517,23 @@ k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__r
 {
     lbf_rhs(slab, sigma, loc, mp, bsig, v, gate);
     if (fmm::gate_closed(gate)) return;
-    constexpr int G = SHARE == kWhole ? kGroups : kGroupsSmall;
     __shared__ double part[4][32];
     __shared__ int2 xs[4][8 * kDotChunks];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t k = SHARE == kWarps ? (int64_t)blockIdx.x : blockIdx.x * (int64_t)(blockDim.x >> 5) + wid;
+    const int64_t k = SPLIT ? (int64_t)blockIdx.x : blockIdx.x * (int64_t)(blockDim.x >> 5) + wid;
     if (k >= nitem) return;
     const int4 i0 = ((const int4 *)items)[2 * k], i1 = ((const int4 *)items)[2 * k + 1];
     const RowItem it{i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
     const int nk = it.nchunk + lchunks;
+    const int k0 = SPLIT ? nk * wid / 4 : 0, k1 = SPLIT ? nk * (wid + 1) / 4 : nk;
     int row;
-    auto sum = [&](int k0, int k1) {
-        return block_rows<G>(it, rows, rexp, cols, sigma, loc, mp, P, k0, k1, xs[wid], lane, row);
-    };
-    double s;
-    if (SHARE == kWarps) {
-        part[wid][lane] = sum(nk * wid / 4, nk * (wid + 1) / 4);
+    double s = block_rows<SPLIT ? kGroupsSmall : kGroups>(it, rows, rexp, cols, sigma, loc, mp, P, k0, k1,
+                                                          xs[wid], lane, row);
+    if (SPLIT) {
+        part[wid][lane] = s;
         __syncthreads();
         if (wid != 0) return;
         s = part[0][lane] + part[1][lane] + part[2][lane] + part[3][lane];
-    } else if (SHARE == kTurns) {
-        s = sum(0, nk / 4);
-#pragma unroll 1
-        for (int w = 1; w < 4; w++) s += sum(nk * w / 4, nk * (w + 1) / 4);
-    } else {
-        s = sum(0, nk);
     }
     if (row < it.nrow) v[it.row0 + row] = s + 2.0 * *bsig;
 }
@@ -908,25 +897,16 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
                    bool df)
 {
     const int64_t n = pl->rows_nitem;
-    // several right-hand sides fill the chip without sharing a block's columns over warps (a
-    // separate solve's sums all the same)
-    const bool full = pl->nrhs > 1 && n * pl->nrhs >= kFullWarps * (int64_t)std::max(pl->nsm, 1);
-    const Share share = !pl->rows_split ? kWhole : full ? kTurns : kWarps;
-    const dim3 grid = lbf_grid(pl, share == kWarps ? n : lbf_cdiv(n, 4));
-#define LBF_ROWS(R, SHARE)                                                                         \
-    LBF_LAUNCH_P(LBF_KERNEL_LEAF, (k_rows_apply<R, SHARE>), grid, 128, 0, s, n, pl->rows_items, pl->rows, \
+    const bool split = pl->rows_split != 0;
+    const dim3 grid = lbf_grid(pl, split ? n : lbf_cdiv(n, 4));
+#define LBF_ROWS(R, SPLIT)                                                                         \
+    LBF_LAUNCH_P(LBF_KERNEL_LEAF, (k_rows_apply<R, SPLIT>), grid, 128, 0, s, n, pl->rows_items, pl->rows, \
                  pl->rows_e, pl->rows_cols, sigma, (const cx<R> *)pl->local,                       \
                  (const cx<R> *)pl->mpole, pl->P, local_chunks(pl->P), pl->bsig, v, gate, pl->slab)
-#define LBF_ROWS_OF(R)                        \
-    if (share == kWarps) LBF_ROWS(R, kWarps); \
-    else if (share == kTurns) LBF_ROWS(R, kTurns); \
-    else LBF_ROWS(R, kWhole)
-    if (df) {
-        LBF_ROWS_OF(df64);
-    } else {
-        LBF_ROWS_OF(double);
-    }
-#undef LBF_ROWS_OF
+    if (df && split) LBF_ROWS(df64, true);
+    else if (df) LBF_ROWS(df64, false);
+    else if (split) LBF_ROWS(double, true);
+    else LBF_ROWS(double, false);
 #undef LBF_ROWS
     LBF_CHECK_LAUNCH();
     return LBF_OK;
