@@ -416,6 +416,31 @@ __device__ __forceinline__ void dot_chunks(const double *__restrict__ t, const i
     }
 }
 
+// The sum of a lane's row over n chunks of double entries whose columns are nodes.  Not inlined:
+// few blocks have any, and beside the integer loops its sums cost them registers (rows of 407
+// ragged islands 143 us inlined, 133 so; the multipoles' loop, which many blocks enter, 152
+// and 133 the other way round).
+template <int G>
+__device__ __noinline__ double wide_rows(const double *__restrict__ t, const int32_t *__restrict__ cl,
+                                         int ncol, int n, int ng, const double *__restrict__ sigma, int lane)
+{
+    double d[G];
+#pragma unroll
+    for (int q = 0; q < G; q++) d[q] = 0.0;
+    for (int k = 0; k < n; k++, t += 32 * ng) {
+        const int m = 8 * k + (lane & 7);
+        const double x = m < ncol ? sigma[cl[m]] : 0.0;
+#pragma unroll
+        for (int q = 0; q < G; q++)
+            if (q < ng) d[q] = fma(t[32 * q], x, d[q]);
+    }
+    fold_rows<G>(lane, [&](int a, int b, bool up, int bit) {
+        const double keep = up ? d[b] : d[a], send = up ? d[a] : d[b];
+        d[a] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+    });
+    return d[0];
+}
+
 // The sum of one row of a block of at most G row groups over its column chunks k0 .. k1 - 1
 // (near chunks, multipole chunks, then the local expansion's), and that row.  The columns'
 // values of a run of chunks are made integers first, a column a lane, and left in xs.
@@ -433,21 +458,26 @@ __device__ __forceinline__ double block_rows(const RowItem &it, const double *__
     const int32_t *cl = cols + (int64_t)it.chunk * 8;
     const int64_t lb = (int64_t)it.box * 2 * P;
     const int nn = (it.ncol + 7) / 8;
-    const bool wide = it.leaf < 0;
     const int grp = fold_rows<G>(lane, [](int, int, bool, int) {});
     row = grp < ng ? 4 * grp + (lane >> 3) : it.nrow;
     prefetch_tiles(t - lane, ng * min(k1 - k0, kAhead), lane);
     double s = 0.0;
     int k = k0;
+    if (it.leaf < 0 && k < min(k1, nn)) {  // near entries kept as doubles
+        const int ke = min(k1, nn);
+        s = wide_rows<G>(t, cl + 8 * k, it.ncol - 8 * k, ke - k, ng, sigma, lane);
+        t += (int64_t)32 * ng * (ke - k);
+        k = ke;
+    }
     while (k < k1) {
-        if (k < it.nchunk && (wide || k >= nn)) {
-            // multipoles of W boxes: few, and in units of their own; near entries kept as doubles
+        if (k < it.nchunk && k >= nn) {
+            // multipoles of W boxes: few, and in units of their own
             double d[G];
 #pragma unroll
             for (int q = 0; q < G; q++) d[q] = 0.0;
             for (const int ke = min(k1, it.nchunk); k < ke; k++, t += 32 * ng) {
-                const int m = 8 * k + (lane & 7), j = cl[m];
-                const double x = m < it.ncol ? sigma[j] : j < 0 ? local_real(mp, -1 - j) : 0.0;
+                const int j = cl[8 * k + (lane & 7)];
+                const double x = j < 0 ? local_real(mp, -1 - j) : 0.0;
 #pragma unroll
                 for (int q = 0; q < G; q++)
                     if (q < ng) d[q] = fma(t[32 * q], x, d[q]);
