@@ -140,12 +140,29 @@ const char *lbf_status_string(int status);
 /* Bytes of device workspace a plan over these islands needs (synchronous, host
  * only).  The quadtree part is an estimate from N and leaf_size unless
  * opt->box_capacity is set; lbf_plan_create reports the exact need if the
- * estimate was short.  The last part holds the accurate forward operator's leaf
- * rows (near field and local evaluation, 8 bytes an entry, up to 64 GB): a plan
- * given a workspace without it, or whose tree needs more, forms them on the fly
- * in every application. */
+ * estimate was short.  Its last parts, LBF_PART_* in this order, hold what of the
+ * accurate operator depends on the geometry alone: a plan given a workspace
+ * without one of them, or whose tree needs more, forms that part on the fly in
+ * every application (as accurate, slower). */
 int lbf_workspace_size(int M, const int64_t *island_ptr /* host, M+1 */, const lbf_options *opt,
                        size_t *bytes /* host out */);
+
+#define LBF_PART_M2L 1    /* the translations' lists and matrices for the tensor cores */
+#define LBF_PART_E 2      /* the multiplier block E (up to 512 islands and 1e8 entries) */
+#define LBF_PART_PAIRS 4  /* else the multiplier potential's (box, centre) expansions */
+#define LBF_PART_ROWS 8   /* the leaf rows (near field and local evaluation, 8 bytes an entry,
+                             up to 64 GB; about 2 KB a node) */
+
+/* The sizes between which a caller short of memory can choose (host call, no GPU work):
+ * sizes[0] is lbf_workspace_size's (nrhs < 2) or lbf_batch_workspace_size's (nrhs >= 2),
+ * each of the next is without one part more, the last first (rows, pairs, E, M2L; equal
+ * where a plan has no such part), and the last size is what a plan cannot do without. */
+#define LBF_WORKSPACE_SIZES 5
+int lbf_workspace_sizes(int M, const int64_t *island_ptr, const lbf_options *opt, int nrhs,
+                        size_t sizes[LBF_WORKSPACE_SIZES] /* host out */);
+
+/* The LBF_PART_* that a plan holds, ORed (host out). */
+int lbf_plan_parts(const lbf_plan *plan, int *parts);
 
 /* Build a plan: project the nodes to the plane (Sec. 3), precompute the
  * trapezoidal weights w_j = h xi'_j, the self terms and the rank-one sphere
@@ -314,11 +331,22 @@ typedef struct lbf_batch_item {
     int64_t box_capacity_needed;            /* see lbf_plan_create */
 } lbf_batch_item;
 int lbf_batch_run(int nitems, lbf_batch_item *items, const lbf_options *opt, int nworkers);
+/* The same run in one workspace for all items: each worker has a slice of it, an item runs in
+ * its worker's (item.bytes: the slice it wants; item.workspace is set by the call).  Results
+ * are those of lbf_batch_run with workspaces of item.bytes.  lbf_batch_shared_size: the bytes
+ * it takes for these items and workers (nworkers slices at most, whatever the number of items;
+ * host call, no GPU work).  LBF_EWORKSPACE when bytes is less. */
+int lbf_batch_shared_size(int nitems, const lbf_batch_item *items, int nworkers, size_t *bytes);
+int lbf_batch_run_shared(int nitems, lbf_batch_item *items, const lbf_options *opt, int nworkers,
+                         void *workspace, size_t bytes);
 /* Workspace of one batch item whose right-hand sides are solved in lockstep
  * (lbf_gmres_solve_many) by lbf_batch_run: the plan's bytes (lbf_workspace_size),
  * rounded up to 256, then lbf_gmres_workspace_many's for nrhs right-hand sides (none
  * where those are solved one after another).  An item whose workspace holds less
- * solves its right-hand sides one after another.  Host call, no GPU work. */
+ * takes the largest of lbf_workspace_sizes that fits, in lockstep with fewer stored
+ * parts; it solves its right-hand sides one after another below the last of them and
+ * in a workspace of a plan's own size (nrhs < 2, up to 64 KB more).  Host call, no GPU
+ * work. */
 int lbf_batch_workspace_size(int M, const int64_t *island_ptr, const lbf_options *opt, int nrhs,
                              size_t *bytes /* host out */);
 
@@ -334,7 +362,9 @@ int lbf_batch_workspace_size(int M, const int64_t *island_ptr, const lbf_options
  *   geometry and pole_rotation: as lbf_plan_create (device arrays; rotation host/NULL)
  *   base: options to start from (precision, fmm64, ...: kept in *best)
  *   target: the largest acceptable rel-l2 error of the operator
- *   workspace, bytes: device memory; with workspace = NULL only *bytes_needed is set
+ *   workspace, bytes: device memory; with workspace = NULL only *bytes_needed is set.
+ *   *bytes_needed is the size with every stored part (lbf_workspace_sizes) of every
+ *   trial; down to the size without any is accepted, the trials then storing what fits
  *   best: host out, base with p, leaf_size and p2p_warps chosen
  *   table, table_len: host out (nullable), every trial as JSON text
  * Synchronous.  LBF_NOCONV (soft) when no trial met the target (best = base). */

@@ -143,9 +143,9 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
         pl->upcnt = A.get<int32_t>(cap);
         pl->pull = A.get<uint32_t>(2 * cap + 4);
         pl->lx_pitch = 2 * std::min(32, o.border ? 32 : P);
-        pl->loc_X = A.get<long long>(cap * pl->lx_pitch);
-        pl->loc_e = A.get<int32_t>(cap + LBF_PASS_WORDS);
     }
+    pl->xcap = o.box_capacity > 0 ? cap : std::min<int64_t>(cap, 8 * N / std::max(1, o.leaf_size) + 1024);
+    pl->use_loc = false;
     if (o.matvec == LBF_MATVEC_FMM && o.fmm64) {
         pl->qdf = A.get<double2>(N);   // cx<df64>: 16 B per node
         pl->udf = A.get<double2>(N);
@@ -277,6 +277,12 @@ void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o, int64_t ca
     lbf_rows_layout(pl, N, o, cap);
 }
 
+void lbf_loc_layout(const lbf_plan *pl, lbf_plan *v, Arena &A)
+{
+    v->loc_X = A.get<long long>(pl->xcap * pl->lx_pitch);
+    v->loc_e = A.get<int32_t>(pl->xcap + LBF_PASS_WORDS);
+}
+
 // The buffers one right-hand side's solve writes, in the sizes lbf_layout gives them
 // (which of them exist follows the options, as there), carved from A for a plan view of
 // lbf_gmres_solve_many: each right-hand side has its own copy, while the geometry, the
@@ -296,8 +302,7 @@ static void layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A)
     v->local = fmm ? A.get<double2>(cap * P) : nullptr;
     v->upcnt = fmm || o.border ? A.get<int32_t>(cap) : nullptr;
     v->pull = fmm || o.border ? A.get<uint32_t>(2 * cap + 4) : nullptr;
-    v->loc_X = fmm || o.border ? A.get<long long>(cap * pl->lx_pitch) : nullptr;
-    v->loc_e = fmm || o.border ? A.get<int32_t>(cap + LBF_PASS_WORDS) : nullptr;
+    if (pl->use_loc) lbf_loc_layout(pl, v, A);
     v->qdf = fmm && o.fmm64 ? (void *)A.get<double2>(N) : nullptr;
     v->q32 = f32 ? A.get<float2>(N) : nullptr;
     v->mpole32 = f32 && fmm ? A.get<float2>(cap * (o.p32 + 1)) : nullptr;
@@ -478,45 +483,63 @@ static int check_islands(int M, const int64_t *ptr, int64_t *N)
     return LBF_OK;
 }
 
-int lbf_workspace_size(int M, const int64_t *island_ptr, const lbf_options *opt, size_t *bytes)
+}  // extern "C"
+
+int lbf_rung_size(int M, const int64_t *island_ptr, const lbf_options &opt, int nrhs, int rung,
+                  size_t *plan_bytes, size_t *item_bytes)
 {
-    if (!opt || !bytes || !valid(*opt)) return LBF_EINVAL;
+    static const unsigned parts[LBF_WORKSPACE_SIZES] = {
+        LBF_PART_M2L | LBF_PART_E | LBF_PART_PAIRS | LBF_PART_ROWS,
+        LBF_PART_M2L | LBF_PART_E | LBF_PART_PAIRS, LBF_PART_M2L | LBF_PART_E, LBF_PART_M2L, 0};
     int64_t N;
     int rc = check_islands(M, island_ptr, &N);
     if (rc) return rc;
     lbf_plan tmp;
+    tmp.N = N;
+    tmp.M = M;
+    tmp.n = N + M;
+    tmp.opt = opt;
+    tmp.P = opt.p + 1;
+    tmp.parts = parts[rung];
     tmp.arena.base = nullptr;
     tmp.arena.cap = ~size_t(0);
-    lbf_layout(&tmp, N, M, *opt, box_capacity_estimate(N, *opt));
-    *bytes = tmp.arena.off + 256;
+    lbf_layout(&tmp, N, M, opt, box_capacity_estimate(N, opt));
+    *plan_bytes = *item_bytes = tmp.arena.off + 256;
+    const bool lu = opt.schur == LBF_SCHUR_LU || (opt.schur == LBF_SCHUR_AUTO && M > 1024);
+    if (nrhs < 2 || !opt.border || lu) return LBF_OK;
+    size_t need = 0;
+    if ((rc = lbf_many_view(&tmp, std::min(nrhs, LBF_LOCKSTEP_MAX), nullptr, 0, nullptr, &need))) return rc;
+    *item_bytes = ((*plan_bytes + 255) & ~size_t(255)) + need;
+    return LBF_OK;
+}
+
+extern "C" {
+
+int lbf_workspace_size(int M, const int64_t *island_ptr, const lbf_options *opt, size_t *bytes)
+{
+    if (!opt || !bytes || !valid(*opt)) return LBF_EINVAL;
+    size_t item = 0;
+    return lbf_rung_size(M, island_ptr, *opt, 0, 0, bytes, &item);
+}
+
+int lbf_workspace_sizes(int M, const int64_t *island_ptr, const lbf_options *opt, int nrhs,
+                        size_t sizes[LBF_WORKSPACE_SIZES])
+{
+    if (nrhs < 0 || !opt || !sizes || !valid(*opt)) return LBF_EINVAL;
+    for (int r = 0; r < LBF_WORKSPACE_SIZES; r++) {
+        size_t pb = 0;
+        const int rc = lbf_rung_size(M, island_ptr, *opt, nrhs, r, &pb, &sizes[r]);
+        if (rc) return rc;
+    }
     return LBF_OK;
 }
 
 int lbf_batch_workspace_size(int M, const int64_t *island_ptr, const lbf_options *opt, int nrhs,
                              size_t *bytes)
 {
-    if (nrhs < 0 || !bytes) return LBF_EINVAL;
+    if (nrhs < 0 || !bytes || !opt || !valid(*opt)) return LBF_EINVAL;
     size_t pb = 0;
-    int rc = lbf_workspace_size(M, island_ptr, opt, &pb);
-    if (rc) return rc;
-    *bytes = pb;
-    const bool lu = opt->schur == LBF_SCHUR_LU || (opt->schur == LBF_SCHUR_AUTO && M > 1024);
-    if (nrhs < 2 || !opt->border || lu) return LBF_OK;
-    const int64_t N = island_ptr[M];
-    lbf_plan tmp;
-    tmp.N = N;
-    tmp.M = M;
-    tmp.n = N + M;
-    tmp.opt = *opt;
-    tmp.P = opt->p + 1;
-    tmp.arena.base = nullptr;
-    tmp.arena.cap = ~size_t(0);
-    lbf_layout(&tmp, N, M, *opt, box_capacity_estimate(N, *opt));
-    size_t need = 0;
-    if ((rc = lbf_many_view(&tmp, std::min(nrhs, LBF_LOCKSTEP_MAX), nullptr, 0, nullptr, &need)))
-        return rc;
-    *bytes = ((pb + 255) & ~size_t(255)) + need;
-    return LBF_OK;
+    return lbf_rung_size(M, island_ptr, *opt, nrhs, 0, &pb, bytes);
 }
 
 static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const double *x,
@@ -622,12 +645,12 @@ static int plan_create(lbf_plan **plan, int M, const int64_t *island_ptr, const 
     if (pl->dcount) CK(cudaMemsetAsync(pl->dcount, 0, sizeof(unsigned) * lbf_cdiv(N, 32), s));
     if (pl->upcnt) CK(cudaMemsetAsync(pl->upcnt, 0, sizeof(int32_t) * cap, s));
     if (pl->loc_X) {  // no word carries the first application's tag
-        CK(cudaMemsetAsync(pl->loc_X, 0, sizeof(long long) * cap * pl->lx_pitch, s));
-        CK(cudaMemsetAsync(pl->loc_e, 0, sizeof(int32_t) * (cap + LBF_PASS_WORDS), s));
+        CK(cudaMemsetAsync(pl->loc_X, 0, sizeof(long long) * pl->xcap * pl->lx_pitch, s));
+        CK(cudaMemsetAsync(pl->loc_e, 0, sizeof(int32_t) * (pl->xcap + LBF_PASS_WORDS), s));
     }
     if (pl->m2l_cap) {
-        CK(cudaMemsetAsync(pl->m2l_X, 0, sizeof(long long) * cap * ((2 * pl->P + 7) / 8 * 8), s));
-        CK(cudaMemsetAsync(pl->m2l_e, 0, sizeof(int32_t) * cap, s));
+        CK(cudaMemsetAsync(pl->m2l_X, 0, sizeof(long long) * pl->xcap * ((2 * pl->P + 7) / 8 * 8), s));
+        CK(cudaMemsetAsync(pl->m2l_e, 0, sizeof(int32_t) * pl->xcap, s));
     }
     if (pl->pull) CK(cudaMemsetAsync(pl->pull, 0, sizeof(uint32_t) * (2 * cap + 4), s));
     CK(cudaMemcpyAsync(pl->tab_tpow, tpow.data(), sizeof(double2) * tpow.size(), cudaMemcpyHostToDevice, s));
@@ -715,6 +738,14 @@ int lbf_plan_destroy(lbf_plan *pl)
     if (pl->host_scalars) cudaFreeHost(pl->host_scalars);
     delete[] pl->island_ptr_h;
     delete pl;
+    return LBF_OK;
+}
+
+int lbf_plan_parts(const lbf_plan *pl, int *parts)
+{
+    if (!pl || !parts) return LBF_EINVAL;
+    *parts = (pl->m2l_cap ? LBF_PART_M2L : 0) | (pl->bd.E ? LBF_PART_E : 0) |
+             (pl->bd.p2l_exp ? LBF_PART_PAIRS : 0) | (pl->rows ? LBF_PART_ROWS : 0);
     return LBF_OK;
 }
 

@@ -12,27 +12,43 @@
 
 namespace {
 
+constexpr size_t kRoundUp = 65536;  // what a caller may round a workspace's size up by
+
 int run_item(lbf_batch_item &it, const lbf_options &opt_all, cudaStream_t s)
 {
     lbf_plan *pl = nullptr;
     int64_t need = 0;
     lbf_options opt = opt_all;
     opt.box_capacity = it.box_capacity;
+    // the right-hand sides in lockstep when the item's workspace holds their buffers after the
+    // plan's: with as many stored parts as leave room for them (lbf_workspace_sizes); one after
+    // another in a workspace of a plan's own size, whole
+    size_t pbytes = it.bytes;
+    bool lock = false, plans = false;
+    for (int r = 0; r < LBF_WORKSPACE_SIZES && it.nrhs > 1; r++) {
+        size_t pb = 0, ib = 0;
+        if (lbf_rung_size(it.M, it.island_ptr, opt, it.nrhs, r, &pb, &ib) != LBF_OK || ib == pb) break;
+        plans = plans || (it.bytes >= pb && it.bytes < pb + kRoundUp);
+        if (!lock && ib <= it.bytes) {
+            lock = true;
+            pbytes = (pb + 255) & ~size_t(255);
+        }
+    }
+    if (plans) {
+        lock = false;
+        pbytes = it.bytes;
+    }
     int rc = lbf_plan_create(&pl, it.M, it.island_ptr, it.x, it.dx, it.d2x, it.centres, nullptr,
-                             &opt, it.workspace, it.bytes, &need, (lbf_stream_t)s);
+                             &opt, it.workspace, pbytes, &need, (lbf_stream_t)s);
     if (rc) {
         it.box_capacity_needed = need;
         return rc;
     }
     const int64_t N = pl->N;
     int worst = LBF_OK;
-    // the right-hand sides in lockstep when the item's workspace holds their buffers
-    // after the plan's (lbf_batch_workspace_size)
-    size_t pbytes = 0, mbytes = 0;
-    const bool sized = lbf_workspace_size(it.M, it.island_ptr, &opt, &pbytes) == LBF_OK;
-    pbytes = (pbytes + 255) & ~size_t(255);
-    const bool lock = sized && it.nrhs > 1 && lbf_gmres_workspace_many(pl, it.nrhs, &mbytes) == LBF_OK &&
-                      mbytes > 0 && it.bytes >= pbytes + mbytes;
+    size_t mbytes = 0;
+    lock = lock && lbf_gmres_workspace_many(pl, it.nrhs, &mbytes) == LBF_OK && mbytes > 0 &&
+           it.bytes >= pbytes + mbytes;
     if (lock) {
         std::vector<int> its(it.nrhs, 0);
         std::vector<double> rr(it.nrhs, 0.0);
@@ -86,24 +102,9 @@ int run_item(lbf_batch_item &it, const lbf_options &opt_all, cudaStream_t s)
     return worst;
 }
 
-}  // namespace
-
-extern "C" int lbf_batch_run(int nitems, lbf_batch_item *items, const lbf_options *opt,
-                             int nworkers)
+// largest first: nodes times right-hand sides
+std::vector<int> order_of(int nitems, const lbf_batch_item *items)
 {
-    if (nitems < 0 || (nitems > 0 && !items) || !opt || nworkers < 1) return LBF_EINVAL;
-    for (int q = 0; q < nitems; q++) {
-        lbf_batch_item &it = items[q];
-        if (it.nrhs < 0 || it.M < 1 || !it.island_ptr || !it.workspace || (it.nrhs > 0 && (!it.g || !it.sigma)) ||
-            it.T < 0 || (it.T > 0 && it.u && !it.targets))
-            return LBF_EINVAL;
-        it.status = LBF_OK;
-        it.iters = 0;
-        it.fp64_applies = it.fp32_applies = 0;
-        it.max_rel_res = 0.0;
-        it.box_capacity_needed = 0;
-    }
-    // largest first: sum of nodes times right-hand sides
     std::vector<int> order(nitems);
     for (int q = 0; q < nitems; q++) order[q] = q;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
@@ -111,11 +112,54 @@ extern "C" int lbf_batch_run(int nitems, lbf_batch_item *items, const lbf_option
         const int64_t wy = items[y].island_ptr[items[y].M] * std::max(items[y].nrhs, 1);
         return wx > wy;
     });
+    return order;
+}
+
+// Offsets of the workers' slices of a shared workspace, and its end: worker w begins with the
+// w-th item of the order and later takes some behind the nw-th
+std::vector<size_t> slices_of(const std::vector<int> &order, const lbf_batch_item *items, int nw)
+{
+    size_t later = 0;
+    for (size_t k = nw; k < order.size(); k++) later = std::max(later, items[order[k]].bytes);
+    std::vector<size_t> at(nw + 1, 0);
+    for (int w = 0; w < nw; w++) {
+        const size_t first = (size_t)w < order.size() ? items[order[w]].bytes : 0;
+        at[w + 1] = at[w] + ((std::max(first, later) + 255) & ~size_t(255));
+    }
+    return at;
+}
+
+int workers_of(int nitems, int nworkers) { return std::max(1, std::min(nworkers, std::max(nitems, 1))); }
+
+bool valid_items(int nitems, const lbf_batch_item *items, bool shared)
+{
+    for (int q = 0; q < nitems; q++) {
+        const lbf_batch_item &it = items[q];
+        if (it.nrhs < 0 || it.M < 1 || !it.island_ptr || (!shared && !it.workspace) ||
+            (it.nrhs > 0 && (!it.g || !it.sigma)) || it.T < 0 || (it.T > 0 && it.u && !it.targets))
+            return false;
+    }
+    return true;
+}
+
+// pool: the shared workspace, or null (every item has its own)
+int run(int nitems, lbf_batch_item *items, const lbf_options *opt, int nworkers, char *pool,
+        const std::vector<int> &order, const std::vector<size_t> &slice)
+{
+    for (int q = 0; q < nitems; q++) {
+        lbf_batch_item &it = items[q];
+        it.status = LBF_OK;
+        it.iters = 0;
+        it.fp64_applies = it.fp32_applies = 0;
+        it.max_rel_res = 0.0;
+        it.box_capacity_needed = 0;
+    }
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return LBF_ECUDA;
-    std::atomic<int> next{0};
+    const int nw = workers_of(nitems, nworkers);
+    std::atomic<int> next{nw};  // worker w begins with item w
     std::atomic<int> fail{0};
-    auto worker = [&]() {
+    auto worker = [&](int w) {
         if (cudaSetDevice(dev) != cudaSuccess) {
             fail.store(1);
             return;
@@ -125,19 +169,47 @@ extern "C" int lbf_batch_run(int nitems, lbf_batch_item *items, const lbf_option
             fail.store(1);
             return;
         }
-        for (;;) {
-            int k = next.fetch_add(1);
-            if (k >= nitems) break;
+        for (int k = w; k < nitems; k = next.fetch_add(1)) {
             lbf_batch_item &it = items[order[k]];
+            if (pool) it.workspace = pool + slice[w];
             it.status = run_item(it, *opt, s);
         }
         cudaStreamSynchronize(s);
         cudaStreamDestroy(s);
     };
-    const int nw = std::max(1, std::min(nworkers, std::max(nitems, 1)));
-    std::vector<std::thread> pool;
-    pool.reserve(nw);
-    for (int w = 0; w < nw; w++) pool.emplace_back(worker);
-    for (auto &t : pool) t.join();
+    std::vector<std::thread> threads;
+    threads.reserve(nw);
+    for (int w = 0; w < nw; w++) threads.emplace_back(worker, w);
+    for (auto &t : threads) t.join();
     return fail.load() ? LBF_ECUDA : LBF_OK;
+}
+
+}  // namespace
+
+extern "C" int lbf_batch_run(int nitems, lbf_batch_item *items, const lbf_options *opt,
+                             int nworkers)
+{
+    if (nitems < 0 || (nitems > 0 && !items) || !opt || nworkers < 1) return LBF_EINVAL;
+    if (!valid_items(nitems, items, false)) return LBF_EINVAL;
+    return run(nitems, items, opt, nworkers, nullptr, order_of(nitems, items), {});
+}
+
+extern "C" int lbf_batch_shared_size(int nitems, const lbf_batch_item *items, int nworkers, size_t *bytes)
+{
+    if (nitems < 0 || (nitems > 0 && !items) || nworkers < 1 || !bytes) return LBF_EINVAL;
+    if (!valid_items(nitems, items, true)) return LBF_EINVAL;
+    *bytes = slices_of(order_of(nitems, items), items, workers_of(nitems, nworkers)).back() + 256;
+    return LBF_OK;
+}
+
+extern "C" int lbf_batch_run_shared(int nitems, lbf_batch_item *items, const lbf_options *opt,
+                                    int nworkers, void *workspace, size_t bytes)
+{
+    if (nitems < 0 || (nitems > 0 && !items) || !opt || nworkers < 1 || !workspace) return LBF_EINVAL;
+    if (!valid_items(nitems, items, true)) return LBF_EINVAL;
+    const std::vector<int> order = order_of(nitems, items);
+    const std::vector<size_t> slice = slices_of(order, items, workers_of(nitems, nworkers));
+    char *base = (char *)(((uintptr_t)workspace + 255) & ~(uintptr_t)255);
+    if ((size_t)(base - (char *)workspace) + slice.back() > bytes) return LBF_EWORKSPACE;
+    return run(nitems, items, opt, nworkers, base, order, slice);
 }

@@ -1144,7 +1144,7 @@ int lbf_mp_build(lbf_plan *pl, cudaStream_t s, int32_t *work, int64_t work_len, 
         B.npartial = np;
         if (B.npartial > B.partial_cap) return LBF_EWORKSPACE;
     }
-    if (n_p2l > B.p2l_exp_cap) B.p2l_exp = nullptr;
+    if (n_p2l > B.p2l_exp_cap || T.nbox > pl->xcap) B.p2l_exp = nullptr;
     if (B.p2l_exp && n_p2l > 0) {
         LBF_LAUNCH(k_mp_pair_exp, lbf_cdiv(n_p2l, 128), 128, 0, s, n_p2l, T.nbox, B.Pe, B.p2l_ptr, B.p2l_src,
                    T.level, T.ix, T.iy, g, B.xc, (cz<double> *)B.p2l_exp);
@@ -1160,10 +1160,12 @@ void lbf_mp_layout_pairs(lbf_plan *pl, int M)
     Border &B = pl->bd;
     B.p2l_exp = nullptr;
     B.p2l_exp_cap = 0;
-    if (B.use_E) return;  // E y needs no expansions
+    if (B.use_E || !(pl->parts & LBF_PART_PAIRS)) return;  // (with E, E y needs no expansions)
     Arena &A = pl->arena;
     const size_t off = A.off;
     const bool full = A.overflow;
+    lbf_loc_layout(pl, pl, A);
+    pl->use_loc = true;
     B.p2l_exp_cap = std::min<int64_t>(400 * (int64_t)M, B.pair_cap);
     B.p2l_exp = A.get<double2>(B.p2l_exp_cap * B.Pe);
     if (A.overflow && !full) {
@@ -1171,6 +1173,9 @@ void lbf_mp_layout_pairs(lbf_plan *pl, int M)
         A.overflow = false;
         B.p2l_exp_cap = 0;
         B.p2l_exp = nullptr;
+        pl->use_loc = false;
+        pl->loc_X = nullptr;
+        pl->loc_e = nullptr;
     }
 }
 

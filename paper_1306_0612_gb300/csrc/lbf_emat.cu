@@ -162,7 +162,7 @@ void lbf_emat_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &o)
     B.E = nullptr;
     B.use_E = false;
     B.nch = (M + 7) / 8;
-    if (!o.border || M > kEmatIslands || N * (int64_t)M > kEmatEntries) return;
+    if (!o.border || M > kEmatIslands || N * (int64_t)M > kEmatEntries || !(pl->parts & LBF_PART_E)) return;
     Arena &A = pl->arena;
     const size_t off = A.off;
     const bool full = A.overflow;

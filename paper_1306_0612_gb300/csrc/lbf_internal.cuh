@@ -137,6 +137,7 @@ struct lbf_plan {
     lbf_options opt{};
     int P = 0;      // expansion terms p + 1
     Arena arena;
+    unsigned parts = ~0u;  // LBF_PART_* that the layout may hold
     int64_t *island_ptr_h = nullptr;  // host copy
     int64_t *island_ptr = nullptr;    // device copy
     // per node, sorted (Morton) order
@@ -191,11 +192,15 @@ struct lbf_plan {
     int32_t *m2l_vptr = nullptr, *m2l_tile0 = nullptr, *m2l_f = nullptr, *m2l_e = nullptr;
     uint4 *m2l_img = nullptr;
     long long *m2l_X = nullptr;
-    // integer local expansions (lbf_passes.cu): lx_pitch reals a box, exponents, and after
-    // them the passes' words (kPassWords)
+    // integer local expansions (lbf_passes.cu; use_loc: whether the layout holds them): lx_pitch
+    // reals a box, exponents, and after them the passes' words (LBF_PASS_WORDS)
     long long *loc_X = nullptr;
     int32_t *loc_e = nullptr;
     int lx_pitch = 0;
+    bool use_loc = false;
+    // boxes that the integer expansions have room for: half as many again as the trees met have,
+    // where the tree's own arrays reserve for the deepest
+    int64_t xcap = 0;
     double *m2l_out = nullptr;
     // stored leaf rows of the accurate forward operator (lbf_rows.cu; rows null: not stored)
     // direct sums: partial sums of the runs of sources, finished runs per 32 nodes
@@ -295,6 +300,12 @@ void lbf_inject_barrier(unsigned *count, cudaStream_t s);
 
 // ---- layout ------------------------------------------------------------------
 void lbf_layout(lbf_plan *pl, int64_t N, int M, const lbf_options &opt, int64_t box_cap);
+// the integer local expansions (a plan's, or a view's)
+void lbf_loc_layout(const lbf_plan *pl, lbf_plan *v, Arena &A);
+// bytes of a plan, and of a batch item with nrhs right-hand sides in lockstep, of
+// lbf_workspace_sizes' entry `rung`
+int lbf_rung_size(int M, const int64_t *island_ptr, const lbf_options &opt, int nrhs, int rung,
+                  size_t *plan_bytes, size_t *item_bytes);
 
 struct SortBufs {  // plan-time scratch of a pair sort (capacity max(N, pair capacity))
     uint64_t *key, *key_alt;

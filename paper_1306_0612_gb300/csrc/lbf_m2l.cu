@@ -416,26 +416,26 @@ k_m2l_tc(int P, const int32_t *__restrict__ tile0, const int2 *__restrict__ pair
 
 }  // namespace
 
-// Room for the translations: 4 a reserved box (measured 2.3), dropped when the workspace has
-// none.  The buffers an application writes are a right-hand side's own (layout of views too).
+// Room for the translations: 4 a reserved box (measured 2.3), in a small system, whose reserve is
+// mostly for depth, 6 a box of 8 N / leaf_size (measured 3 to 4.4), dropped when the workspace
+// has none.  The buffers an application writes are a right-hand side's own (layout of views too).
 void lbf_m2l_layout_rhs(const lbf_plan *pl, lbf_plan *v, Arena &A)
 {
-    const int64_t cap = pl->tree.cap;
     const bool on = pl->m2l_cap > 0;
-    v->m2l_X = on ? A.get<long long>(cap * real_pitch(pl->P)) : nullptr;
-    v->m2l_e = on ? A.get<int32_t>(cap) : nullptr;
+    v->m2l_X = on ? A.get<long long>(pl->xcap * real_pitch(pl->P)) : nullptr;
+    v->m2l_e = on ? A.get<int32_t>(pl->xcap) : nullptr;
     v->m2l_out = on ? A.get<double>(pl->m2l_cap * 2 * pl->P) : nullptr;
 }
 
 void lbf_m2l_layout(lbf_plan *pl, const lbf_options &o, int64_t cap)
 {
     pl->m2l_cap = 0;
-    if (o.matvec != LBF_MATVEC_FMM || o.p + 1 > 32) return;
+    if (o.matvec != LBF_MATVEC_FMM || o.p + 1 > 32 || !(pl->parts & LBF_PART_M2L)) return;
     Arena &A = pl->arena;
     const size_t off = A.off;
     const bool full = A.overflow;
     pl->P = o.p + 1;
-    pl->m2l_cap = 4 * cap;
+    pl->m2l_cap = std::min<int64_t>(4 * cap, 6 * pl->xcap);
     pl->m2l_pairs = A.get<int2>(pl->m2l_cap + kNoffs * kRowsT);
     pl->m2l_vptr = A.get<int32_t>(cap + 1);
     pl->m2l_tile0 = A.get<int32_t>(2 * (kNoffs + 1));
@@ -474,7 +474,7 @@ int lbf_m2l_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch, int64_t scratc
     LBF_CUDA(cudaMemcpyAsync(&n, pl->m2l_vptr + nb, sizeof(n), cudaMemcpyDeviceToHost, s));
     LBF_CUDA(cudaMemcpyAsync(&tiles, pl->m2l_tile0 + kNoffs, sizeof(tiles), cudaMemcpyDeviceToHost, s));
     LBF_CUDA(cudaStreamSynchronize(s));
-    if (n > pl->m2l_cap) {
+    if (n > pl->m2l_cap || nb > pl->xcap) {
         pl->m2l_cap = 0;
         return LBF_OK;
     }

@@ -642,7 +642,7 @@ BoxGeo geo_of(const Tree &T)
 
 }  // namespace
 
-static unsigned *pass_words(const lbf_plan *pl) { return (unsigned *)(pl->loc_e + pl->tree.cap); }
+static unsigned *pass_words(const lbf_plan *pl) { return (unsigned *)(pl->loc_e + pl->xcap); }
 
 static int l2l(lbf_plan *pl, int P, const Own &w, cx<double> *loc, int kid, const int *gate,
                cudaStream_t s)
@@ -657,7 +657,7 @@ static int l2l(lbf_plan *pl, int P, const Own &w, cx<double> *loc, int kid, cons
 }
 
 // whether the plan's double applications take these passes
-bool lbf_passes_ready(const lbf_plan *pl) { return pl->rows && pl->m2l_cap && pl->nbigx >= 0; }
+bool lbf_passes_ready(const lbf_plan *pl) { return pl->rows && pl->m2l_cap && pl->loc_X && pl->nbigx >= 0; }
 
 int lbf_passes_build(lbf_plan *pl, cudaStream_t s, int32_t *scratch)
 {

@@ -815,7 +815,7 @@ int local_chunks(int P) { return (2 * P + 7) / 8; }
 void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap)
 {
     pl->rows = nullptr;
-    if (o.matvec != LBF_MATVEC_FMM) return;
+    if (o.matvec != LBF_MATVEC_FMM || !(pl->parts & LBF_PART_ROWS)) return;
     // local columns for the density's expansions and, where E y is one, the multipliers'
     const int Pl = std::max(o.p + 1, pl->bd.p2l_exp_cap ? pl->bd.Pe : 0);
     pl->rows_lch = local_chunks(Pl);
@@ -826,7 +826,11 @@ void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap)
     if (tiles > (int64_t)250000000) return;
     Arena &A = pl->arena;
     const size_t off = A.off;
-    const bool full = A.overflow;
+    const bool full = A.overflow, had_loc = pl->use_loc;
+    if (!had_loc && pl->m2l_cap) {  // the passes over the stored parts
+        lbf_loc_layout(pl, pl, A);
+        pl->use_loc = true;
+    }
     pl->rows_tiles = tiles;
     pl->rows_chunks = chunks;
     pl->rows_items_cap = N / 4 + cap;
@@ -845,6 +849,11 @@ void lbf_rows_layout(lbf_plan *pl, int64_t N, const lbf_options &o, int64_t cap)
         A.off = off;
         A.overflow = false;
         pl->rows = nullptr;
+        if (!had_loc) {
+            pl->use_loc = false;
+            pl->loc_X = nullptr;
+            pl->loc_e = nullptr;
+        }
     }
 }
 

@@ -104,20 +104,22 @@ extern "C" int lbf_autotune(int M, const int64_t *island_ptr, const double *x, c
     o.border = 0;
     o.matvec = LBF_MATVEC_FMM;
     o.box_capacity = 0;
-    size_t plan_bytes = 0;
+    size_t plan_bytes = 0, plan_least = 0;
     for (int lf : {16, 32, 48, 64}) {
         o.leaf_size = lf;
         o.p = p_ref;
-        size_t b = 0;
-        int rc = lbf_workspace_size(M, island_ptr, &o, &b);
+        size_t b[LBF_WORKSPACE_SIZES];
+        int rc = lbf_workspace_sizes(M, island_ptr, &o, 0, b);
         if (rc) return rc;
-        plan_bytes = std::max(plan_bytes, b);
+        plan_bytes = std::max(plan_bytes, b[0]);
+        plan_least = std::max(plan_least, b[LBF_WORKSPACE_SIZES - 1]);
     }
     plan_bytes = (plan_bytes + 255) & ~size_t(255);
-    const size_t vec_bytes = sizeof(double) * (size_t)(4 * N + 2 * kErrBlocks + 8);
-    const size_t need = plan_bytes + vec_bytes + 256;
-    if (bytes_needed) *bytes_needed = need;
-    if (!workspace || bytes < need) return workspace ? LBF_EWORKSPACE : LBF_OK;
+    plan_least = (plan_least + 255) & ~size_t(255);
+    const size_t vec_bytes = sizeof(double) * (size_t)(4 * N + 2 * kErrBlocks + 8) + 256;
+    if (bytes_needed) *bytes_needed = plan_bytes + vec_bytes;
+    if (!workspace || bytes < plan_least + vec_bytes) return workspace ? LBF_EWORKSPACE : LBF_OK;
+    plan_bytes = std::min(plan_bytes, (bytes - vec_bytes) & ~size_t(255));
     if (!x || !dx || !d2x || !centres) return LBF_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     char *wsp = (char *)workspace;

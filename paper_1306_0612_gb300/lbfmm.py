@@ -109,6 +109,13 @@ def load():
             "lbf_gmres_solve_transpose": (C.c_int, [_P, _P, _P, _P, _P, _P, _P]),
             "lbf_batch_run": (C.c_int, [C.c_int, C.POINTER(lbf_batch_item), C.POINTER(lbf_options),
                                         C.c_int]),
+            "lbf_batch_run_shared": (C.c_int, [C.c_int, C.POINTER(lbf_batch_item),
+                                               C.POINTER(lbf_options), C.c_int, _P, C.c_size_t]),
+            "lbf_batch_shared_size": (C.c_int, [C.c_int, C.POINTER(lbf_batch_item), C.c_int,
+                                                C.POINTER(C.c_size_t)]),
+            "lbf_workspace_sizes": (C.c_int, [C.c_int, _P, C.POINTER(lbf_options), C.c_int,
+                                              C.POINTER(C.c_size_t)]),
+            "lbf_plan_parts": (C.c_int, [_P, C.POINTER(C.c_int)]),
             "lbf_evaluate_transpose": (C.c_int, [_P, i64, _P, _P, _P, _P, _P]),
             "lbf_gradient_nodes": (C.c_int, [_P, _P, _P, _P, i64, _P, _P, _P, _P]),
             "lbf_gradient_data": (C.c_int, [_P, _P, _P, _P]),
@@ -144,7 +151,8 @@ def exported_symbols():
             "lbf_profile_reset", "lbf_profile_read", "lbf_gmres_solve_transpose",
             "lbf_evaluate_transpose", "lbf_gradient_nodes", "lbf_gradient_data", "lbf_batch_run", "lbf_evaluate_noalloc", "lbf_solve_stats", "lbf_sync_status", "lbf_selftest_rcp", "lbf_autotune", "lbf_debug_inject", "lbf_debug_clear", "lbf_point_vortices", "lbf_dipole_sum",
             "lbf_launch_count", "lbf_gmres_workspace_many", "lbf_gmres_solve_many",
-            "lbf_batch_workspace_size"]
+            "lbf_batch_workspace_size", "lbf_workspace_sizes", "lbf_plan_parts",
+            "lbf_batch_run_shared", "lbf_batch_shared_size"]
 
 
 def lbf_status_string(status: int) -> str:
@@ -201,6 +209,20 @@ def lbf_batch_workspace_size(island_ptr: np.ndarray, opt: lbf_options, nrhs: int
     return n.value
 
 
+LBF_WORKSPACE_SIZES = 5
+LBF_PART_M2L, LBF_PART_E, LBF_PART_PAIRS, LBF_PART_ROWS = 1, 2, 4, 8
+
+
+def lbf_workspace_sizes(island_ptr: np.ndarray, opt: lbf_options, nrhs: int = 0) -> list[int]:
+    """The plan's sizes (nrhs < 2), or a lockstep batch item's, with all stored parts, then
+    without one more each, the least last."""
+    ptr = np.ascontiguousarray(island_ptr, dtype=np.int64)
+    out = (C.c_size_t * LBF_WORKSPACE_SIZES)()
+    _check(load().lbf_workspace_sizes(len(ptr) - 1, ptr.ctypes.data, C.byref(opt), int(nrhs), out),
+           "lbf_workspace_sizes")
+    return [int(v) for v in out]
+
+
 class Plan:
     """A plan and the torch-owned workspace it lives in."""
 
@@ -218,14 +240,21 @@ class Plan:
             self.handle = None
 
 
-def _plan_workspace(nbytes, dev):
-    """(workspace, error): nbytes on dev, or what is free there with the allocator's error (a
-    plan without room for its stored rows forms them on the fly)."""
-    try:
-        return torch.empty(nbytes, dtype=torch.uint8, device=dev), None
-    except torch.cuda.OutOfMemoryError as e:
-        free = torch.cuda.mem_get_info(dev)[0]
-        return torch.empty(min(nbytes, int(0.95 * free)), dtype=torch.uint8, device=dev), e
+def _allocate(sizes, dev):
+    """A workspace of one of the sizes (descending; all but the last hold stored parts that a plan
+    can do without).  Stored parts of more than an eighth of the device are taken only while
+    they leave free what the plan cannot do without once more, for the caller's own arrays; and
+    where the allocator has no room the next size is tried."""
+    least = sizes[-1]
+    if sizes[0] - least > torch.cuda.get_device_properties(dev).total_memory // 8:
+        free = torch.cuda.mem_get_info(dev)[0] + torch.cuda.memory_reserved(dev) - torch.cuda.memory_allocated(dev)
+        sizes = [n for n in sizes if n + least <= free] or [least]
+    for n in sizes:
+        try:
+            return torch.empty(n, dtype=torch.uint8, device=dev)
+        except torch.cuda.OutOfMemoryError:
+            if n <= sizes[-1]:
+                raise
 
 
 def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream, device):
@@ -240,7 +269,7 @@ def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream,
     name = "lbf_plan_create_planar" if planar else "lbf_plan_create"
     for _ in range(6):
         nbytes = lbf_workspace_size(ptr, opt)
-        ws, short = _plan_workspace(nbytes, dev)
+        ws = _allocate([nbytes] + [n for n in lbf_workspace_sizes(ptr, opt) if n < nbytes], dev)
         nbytes = ws.numel()
         h = C.c_void_p()
         need = C.c_int64(0)
@@ -253,8 +282,6 @@ def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream,
         else:
             rc = lib.lbf_plan_create(C.byref(h), M, ptr.ctypes.data_as(_P), *geo,
                                      None if rot is None else rot.ctypes.data_as(_P), *tail)
-        if rc == LBF_EWORKSPACE and short is not None:
-            raise short
         if rc == LBF_EWORKSPACE and need.value > opt.box_capacity:
             opt = lbf_options.from_buffer_copy(opt)
             opt.box_capacity = int(need.value)
@@ -282,6 +309,13 @@ def lbf_plan_destroy(plan: Plan):
     if plan.handle:
         _check(load().lbf_plan_destroy(plan.handle), "lbf_plan_destroy")
         plan.handle = None
+
+
+def lbf_plan_parts(plan: Plan) -> int:
+    """The LBF_PART_* that the plan holds."""
+    parts = C.c_int(0)
+    _check(load().lbf_plan_parts(plan.handle, C.byref(parts)), "lbf_plan_parts")
+    return parts.value
 
 
 def lbf_plan_info(plan: Plan) -> dict:
@@ -403,8 +437,10 @@ def lbf_batch_run(instances, opt=None, nworkers=8, lockstep=True):
     list of dicts with sigma (nrhs x N), a (nrhs x M), u (nrhs x T or None) and the
     item's status, iters, fp64_applies, fp32_applies, max_rel_res.  Instances whose
     quadtree outgrew the workspace estimate are rerun with the size they reported.
-    lockstep: size each workspace for lbf_gmres_solve_many (lbf_batch_workspace_size), so
-    that an instance's right-hand sides advance together; else one after another."""
+    lockstep: size the workspaces for lbf_gmres_solve_many (lbf_batch_workspace_size), so
+    that an instance's right-hand sides advance together; else one after another.  The
+    instances share one workspace of a slice a worker (lbf_batch_run_shared), with fewer
+    stored parts (lbf_workspace_sizes) where memory is short."""
     lib = load()
     opt = opt or lbf_default_options()
     n = len(instances)
@@ -415,7 +451,7 @@ def lbf_batch_run(instances, opt=None, nworkers=8, lockstep=True):
         if not todo:
             break
         items = (lbf_batch_item * len(todo))()
-        keep = []
+        keep, sizes = [], []
         for slot, q in enumerate(todo):
             ins = instances[q]
             ptr = np.ascontiguousarray(ins["island_ptr"], dtype=np.int64)
@@ -424,9 +460,8 @@ def lbf_batch_run(instances, opt=None, nworkers=8, lockstep=True):
             o.box_capacity = caps[q]
             g = ins["g"].reshape(-1)
             nrhs = g.numel() // N
-            nbytes = lbf_batch_workspace_size(ptr, o, nrhs) if lockstep else lbf_workspace_size(ptr, o)
+            sizes.append(lbf_workspace_sizes(ptr, o, nrhs if lockstep else 0))
             dev = ins["x"].device
-            ws = torch.empty(nbytes, dtype=torch.uint8, device=dev)
             sigma = torch.empty(nrhs * N, dtype=torch.float64, device=dev)
             a = torch.empty(nrhs * M, dtype=torch.float64, device=dev)
             t = ins.get("targets")
@@ -438,17 +473,29 @@ def lbf_batch_run(instances, opt=None, nworkers=8, lockstep=True):
             it.dx = _dptr(ins["dx"], 3 * N, "dx").value
             it.d2x = _dptr(ins["d2x"], 3 * N, "d2x").value
             it.centres = _dptr(ins["centres"], 3 * M, "centres").value
-            it.workspace, it.bytes = ws.data_ptr(), nbytes
             it.nrhs, it.g = nrhs, _dptr(g, nrhs * N, "g").value
             it.sigma, it.a = sigma.data_ptr(), a.data_ptr()
             it.T = T
             it.targets = None if T == 0 else _dptr(t, 3 * T, "targets").value
             it.u = None if u is None else u.data_ptr()
             it.box_capacity = caps[q]
-            keep.append((q, ptr, ws, sigma, a, u, nrhs, N, M, T))
-        _check(lib.lbf_batch_run(len(todo), items, C.byref(opt), int(nworkers)), "lbf_batch_run")
+            keep.append((q, ptr, sigma, a, u, nrhs, N, M, T))
+        totals = []
+        for r in range(LBF_WORKSPACE_SIZES):
+            for it, s in zip(items, sizes):
+                it.bytes = s[r]
+            total = C.c_size_t(0)
+            _check(lib.lbf_batch_shared_size(len(todo), items, int(nworkers), C.byref(total)),
+                   "lbf_batch_run")
+            totals.append(total.value)
+        ws = _allocate(totals, instances[todo[0]]["x"].device)
+        for it, s in zip(items, sizes):
+            it.bytes = s[totals.index(ws.numel())]
+        _check(lib.lbf_batch_run_shared(len(todo), items, C.byref(opt), int(nworkers),
+                                        C.c_void_p(ws.data_ptr()), ws.numel()), "lbf_batch_run")
+        del ws
         nxt = []
-        for slot, (q, ptr, ws, sigma, a, u, nrhs, N, M, T) in enumerate(keep):
+        for slot, (q, ptr, sigma, a, u, nrhs, N, M, T) in enumerate(keep):
             it = items[slot]
             if it.status == LBF_EWORKSPACE and it.box_capacity_needed > caps[q]:
                 caps[q] = int(it.box_capacity_needed)
@@ -602,12 +649,19 @@ def lbf_autotune(island_ptr, x, dx, d2x, centres, target: float, opt=None, pole_
     _check(lib.lbf_autotune(M, ptr.ctypes.data_as(_P), None, None, None, None, None, C.byref(opt),
                             float(target), None, 0, C.byref(need), C.byref(best), None, 0,
                             _stream(stream)), "lbf_autotune")
-    ws = torch.empty(int(need.value), dtype=torch.uint8, device=x.device)
+    trial = lbf_options.from_buffer_copy(opt)
+    trial.border, trial.matvec, trial.box_capacity, trial.p = 0, LBF_MATVEC_FMM, 0, 44
+    least = 0  # every trial without stored parts, beside the vectors of the whole need
+    most = 0
+    for trial.leaf_size in (16, 32, 48, 64):
+        s = lbf_workspace_sizes(ptr, trial)
+        least, most = max(least, s[-1]), max(most, s[0])
+    ws = _allocate([int(need.value), int(need.value) - most + least + 512], x.device)
     buf = C.create_string_buffer(1 << 16)
     rc = lib.lbf_autotune(M, ptr.ctypes.data_as(_P), _dptr(x, 3 * N, "x"), _dptr(dx, 3 * N, "dx"),
                           _dptr(d2x, 3 * N, "d2x"), _dptr(centres, 3 * M, "centres"),
                           None if rot is None else rot.ctypes.data_as(_P), C.byref(opt),
-                          float(target), C.c_void_p(ws.data_ptr()), int(need.value), C.byref(need),
+                          float(target), C.c_void_p(ws.data_ptr()), ws.numel(), C.byref(need),
                           C.byref(best), buf, len(buf), _stream(stream))
     _check(rc, "lbf_autotune")
     del ws
