@@ -87,7 +87,9 @@ typedef struct lbf_options {
     int graphs;           /* GMRES steps replayed from a CUDA graph captured once per plan
                              (for the legacy default stream on a stream of its own): 1 on,
                              0 off, -1 automatic (on for N <= 4194304, where launches count);
-                             per-kernel tracing skips graph-replayed kernels */
+                             per-kernel tracing skips graph-replayed kernels, so while it is
+                             on the default stream launches directly, and -1 means on for
+                             N <= 262144 */
     int fmm64;            /* arithmetic of the accurate (double) FMM operator: 0 double,
                              1 double-float (pairs of floats, ~48-bit significands; this
                              GPU issues float 64 times faster than double).  Stored leaf

@@ -26,6 +26,7 @@ extern std::atomic<int64_t> g_lbf_launches;
 // Tracing: event pair around a launch when lbf_profile_enable(1) is on.
 void lbf_prof_mark(int id, int begin, cudaStream_t s);
 void lbf_prof_capture(bool on);  // this thread is capturing a CUDA graph: no marks
+bool lbf_prof_enabled();
 #define LBF_LAUNCH_P(id, kernel, grid, block, smem, stream, ...)           \
     do {                                                                   \
         lbf_prof_mark((id), 1, (stream));                                  \

@@ -725,6 +725,9 @@ static int arnoldi_step(lbf_plan *pl, int opc, int prec, int k, bool from_state,
 // included, with graphs and without: 131,072 nodes, gradient of a solve, 45.9 and 47.7 ms;
 // 416,768 nodes 22.6 and 23.7; 524,288 refined 20.4 and 22.2; 2.1 million 115.6 and 117.1.
 constexpr int64_t kGraphNodes = 1 << 22;
+// While kernels are traced (a replay leaves no marks) only small plans' steps, and none on the
+// default stream.
+constexpr int64_t kTracedGraphNodes = 1 << 18;
 
 // The captured step graph of (prec, transpose), built on first use; null when graphs
 // are off for this plan.  The legacy default stream cannot capture (but runs graphs): the
@@ -732,13 +735,15 @@ constexpr int64_t kGraphNodes = 1 << 22;
 static cudaGraphExec_t step_graph(lbf_plan *pl, int opc, int prec, cudaStream_t s)
 {
     const int g = pl->opt.graphs;
-    if (g == 0 || (g < 0 && pl->N > kGraphNodes) || !pl->vstep) return nullptr;
+    const bool legacy = s == nullptr || s == cudaStreamLegacy, traced = lbf_prof_enabled();
+    if (g == 0 || (g < 0 && pl->N > (traced ? kTracedGraphNodes : kGraphNodes)) || !pl->vstep) return nullptr;
+    if (traced && legacy) return nullptr;
     if (!(opc & LBF_OP_PRECONDITIONED)) return nullptr;  // the graphs hold the preconditioned step
     const int pi = prec == LBF_PREC_FP32 ? 1 : 0, ti = (opc & LBF_OP_TRANSPOSE) ? 1 : 0;
     if (pl->gexec[pi][ti]) return pl->gexec[pi][ti];
     cudaGraph_t graph = nullptr;
     cudaStream_t own = nullptr;
-    if (s == nullptr || s == cudaStreamLegacy) {
+    if (legacy) {
         if (cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;

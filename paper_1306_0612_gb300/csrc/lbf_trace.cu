@@ -58,6 +58,12 @@ thread_local bool t_capturing = false;
 
 void lbf_prof_capture(bool on) { t_capturing = on; }
 
+bool lbf_prof_enabled()
+{
+    std::lock_guard<std::mutex> lk(g_prof.mu);
+    return g_prof.on;
+}
+
 void lbf_prof_mark(int id, int begin, cudaStream_t s)
 {
     if (!g_prof.on || t_capturing) return;
