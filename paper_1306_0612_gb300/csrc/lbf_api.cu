@@ -31,7 +31,7 @@ int64_t box_capacity_estimate(int64_t N, const lbf_options &o)
 
 bool valid(const lbf_options &o)
 {
-    return o.tol > 0 && o.restart >= 1 && o.restart <= 200 && o.maxit >= 1 && o.p >= 4 &&
+    return o.tol > 0 && o.restart >= 1 && o.restart <= LBF_MAX_RESTART && o.maxit >= 1 && o.p >= 4 &&
            o.p + 1 <= LBF_MAX_TERMS && o.leaf_size >= 1 && o.leaf_size <= 1024 &&
            o.max_depth >= 1 && o.max_depth <= 30 &&
            (o.matvec == LBF_MATVEC_FMM || o.matvec == LBF_MATVEC_DIRECT) &&

@@ -11,6 +11,7 @@
 #define LBF_PI 3.14159265358979323846
 #define LBF_MAX_TERMS 64  // expansion terms p + 1 supported by the kernels
 #define LBF_MAX_LEVELS 31
+#define LBF_MAX_RESTART 200  // GMRES restart length
 #define LBF_ANC_STRIDE 32
 #define LBF_PASS_WORDS 8  // of lbf_passes.cu: up ticket, warps done, application; down application
 

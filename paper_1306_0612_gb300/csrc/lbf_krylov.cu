@@ -27,6 +27,8 @@ struct GmresState {
 namespace {
 
 constexpr int kRowsPerChunk = 1024;
+// (k_arnoldi's rotations take the place of the chunk)
+static_assert(3 * (LBF_MAX_RESTART + 2) <= kRowsPerChunk, "rotations and Hessenberg column");
 constexpr int kDotBlocks = 152 * 2;
 
 __device__ __forceinline__ bool gate_closed(const int *gate) { return gate && *gate == 0; }

@@ -211,15 +211,15 @@ struct Own {
     int M;
 };
 
-__device__ __forceinline__ cx<double> own_part(const Own &w, int64_t b, int P, int lane, int v0, int dv,
-                                               double ir, const cx<double> *loc)
+__device__ __forceinline__ cx<double> own_part(const Own &w, int64_t b, int P, int lane, double ir,
+                                               const cx<double> *loc)
 {
     cx<double> o = mk<double>(0, 0);
     if (lane >= P) return o;
     const int v1 = w.ptr[b + 1];
     if (w.src) {
 #pragma unroll 4
-        for (int v = w.ptr[b] + v0; v < v1; v += dv) {
+        for (int v = w.ptr[b]; v < v1; v++) {
             const cx<double> a = w.part[(int64_t)v * P + lane];
             const double y = w.y[w.src[v]];
             o.x = fma(y, a.x, o.x);
@@ -228,14 +228,14 @@ __device__ __forceinline__ cx<double> own_part(const Own &w, int64_t b, int P, i
         return o;
     }
 #pragma unroll 4
-    for (int v = w.ptr[b] + v0; v < v1; v += dv) {
+    for (int v = w.ptr[b]; v < v1; v++) {
         const cx<double> a = w.part[(int64_t)v * P + lane];
         o.x += a.x;
         o.y += a.y;
     }
     o.x *= ir;
     o.y *= ir;
-    if (v0 == 0 && w.nx[b] && w.en[b] - w.bg[b] > w.thr) {
+    if (w.nx[b] && w.en[b] - w.bg[b] > w.thr) {
         const cx<double> x = fmm::ldcg_cx(&loc[b * P + lane]);
         o.x += x.x;
         o.y += x.y;
@@ -556,7 +556,7 @@ k_l2l(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_t *__r
         const int lv = level[b], p = parent[b], h2 = quadrant(ix[b], iy[b]);
         const bool leaf = nchild[b] == 0;
         if (w.sums && b == 0) strength_sums(w, lane);
-        const cx<double> own = own_part(w, b, P, lane, 0, 1, g.invL * fmm::pow2<double>(lv + 1), loc);
+        const cx<double> own = own_part(w, b, P, lane, g.invL * fmm::pow2<double>(lv + 1), loc);
         // its exponent, and the row of this lane
         const int Ex = (int)((__double_as_longlong(own.x) >> 52) & 0x7ff);
         const int Ey = (int)((__double_as_longlong(own.y) >> 52) & 0x7ff);
