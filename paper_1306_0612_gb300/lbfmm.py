@@ -489,6 +489,9 @@ def lbf_batch_run(instances, opt=None, nworkers=8, lockstep=True):
                    "lbf_batch_run")
             totals.append(total.value)
         ws = _allocate(totals, instances[todo[0]]["x"].device)
+        # the workers' streams wait for nothing: what the caller's stream still does to the inputs, or
+        # to memory the allocator has just given out again, is done first
+        torch.cuda.current_stream(ws.device).synchronize()
         for it, s in zip(items, sizes):
             it.bytes = s[totals.index(ws.numel())]
         _check(lib.lbf_batch_run_shared(len(todo), items, C.byref(opt), int(nworkers),

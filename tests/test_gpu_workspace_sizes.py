@@ -103,3 +103,20 @@ def test_shared_workspace_gives_what_own_workspaces_give():
         for (_, s, a, _), it, (s0, a0, n) in zip(keep, items, own):
             assert it.status == L.LBF_OK and it.iters == n
             assert np.array_equal(host(s), s0) and np.array_equal(host(a), a0)
+
+
+def test_batch_waits_for_its_inputs():
+    """Data still being written on the caller's stream (behind a wait of about 50 ms) when the batch
+    is called: its own streams read them after that."""
+    inst, opt = _instances(2), L.lbf_default_options(tol=1e-12)
+    ref = [host(r["sigma"]) for r in L.lbf_batch_run(inst, opt=opt, nworkers=4)]
+    data = [ins["g"].clone() for ins in inst]
+    for ins in inst:
+        ins["g"] = torch.zeros_like(ins["g"])
+    torch.cuda.synchronize()
+    torch.cuda._sleep(100_000_000)
+    for ins, d in zip(inst, data):
+        ins["g"].copy_(d)
+    res = L.lbf_batch_run(inst, opt=opt, nworkers=4)
+    for r, s in zip(res, ref):
+        assert np.array_equal(host(r["sigma"]), s)
