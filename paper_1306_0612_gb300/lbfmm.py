@@ -257,7 +257,7 @@ def _allocate(sizes, dev):
                 raise
 
 
-def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream, device):
+def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream, device, stored):
     lib = load()
     opt = opt or lbf_default_options()
     ptr = np.ascontiguousarray(island_ptr, dtype=np.int64)
@@ -268,8 +268,9 @@ def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream,
     dev = a.device if device is None else device
     name = "lbf_plan_create_planar" if planar else "lbf_plan_create"
     for _ in range(6):
-        nbytes = lbf_workspace_size(ptr, opt)
-        ws = _allocate([nbytes] + [n for n in lbf_workspace_sizes(ptr, opt) if n < nbytes], dev)
+        sizes = lbf_workspace_sizes(ptr, opt)
+        nbytes = lbf_workspace_size(ptr, opt) if stored else sizes[-1]
+        ws = _allocate([nbytes] + [n for n in sizes if n < nbytes], dev)
         nbytes = ws.numel()
         h = C.c_void_p()
         need = C.c_int64(0)
@@ -293,16 +294,18 @@ def _create(planar, island_ptr, a, da, d2a, centres, pole_rotation, opt, stream,
 
 
 def lbf_plan_create(island_ptr, x, dx, d2x, centres, pole_rotation=None, opt=None, stream=None,
-                    device=None) -> Plan:
+                    device=None, stored=True) -> Plan:
     """Build a plan from nodes on the sphere (synchronous).  Retries with a larger
-    box capacity when the quadtree outgrows the first workspace estimate."""
-    return _create(False, island_ptr, x, dx, d2x, centres, pole_rotation, opt, stream, device)
+    box capacity when the quadtree outgrows the first workspace estimate.
+    stored=False: without the stored parts (lbf_workspace_sizes), for a plan applied or
+    evaluated only a few times: half the time to create, slower to use."""
+    return _create(False, island_ptr, x, dx, d2x, centres, pole_rotation, opt, stream, device, stored)
 
 
 def lbf_plan_create_planar(island_ptr, xi, dxi, d2xi, centres, opt=None, stream=None,
-                           device=None) -> Plan:
+                           device=None, stored=True) -> Plan:
     """Build a plan from planar nodes xi, xi', xi'' (N x 2 each, synchronous)."""
-    return _create(True, island_ptr, xi, dxi, d2xi, centres, None, opt, stream, device)
+    return _create(True, island_ptr, xi, dxi, d2xi, centres, None, opt, stream, device, stored)
 
 
 def lbf_plan_destroy(plan: Plan):

@@ -32,6 +32,13 @@ def test_a_plan_holds_the_parts_its_workspace_has_room_for(monkeypatch, M, rung,
     assert rel_l2(host(o)[rows], oracle.apply_rows(g, v, rows, 0)) < 1e-10
 
 
+def test_a_plan_asked_to_store_nothing():
+    g = wl.star_caps(5, 40, 33)
+    args = (g.island_ptr, dev(g.x), dev(g.dx), dev(g.d2x), dev(g.centres))
+    assert L.lbf_plan_parts(L.lbf_plan_create(*args, stored=False)) == 0
+    assert L.lbf_plan_parts(L.lbf_plan_create(*args)) == 11
+
+
 def _instances(nrhs):
     out = []
     for k, M in enumerate((3, 9, 1, 6, 14, 2, 5)):
