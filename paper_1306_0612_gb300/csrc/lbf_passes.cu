@@ -617,11 +617,11 @@ k_l2l(int64_t nbox, int P, const int32_t *__restrict__ level, const int32_t *__r
             if (on)
                 st_words(&LX[b * pitch + 2 * row], tag_word(rescale(sx, sh), tag),
                          tag_word(rescale(sy, sh), tag));
+            if (lane == 0) st_word(&ex[b], tag_exp(bad ? kBadExp : nb == 0 ? kZeroExp : e + sh, tag));
             // the rows past P too: the two chains have orders of their own, and rows left with an
             // earlier launch's tag would pass for this kind's 255 launches on
             for (int r = P + lane; 2 * r < pitch; r += 32)
                 st_words(&LX[b * pitch + 2 * r], tag_word(0, tag), tag_word(0, tag));
-            if (lane == 0) st_word(&ex[b], tag_exp(bad ? kBadExp : nb == 0 ? kZeroExp : e + sh, tag));
         }
     }
     if (lane == 0) {

@@ -18,9 +18,11 @@ def _plan():
     return g, plan_for(g, p=26, leaf_size=24)
 
 
-def test_a_chain_leaves_no_word_of_an_earlier_launch():
+def test_a_chain_leaves_no_word_of_an_earlier_launch(monkeypatch):
     """After a whole application (a chain of each kind) and one of the density alone, all 64
-    words of every box with children carry the last chain's tag, the third."""
+    words of every box with children carry the last chain's tag, the third (in a workspace of
+    zeros, without another plan's words)."""
+    monkeypatch.setattr(L, "_allocate", lambda sizes, d: torch.zeros(sizes[0], dtype=torch.uint8, device=d))
     g, plan = _plan()
     v = dev(np.random.default_rng(1).standard_normal(g.N + g.M))
     o = zeros(g.N + g.M)
