@@ -70,8 +70,10 @@ constexpr int kGroups = 8, kGroupsSmall = 2;
 // (8192 nodes: 458 us an application with whole leaves a warp, 408 shared; at 7130 leaves
 // the two are within 1 %, at 16,150 sharing costs 4 % of a solve)
 constexpr int64_t kSmallLeaves = 4864;
-// (several right-hand sides in lockstep share columns too, so that their sums are those of a
-// separate solve: 16 of 10,000 nodes 134 us, 157 with the quarters taken in turn by one warp)
+// (several right-hand sides in lockstep share no columns once their blocks make this many warps
+// an SM, four times what is resident; their sums are those of a separate solve all the same:
+// 16 of 64,000 nodes 1003 us shared, 850 not)
+constexpr int64_t kFullWarps = 64;
 constexpr int kLocalTop = 1021;  // exponent field of the local columns' largest: [1/4, 1/2)
 constexpr int kRowBlocks = 4;    // thread blocks an SM
 constexpr int kRun = 4;          // chunks read at a time (2 or 4)
@@ -416,18 +418,20 @@ __device__ __forceinline__ void dot_chunks(const double *__restrict__ t, const i
     }
 }
 
-// The sum of a lane's row over n chunks of double entries whose columns are nodes.  Not inlined:
-// few blocks have any, and beside the integer loops its sums cost them registers (rows of 407
-// ragged islands 143 us inlined, 133 so; the multipoles' loop, which many blocks enter, 152
-// and 133 the other way round).
+// The sum of a lane's row over the chunks w, w + step, .. of n of double entries whose columns are
+// nodes.  Not inlined: few blocks have any, and beside the integer loops its sums cost them
+// registers (rows of 407 ragged islands 143 us inlined, 133 so; the multipoles' loop, which many
+// blocks enter, 152 and 133 the other way round).
 template <int G>
 __device__ __noinline__ double wide_rows(const double *__restrict__ t, const int32_t *__restrict__ cl,
-                                         int ncol, int n, int ng, const double *__restrict__ sigma, int lane)
+                                         int ncol, int w, int step, int n, int ng,
+                                         const double *__restrict__ sigma, int lane)
 {
     double d[G];
 #pragma unroll
     for (int q = 0; q < G; q++) d[q] = 0.0;
-    for (int k = 0; k < n; k++, t += 32 * ng) {
+    t += (int64_t)32 * ng * w;
+    for (int k = w; k < n; k += step, t += 32 * step * ng) {
         const int m = 8 * k + (lane & 7);
         const double x = m < ncol ? sigma[cl[m]] : 0.0;
 #pragma unroll
@@ -441,103 +445,227 @@ __device__ __noinline__ double wide_rows(const double *__restrict__ t, const int
     return d[0];
 }
 
-// The sum of one row of a block of at most G row groups over its column chunks k0 .. k1 - 1
-// (near chunks, multipole chunks, then the local expansion's), and that row.  The columns'
-// values of a run of chunks are made integers first, a column a lane, and left in xs.
+// The values of n column chunks from chunk k on (near nodes, or far: the local expansion's) in xs,
+// zeros up to a multiple of four chunks, as they are (each lane's its own); the lane's largest
+// exponent field, kBadExp where one is not finite
+template <typename R>
+__device__ __forceinline__ int run_values(const RowItem &it, const int32_t *__restrict__ cl,
+                                          const double *__restrict__ sigma, const cx<R> *__restrict__ loc,
+                                          int P, bool far, int k, int n, int2 *xs, int lane)
+{
+    const int64_t lb = (int64_t)it.box * 2 * P;
+    const int off = 8 * (far ? it.nchunk : 0), end = min(far ? off + 2 * P : it.ncol, 8 * (k + n));
+    const int m1 = 8 * (k + (n + 3) / 4 * 4);
+    int top = 0;
+#pragma unroll 2
+    for (int m = 8 * k + lane; m < m1; m += 32) {
+        double v = 0.0;
+        if (m < end) v = far ? local_real(loc, lb + m - off) : sigma[cl[m]];
+        const int E = exp_field(v);
+        if (E) top = max(top, E == 0x7ff ? kBadExp : E + (far ? (m - off) >> 2 : 0));
+        xs[m - 8 * k] = make_int2(__double2loint(v), __double2hiint(v));
+    }
+    return top;
+}
+// and the values as words in the unit of top (of the local expansion from its chunk k on)
+__device__ __forceinline__ void run_words(bool far, int k, int n, int top, int2 *xs, int lane)
+{
+#pragma unroll 2
+    for (int m = lane; m < 8 * ((n + 3) / 4 * 4); m += 32) {
+        const int2 b = xs[m];
+        xs[m] = dot_word(__hiloint2double(b.y, b.x), far ? (8 * k + m) >> 2 : 0, top);
+    }
+}
+// the lane's row's sum over n integer chunks at t
+template <int G>
+__device__ __forceinline__ Dot run_dot(const double *__restrict__ t, const int2 *xs, int n, int ng, int lane)
+{
+    Dot acc[G];
+#pragma unroll
+    for (int q = 0; q < G; q++) acc[q] = Dot{0, 0};
+#define LBF_DOT(NG) dot_chunks<(NG <= G ? NG : G)>(t, xs + (lane & 7), n, lane, acc)
+    if (G <= 2) {
+        if (ng == 1) LBF_DOT(1);
+        else LBF_DOT(2);
+    } else {
+        LBF_GROUPS(ng, LBF_DOT)
+    }
+#undef LBF_DOT
+    fold_rows<G>(lane, [&](int a, int b, bool up, int bit) { acc[a] = dot_meet(acc[a], acc[b], up, bit); });
+    return acc[0];
+}
+// its sum over the multipole chunks w, w + step, .. of W boxes (few, and in units of their own), t at
+// the first
+template <int G, typename R>
+__device__ __forceinline__ double far_chunks(const double *__restrict__ t, const RowItem &it,
+                                             const int32_t *__restrict__ cl, const cx<R> *__restrict__ mp,
+                                             int w, int step, int ng, int lane)
+{
+    double d[G];
+#pragma unroll
+    for (int q = 0; q < G; q++) d[q] = 0.0;
+    t += (int64_t)32 * ng * w;
+    for (int c = (it.ncol + 7) / 8 + w; c < it.nchunk; c += step, t += 32 * step * ng) {
+        const int j = cl[8 * c + (lane & 7)];
+        const double x = j < 0 ? local_real(mp, -1 - j) : 0.0;
+#pragma unroll
+        for (int q = 0; q < G; q++)
+            if (q < ng) d[q] = fma(t[32 * q], x, d[q]);
+    }
+    fold_rows<G>(lane, [&](int a, int b, bool up, int bit) {
+        const double keep = up ? d[b] : d[a], send = up ? d[a] : d[b];
+        d[a] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+    });
+    return d[0];
+}
+__device__ __forceinline__ double run_double(const Dot &d, int top, int unit)
+{
+    return top >= kBadExp ? __longlong_as_double(0x7ff8000000000000ll) : dot_double(d, top + unit);
+}
+
+// The sum of a lane's row of a block of at most G row groups over its columns, by one warp: near
+// chunks, multipole chunks, then the local expansion's.  Near nodes are taken in runs of up to
+// kDotChunks chunks, in units of the run's largest density and the row's largest entry, the local
+// expansion in that of its largest b_l 2^(l/2).  (Blocks that may be shared add four sums of
+// double chunks, as shared_rows does.)
 template <int G, typename R>
 __device__ __forceinline__ double block_rows(const RowItem &it, const double *__restrict__ rows,
                                              const int32_t *__restrict__ rexp,
                                              const int32_t *__restrict__ cols,
                                              const double *__restrict__ sigma,
                                              const cx<R> *__restrict__ loc,
-                                             const cx<R> *__restrict__ mp, int P, int k0, int k1,
-                                             int2 *xs, int lane, int &row)
+                                             const cx<R> *__restrict__ mp, int P, int lchunks,
+                                             int2 *xs, int lane, int row)
 {
+    constexpr int kStep = G == kGroupsSmall ? 4 : 1;
     const int ng = (it.nrow + 3) / 4;
-    const double *t = rows + ((int64_t)it.tile + (int64_t)k0 * ng) * 32 + lane;
+    const double *t = rows + (int64_t)it.tile * 32 + lane;
     const int32_t *cl = cols + (int64_t)it.chunk * 8;
-    const int64_t lb = (int64_t)it.box * 2 * P;
-    const int nn = (it.ncol + 7) / 8;
-    const int grp = fold_rows<G>(lane, [](int, int, bool, int) {});
-    row = grp < ng ? 4 * grp + (lane >> 3) : it.nrow;
-    prefetch_tiles(t - lane, ng * min(k1 - k0, kAhead), lane);
+    const int nn = (it.ncol + 7) / 8, nk = it.nchunk + lchunks;
+    prefetch_tiles(t - lane, ng * min(nk, kAhead), lane);
     double s = 0.0;
-    int k = k0;
-    if (it.leaf < 0 && k < min(k1, nn)) {  // near entries kept as doubles
-        const int ke = min(k1, nn);
-        s = wide_rows<G>(t, cl + 8 * k, it.ncol - 8 * k, ke - k, ng, sigma, lane);
-        t += (int64_t)32 * ng * (ke - k);
-        k = ke;
+    int k = 0;
+    if (it.leaf < 0) {  // near entries kept as doubles
+        s = wide_rows<G>(t, cl, it.ncol, 0, kStep, nn, ng, sigma, lane);
+#pragma unroll 1
+        for (int w = 1; w < kStep; w++) s += wide_rows<G>(t, cl, it.ncol, w, kStep, nn, ng, sigma, lane);
+        t += (int64_t)32 * nn * ng;
+        k = nn;
     }
-    while (k < k1) {
-        if (k < it.nchunk && k >= nn) {
-            // multipoles of W boxes: few, and in units of their own
-            double d[G];
-#pragma unroll
-            for (int q = 0; q < G; q++) d[q] = 0.0;
-            for (const int ke = min(k1, it.nchunk); k < ke; k++, t += 32 * ng) {
-                const int j = cl[8 * k + (lane & 7)];
-                const double x = j < 0 ? local_real(mp, -1 - j) : 0.0;
-#pragma unroll
-                for (int q = 0; q < G; q++)
-                    if (q < ng) d[q] = fma(t[32 * q], x, d[q]);
-            }
-            fold_rows<G>(lane, [&](int a, int b, bool up, int bit) {
-                const double keep = up ? d[b] : d[a], send = up ? d[a] : d[b];
-                d[a] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
-            });
-            s += d[0];
+    while (k < nk) {
+        if (k >= nn && k < it.nchunk) {
+            double m = far_chunks<G>(t, it, cl, mp, 0, kStep, ng, lane);
+#pragma unroll 1
+            for (int w = 1; w < kStep; w++) m += far_chunks<G>(t, it, cl, mp, w, kStep, ng, lane);
+            s += m;
+            t += (int64_t)32 * (it.nchunk - k) * ng;
+            k = it.nchunk;
             continue;
         }
-        // near nodes, in units of the run's largest density and the row's largest entry; the
-        // local expansion, in those of the run's largest b_l 2^(l/2)
         const bool far = k >= nn;
-        const int n = min((far ? k1 : min(k1, nn)) - k, kDotChunks);
-        if (k > k0) prefetch_tiles(t - lane, ng * min(n, kAhead), lane);
-        const int off = 8 * (far ? it.nchunk : 0), end = min(far ? off + 2 * P : it.ncol, 8 * (k + n));
-        const int m1 = 8 * (k + (n + 3) / 4 * 4);
-        int top = 0;
+        const int n = min((far ? nk : nn) - k, kDotChunks);
+        if (k > 0) prefetch_tiles(t - lane, ng * min(n, kAhead), lane);
         __syncwarp();
-#pragma unroll 2
-        for (int m = 8 * k + lane; m < m1; m += 32) {
-            double v = 0.0;
-            if (m < end) v = far ? local_real(loc, lb + m - off) : sigma[cl[m]];
-            const int E = exp_field(v);
-            if (E) top = max(top, E == 0x7ff ? kBadExp : E + (far ? (m - off) >> 2 : 0));
-            xs[m - 8 * k] = make_int2(__double2loint(v), __double2hiint(v));  // a lane's own until they are words
-        }
-        top = __reduce_max_sync(0xffffffffu, top);
-        const bool bad = top >= kBadExp;
-#pragma unroll 2
-        for (int m = 8 * k + lane; m < m1; m += 32) {
-            const int2 b = xs[m - 8 * k];
-            xs[m - 8 * k] = dot_word(__hiloint2double(b.y, b.x), far ? (m - off) >> 2 : 0, top);
-        }
+        const int top = __reduce_max_sync(0xffffffffu, run_values(it, cl, sigma, loc, P, far, k, n, xs, lane));
+        run_words(far, k - it.nchunk, n, top, xs, lane);
         __syncwarp();
-        Dot acc[G];
-#pragma unroll
-        for (int q = 0; q < G; q++) acc[q] = Dot{0, 0};
-#define LBF_DOT(NG) dot_chunks<(NG <= G ? NG : G)>(t, xs + (lane & 7), n, lane, acc)
-        if (G <= 2) {
-            if (ng == 1) LBF_DOT(1);
-            else LBF_DOT(2);
-        } else {
-            LBF_GROUPS(ng, LBF_DOT)
-        }
-#undef LBF_DOT
+        const Dot d = run_dot<G>(t, xs, n, ng, lane);
         k += n;
         t += (int64_t)32 * n * ng;
-        fold_rows<G>(lane, [&](int a, int b, bool up, int bit) { acc[a] = dot_meet(acc[a], acc[b], up, bit); });
-        if (row < it.nrow)
-            s += bad ? __longlong_as_double(0x7ff8000000000000ll)
-                     : dot_double(acc[0], top + (far ? -1129 : rexp[it.row0 + row] - 2150));
+        if (row < it.nrow) s += run_double(d, top, far ? -1129 : rexp[it.row0 + row] - 2150);
     }
     return s;
 }
 
-// v of a block's rows: a warp per block, or (SPLIT, blocks of kGroupsSmall groups) the four
-// warps of a thread block, each over a quarter of the columns, the quarters added in order.
-template <typename R, bool SPLIT>
+// What four warps share of a block
+struct Shared {
+    int top[2][4];
+    Dot dot[2][4][32];
+    double part[4][32];
+};
+
+// The same sums by the four warps of a thread block, the first warp's valid, and the same bits: the
+// warps take quarters of every run, find its unit together and add their integer sums exactly
+// before one is turned into a double; double chunks are four sums, of every fourth chunk, added in
+// order.  The last run of near nodes and the local expansion go together (two barriers for most
+// blocks).
+template <typename R>
+__device__ __forceinline__ double shared_rows(const RowItem &it, const double *__restrict__ rows,
+                                              const int32_t *__restrict__ rexp,
+                                              const int32_t *__restrict__ cols,
+                                              const double *__restrict__ sigma,
+                                              const cx<R> *__restrict__ loc,
+                                              const cx<R> *__restrict__ mp, int P, int lchunks,
+                                              int2 *xs, Shared &sh, int wid, int lane, int row)
+{
+    constexpr int G = kGroupsSmall;
+    const int ng = (it.nrow + 3) / 4;
+    const double *tiles = rows + (int64_t)it.tile * 32 + lane;
+    const int32_t *cl = cols + (int64_t)it.chunk * 8;
+    const int nn = (it.ncol + 7) / 8;
+    auto add_parts = [&](double mine) {
+        sh.part[wid][lane] = mine;
+        __syncthreads();
+        const double s = ((sh.part[0][lane] + sh.part[1][lane]) + sh.part[2][lane]) + sh.part[3][lane];
+        __syncthreads();
+        return s;
+    };
+    auto add_dots = [&](int i) {
+        Dot d = sh.dot[i][0][lane];
+#pragma unroll
+        for (int w = 1; w < 4; w++) {
+            d.h += sh.dot[i][w][lane].h;
+            d.m += sh.dot[i][w][lane].m;
+        }
+        return d;
+    };
+    const int re = row < it.nrow ? rexp[it.row0 + row] : 0;  // (not at the end, where nothing hides the load)
+    double s = 0.0, local = 0.0;
+    int k = 0;
+    if (it.leaf < 0) {
+        s = add_parts(wide_rows<G>(tiles, cl, it.ncol, wid, 4, nn, ng, sigma, lane));
+        k = nn;
+    }
+    const int l0 = it.nchunk + lchunks * wid / 4, ln = it.nchunk + lchunks * (wid + 1) / 4 - l0;
+    const double *tl = tiles + (int64_t)32 * ng * l0;
+    prefetch_tiles(tl - lane, ng * ln, lane);
+    for (bool last = false; !last;) {
+        const int n = min(nn - k, kDotChunks);
+        const int c0 = k + n * wid / 4, cn = k + n * (wid + 1) / 4 - c0;
+        const double *t = tiles + (int64_t)32 * ng * c0;
+        int2 *xl = xs + 8 * ((cn + 3) / 4 * 4);
+        k += n;
+        last = k >= nn;
+        prefetch_tiles(t - lane, ng * min(cn, kAhead), lane);
+        __syncwarp();
+        int top = __reduce_max_sync(0xffffffffu, run_values(it, cl, sigma, loc, P, false, c0, cn, xs, lane));
+        int topl = last ? __reduce_max_sync(0xffffffffu, run_values(it, cl, sigma, loc, P, true, l0, ln, xl, lane)) : 0;
+        if (lane == 0) {
+            sh.top[0][wid] = top;
+            sh.top[1][wid] = topl;
+        }
+        __syncthreads();
+        top = max(max(sh.top[0][0], sh.top[0][1]), max(sh.top[0][2], sh.top[0][3]));
+        topl = max(max(sh.top[1][0], sh.top[1][1]), max(sh.top[1][2], sh.top[1][3]));
+        run_words(false, 0, cn, top, xs, lane);
+        if (last) run_words(true, l0 - it.nchunk, ln, topl, xl, lane);
+        __syncwarp();
+        sh.dot[0][wid][lane] = run_dot<G>(t, xs, cn, ng, lane);
+        if (last) sh.dot[1][wid][lane] = run_dot<G>(tl, xl, ln, ng, lane);
+        __syncthreads();
+        if (wid == 0 && row < it.nrow) {
+            if (n > 0) s += run_double(add_dots(0), top, re - 2150);
+            if (last) local = run_double(add_dots(1), topl, -1129);
+        }
+    }
+    if (nn < it.nchunk)
+        s += add_parts(far_chunks<G>(tiles + (int64_t)32 * ng * nn, it, cl, mp, wid, 4, ng, lane));
+    return s + local;
+}
+
+// v of a block's rows: a warp per block of at most G row groups, or (SPLIT) the four warps of a
+// thread block
+template <typename R, int G, bool SPLIT>
 __global__ void __launch_bounds__(128, kRowBlocks)
 k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__restrict__ rows,
              const int32_t *__restrict__ rexp, const int32_t *__restrict__ cols,
@@ -547,25 +675,23 @@ k_rows_apply(int64_t nitem, const RowItem *__restrict__ items, const double *__r
 {
     lbf_rhs(slab, sigma, loc, mp, bsig, v, gate);
     if (fmm::gate_closed(gate)) return;
-    __shared__ double part[4][32];
-    __shared__ int2 xs[4][8 * kDotChunks];
+    __shared__ int2 xs[4][8 * (SPLIT ? kDotChunks / 4 + 16 : kDotChunks)];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t k = SPLIT ? (int64_t)blockIdx.x : blockIdx.x * (int64_t)(blockDim.x >> 5) + wid;
     if (k >= nitem) return;
     const int4 i0 = ((const int4 *)items)[2 * k], i1 = ((const int4 *)items)[2 * k + 1];
     const RowItem it{i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
-    const int nk = it.nchunk + lchunks;
-    const int k0 = SPLIT ? nk * wid / 4 : 0, k1 = SPLIT ? nk * (wid + 1) / 4 : nk;
-    int row;
-    double s = block_rows<SPLIT ? kGroupsSmall : kGroups>(it, rows, rexp, cols, sigma, loc, mp, P, k0, k1,
-                                                          xs[wid], lane, row);
-    if (SPLIT) {
-        part[wid][lane] = s;
-        __syncthreads();
-        if (wid != 0) return;
-        s = part[0][lane] + part[1][lane] + part[2][lane] + part[3][lane];
+    const int grp = fold_rows<G>(lane, [](int, int, bool, int) {});
+    const int row = 4 * grp + (lane >> 3) < it.nrow ? 4 * grp + (lane >> 3) : it.nrow;
+    const double beta = SPLIT ? *bsig : 0.0;
+    double s;
+    if constexpr (SPLIT) {
+        __shared__ Shared sh;
+        s = shared_rows(it, rows, rexp, cols, sigma, loc, mp, P, lchunks, xs[wid], sh, wid, lane, row);
+    } else {
+        s = block_rows<G>(it, rows, rexp, cols, sigma, loc, mp, P, lchunks, xs[wid], lane, row);
     }
-    if (row < it.nrow) v[it.row0 + row] = s + 2.0 * *bsig;
+    if ((!SPLIT || wid == 0) && row < it.nrow) v[it.row0 + row] = s + 2.0 * (SPLIT ? beta : *bsig);
 }
 
 // a[h] += the tiles of chunk h (of n, at most 4) times the rows' values
@@ -936,16 +1062,23 @@ int lbf_rows_apply(lbf_plan *pl, const double *sigma, double *v, const int *gate
                    bool df)
 {
     const int64_t n = pl->rows_nitem;
-    const bool split = pl->rows_split != 0;
+    const bool small = pl->rows_split != 0;
+    const bool split = small && (pl->nrhs == 1 || n * pl->nrhs < kFullWarps * (int64_t)std::max(pl->nsm, 1));
     const dim3 grid = lbf_grid(pl, split ? n : lbf_cdiv(n, 4));
-#define LBF_ROWS(R, SPLIT)                                                                         \
-    LBF_LAUNCH_P(LBF_KERNEL_LEAF, (k_rows_apply<R, SPLIT>), grid, 128, 0, s, n, pl->rows_items, pl->rows, \
+#define LBF_ROWS(R, G, SPLIT)                                                                      \
+    LBF_LAUNCH_P(LBF_KERNEL_LEAF, (k_rows_apply<R, G, SPLIT>), grid, 128, 0, s, n, pl->rows_items, pl->rows, \
                  pl->rows_e, pl->rows_cols, sigma, (const cx<R> *)pl->local,                       \
                  (const cx<R> *)pl->mpole, pl->P, local_chunks(pl->P), pl->bsig, v, gate, pl->slab)
-    if (df && split) LBF_ROWS(df64, true);
-    else if (df) LBF_ROWS(df64, false);
-    else if (split) LBF_ROWS(double, true);
-    else LBF_ROWS(double, false);
+#define LBF_ROWS_OF(R)                                  \
+    if (split) LBF_ROWS(R, kGroupsSmall, true);         \
+    else if (small) LBF_ROWS(R, kGroupsSmall, false);   \
+    else LBF_ROWS(R, kGroups, false)
+    if (df) {
+        LBF_ROWS_OF(df64);
+    } else {
+        LBF_ROWS_OF(double);
+    }
+#undef LBF_ROWS_OF
 #undef LBF_ROWS
     LBF_CHECK_LAUNCH();
     return LBF_OK;
