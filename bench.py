@@ -110,9 +110,12 @@ def make_geometry(name):
 
 def workload_config(name, g, T, tol, precision):
     w = WORKLOADS[name]
-    arith = {"fp64": "native double throughout",
-             "df64": "double-float FMM (pairs of floats), double elsewhere",
-             "fp32r": "float FMM in the inner solves, native double residuals (refinement)"}[precision]
+    stored = ("FMM from stored parts: near rows, densities and expansions as 54-bit integers summed exactly on "
+              "the integer pipes, M2L as digit products on the tensor cores, rounding as of double; ")
+    arith = {"fp64": stored + "geometry, border and GMRES in double",
+             "df64": stored + "the double-float option's passes only without the stored parts",
+             "fp32r": "float FMM in the inner solves; residuals (refinement): " + stored +
+                      "geometry, border and GMRES in double"}[precision]
     return {"workload": f"{name}: {w['M']} star-cap islands x {w['nodes']} nodes "
                         f"(N={g.N}), Green's-pair data, GMRES(50) tol {tol:g}, {T} targets",
             "islands": g.M, "nodes": g.N, "targets": T, "precision": precision,

@@ -90,10 +90,13 @@ typedef struct lbf_options {
                              per-kernel tracing skips graph-replayed kernels, so while it is
                              on the default stream launches directly, and -1 means on for
                              N <= 262144 */
-    int fmm64;            /* arithmetic of the accurate (double) FMM operator: 0 double,
-                             1 double-float (pairs of floats, ~48-bit significands; this
-                             GPU issues float 64 times faster than double).  Stored leaf
-                             rows are double in both */
+    int fmm64;            /* arithmetic of the accurate FMM operator where it does not run from
+                             stored parts (p >= 32, a workspace without LBF_PART_M2L and
+                             LBF_PART_ROWS, derivative rows): 0 double, 1 double-float (pairs
+                             of floats, ~48-bit significands; this GPU issues float 64 times
+                             faster than double).  From stored parts both are the same:
+                             integers of 54 bits below a common size (a row's entries, a
+                             box's expansion), summed exactly */
     int schur;            /* how the preconditioner applies S^-1 (S = D - F E, Sec. 5, Eq.
                              matrix_eqns_c): LBF_SCHUR_AUTO, LBF_SCHUR_GJ or LBF_SCHUR_LU */
     int p2p_warps;        /* near-field tile: warps (leaves) per block of the leaf pass,
@@ -239,11 +242,12 @@ int lbf_gmres_solve(lbf_plan *plan, const double *g, double *sigma, double *a, c
  * when graphs are on; with FP32_REFINE every refinement round forms the FP64 residuals
  * of the open right-hand sides together and runs their float inner solves in lockstep.
  * Each right-hand side runs the kernels and fixed-order reductions of lbf_gmres_solve on
- * its own buffers, except the near field of the native-double FMM operator (fmm64 = 0),
- * which one pass forms for the whole group, a pair's geometry once for all densities (a
- * different rounding: results agree with separate solves to the solver's tolerance).
- * With direct sums, the double-float operator, or the float one alone, sigma, a, iters
- * and rel_res equal those of nrhs separate lbf_gmres_solve calls bit for bit.  A
+ * its own buffers, except, on a plan without LBF_PART_ROWS, the near field of the
+ * native-double FMM operator (fmm64 = 0), which one pass forms for the whole group, a
+ * pair's geometry once for all densities (a different rounding: results agree with
+ * separate solves to the solver's tolerance).  With stored rows, direct sums, the
+ * double-float operator, or the float one alone, sigma, a, iters and rel_res equal those
+ * of nrhs separate lbf_gmres_solve calls bit for bit.  A
  * right-hand side that converges stops while the others go on.  Plans whose S^-1 is
  * applied by LU factors (LBF_SCHUR_LU, or M > 1024 with LBF_SCHUR_AUTO) solve the
  * right-hand sides one after another with lbf_gmres_solve (workspace 0).

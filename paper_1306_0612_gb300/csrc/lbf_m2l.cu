@@ -31,7 +31,8 @@
 // one CTA an SM: eight warps expand the gathered rows' digits into shared memory (112 KB; the
 // next tile's integers are fetched before the wait for the MMAs) and one of their threads
 // issues the MMAs, eight warps read the accumulators back and write each translation's local
-// expansion; the expansion of one tile's digits overlaps the readout of the one before.  The
+// expansion; the expansion of one tile's digits overlaps the readout of the one before: 2.9 ms for
+// the 6.6 million translations at 16.8 million nodes (2.65 without the products of place 7).  The
 // target's warp in k_down then adds its translations in list order (two additions a
 // coefficient).
 //

@@ -28,22 +28,24 @@
 // On the integer pipes: a double multiply-add leaves a scheduler every 64 cycles, the three
 // 32 x 32 -> 64 bit products that stand for one every 17 (lbf_fixed.cuh).  An entry is an integer
 // of 54 bits below its row's largest near entry (rexp), the density below the largest of the run
-// of up to 512 columns it is summed with, the local columns and the expansion below fixed sizes (|u_i^l| 2^-(l/2) < 3/2); the sums are exact
-// but for the products' last 52 bits.  Errors of whole applications against 64 bits are what they
-// were with double entries, to three digits, at orders 22 to 31.  The multipole columns, few and in units
-// of their own, stay double.
+// of up to 512 columns it is summed with, the local columns and the expansion below fixed sizes
+// (|u_i^l| 2^-(l/2) < 3/2); the sums are exact but for the products' last 52 bits.  Errors of whole
+// applications against 64 bits are what they were with double entries, to three digits, at orders
+// 22 to 31; of single rows, relative to the sums of their terms' sizes, they are a few 2^-53 or less,
+// also where densities of 1 and 1e-12 meet, and blocks whose entries differ too much stay double
+// (kWideTop).  The multipole columns, few and in units of their own, stay double.
 //
 // Layout: a leaf's rows are cut into blocks of at most kGroups groups of four rows, its
 // columns into chunks of eight; a tile is one group x one chunk, 32 doubles, row-major,
 // so lane = 8 (row mod 4) + (column mod 8) and a warp's load is 256 contiguous bytes.  A
 // block's tiles are stored chunk by chunk: the near nodes, the W multipoles' reals, then
-// the 2 P reals of the local expansion.  Each lane holds one sum per group; eight lanes share a row, and a butterfly
-// that halves the groups at each step adds them in 7 additions for 8 groups (lanes on
+// the 2 P reals of the local expansion.  Each lane holds one sum per group; eight lanes share a
+// row, and a butterfly that halves the groups at each step adds them in 7 additions for 8 groups (lanes on
 // rows alone would leave 19 % of the lanes idle at 26 nodes a leaf, lanes on columns
 // alone would add 31 shuffled sums to 4 x 26 multiply-adds).
 //
-// Measured, rows of one application at 16.8 million nodes, 416,768 and 8192: 6.5 ms, 127 us
-// and 14 us (double entries 7.4 ms, 201 us, 22 us); transposed, 131,072 nodes, 89 and 97 us
+// Measured, rows of one application at 16.8 million nodes, 416,768 and 8192: 6.6 ms, 128 us
+// and 16 us (double entries 7.4 ms, 201 us, 22 us); transposed, 131,072 nodes, 93 and 97 us
 // (147 and 137).  Bound by the latency of the tiles' loads, 3.9 of 6.7 TB/s at the large end: the
 // next eight chunks are asked for ahead, four are read at once; more warps with fewer loads
 // each were slower (6.9 ms with two chunks at once, 8.8 with 24 warps an SM).
