@@ -26,7 +26,8 @@
 // carries the launch's tag (lbf_fixed.cuh), so a level costs one trip through L2 and no fence.
 // Measured, microseconds at 8192 nodes and at 16.8 million: up 50 and 3300 (double shifts
 // and P2M 8000 at the latter; integer shifts with arrival counters 91 and 6100, P2M still
-// double), a chain 27 and 3060 (5400; with flags 70 and 3600).  What is left is bound by the
+// double), a chain 27 and, at the latter, the density's 1710, the potential's 4330 (5400 in the mean;
+// with flags 70 and 3600).  What is left is bound by the
 // dependent loads of a box (a third fewer instructions for its sums changed nothing) and by
 // the depth of the tree.
 #include <algorithm>

@@ -46,8 +46,9 @@
 //
 // Measured, rows of one application at 16.8 million nodes, 416,768 and 8192: 6.6 ms, 128 us
 // and 16 us (double entries 7.4 ms, 201 us, 22 us); transposed, 131,072 nodes, 93 and 97 us
-// (147 and 137).  Bound by the latency of the tiles' loads, 3.9 of 6.7 TB/s at the large end: the
-// next eight chunks are asked for ahead, four are read at once; more warps with fewer loads
+// (147 and 137).  Bound by memory at the large end, 36.4 GB (25.6 of entries, the rest the padding of
+// rows to four and columns to eight) at 5.55 of 6.68 TB/s, by the latency of the tiles' loads below:
+// the next eight chunks are asked for ahead, four are read at once; more warps with fewer loads
 // each were slower (6.9 ms with two chunks at once, 8.8 with 24 warps an SM).
 //
 // The transposed rows (K^T tau)_i read the same tiles: near pairs are symmetric (b's columns
@@ -867,7 +868,7 @@ k_rows_t_out(int64_t nitem, const RowItem *__restrict__ items, const double *__r
 // (P terms) through the stored columns, a warp per row block, Re(b_l u^l) as -pi times column
 // 2 l against -Im b_l and column 2 l + 1 against Re b_l; then the node's direct centres
 // (partial), the centres summed directly everywhere and the constants.
-// Bound by the columns' bytes: 1.9 ms at 16.8 million nodes, 4.2 as a Horner chain a node
+// Bound by the columns' bytes: 1.9 ms at 16.8 million nodes (10.2 GB at 5.3 TB/s), 4.2 as a Horner chain a node
 // (four double multiply-adds a term).
 __global__ void __launch_bounds__(128, 4)
 k_rows_mp(int64_t nitem, const RowItem *__restrict__ items, const double *__restrict__ rows, int P,
